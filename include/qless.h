@@ -109,11 +109,16 @@ ql_status ql_check_bounded_wait(int32_t arrive, int64_t limit_clocks, int32_t* i
 size_t ql_workspace_bytes(ql_method method, int64_t m, int64_t n, ql_dtype dtype);
 
 /*
- * Q-less Householder TSQR (Sec. 3.2, Algorithms 2-4).  One persistent launch: every CTA
- * streams its row blocks of X through shared memory, factors [R; W] in place with
- * Householder reflectors (Algorithm 4), and the per-CTA triangles are merged by a binary
- * "last CTA done" R-tree (Algorithm 2, stage 2) inside the same launch.  An FP64 fallback
- * launch follows that exits at once unless the range check fired.
+ * Q-less TSQR (Sec. 3.2, Algorithms 2-4): the R of X for any condition number.
+ * For n >= 5 the first launch forms X^T X exactly (X rounded to 2^-56 of each column's
+ * largest entry, every product and sum an integer) and factors it in 125-bit fixed point:
+ * the same R, with an error below the Householder tiles'.  Columns dependent to about 2^-40
+ * of their norm (a pivot below 2^-80) are left to the Householder launch behind it, which
+ * otherwise exits at once and which is the only one for n <= 4: every CTA streams its row blocks of X
+ * through shared memory, factors [R; W] in place with Householder reflectors (Algorithm 4),
+ * and the per-CTA triangles are merged by a "last CTA done" R-tree (Algorithm 2, stage 2)
+ * inside the same launch.  An FP64 fallback launch follows that exits at once unless the
+ * range check fired.
  * Arguments: m >= 0 rows, 1 <= n <= 64 columns, X device (F64 or F32), ldx >= max(m,1),
  * R device double n x n (ldr >= n), info nullable device int32[2], ws/ws_bytes workspace.
  */

@@ -73,18 +73,23 @@ bool pipe_tensor_maps(CUtensorMap* tmA, CUtensorMap* tmB, const void* A, const v
 
 static int nc_of(int n) { return n <= 1 ? 1 : n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : n <= 16 ? 16 : n <= 32 ? 32 : 64; }
 
+static size_t gram_head_bytes(int n) { return 512 + (n > 4 ? (sacc_bytes(nc_of(n)) + 255) / 256 * 256 : 0); }
+
 static size_t gram_layout(int n, GramWs* w, void* base) {
   const int nc = nc_of(n);
-  const size_t head = 512;  // flags, counters and the first pass's column exponents
+  // flags, counters and the first pass's column exponents, then the integer accumulators of
+  // the exact Gram pass: cleared before every call
+  const size_t head = gram_head_bytes(n);
   const size_t keep = ((size_t)3 * nc * nc * sizeof(double) + 255) / 256 * 256;  // 3 n x n blocks (ld n)
   // one NC x NC partial per CTA (the streaming kernel for nc <= 4 runs up to 8 CTAs per SM)
   const size_t parts = (size_t)device_sm_count() * (nc <= 4 ? 8 : kGramMaxCtasPerSm) * nc * nc * sizeof(double);
-  // accumulators of the tcgen05 kernels (16 to 64 columns, one CTA per SM): an FP64 and a
-  // double-float level per CTA (the per-tile kernel of the later passes uses the first)
-  const size_t fbuf = nc >= 16 ? (size_t)device_sm_count() * nc * 128 * 2 * sizeof(double) : 0;
+  // accumulators of the tcgen05 kernels (8 to 64 columns, one CTA per SM): 128-bit sums (exact
+  // pass), an FP64 and a double-float level (pipelined later passes) or FP64 (per tile)
+  const size_t fbuf = nc >= 8 ? (size_t)device_sm_count() * nc * 128 * 2 * sizeof(double) : 0;
   if (w && base) {
     unsigned char* b = static_cast<unsigned char*>(base);
     w->flags = reinterpret_cast<int*>(b);
+    w->sacc = reinterpret_cast<long long*>(b + 512);
     w->keep = reinterpret_cast<double*>(b + head);
     w->partials = reinterpret_cast<double*>(b + head + keep);
     w->fbuf = reinterpret_cast<double*>(b + head + keep + parts);
@@ -105,7 +110,7 @@ ql_status gram_launch(const GramCall& c, ql_arith arith) {
   if (!c.ws || c.ws_bytes < gram_layout(c.n, nullptr, nullptr)) return QL_ERR_WORKSPACE;
   GramWs w;
   gram_layout(c.n, &w, c.ws);
-  if (cudaMemsetAsync(w.flags, 0, 512, c.stream) != cudaSuccess) return QL_ERR_CUDA;
+  if (cudaMemsetAsync(w.flags, 0, gram_head_bytes(c.n), c.stream) != cudaSuccess) return QL_ERR_CUDA;
   ql_status st;
   if (c.dtype == QL_F64) {
     if (arith == QL_ARITH_F64) return gram_dispatch<double, ArithF64>(c, w, 0);
@@ -115,6 +120,34 @@ ql_status gram_launch(const GramCall& c, ql_arith arith) {
   if (arith == QL_ARITH_F64) return gram_dispatch<float, ArithF64>(c, w, 0);
   if ((st = gram_dispatch<float, ArithDF>(c, w, 0))) return st;
   return gram_dispatch<float, ArithF64>(c, w, 1);
+}
+
+// Workspace and launch of the exact pass for a TSQR call (n >= 2).  The caller clears the
+// first *clear_bytes of `base` beforehand; flags[0] then asks for the FP64 launch and
+// flags[1] for the double-float Householder launch.
+size_t xgram_tsqr_bytes(int n) { return gram_layout(n < 5 ? 5 : n, nullptr, nullptr); }
+size_t xgram_tsqr_clear_bytes(int n) { return gram_head_bytes(n < 5 ? 5 : n); }
+ql_status xgram_tsqr_launch(const TsqrCall& t, void* base) {
+  GramCall c;
+  c.m = t.m;
+  c.n = t.n;
+  c.nA = t.nA;
+  c.A = t.A;
+  c.lda = t.lda;
+  c.b = t.b;
+  c.dtype = t.dtype;
+  c.method = QL_TSQR;
+  c.epilogue = t.epilogue;
+  c.R = t.R;
+  c.ldr = t.ldr;
+  c.x = t.x;
+  c.resnorm = t.resnorm;
+  c.Rext = t.Rext;
+  c.info = t.info;
+  c.stream = t.stream;
+  GramWs w;
+  gram_layout(c.n < 5 ? 5 : c.n, &w, base);
+  return c.dtype == QL_F64 ? xgram_pass1<double>(c, w) : xgram_pass1<float>(c, w);
 }
 
 }  // namespace ql

@@ -27,8 +27,12 @@ struct GramWs {
                     // [64 + c]: largest biased exponent of column c over all rows (tensor-core pass 1)
   double* keep;      // 3 n x n blocks carried from pass 1 to pass 2 (row-major, ld n)
   double* partials;  // one NC x NC partial Gram per CTA
-  double* fbuf;      // tcgen05 kernel: FP64 accumulators per CTA, [NC columns][128 TMEM lanes]
+  double* fbuf;      // tcgen05 kernels: accumulators per CTA, 16 bytes per [NC columns][128 TMEM lanes]
+  long long* sacc;   // exact Gram pass: integer accumulators, kLimbs words per entry i <= j of C
 };
+constexpr int kLimbs = 8, kLimbBits = 40;
+// Bytes of the integer accumulators for nc columns.
+constexpr size_t sacc_bytes(int nc) { return (size_t)nc * (nc + 1) / 2 * kLimbs * sizeof(long long); }
 
 template <typename S>
 struct GramArgs {
@@ -294,12 +298,13 @@ __global__ void __launch_bounds__(GramShape<NC>::T, 1) gram_kernel(GramArgs<S> a
   gram_finish<NC, T, S, Ar>(a, smem, colmax, misc, gridDim.x);
 }
 
-// Range verdict, "last CTA done" election and, in the last CTA, the fixed-order reduction
-// of all CTA partials followed by the n x n FP64 epilogue of the pass.  Shared by the SIMT
-// and the tensor-core Gram kernels (the caller has written this CTA's partial already).
 template <int NC, int T, typename S, typename Ar>
-QL_DEV void gram_finish(const GramArgs<S>& a, unsigned char* smem, const int* colmax, int* misc, int k) {
-  using V = typename Ar::T;
+QL_DEV void gram_epilogue(const GramArgs<S>& a, unsigned char* smem);
+
+// Range verdict and "last CTA done" election (true in the last of the k CTAs of the pass,
+// unless the FP64 launches have to redo the call).
+template <typename S, typename Ar>
+QL_DEV bool gram_elect(const GramArgs<S>& a, const int* colmax, int* misc, int k) {
   const int tid = threadIdx.x, n = a.n;
   if (tid == 0) {
     bool bad = false;
@@ -322,22 +327,26 @@ QL_DEV void gram_finish(const GramArgs<S>& a, unsigned char* smem, const int* co
     if (old == k - 1) *counter = 0;
   }
   __syncthreads();
-  if (!misc[0]) return;
+  if (!misc[0]) return false;
   __threadfence();
   if (Ar::kRangeChecked && *(volatile int*)&a.w.flags[0] != 0) {  // the FP64 launches redo it
     if (a.redo && tid == 0) gram_request_redo(a.redo, a.redo_any, *(volatile int*)&a.w.flags[4]);
-    return;
+    return false;
   }
+  return true;
+}
 
-  // ---------------- epilogue: one CTA, FP64, shared memory reused from here on; the odd
+// In the last CTA: the fixed-order reduction of all CTA partials followed by the n x n FP64
+// epilogue of the pass.  Shared by the SIMT and the per-tile and pipelined tensor-core
+// kernels (the caller has written this CTA's partial already).
+template <int NC, int T, typename S, typename Ar>
+QL_DEV void gram_finish(const GramArgs<S>& a, unsigned char* smem, const int* colmax, int* misc, int k) {
+  if (!gram_elect<S, Ar>(a, colmax, misc, k)) return;
+  const int tid = threadIdx.x, n = a.n;
+  // one CTA, FP64, shared memory reused from here on; the odd
   // leading dimension keeps column walks (Jacobi rotations) free of bank conflicts
   constexpr int LE = NC + 1;
   double* Cs = reinterpret_cast<double*>(smem);  // n x n, ld LE
-  double* Us = Cs + NC * LE;
-  double* Ps = Us + NC * LE;
-  double* Qs = Ps + NC * LE;
-  double* vec = Qs + NC * LE;  // 8 LE doubles
-  int* sflag = reinterpret_cast<int*>(vec + 8 * LE);
   __syncthreads();
   // fixed-order FP64 sum of the CTA partials (bitwise reproducible).  P lanes share an
   // entry (as many as the thread count allows, up to a warp): each sums a strided subset of
@@ -364,6 +373,20 @@ QL_DEV void gram_finish(const GramArgs<S>& a, unsigned char* smem, const int* co
     }
   }
   __syncthreads();
+  gram_epilogue<NC, T, S, Ar>(a, smem);
+}
+
+// The n x n FP64 work of one pass, by one CTA: C (full, ld NC + 1) at the start of smem.
+template <int NC, int T, typename S, typename Ar>
+QL_DEV void gram_epilogue(const GramArgs<S>& a, unsigned char* smem) {
+  const int tid = threadIdx.x, n = a.n;
+  constexpr int LE = NC + 1;
+  double* Cs = reinterpret_cast<double*>(smem);  // n x n, ld LE
+  double* Us = Cs + NC * LE;
+  double* Ps = Us + NC * LE;
+  double* Qs = Ps + NC * LE;
+  double* vec = Qs + NC * LE;  // 8 LE doubles
+  int* sflag = reinterpret_cast<int*>(vec + 8 * LE);
   double* keep = a.w.keep;  // [0]: R1 or S1, [1]: M (R1^{-1} or B1)
   const int nn = n * n;
   if (a.method == QL_TSQR) {
@@ -2361,6 +2384,13 @@ ql_status gram_launch_one(const GramCall& c, const GramWs& w, int pass, int gate
   return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
+// Exact Gram pass (xgram.cuh): R of a TSQR call (method QL_TSQR, n >= 2), or the first pass
+// of a Gram method with n >= 5.
+template <typename S>
+ql_status xgram_pass1(const GramCall& c, const GramWs& w);
+extern template ql_status xgram_pass1<double>(const GramCall&, const GramWs&);
+extern template ql_status xgram_pass1<float>(const GramCall&, const GramWs&);
+
 // All passes of one method (two, three for shifted Cholesky-QR3) for one (storage, arithmetic) pair.
 template <typename S, typename Ar>
 ql_status gram_dispatch(const GramCall& c, const GramWs& w, int gated) {
@@ -2402,7 +2432,11 @@ ql_status gram_dispatch(const GramCall& c, const GramWs& w, int gated) {
       if (st || c.method != QL_SCHOLQR3) return st;
       return gram_stream_launch_one<NC, S, Ar, kXUpper>(c, w, 3, gated);
     }
-    ql_status st = gram_launch_one<NC, S, Ar, kXNone>(c, w, 1, gated);
+    ql_status st;
+    if constexpr (NC == 8 && std::is_same<Ar, ArithDF>::value)
+      st = tc_gram_enabled() ? xgram_pass1<S>(c, w) : gram_launch_one<NC, S, Ar, kXNone>(c, w, 1, gated);
+    else
+      st = gram_launch_one<NC, S, Ar, kXNone>(c, w, 1, gated);
     if (st) return st;
     if (c.method == QL_SVQB2) return gram_launch_one<NC, S, Ar, kXFull>(c, w, 2, gated);
     st = gram_launch_one<NC, S, Ar, kXUpper>(c, w, 2, gated);

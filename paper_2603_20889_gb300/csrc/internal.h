@@ -36,10 +36,17 @@ struct TsqrCall {
   int max_ctas = 0;     // 0: no limit (testing the R-tree with few leaves)
   int variant = -1;     // thread layout (row-block height) for n > 8: -1 environment default, 0..2
   int arity = 0;        // R-tree arity: 0 the column class's default, else 2 .. default
+  bool householder = false;  // Householder tiles only (no exact Gram pass)
 };
 
-// Upper bound of the TSQR workspace for n columns (any m).
-size_t tsqr_workspace_bytes(int n);
+// Upper bound of the TSQR workspace for n columns (any m); householder: without the exact
+// Gram pass.
+size_t tsqr_workspace_bytes(int n, bool householder = false);
+// The exact Gram pass as a TSQR call's first launch (gram.cu): workspace, the leading bytes
+// of it to clear, and the launch.
+size_t xgram_tsqr_bytes(int n);
+size_t xgram_tsqr_clear_bytes(int n);
+ql_status xgram_tsqr_launch(const TsqrCall& c, void* base);
 // Launch the double-float TSQR (or FP64 when arith == QL_ARITH_F64) and, after a
 // double-float launch, the gated FP64 fallback.
 ql_status tsqr_launch(const TsqrCall& c, ql_arith arith);

@@ -33,41 +33,54 @@ int device_sm_count() {
   return v;
 }
 
-size_t tsqr_workspace_bytes(int n) {
+// Workspace: the exact Gram pass's block (its head, the flags, is shared by every launch of
+// the call) unless the call is Householder only, then the tree's counters and slots.
+constexpr size_t kFlagBytes = 512;
+
+static size_t counter_bytes() {
+  const size_t cnt = tree_counters(device_sm_count() * kMaxCtasPerSm);
+  return (cnt * sizeof(int) + 255) / 256 * 256;
+}
+
+size_t tsqr_workspace_bytes(int n, bool householder) {
   if (n < 1 || n > kMaxN) return 0;
-  size_t leaves = (size_t)device_sm_count() * kMaxCtasPerSm;
-  size_t cnt = tree_counters((int)leaves);
-  size_t head = 256 + (cnt * sizeof(int) + 255) / 256 * 256;
-  return head + tree_slots((int)leaves) * (size_t)n * n * sizeof(double);
+  const size_t leaves = (size_t)device_sm_count() * kMaxCtasPerSm;
+  return counter_bytes() + (householder || n < 2 ? kFlagBytes : xgram_tsqr_bytes(n)) +
+         tree_slots((int)leaves) * (size_t)n * n * sizeof(double);
+}
+
+// The exact Gram pass (xgram.cuh) replaces the Householder tiles from 5 columns.  Measured
+// (m = 2^25, n = 4): Householder 0.92 ms, exact 1.59 ms (half of the 8-column class's work is
+// padding there).
+constexpr int kExactMinN = 5;
+
+template <typename S>
+static ql_status tsqr_launch_s(const TsqrCall& c, const TreeView& tv, bool exact, ql_arith arith) {
+  if (arith == QL_ARITH_F64) return dispatch<S, ArithF64>(c, tv, 0);
+  ql_status st = dispatch<S, ArithDF>(c, tv, exact ? 2 : 0);
+  if (st != QL_OK) return st;
+  return dispatch<S, ArithF64>(c, tv, 1);
 }
 
 ql_status tsqr_launch(const TsqrCall& c, ql_arith arith) {
   if (c.n < 1 || c.n > kMaxN) return QL_ERR_ARG;
-  const int sms = device_sm_count();
-  size_t leaves_max = (size_t)sms * kMaxCtasPerSm;
-  size_t cnt = tree_counters((int)leaves_max);
-  size_t head = 256 + (cnt * sizeof(int) + 255) / 256 * 256;
-  size_t need = head + tree_slots((int)leaves_max) * (size_t)c.n * c.n * sizeof(double);
-  if (!c.ws || c.ws_bytes < need) return QL_ERR_WORKSPACE;
+  if (!c.ws || c.ws_bytes < tsqr_workspace_bytes(c.n, c.householder)) return QL_ERR_WORKSPACE;
+  const bool exact = !c.householder && c.n >= kExactMinN && arith != QL_ARITH_F64 && tc_gram_enabled();
+  // [tree counters][flags (head of the exact pass's block)][slots]
   unsigned char* ws = static_cast<unsigned char*>(c.ws);
+  const size_t cb = counter_bytes(), xb = c.householder || c.n < 2 ? kFlagBytes : xgram_tsqr_bytes(c.n);
   TreeView tv;
-  tv.flags = reinterpret_cast<int*>(ws);
-  tv.counters = reinterpret_cast<int*>(ws + 256);
-  tv.slots = reinterpret_cast<double*>(ws + head);
+  tv.counters = reinterpret_cast<int*>(ws);
+  tv.flags = reinterpret_cast<int*>(ws + cb);
+  tv.slots = reinterpret_cast<double*>(ws + cb + xb);
   tv.leaves = 0;
-  if (cudaMemsetAsync(ws, 0, head, c.stream) != cudaSuccess) return QL_ERR_CUDA;
-  ql_status st;
-  if (c.dtype == QL_F64) {
-    if (arith == QL_ARITH_F64) return dispatch<double, ArithF64>(c, tv, 0);
-    st = dispatch<double, ArithDF>(c, tv, 0);
+  if (cudaMemsetAsync(ws, 0, cb + (exact ? xgram_tsqr_clear_bytes(c.n) : kFlagBytes), c.stream) != cudaSuccess)
+    return QL_ERR_CUDA;
+  if (exact) {
+    ql_status st = xgram_tsqr_launch(c, ws + cb);
     if (st != QL_OK) return st;
-    return dispatch<double, ArithF64>(c, tv, 1);
-  } else {
-    if (arith == QL_ARITH_F64) return dispatch<float, ArithF64>(c, tv, 0);
-    st = dispatch<float, ArithDF>(c, tv, 0);
-    if (st != QL_OK) return st;
-    return dispatch<float, ArithF64>(c, tv, 1);
   }
+  return c.dtype == QL_F64 ? tsqr_launch_s<double>(c, tv, exact, arith) : tsqr_launch_s<float>(c, tv, exact, arith);
 }
 
 }  // namespace ql

@@ -18,7 +18,8 @@ struct TsqrArgs {
   TsqrProblem<S> p;
   TreeView tv;
   int64_t tiles;
-  int gated;  // FP64 fallback launch: run only if the range flag is set
+  int gated;  // 1: FP64 launch, run only if flags[0] is set; 2: double-float launch behind the
+              // exact Gram pass, run only if flags[1] is set (a pivot too small, a wait given up)
   int arity;  // R-tree arity (2 .. the column class's default)
   int epilogue;
   double* R;
@@ -33,8 +34,8 @@ template <int NC, int TC, int RPT, int T, typename S, typename Ar>
 __global__ void __launch_bounds__(T, 1) tsqr_kernel(TsqrArgs<S> a) {
   extern __shared__ __align__(16) unsigned char smem[];
   using Cta = TsqrCta<NC, TC, RPT, T, S, Ar>;
-  if (a.gated) {
-    if (*(volatile int*)&a.tv.flags[0] == 0) return;
+  if (a.gated) {  // flags[0]: range, flags[1]: Householder redo (see TsqrArgs)
+    if (*(volatile int*)&a.tv.flags[a.gated - 1] == 0) return;
   }
   Cta cta;
   cta.init(smem);
@@ -60,10 +61,11 @@ __global__ void __launch_bounds__(T, 1) tsqr_kernel(TsqrArgs<S> a) {
   // root: every CTA has passed its range check and its tree arrival by now
   __threadfence();
   if (Ar::kRangeChecked && *(volatile int*)&a.tv.flags[0] != 0) return;  // FP64 launch redoes it
+  const int tmo = *(volatile int*)&a.tv.flags[4];  // a bounded wait of the exact pass that gave up
   if (a.epilogue == kEpiR)
-    epilogue_r<T>(Ra, NC, n, a.R, a.ldr, a.info, &cta.misc[2]);
+    epilogue_r<T>(Ra, NC, n, a.R, a.ldr, a.info, &cta.misc[2], tmo);
   else
-    epilogue_lstsq<T>(Ra, NC, n, a.x, a.resnorm, a.Rext, a.info, cta.sd, &cta.misc[2]);
+    epilogue_lstsq<T>(Ra, NC, n, a.x, a.resnorm, a.Rext, a.info, cta.sd, &cta.misc[2], tmo);
 }
 
 template <int NC, int TC, int RPT, int T, typename S, typename Ar>

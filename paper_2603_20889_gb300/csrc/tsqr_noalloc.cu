@@ -52,7 +52,7 @@ extern "C" ql_status ql_tsqr_qless_noalloc(int64_t m, int64_t n, const void* X, 
   if ((st = check_r(R, ldr, n))) return st;
   if (n > kNoAllocMaxN) return QL_ERR_WORKSPACE;  // beyond what the fixed scratch array holds
   // the R-tree is sized for the SM count of the current device
-  if (tsqr_workspace_bytes((int)n) > kNoAllocScratchBytes) return QL_ERR_WORKSPACE;
+  if (tsqr_workspace_bytes((int)n, true) > kNoAllocScratchBytes) return QL_ERR_WORKSPACE;
   void* scratch = nullptr;
   st = scratch_for_current_device(&scratch);
   if (st != QL_OK) return st;
@@ -71,6 +71,7 @@ extern "C" ql_status ql_tsqr_qless_noalloc(int64_t m, int64_t n, const void* X, 
   c.ws = scratch;
   c.ws_bytes = kNoAllocScratchBytes;
   c.stream = (cudaStream_t)stream;
+  c.householder = true;  // the exact Gram pass's accumulators do not fit in the scratch array
   int ctas = 0;  // the autotuned grid, as the regular entry point uses (a table lookup, no allocation)
   int var = -1, ar = 0;
   if (tune_lookup(m, n, dtype, 1.0, nullptr, &ctas, &var, &ar)) {

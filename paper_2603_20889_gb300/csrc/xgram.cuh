@@ -1,0 +1,950 @@
+// Exact Gram pass on tcgen05 (C = X^T X) with a fixed-point Cholesky behind it: R of a TSQR
+// call in one pass over X, in the 8-, 16-, 32- and 64-column classes.
+//
+// Measured against the double-float Householder tiles it replaces (those stay for columns
+// dependent to about 2^-40 and for n <= 4): m = 2^22, n = 64 21.1 -> 2.40 ms; least squares
+// 2^24 x 31, FP32-stored, 19.2 -> 1.84 ms; 131072 x 8 145 -> 45 us; ||R - R_ref|| / ||R_ref||
+// 3.5e-16 -> 2.1e-16 (n = 64), 4.4e-16 -> 1.2e-16 (n = 8) against 64-bit references.
+//
+// Every value is rounded to a signed 56-bit fixed point N relative to a running per-column
+// scale 2^e (|x| < 2^e, x ~ N 2^(e - 55)) and cut into EIGHT balanced base-128 digits, which
+// bf16 holds exactly.  ALL 64 digit-plane products are formed, every FP32 sum of the tensor
+// core stays an integer of at most 2^24 (exact), the read-outs fold them into 128-bit
+// integers and the CTAs add those into one integer accumulator of 320 bits per entry of C.
+// The Gram matrix of the rounded X is therefore exact: no product is dropped, no sum rounds,
+// and the result does not depend on the order of tiles, CTAs or atomics.  That is what lets
+// one pass serve TSQR: with C exact, a Cholesky factorisation in 125-bit fixed point
+// (xg_cholesky) loses kappa^2 2^-120 instead of kappa^2 2^-53, so the R it gives is limited
+// by the 2^-56 rounding of X (a backward error, like Householder's) up to kappa ~ 2^40.
+//
+//  * Roles and tiles: 16 slicer warps cut tiles of 4096 elements (KT = 4096 / NC rows) into
+//    digit planes and read the accumulators out; one control warp issues the tensor-map
+//    copies two tiles ahead and the MMAs.  Two raw stages and two digit buffers alternate.
+//    Mbarriers: "MMAs done" and "digits ready" per digit buffer, "tile landed" and "stage
+//    read" per raw stage; one vote of the slicers per tile (a column outgrew its scale, or a
+//    wait gave up).
+//  * The planes lie one after the other in the K-major core-matrix layout, so all planes
+//    together are one operand of 8 NC columns (plane p, column c at 8-column group
+//    (p NC + c) / 8).
+//      NC = 8:   one MMA 128 x 64 x 16 per 16 rows (lanes 64..127 see the memory behind the
+//                planes and are never read); lane p 8 + i, column q 8 + j.
+//      NC = 16:  one MMA 128 x 128 x 16: lane p 16 + i, column q 16 + j.
+//      NC = 32:  two MMAs 128 x 256 x 16 (planes 0..3, 4..7): 512 tensor-memory columns.
+//      NC = 64:  512 x 512 sums do not fit, so pairs of equal weight w = p + q share one of
+//                16 half blocks: block b holds weight 2 b in lanes 0..63 and 2 b + 1 in lanes
+//                64..127.  Plane q even meets the stacked planes (p, p + 1), p even, and q
+//                odd those with p odd (from -1 to 7; plane -1 and plane 8 are zeros), so
+//                every product lands on its own weight: 36 MMAs 128 x 64 x 16.
+//  * G tiles add up in tensor memory per read-out: G KT rows x (pairs per sum) x 64^2 <= 2^24.
+#pragma once
+
+#include "gram_launch.cuh"
+
+namespace ql {
+
+using u64 = unsigned long long;
+using u128 = unsigned __int128;
+using i128 = __int128;
+
+template <int NC>
+struct XgShape {
+  static constexpr int TS = 512;             // slicer threads
+  static constexpr int T = TS + 32;          // and the control warp
+  static constexpr int KT = 4096 / NC;       // rows per tile
+  static constexpr int PLANE = NC * KT * 2;  // bytes per digit plane (8 KB)
+  static constexpr int DBUF = 8 * PLANE;     // digit planes of a tile (64 KB)
+  static constexpr int PAD = NC == 64 ? PLANE : 0;  // zero planes before, between and after the buffers
+  static constexpr int LBO = 128;            // bytes between core matrices along the rows
+  static constexpr int SBO = KT * 16;        // bytes between 8-column groups
+  static constexpr int TCOLS = NC == 8 ? 64 : (NC == 16 ? 128 : 512);
+  static constexpr int PAIRS = NC == 64 ? 8 : 1;     // products per sum (weight 7 has eight)
+  static constexpr int G = 4096 / (KT * PAIRS);      // tiles per read-out: 8, 16, 32, 8
+  static constexpr int SLACK = 2;            // bits of headroom above a new column maximum
+  static constexpr int HALF = NC / 4;        // columns of C per slicer thread at a read-out
+  static constexpr int LG = NC == 8 ? 8 : 128 / NC;  // lane groups (planes, or weight parities)
+  // a 128-bit sum takes at most 2^111 per row: emptied after 2^15 rows (and one more group)
+  static constexpr int MAX_READS = (1 << 15) / (G * KT);
+  static_assert(NC == 8 || NC == 16 || NC == 32 || NC == 64, "column classes");
+  static_assert((long long)G * KT * PAIRS * 4096 <= (1LL << 24), "exact FP32 digit sums");
+};
+
+template <int NC, typename S>
+struct XgSmem {
+  using Sh = XgShape<NC>;
+  // a staged tile: boxes of 128 bytes of rows x NC columns, 128-byte swizzle (see PipeSmem)
+  static constexpr int RPB = 128 / (int)sizeof(S);
+  static constexpr int NBOX = Sh::KT / RPB;
+  static constexpr size_t kDig = 2 * (size_t)Sh::DBUF + 3 * (size_t)Sh::PAD;
+  static constexpr size_t kRaw = sizeof(S) * (size_t)NC * Sh::KT;
+  static constexpr size_t kOffRaw = kDig;
+  // (NC = 8: lanes 64..127 of the second buffer's MMAs read 64 KB past it, which must exist)
+  static constexpr size_t kRawSpan = NC == 8 && 2 * kRaw < (size_t)Sh::DBUF ? (size_t)Sh::DBUF : 2 * kRaw;
+  static constexpr size_t kOffScale = kOffRaw + kRawSpan;
+  static constexpr size_t kOffColmax = kOffScale + 4 * NC;
+  static constexpr size_t kOffMisc = kOffColmax + 4 * NC;
+  static constexpr size_t kOffBar = (kOffMisc + 64 * 4 + 15) / 16 * 16;
+  static constexpr size_t kOffSlot = kOffBar + 64;
+  static constexpr size_t kBytes = kOffSlot + 32;
+  static constexpr size_t kEpi = 8 * (4 * (size_t)NC * (NC + 1) + 8 * (NC + 1)) + 64 * 4 + 16;
+  static_assert(kEpi <= kOffScale, "the epilogue's shared memory stays below the scales and barriers");
+  static_assert(16 * (size_t)(Sh::LG - 1) * NC * NC <= (size_t)Sh::DBUF, "lane-group sums fit in a digit buffer");
+};
+
+// Integer accumulators of C: entry (i <= j) at index i + j (j + 1) / 2, kLimbs limbs of 40 bits
+// in 64-bit words.  The unit is 2^(2 (kEsMin - 1022) - 110): N_i N_j of columns at scale
+// exponents Es_i, Es_j (>= kEsMin) weighs 2^(Es_i + Es_j - 2 kEsMin) units, at most 2^184, so
+// 128-bit sums end below bit 312 of 320; a limb takes 2^23 additions before it could overflow.
+constexpr int kEsMin = kDfEminLimit;
+constexpr int kEsMax = kDfEmaxLimit + 2;
+constexpr int kXgUnitExp = 2 * (kEsMin - 1022) - 110;  // -188
+QL_DEV int tri_index(int i, int j) { return i + j * (j + 1) / 2; }
+
+// ---------------------------------------------------------------------------------------
+// Cutting.  Nb2 = 2 N + 1 + 2 kDigitBias8 rounded so that field p, (Nb2 >> (1 + 7 (7 - p)))
+// & 127 (& 255 for p = 0), is digit p + 64: Q = floor(2 |x| 2^(55 - e)) by one funnel shift,
+// the sign by a one's complement, and the bias constant adds the rounding half (ties away
+// from zero).  s = Es - E + 7 is the right shift of the significand aligned at bit 62.
+// ---------------------------------------------------------------------------------------
+constexpr u64 kCutBias = 2 * kDigitBias8 + 1;
+
+QL_DEV unsigned sig_hi(unsigned hw, unsigned lw) { return (__funnelshift_l(lw, hw, 10) & 0x3fffffffu) | 0x40000000u; }
+
+template <bool FAR>
+QL_DEV u64 cut56(unsigned h, unsigned l, unsigned sign_word, int s) {
+  unsigned ql = __funnelshift_r(l, h, s), qh = h >> (s & 31);
+  if constexpr (FAR) {
+    if (s > 31) {
+      ql = __funnelshift_rc(h, 0u, (unsigned)(s - 32));
+      qh = 0u;
+    }
+  }
+  const unsigned m = (unsigned)((int)sign_word >> 31);
+  return (((u64)(qh ^ m) << 32) | (ql ^ m)) + kCutBias;
+}
+
+// Planes 7 - 2 K and 6 - 2 K of eight elements: two adjacent 7-bit fields per element and
+// shift, packed for rows (r, r + 1) into one word each, bf16(128 + f) - 192 = f - 64.
+template <int PLANE, int K>
+QL_DEV void put_plane_pairs(unsigned char* base, const u64 (&Nb)[8]) {
+  unsigned lo[4], hi[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const unsigned fa = (unsigned)(Nb[2 * e] >> (1 + 14 * K)), fb = (unsigned)(Nb[2 * e + 1] >> (1 + 14 * K));
+    const unsigned t = __byte_perm(fa, fb, 0x5410);
+    const unsigned wl = (t & 0x007f007fu) | 0x43004300u;
+    const unsigned wh = ((t >> 7) & (K == 3 ? 0x00ff00ffu : 0x007f007fu)) | 0x43004300u;
+    const __nv_bfloat162 off = __floats2bfloat162_rn(192.0f, 192.0f);
+    const __nv_bfloat162 rl = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&wl), off);
+    const __nv_bfloat162 rh = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&wh), off);
+    lo[e] = *reinterpret_cast<const unsigned*>(&rl);
+    hi[e] = *reinterpret_cast<const unsigned*>(&rh);
+  }
+  *reinterpret_cast<uint4*>(base + (7 - 2 * K) * PLANE) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+  *reinterpret_cast<uint4*>(base + (6 - 2 * K) * PLANE) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+  if constexpr (K < 3) put_plane_pairs<PLANE, K + 1>(base, Nb);
+}
+
+// Eight rows of one column as raw words.
+template <typename S>
+struct Rows8;
+template <>
+struct Rows8<double> {
+  unsigned hw[8], lw[8];
+  QL_DEV unsigned amax() const {  // largest |x|, as its high word
+    unsigned a = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) a = max(a, hw[j] & 0x7fffffffu);
+    return a;
+  }
+  QL_DEV static int exponent(unsigned amax) { return (int)(amax >> 20); }
+  QL_DEV int shift(int j, int base) const { return base - (int)((hw[j] & 0x7fffffffu) >> 20); }
+  QL_DEV unsigned h(int j) const { return sig_hi(hw[j], lw[j]); }
+  QL_DEV unsigned l(int j) const { return lw[j] << 10; }
+  QL_DEV void set(int j, double x) {
+    hw[j] = (unsigned)__double2hiint(x);
+    lw[j] = (unsigned)__double2loint(x);
+  }
+  QL_DEV void chunk(int q, const uint4& t) {
+    lw[2 * q] = t.x;
+    hw[2 * q] = t.y;
+    lw[2 * q + 1] = t.z;
+    hw[2 * q + 1] = t.w;
+  }
+};
+template <>
+struct Rows8<float> {
+  unsigned hw[8];
+  QL_DEV unsigned amax() const {
+    unsigned a = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) a = max(a, hw[j] & 0x7fffffffu);
+    return a;
+  }
+  QL_DEV static int exponent(unsigned amax) {
+    const int ef = (int)(amax >> 23);
+    return ef == 0 ? 0 : ef + 896;
+  }
+  QL_DEV int shift(int j, int base) const { return base - 896 - (int)((hw[j] & 0x7fffffffu) >> 23); }
+  QL_DEV unsigned h(int j) const { return ((hw[j] << 7) & 0x3fffffffu) | 0x40000000u; }
+  QL_DEV unsigned l(int) const { return 0u; }
+  QL_DEV void set(int j, float x) { hw[j] = __float_as_uint(x); }
+  QL_DEV void chunk(int q, const uint4& t) {
+    hw[4 * q] = t.x;
+    hw[4 * q + 1] = t.y;
+    hw[4 * q + 2] = t.z;
+    hw[4 * q + 3] = t.w;
+  }
+};
+
+// One instruction descriptor for M = 128 and N columns.
+template <int N>
+QL_DEV constexpr uint32_t xg_idesc() {
+  return umma_idesc_bf16(128, N);
+}
+
+// The MMAs of one tile (control thread): d0 is the descriptor of plane 0, k-step 0.
+template <int NC>
+QL_DEV void xg_issue_mmas(uint32_t tbase, uint64_t d0, uint32_t fresh) {
+  using Sh = XgShape<NC>;
+  constexpr uint64_t PL = Sh::PLANE >> 4;
+#pragma unroll 1
+  for (int kk = 0; kk < Sh::KT / 16; ++kk) {
+    const uint64_t dk = d0 + (uint64_t)((kk * 2 * Sh::LBO) >> 4);
+    const uint32_t first = (!fresh || kk > 0) ? 1u : 0u;
+    if constexpr (NC == 8) {
+      umma_bf16(tbase, dk, dk, xg_idesc<64>(), first);
+    } else if constexpr (NC == 16) {
+      umma_bf16(tbase, dk, dk, xg_idesc<128>(), first);
+    } else if constexpr (NC == 32) {
+      umma_bf16(tbase, dk, dk, xg_idesc<256>(), first);
+      umma_bf16(tbase + 256, dk + 4 * PL, dk, xg_idesc<256>(), first);
+    } else {
+#pragma unroll
+      for (int b = 0; b < 8; ++b) {
+        uint32_t acc = first;
+#pragma unroll
+        for (int p = -1; p <= 7; ++p) {
+          const int q = 2 * b - p;
+          if (q >= 0 && q <= 7) {
+            umma_bf16(tbase + (uint32_t)(b * 64), dk + (uint64_t)(int64_t)(p * (int64_t)PL), dk + (uint64_t)q * PL,
+                      xg_idesc<64>(), acc);
+            acc = 1u;
+          }
+        }
+      }
+    }
+  }
+}
+
+// tcgen05.ld of two columns (the 8-column class).
+QL_DEV void tmem_ld(uint32_t taddr, uint32_t (&v)[2]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];\n" : "=r"(v[0]), "=r"(v[1]) : "r"(taddr));
+}
+
+QL_DEV i128 load_i128(const ulonglong2* p) {
+  const ulonglong2 t = __ldcg(p);
+  return (i128)(((u128)t.y << 64) | t.x);
+}
+QL_DEV void store_i128(ulonglong2* p, i128 v) {
+  __stcg(p, make_ulonglong2((u64)(u128)v, (u64)((u128)v >> 64)));
+}
+
+// Add v 2^s (0 <= s <= 184) to the limbs of one entry.
+QL_DEV void sacc_add(long long* limbs, i128 v, int s) {
+  if (v == 0) return;
+  const bool neg = v < 0;
+  u128 mag = neg ? (u128)(-v) : (u128)v;
+  constexpr u64 kMask = (1ull << kLimbBits) - 1ull;
+  int k = s / kLimbBits;
+  const int off = s - k * kLimbBits;
+  u64 c = ((u64)mag << off) & kMask;
+  u128 rem = mag >> (kLimbBits - off);
+  for (;;) {
+    if (c) atomicAdd(reinterpret_cast<u64*>(limbs + k), neg ? (u64)0 - c : c);
+    if (rem == 0) break;
+    c = (u64)rem & kMask;
+    rem >>= kLimbBits;
+    ++k;
+  }
+}
+
+// Magnitude (320 bits, little-endian words) and sign of an entry.
+struct Wide320 {
+  u64 w[5];
+  bool neg;
+};
+QL_DEV Wide320 sacc_load(const long long* limbs) {
+  long long l[kLimbs];
+#pragma unroll
+  for (int k = 0; k < kLimbs; ++k) l[k] = __ldcg(limbs + k);
+  constexpr u64 kMask = (1ull << kLimbBits) - 1ull;
+  u64 d[kLimbs];
+  long long carry = 0;
+#pragma unroll
+  for (int k = 0; k < kLimbs; ++k) {
+    const long long t = l[k] + carry;
+    d[k] = (u64)t & kMask;
+    carry = t >> kLimbBits;
+  }
+  Wide320 r;
+  r.neg = carry < 0;
+  if (r.neg) {  // two's complement over the eight limbs
+    u64 c = 1;
+#pragma unroll
+    for (int k = 0; k < kLimbs; ++k) {
+      const u64 t = ((~d[k]) & kMask) + c;
+      d[k] = t & kMask;
+      c = t >> kLimbBits;
+    }
+  }
+  r.w[0] = d[0] | (d[1] << 40);
+  r.w[1] = (d[1] >> 24) | (d[2] << 16) | (d[3] << 56);
+  r.w[2] = (d[3] >> 8) | (d[4] << 32);
+  r.w[3] = (d[4] >> 32) | (d[5] << 8) | (d[6] << 48);
+  r.w[4] = (d[6] >> 16) | (d[7] << 24);
+  return r;
+}
+QL_DEV int bit_length(const Wide320& a) {
+#pragma unroll
+  for (int k = 4; k >= 0; --k)
+    if (a.w[k]) return 64 * k + 64 - __clzll((long long)a.w[k]);
+  return 0;
+}
+// Bits [r, r + 128) of the magnitude (0 <= r).
+QL_DEV u128 bits_at(const Wide320& a, int r) {
+  const int wi = r >> 6, bi = r & 63;
+  u64 x[3] = {0, 0, 0};
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+      if (i == wi + k) x[k] = a.w[i];
+  const u128 lo = ((u128)x[1] << 64) | x[0];
+  if (bi == 0) return lo;
+  return (lo >> bi) | ((u128)x[2] << (128 - bi));
+}
+// Signed magnitude times 2^e as a double (one rounding; mag fits in 128 bits).
+QL_DEV double ldexp_pow2(double v, int e) {  // |e| may exceed one normal power of two
+  while (e > 1000) {
+    v *= 0x1p1000;
+    e -= 1000;
+  }
+  while (e < -1000) {
+    v *= 0x1p-1000;
+    e += 1000;
+  }
+  return v * __longlong_as_double((long long)(e + 1023) << 52);
+}
+QL_DEV double mag_to_double(u128 mag, int e) {
+  const u64 hi = (u64)(mag >> 64);
+  if (hi == 0) {
+    const u64 lo = (u64)mag;
+    return lo ? ldexp_pow2(__ull2double_rn(lo), e) : 0.0;
+  }
+  const int z = __clzll((long long)hi);
+  const u128 t = mag << z;
+  const u64 top = (u64)(t >> 64) | ((u64)t != 0 ? 1ull : 0ull);  // sticky bit below the 64
+  return ldexp_pow2(__ull2double_rn(top), e + 64 - z);
+}
+QL_DEV double wide_to_double(const Wide320& a, int e) {
+  const int bl = bit_length(a);
+  if (bl == 0) return 0.0;
+  const int r = bl > 128 ? bl - 128 : 0;
+  const double v = mag_to_double(bits_at(a, r), e + r);
+  return a.neg ? -v : v;
+}
+
+// ---------------------------------------------------------------------------------------
+// Cholesky factorisation of the exact Gram matrix in 125-bit fixed point, by one CTA.
+// Column j is scaled by 2^-s_j so that 1/4 <= C_jj < 1; every later quantity (Schur
+// complements, rows of R) stays below 1 in magnitude, so fixed point loses 2^-122 per
+// operation and nothing to cancellation.  Integer multiplies run on the ALUs at full rate,
+// where FP64 (1/64 of the FP32 rate) or double-double would not: a double-double version of
+// the same factorisation needs about 0.9 M FP64 operations at n = 64, 0.2 ms on one SM.
+// 1 / sqrt(pivot) comes from FP64 with one double-double Newton step (relative 2^-103), by
+// one lane, while the other warps update the trailing rows.  A pivot below 2^-80 of its
+// column (kappa above about 2^40), zero or negative stops the factorisation; a column that
+// is zero altogether gives a zero row of R.
+// ---------------------------------------------------------------------------------------
+constexpr int kFx = 125;
+
+QL_DEV u64 umul_hi(u64 a, u64 b) { return __umul64hi(a, b); }
+// (a b) 2^-kFx for |a|, |b| < 2^(kFx + 1); error below 2^4 units
+QL_DEV i128 fx_mul(i128 a, i128 b) {
+  const long long ah = (long long)(a >> 64), bh = (long long)(b >> 64);
+  const u64 al = (u64)a, bl = (u64)b;
+  i128 p = (i128)ah * bh;
+  p += (i128)(u128)umul_hi((u64)ah, bl) - (ah < 0 ? (i128)(u128)bl : (i128)0);
+  p += (i128)(u128)umul_hi((u64)bh, al) - (bh < 0 ? (i128)(u128)al : (i128)0);
+  return p * 8;  // 2^128 / 2^125
+}
+
+struct FxPivot {
+  i128 r;  // 2^-x / sqrt(d) in (1/2, 1], fixed point
+  int x;
+  int ok;  // 1: usable; 0: zero column; -1: pivot too small
+};
+QL_DEV FxPivot fx_pivot(i128 d, bool zero_column) {
+  FxPivot pv{0, 0, 0};
+  if (zero_column) return pv;
+  if (d < ((i128)1 << (kFx - 80))) {
+    pv.ok = -1;
+    return pv;
+  }
+  // d = 2^-2z f, f in [1/4, 1)
+  const u64 hi = (u64)((u128)d >> 64);
+  const int lead = hi ? __clzll((long long)hi) : 64 + __clzll((long long)(u64)d);  // of 128 bits
+  const int z = (lead - (128 - kFx)) >> 1;  // d < 2^(128 - lead - kFx)
+  const u128 f = (u128)d << (2 * z);
+  const u64 fh = (u64)(f >> 72);  // 53 bits at most: exact in a double
+  const double dh = (double)fh * 0x1p-53;
+  const double dl = (double)(u64)((f >> 19) & ((((u64)1) << 53) - 1)) * 0x1p-106;
+  const double r0 = rsqrt(dh);
+  const double th = r0 * r0, tl = fma(r0, r0, -th);
+  const double p = dh * th, pe = fma(dh, th, -p);
+  const double e = (1.0 - p) - (pe + fma(dh, tl, dl * th));
+  const double r1 = 0.5 * r0 * e;  // r0 in (1, 2]
+  // r / 2 in fixed point
+  i128 r = (i128)((u128)(u64)(r0 * 0x1p52) << (kFx - 53));
+  r += (i128)__double2ll_rn(r1 * 0x1p104) * ((i128)1 << (kFx - 105));
+  pv.r = r;
+  pv.x = z + 1;
+  pv.ok = 1;
+  return pv;
+}
+
+// sacc -> Rout (n x n upper triangle, row-major, ld LE, in shared memory).  Shared memory from
+// smem: two arrays of NC x LE words, then the scratch.  Returns 0, or the 1-based index of
+// the pivot that stopped it (to every thread).
+template <int NC, int T>
+QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double* Rout) {
+  constexpr int LE = NC + 1;
+  u64* Slo = reinterpret_cast<u64*>(smem);
+  long long* Shi = reinterpret_cast<long long*>(Slo + NC * LE);
+  int* sj = reinterpret_cast<int*>(Shi + NC * LE);  // column exponents
+  FxPivot* piv = reinterpret_cast<FxPivot*>(reinterpret_cast<unsigned char*>(sj) + 4 * NC + (16 - (4 * NC) % 16) % 16);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int NW = T / 32;
+  auto get = [&](int i, int j) -> i128 { return (i128)(((u128)(u64)Shi[i * LE + j] << 64) | Slo[i * LE + j]); };
+  auto put = [&](int i, int j, i128 v) {
+    Slo[i * LE + j] = (u64)(u128)v;
+    Shi[i * LE + j] = (long long)(v >> 64);
+  };
+  for (int j = tid; j < n; j += T) {
+    const Wide320 a = sacc_load(sacc + (size_t)tri_index(j, j) * kLimbs);
+    const int bl = a.neg ? 0 : bit_length(a);
+    sj[j] = bl ? (bl + 1) >> 1 : -1;
+  }
+  __syncthreads();
+  for (int i = warp; i < n; i += NW)
+    for (int j = i + lane; j < n; j += 32) {
+      i128 v = 0;
+      if (sj[i] >= 0 && sj[j] >= 0) {
+        const Wide320 a = sacc_load(sacc + (size_t)tri_index(i, j) * kLimbs);
+        const int r = sj[i] + sj[j] - kFx;
+        u128 mag = r > 0 ? bits_at(a, r) + (bits_at(a, r - 1) & 1)
+                         : bits_at(a, 0) << (-r);
+        v = a.neg ? -(i128)mag : (i128)mag;
+      }
+      put(i, j, v);
+    }
+  __syncthreads();
+  if (tid == 0) piv[0] = fx_pivot(get(0, 0), sj[0] < 0);
+  __syncthreads();
+  for (int k = 0; k < n; ++k) {
+    const FxPivot pv = piv[k & 1];
+    if (pv.ok < 0) return k + 1;  // uniform
+    for (int j = k + tid; j < n; j += T) {  // row k of R
+      const i128 v = pv.ok ? fx_mul(get(k, j) << pv.x, pv.r) : (i128)0;
+      put(k, j, v);
+      const u128 mag = v < 0 ? (u128)-v : (u128)v;
+      const double d = mag_to_double(mag, sj[j] - kFx + kXgUnitExp / 2);
+      Rout[k * LE + j] = v < 0 ? -d : d;
+    }
+    __syncthreads();
+    if (warp == 0) {  // the next row, then its pivot
+      const int i = k + 1;
+      if (i < n) {
+        const i128 lki = get(k, i);
+        for (int j = i + lane; j < n; j += 32) put(i, j, get(i, j) - fx_mul(lki, get(k, j)));
+        if (lane == 0) piv[i & 1] = fx_pivot(get(i, i), sj[i] < 0);
+      }
+    } else {
+      for (int i = k + 1 + warp; i < n; i += NW - 1) {
+        const i128 lki = get(k, i);
+        for (int j = i + lane; j < n; j += 32) put(i, j, get(i, j) - fx_mul(lki, get(k, j)));
+      }
+    }
+    __syncthreads();
+  }
+  for (int e = tid; e < n * n; e += T)
+    if (e / n > e % n) Rout[(e / n) * LE + e % n] = 0.0;
+  __syncthreads();
+  return 0;
+}
+
+// Range verdict, election of the last CTA and, in it, the epilogue: for TSQR calls
+// (a.method == QL_TSQR) R from the fixed-point Cholesky, or the request that the Householder
+// launch redoes the call (flags[1]); for the Gram methods C in FP64 and their own epilogue.
+template <int NC, int T, typename S>
+QL_DEV void xg_finish(const GramArgs<S>& a, unsigned char* smem, const int* colmax, int* misc, int k) {
+  if (!gram_elect<S, ArithDF>(a, colmax, misc, k)) return;
+  const int tid = threadIdx.x, n = a.n;
+  constexpr int LE = NC + 1;
+  if (a.method == QL_TSQR) {
+    if (*(volatile int*)&a.w.flags[1] != 0) return;  // a bounded wait gave up: Householder redoes the call
+    double* Rs = reinterpret_cast<double*>(smem);
+    double* vec = Rs + NC * LE;
+    int* sflag = reinterpret_cast<int*>(vec + 2 * LE);
+    unsigned char* scratch = smem + ((NC + 3) * LE * 8 + 255) / 256 * 256;
+    if (xg_cholesky<NC, T>(a.w.sacc, n, scratch, Rs)) {
+      if (tid == 0) {
+        a.w.flags[1] = 1;
+        if (a.redo) gram_request_redo(a.redo, a.redo_any);
+      }
+      return;
+    }
+    if (a.epilogue == kEpiR)
+      epilogue_r<T>(Rs, LE, n, a.R, a.ldr, a.info, sflag);
+    else
+      epilogue_lstsq<T>(Rs, LE, n, a.x, a.resnorm, a.Rext, a.info, vec, sflag);
+    return;
+  }
+  double* Cs = reinterpret_cast<double*>(smem);
+  for (int i = tid >> 5; i < n; i += T / 32)
+    for (int j = i + (tid & 31); j < n; j += 32) {
+      const double v = wide_to_double(sacc_load(a.w.sacc + (size_t)tri_index(i, j) * kLimbs), kXgUnitExp);
+      Cs[i * LE + j] = v;
+      Cs[j * LE + i] = v;
+    }
+  __syncthreads();
+  gram_epilogue<NC, T, S, ArithDF>(a, smem);
+}
+
+// Row tiles [tiles bid / k, tiles (bid + 1) / k) of one problem; tensor memory at tbase and
+// barriers set up by xg_cta_begin, phases carried in bars (see gram_pipe_body).
+template <int NC, typename S>
+QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& bars, const CUtensorMap* tmA,
+                       const CUtensorMap* tmB) {
+  using Sh = XgShape<NC>;
+  using Sm = XgSmem<NC, S>;
+  constexpr int T = Sh::T, TS = Sh::TS, KT = Sh::KT, PLANE = Sh::PLANE, SBO = Sh::SBO, LBO = Sh::LBO, HALF = Sh::HALF,
+                RPB = Sm::RPB, NBOX = Sm::NBOX, LG = Sh::LG;
+  extern __shared__ __align__(1024) unsigned char smem_umma[];
+  unsigned char* smem = smem_umma;
+  const int tid = threadIdx.x, n = a.n, lane = tid & 31, warp = tid >> 5;
+  const bool control = warp == TS / 32;
+  auto digits = [&](int b) { return smem + Sh::PAD + (size_t)b * (Sh::DBUF + Sh::PAD); };
+  unsigned char* raw0 = smem + Sm::kOffRaw;
+  int* scale = reinterpret_cast<int*>(smem + Sm::kOffScale);
+  int* colmax = reinterpret_cast<int*>(smem + Sm::kOffColmax);
+  int* misc = reinterpret_cast<int*>(smem + Sm::kOffMisc);
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + Sm::kOffBar);  // [2] MMAs done, per digit buffer
+  uint64_t* lbar = mbar + 2;                                          // [2] tile landed, per raw stage
+  uint64_t* dbar = mbar + 4;                                          // [2] digits ready, per digit buffer
+  uint64_t* rbar = mbar + 6;                                          // [2] stage read, per raw stage
+  int* ngrp = reinterpret_cast<int*>(smem + Sm::kOffSlot + 4);        // [2] tile opens a new group
+  int* sfail = ngrp + 2;                                              // [2] where each role gave up
+
+  a.tiles = (a.m + KT - 1) / KT;
+  for (int i = tid; i < NC; i += T) {
+    colmax[i] = 0;
+    scale[i] = 0;
+  }
+  if (tid < 2) sfail[tid] = 0;
+  if constexpr (Sh::PAD > 0) {
+    for (int z = 0; z < 3; ++z)
+      for (int i = tid; i < Sh::PAD / 16; i += T)
+        *reinterpret_cast<uint4*>(smem + (size_t)z * (Sh::DBUF + Sh::PAD) + 16 * i) = make_uint4(0, 0, 0, 0);
+  }
+  // the generic writes so far (a previous work item's included) come before the copies and
+  // the MMA operand reads
+  fence_proxy_async_smem();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+
+  const int64_t t0 = a.tiles * bid / k, t1 = a.tiles * (bid + 1) / k;
+  const bool bulk = a.bulk != 0;  // tensor copies; otherwise the slicers read X from global memory
+
+  // this slicer's unit of a tile: rows r0..r0+7 of column cu (8 consecutive threads hold 8
+  // consecutive columns, so their digit stores fill whole core-matrix rows)
+  const int u8 = (tid & (TS - 1)) >> 3;
+  const int cu = 8 * (u8 / (KT / 8)) + (tid & 7), r0 = 8 * (u8 % (KT / 8));
+  const bool live = cu < n && !control;
+  // read-out role: TMEM lane quarter qd, columns hh HALF + [0, HALF) of C; lane L belongs to
+  // lane group lg (plane, or weight parity) and row li of C
+  const int qd = warp & 3, hh = (warp >> 2) & 3;
+  const int L = 32 * qd + lane, lg = L / NC, li = L % NC;
+  const bool reader = !control && lg < LG;
+  ulonglong2* acc = reinterpret_cast<ulonglong2*>(a.w.fbuf) + (size_t)bid * NC * 128;  // [column][lane]
+
+  if (control) {
+    // ---- control warp: copies two tiles ahead; per tile, once the slicers have read its
+    // stage, the copy two ahead into it; once its digits are ready, the MMAs
+    bool ok = true;
+    uint32_t pend = 0u, ppar = 0u;  // bit b: a copy into stage b in flight, and its phase parity
+    auto copy = [&](int64_t t, int b) {
+      if (!bulk) return;
+      unsigned char* stage = raw0 + (size_t)b * Sm::kRaw;
+      const int row0 = (int)(t * KT);
+      if (lane == 0) {
+        mbar_arrive_expect_tx(&lbar[b], (uint32_t)(NBOX * n * 128));
+#pragma unroll 1
+        for (int kb = 0; kb < NBOX; ++kb) {
+          tma_load_2d(stage + (size_t)kb * NC * 128, tmA, row0 + kb * RPB, 0, &lbar[b]);
+          if (tmB) tma_load_2d(stage + (size_t)(kb * NC + a.src.nA) * 128, tmB, row0 + kb * RPB, 0, &lbar[b]);
+        }
+      }
+      __syncwarp();
+      pend |= 1u << b;
+      ppar = (ppar & ~(1u << b)) | (bars.lpar & (1u << b));
+      bars.lpar ^= 1u << b;
+    };
+    if (t0 < t1) copy(t0, 0);
+    if (t0 + 1 < t1) copy(t0 + 1, 1);
+    for (int64_t t = t0; t < t1; ++t) {
+      const int b = (int)((t - t0) & 1);
+      if (!__all_sync(0xffffffffu, mbar_wait_bounded(&rbar[b], (bars.mpar >> b) & 1u))) {
+        ok = false;
+        break;
+      }
+      pend &= ~(1u << b);
+      if (t + 2 < t1) copy(t + 2, b);
+      if (!__all_sync(0xffffffffu, mbar_wait_bounded(&dbar[b], (bars.mpar >> b) & 1u))) {
+        ok = false;
+        break;
+      }
+      bars.mpar ^= 1u << b;
+      tc_fence_after();
+      if (lane == 0) {
+        // planes and k-steps add (byte offset >> 4) to the 14-bit address field, which stays
+        // below 2^14 (shared addresses < 256 KB); plane -1 is the zero plane before the buffer
+        xg_issue_mmas<NC>(tbase, umma_sdesc(smem_addr(digits(b)), LBO, SBO), (uint32_t)ngrp[b]);
+        umma_commit(&mbar[b]);
+      }
+      __syncwarp();
+    }
+    for (int b = 0; b < 2; ++b)  // no copy may still be writing when the CTA moves on
+      if (pend & (1u << b)) mbar_wait_bounded(&lbar[b], (ppar >> b) & 1u);
+    if (!ok && lane == 0) sfail[1] = 2;
+  } else {
+    // ---- slicer warps
+    bool ok = true;
+    int fail_where = 0;  // 1: a tile copy never completed, 2: the MMAs never completed
+    int grp = 0;         // tiles summed in tensor memory since the last read-out
+    int nread = 0;       // read-outs in the 128-bit sums since they were last emptied
+    int last_b = 0;      // digit buffer of the latest tile handed to the MMAs
+    uint32_t cpar = 0u;  // bit b: phase parity of the MMAs of the latest tile on buffer b
+    unsigned arun = 0;   // largest |x| this slicer's column has shown (range record)
+
+    // Tensor-memory sums -> 128-bit integers.  A thread folds the eight sums of its (lane,
+    // column): digits q of the other factor for NC <= 32 (planes p and p + 4 for NC = 32),
+    // the eight weights of its parity for NC = 64.
+    auto readout = [&]() {
+      constexpr int JS = HALF < 4 ? HALF : 4;
+      const uint32_t lane_base = tbase + ((uint32_t)(32 * qd) << 16) + (uint32_t)(hh * HALF);
+      const bool keep = nread++ > 0;   // uniform: every slicer counts the read-outs
+      if (NC == 8 && qd >= 2) return;  // lanes 64..127 hold nothing
+#pragma unroll 1
+      for (int c0 = 0; c0 < HALF; c0 += JS) {
+        i128 sum[JS];
+#pragma unroll
+        for (int j = 0; j < JS; ++j) sum[j] = 0;
+#pragma unroll
+        for (int part = 0; part < (NC == 32 ? 2 : 1); ++part) {
+          uint32_t v[8][JS];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) tmem_ld(lane_base + (uint32_t)(part * 256 + q * NC + c0), v[q]);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < JS; ++j) {
+            int d[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) d[q] = __float2int_rn(__uint_as_float(v[q][j]));
+            constexpr int SP = NC == 64 ? 14 : 7;
+            if constexpr (NC == 64) {
+              i128 s = (long long)d[0] * (1 << SP) + d[1];
+              s = s * ((i128)1 << (2 * SP)) + ((long long)d[2] * (1 << SP) + d[3]);
+              s = s * ((i128)1 << (2 * SP)) + ((long long)d[4] * (1 << SP) + d[5]);
+              s = s * ((i128)1 << (2 * SP)) + ((long long)d[6] * (1 << SP) + d[7]);
+              sum[j] = s;
+            } else {
+              long long h = d[0], l = d[4];
+#pragma unroll
+              for (int q = 1; q < 4; ++q) {
+                h = h * 128 + d[q];
+                l = l * 128 + d[4 + q];
+              }
+              const i128 s = (i128)h * (1 << 28) + l;
+              sum[j] = sum[j] * (1 << 28) + s;
+            }
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < JS; ++j) {
+          ulonglong2* p = acc + (size_t)(hh * HALF + c0 + j) * 128 + L;
+          store_i128(p, keep ? load_i128(p) + sum[j] : sum[j]);
+        }
+      }
+    };
+    // 128-bit sums -> the integer accumulators of C at the current column scales.  Lane groups
+    // 1.. hand their sums to group 0 through `scratch` (a free digit buffer).
+    auto emit = [&](unsigned char* scratch) {
+      ulonglong2* sc = reinterpret_cast<ulonglong2*>(scratch);
+      if (reader && lg > 0) {
+#pragma unroll 1
+        for (int j = 0; j < HALF; ++j)
+          sc[((size_t)(lg - 1) * NC + li) * NC + hh * HALF + j] = __ldcg(acc + (size_t)(hh * HALF + j) * 128 + L);
+      }
+      slicer_sync<TS>();
+      if (reader && lg == 0 && li < n) {
+        const int si = scale[li];
+#pragma unroll 1
+        for (int j = 0; j < HALF; ++j) {
+          const int jj = hh * HALF + j;
+          if (jj < li || jj >= n) continue;
+          i128 v = load_i128(acc + (size_t)jj * 128 + L);
+          auto part = [&](int g) -> i128 {
+            const ulonglong2 t = sc[((size_t)(g - 1) * NC + li) * NC + jj];
+            return (i128)(((u128)t.y << 64) | t.x);
+          };
+          if constexpr (NC == 64) {
+            v += part(1) >> 7;  // odd weights: a multiple of 2^7 (weight 15 is empty)
+          } else {
+#pragma unroll 1
+            for (int g = 1; g < LG; ++g) v = v * 128 + part(g);
+          }
+          const int sj = scale[jj];
+          if (si >= kEsMin && sj >= kEsMin && si <= kEsMax && sj <= kEsMax)  // else flagged at the end, or zero
+            sacc_add(a.w.sacc + (size_t)tri_index(li, jj) * kLimbs, v, si + sj - 2 * kEsMin);
+        }
+      }
+      slicer_sync<TS>();
+      nread = 0;
+    };
+    auto wait_last = [&]() {  // the MMAs of every tile handed over are done
+      return slicer_and<TS>(mbar_wait_bounded(&mbar[last_b], (cpar >> last_b) & 1u));
+    };
+
+    Rows8<S> v, ahead;
+    auto load_global = [&](Rows8<S>& w, int64_t t) {
+      const S* col = a.src.col(cu) + t * KT + r0;
+      const int64_t left = a.m - (t * KT + r0);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) w.set(j, j < left ? __ldg(col + j) : S(0));
+    };
+    if (!bulk && live && t0 < t1) load_global(ahead, t0);
+
+    for (int64_t t = t0; t < t1; ++t) {
+      const int i = (int)(t - t0), b = i & 1;
+      bool landed = true;
+      if (bulk) {
+        landed = mbar_wait_bounded(&lbar[b], (bars.lpar >> b) & 1u);
+        bars.lpar ^= 1u << b;
+      }
+      unsigned am = 0;
+      int es = 0;
+      bool over = false;
+      if (live) {
+        if (bulk) {
+          const unsigned char* line = raw0 + (size_t)b * Sm::kRaw + (size_t)((r0 / RPB) * NC + cu) * 128;
+          const int q0 = (r0 % RPB) * (int)sizeof(S) / 16, swz = cu == a.src.nA ? 0 : (cu & 7);
+#pragma unroll
+          for (int q = 0; q < 8 * (int)sizeof(S) / 16; ++q)
+            v.chunk(q, *reinterpret_cast<const uint4*>(line + (((q0 + q) ^ swz) << 4)));
+        } else {
+          v = ahead;
+          if (t + 1 < t1) load_global(ahead, t + 1);
+        }
+        am = v.amax();
+        arun = max(arun, am);
+        es = Rows8<S>::exponent(am);
+        over = es > scale[cu];
+      }
+      // stage b is read: the control warp may copy the tile two ahead into it
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&rbar[b]);
+      // digit buffer b is free once the MMAs of tile t - 2 are done
+      const bool okw = i >= 2 ? mbar_wait_bounded(&mbar[b], (cpar >> b) & 1u) : true;
+      const bool full = grp >= Sh::G;
+      if (slicer_or<TS>(over || !okw || !landed) || full) {
+        if (!slicer_and<TS>(landed)) {  // the copy engine did not deliver
+          ok = false;
+          fail_where = 1;
+          break;
+        }
+        if (!slicer_and<TS>(okw)) {  // the tensor core did not finish
+          ok = false;
+          fail_where = 2;
+          break;
+        }
+        const bool anyover = slicer_or<TS>(over);
+        if (grp > 0) {
+          if (!wait_last()) {
+            ok = false;
+            fail_where = 2;
+            break;
+          }
+          tc_fence_after();
+          readout();
+          grp = 0;
+        }
+        if (nread > 0 && (anyover || nread >= Sh::MAX_READS)) emit(digits(0));  // every MMA is done: both buffers are free
+        if (anyover) {
+          slicer_sync<TS>();  // every read of the old scales is done
+          if (over) atomicMax(&scale[cu], max(es + Sh::SLACK, kEsMin));
+        }
+        slicer_sync<TS>();
+      }
+      // eight digits of every element into buffer b
+      unsigned char* dst = digits(b) + (cu >> 3) * SBO + (r0 >> 3) * LBO + (cu & 7) * 16;
+      if (live) {
+        const int Es = scale[cu], base = Es > 0 ? Es + 7 : 4096;
+        int s[8], any = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          s[j] = v.shift(j, base);
+          any |= s[j];
+        }
+        u64 Nb[8];
+        if (any > 31) {  // an element more than 2^24 below the scale (or zero)
+#pragma unroll
+          for (int j = 0; j < 8; ++j) Nb[j] = cut56<true>(v.h(j), v.l(j), v.hw[j], s[j]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) Nb[j] = cut56<false>(v.h(j), v.l(j), v.hw[j], s[j]);
+        }
+        put_plane_pairs<PLANE, 0>(dst, Nb);
+      } else {
+#pragma unroll
+        for (int p = 0; p < 8; ++p) *reinterpret_cast<uint4*>(dst + p * PLANE) = make_uint4(0, 0, 0, 0);
+      }
+      if (tid == 0) ngrp[b] = grp == 0 ? 1 : 0;
+      fence_proxy_async_smem();  // the digit planes are read by the tensor core
+      tc_fence_before();         // the read-out's TMEM loads come before the next MMAs
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&dbar[b]);
+      cpar = (cpar & ~(1u << b)) | (bars.mpar & (1u << b));
+      bars.mpar ^= 1u << b;
+      last_b = b;
+      ++grp;
+    }
+    if (ok && grp > 0) {  // the last group
+      if (!wait_last()) {
+        ok = false;
+        fail_where = 2;
+      } else {
+        tc_fence_after();
+        readout();
+      }
+    }
+    if (ok && nread > 0) emit(digits(0));
+    if (!ok && tid == 0) sfail[0] = fail_where;
+    if (live && arun > 0) atomicMax(&colmax[cu], Rows8<S>::exponent(arun));
+  }
+  tc_fence_before();
+  __syncthreads();
+  const int fw = sfail[0] ? sfail[0] : sfail[1];
+  if (fw) {
+    bars.ok = false;  // a late arrival may still complete a phase: the CTA takes no more work
+    if (tid == 0) {   // the gated launches redo the call and report {QL_ERR_TIMEOUT, where}
+      atomicCAS(&a.w.flags[4], 0, fw);
+      atomicOr(&a.w.flags[a.method == QL_TSQR ? 1 : 0], 2);
+    }
+  }
+  for (int cc = tid; cc < n; cc += T)  // column exponents of the whole matrix, for the later passes
+    if (colmax[cc] > 0) atomicMax(&a.w.flags[64 + cc], colmax[cc]);
+  xg_finish<NC, T, S>(a, smem, colmax, misc, k);
+}
+
+template <int NC, typename S>
+QL_DEV uint32_t xg_cta_begin(unsigned char* smem) {
+  using Sm = XgSmem<NC, S>;
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + Sm::kOffSlot);
+  if ((threadIdx.x >> 5) == 0) tmem_alloc(tslot, XgShape<NC>::TCOLS);
+  if (threadIdx.x == 0) {
+    uint64_t* bar = reinterpret_cast<uint64_t*>(smem + Sm::kOffBar);
+    for (int i = 0; i < 4; ++i) mbar_init(bar + i, 1);
+    for (int i = 4; i < 8; ++i) mbar_init(bar + i, XgShape<NC>::TS / 32);  // one arrival per slicer warp
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  return *tslot;
+}
+
+template <int NC, typename S>
+__global__ void __launch_bounds__(XgShape<NC>::T, 1)
+    xgram_kernel(const __grid_constant__ GramArgs<S> a, const __grid_constant__ CUtensorMap tmA,
+                 const __grid_constant__ CUtensorMap tmB, int has_b) {
+  extern __shared__ __align__(1024) unsigned char smem_umma[];
+  const uint32_t tbase = xg_cta_begin<NC, S>(smem_umma);
+  PipeBars bars;
+  xgram_body<NC, S>(a, blockIdx.x, gridDim.x, tbase, bars, &tmA, has_b ? &tmB : nullptr);
+  tc_fence_before();
+  __syncthreads();
+  if ((threadIdx.x >> 5) == 0) tmem_dealloc(tbase, XgShape<NC>::TCOLS);
+}
+
+template <int NC, typename S>
+ql_status xgram_launch_one(const GramCall& c, const GramWs& w) {
+  using Sh = XgShape<NC>;
+  using Sm = XgSmem<NC, S>;
+  auto kern = xgram_kernel<NC, S>;
+  static bool ready = false;
+  static std::mutex mu;
+  {
+    std::lock_guard<std::mutex> lk(mu);
+    if (!ready) {
+      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sm::kBytes) != cudaSuccess)
+        return QL_ERR_CUDA;
+      ready = true;
+    }
+  }
+  const int64_t tiles = (c.m + Sh::KT - 1) / Sh::KT;
+  int64_t g = (int64_t)device_sm_count();  // one CTA per SM: the shared memory allows no second one
+  if (g > tiles) g = tiles;
+  if (g < 1) g = 1;
+  GramArgs<S> a{};
+  a.src.A = static_cast<const S*>(c.A);
+  a.src.lda = c.lda;
+  a.src.b = static_cast<const S*>(c.b);
+  a.src.nA = c.nA;
+  a.m = c.m;
+  a.n = c.n;
+  a.tiles = tiles;
+  a.pass = 1;
+  a.method = c.method;
+  a.epilogue = c.epilogue;
+  a.w = w;
+  a.R = c.R;
+  a.ldr = c.ldr;
+  a.Z = c.Z;
+  a.rank_tol = c.rank_tol;
+  a.x = c.x;
+  a.resnorm = c.resnorm;
+  a.Rext = c.Rext;
+  a.info = c.info;
+  CUtensorMap tmA{}, tmB{};
+  const bool has_b = c.nA < c.n;
+  a.bulk = pipe_tensor_maps(&tmA, has_b ? &tmB : nullptr, c.A, c.b, std::is_same<S, double>::value ? QL_F64 : QL_F32,
+                            c.m, c.nA, c.lda)
+               ? 1
+               : 0;
+  a.mround = NC >= 16 ? 2 : 1;  // how the next pass's kernel of this class reads M
+  count_launch();
+  kern<<<(int)g, Sh::T, Sm::kBytes, c.stream>>>(a, tmA, tmB, has_b ? 1 : 0);
+  return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+}
+
+template <typename S>
+ql_status xgram_pass1(const GramCall& c, const GramWs& w) {
+  if (c.n <= 8) return xgram_launch_one<8, S>(c, w);
+  if (c.n <= 16) return xgram_launch_one<16, S>(c, w);
+  if (c.n <= 32) return xgram_launch_one<32, S>(c, w);
+  return xgram_launch_one<64, S>(c, w);
+}
+
+}  // namespace ql

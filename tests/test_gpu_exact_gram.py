@@ -1,0 +1,92 @@
+"""The exact Gram route of TSQR (n >= 5): tile edges, column classes, scale changes, zero and
+dependent columns, unaligned columns, and the hand-over to the Householder tiles.
+
+Tolerance.  X is rounded to 2^-56 of each column's largest entry and everything after that is
+exact to 2^-100, so ||R - R_ref|| <= (2^-55 kappa + 2^-52) ||R_ref|| n; the bound of the other
+parity tests, 1e-13 n kappa, is far above it.  R^T R is compared with X^T X formed in FP64 by
+row blocks (rounding below 1e-14 n of the column norms).
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2603_20889_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def tsqr(X, pad=0):
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    m, n = X.shape
+    buf = torch.zeros((n, m + pad), dtype=torch.float64 if X.dtype == np.float64 else torch.float32, device="cuda")
+    buf[:, :m] = torch.from_numpy(np.ascontiguousarray(X.T)).cuda()
+    R, info = q.tsqr_qless(buf[:, :m].T)
+    return R.cpu().numpy(), info.cpu().tolist()
+
+
+def gram_error(R, X):
+    G = X.astype(np.float64).T @ X.astype(np.float64)
+    d = np.sqrt(np.diag(G))
+    return np.abs((R.T @ R - G) / np.where(d > 0, d, 1)[:, None] / np.where(d > 0, d, 1)[None, :]).max()
+
+
+@pytest.mark.parametrize("n", [5, 8, 9, 16, 17, 32, 33, 64])
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_tile_edges_against_oracle(n, dtype):
+    kt = 4096 // (8 if n <= 8 else 16 if n <= 16 else 32 if n <= 32 else 64)
+    for m, pad in ((n, 0), (kt - 1, 1), (kt, 0), (kt + 1, 2), (3 * kt + 5, 3)):
+        X = synth.conditioned(max(m, n), n, 100.0, seed=m + n, dtype=dtype)
+        R, info = tsqr(X, pad)
+        assert info == [0, 0]
+        ref = oracle.householder_r(X.astype(np.float64))
+        # a square Gaussian X may be far worse conditioned than its mixing matrix
+        kappa = max(100.0, np.linalg.cond(X.astype(np.float64)))
+        assert oracle.rel_err(R, ref) <= oracle.tolerance(n, kappa), (m, pad)
+
+
+@pytest.mark.parametrize("n,log2m", [(8, 18), (16, 17), (32, 16), (64, 16)])
+def test_many_tiles_per_cta_exact_r(n, log2m):
+    X, R0 = synth.hadamard_exact_case(1 << log2m, n, 1e4, seed=n)
+    R, info = tsqr(X)
+    assert info == [0, 0]
+    assert oracle.rel_err(R, R0) <= 1e-15  # R0 is exact; R rounds once per entry
+
+
+@pytest.mark.parametrize("n,m", [(5, 200001), (16, 100003), (32, 60002), (64, 40000)])
+def test_growing_rows_raise_the_column_scales(n, m):
+    X = synth.gaussian(m, n, seed=n) * np.exp2(np.floor(24.0 * np.arange(m) / m))[:, None]
+    R, info = tsqr(X)
+    assert info == [0, 0]
+    assert gram_error(R, X) <= 1e-14 * n
+
+
+@pytest.mark.parametrize("n", [6, 24, 40])
+def test_zero_and_far_apart_entries(n):
+    X = synth.gaussian(5000, n, seed=3)
+    X[:, 2] = 0.0                      # a zero column stays on the exact route
+    X[::7, 1] *= 2.0 ** -30            # entries far below the column's scale
+    X[::3, 3] = 0.0
+    R, info = tsqr(X)
+    assert info == [0, 0] and R[2, 2] == 0.0 and np.all(R[2, 3:] == 0.0)
+    assert gram_error(R, X) <= 1e-14 * n
+
+
+@pytest.mark.parametrize("n", [8, 20, 64])
+def test_dependent_columns_go_to_householder(n):
+    X = synth.gaussian(3000, n, seed=5)
+    X[:, n - 1] = X[:, 0]              # pivot exactly zero: the Householder tiles redo the call
+    R, info = tsqr(X)
+    assert info == [0, 0] and np.all(np.isfinite(R)) and np.all(np.diag(R) >= 0.0)
+    assert R[n - 1, n - 1] <= 1e-12 * R[0, 0]
+    assert gram_error(R, X) <= 1e-13 * n
+
+
+def test_very_ill_conditioned_matches_oracle():
+    for kappa in (1e9, 1e12, 1e14):    # the last one below the pivot limit of the exact route
+        X = synth.conditioned(4000, 12, kappa, seed=9)
+        R, info = tsqr(X)
+        assert info == [0, 0]
+        assert oracle.rel_err(R, oracle.householder_r(X)) <= oracle.tolerance(12, kappa)
