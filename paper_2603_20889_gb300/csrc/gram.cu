@@ -31,11 +31,10 @@ bool pipe_gram2_enabled() {
   return on;
 }
 
-bool pipe_tensor_maps(CUtensorMap* tmA, CUtensorMap* tmB, const void* A, const void* b, int dtype, int64_t m, int nA,
-                      int64_t lda) {
-  using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                            const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                            CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+static Encode tensor_map_encoder() {
   static const Encode encode = [] {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult q{};
@@ -44,6 +43,12 @@ bool pipe_tensor_maps(CUtensorMap* tmA, CUtensorMap* tmB, const void* A, const v
       return (Encode) nullptr;
     return reinterpret_cast<Encode>(fn);
   }();
+  return encode;
+}
+
+bool pipe_tensor_maps(CUtensorMap* tmA, CUtensorMap* tmB, const void* A, const void* b, int dtype, int64_t m, int nA,
+                      int64_t lda) {
+  const Encode encode = tensor_map_encoder();
   const size_t es = dtype == QL_F64 ? 8 : 4;
   auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
   if (!encode || m < 1 || m >= (int64_t(1) << 31) || nA < 1 || nA > 256 || !aligned(A) || ((size_t)lda * es) % 16 ||
@@ -68,6 +73,21 @@ bool pipe_tensor_maps(CUtensorMap* tmA, CUtensorMap* tmB, const void* A, const v
         CUDA_SUCCESS)
       return false;
   }
+  return true;
+}
+
+bool xg_tensor_maps(XgMaps* maps, int nc, const void* A, const void* b, int dtype, int64_t m, int nA, int64_t lda) {
+  if (!pipe_tensor_maps(&maps->rows, b ? &maps->rhs : nullptr, A, b, dtype, m, nA, lda)) return false;
+  const size_t es = dtype == QL_F64 ? 8 : 4;
+  const cuuint32_t rpb = (cuuint32_t)(128 / es), one[3] = {1, 1, 1};
+  const cuuint64_t dims[3] = {rpb, (cuuint64_t)nA, (cuuint64_t)(m / rpb)}, strides[2] = {(cuuint64_t)lda * es, 128};
+  const cuuint32_t box[3] = {rpb, (cuuint32_t)nc, (cuuint32_t)(4096 / nc / rpb)};
+  maps->full = dims[2] > 0 && tensor_map_encoder()(&maps->tile, dtype == QL_F64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
+                                       const_cast<void*>(A), dims, strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                                       CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+                   ? 1
+                   : 0;
   return true;
 }
 

@@ -18,8 +18,10 @@
 // by the 2^-56 rounding of X (a backward error, like Householder's) up to kappa ~ 2^40.
 //
 //  * Roles and tiles: 16 slicer warps cut tiles of 4096 elements (KT = 4096 / NC rows) into
-//    digit planes and read the accumulators out; one control warp issues the tensor-map
-//    copies two tiles ahead and the MMAs.  Two raw stages and two digit buffers alternate.
+//    digit planes and read the accumulators out; one warp issues the tensor-map copies two
+//    tiles ahead (a whole tile per instruction), one the MMAs, in warp-uniform code with one
+//    elected lane so that descriptors stay in uniform registers.  Two raw stages and two
+//    digit buffers alternate.
 //    Mbarriers: "MMAs done" and "digits ready" per digit buffer, "tile landed" and "stage
 //    read" per raw stage; one vote of the slicers per tile (a column outgrew its scale, or a
 //    wait gave up).
@@ -49,7 +51,7 @@ using i128 = __int128;
 template <int NC>
 struct XgShape {
   static constexpr int TS = 512;             // slicer threads
-  static constexpr int T = TS + 32;          // and the control warp
+  static constexpr int T = TS + 64;          // and the copy warp and the MMA warp
   static constexpr int KT = 4096 / NC;       // rows per tile
   static constexpr int PLANE = NC * KT * 2;  // bytes per digit plane (8 KB)
   static constexpr int DBUF = 8 * PLANE;     // digit planes of a tile (64 KB)
@@ -71,7 +73,8 @@ struct XgShape {
 template <int NC, typename S>
 struct XgSmem {
   using Sh = XgShape<NC>;
-  // a staged tile: boxes of 128 bytes of rows x NC columns, 128-byte swizzle (see PipeSmem)
+  // a staged tile: boxes of 128 bytes of rows x NC columns, 128-byte swizzle (see PipeSmem);
+  // the right-hand side of least squares is staged apart, its rows in order
   static constexpr int RPB = 128 / (int)sizeof(S);
   static constexpr int NBOX = Sh::KT / RPB;
   static constexpr size_t kDig = 2 * (size_t)Sh::DBUF + 3 * (size_t)Sh::PAD;
@@ -79,13 +82,16 @@ struct XgSmem {
   static constexpr size_t kOffRaw = kDig;
   // (NC = 8: lanes 64..127 of the second buffer's MMAs read 64 KB past it, which must exist)
   static constexpr size_t kRawSpan = NC == 8 && 2 * kRaw < (size_t)Sh::DBUF ? (size_t)Sh::DBUF : 2 * kRaw;
-  static constexpr size_t kOffScale = kOffRaw + kRawSpan;
+  static constexpr size_t kStageB = sizeof(S) * (size_t)Sh::KT;
+  static constexpr size_t kOffB = kOffRaw + kRawSpan;
+  static constexpr size_t kOffScale = kOffB + 2 * kStageB;
   static constexpr size_t kOffColmax = kOffScale + 4 * NC;
   static constexpr size_t kOffMisc = kOffColmax + 4 * NC;
   static constexpr size_t kOffBar = (kOffMisc + 64 * 4 + 15) / 16 * 16;
   static constexpr size_t kOffSlot = kOffBar + 64;
   static constexpr size_t kBytes = kOffSlot + 32;
   static constexpr size_t kEpi = 8 * (4 * (size_t)NC * (NC + 1) + 8 * (NC + 1)) + 64 * 4 + 16;
+  static_assert(kBytes <= 232448, "shared memory of one SM");
   static_assert(kEpi <= kOffScale, "the epilogue's shared memory stays below the scales and barriers");
   static_assert(16 * (size_t)(Sh::LG - 1) * NC * NC <= (size_t)Sh::DBUF, "lane-group sums fit in a digit buffer");
 };
@@ -196,15 +202,41 @@ struct Rows8<float> {
   }
 };
 
-// One instruction descriptor for M = 128 and N columns.
-template <int N>
-QL_DEV constexpr uint32_t xg_idesc() {
-  return umma_idesc_bf16(128, N);
+// One lane of the (converged) warp: 1 in it, 0 in the others.
+QL_DEV uint32_t elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p;
+}
+QL_DEV void umma_bf16_if(uint32_t leader, uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %5, 0;\n"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(leader));
+}
+QL_DEV void umma_commit_if(uint32_t leader, uint64_t* mbar) {
+  asm volatile(
+      "{\n.reg .pred q;\nsetp.ne.b32 q, %1, 0;\n"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_addr(mbar)),
+      "r"(leader));
+}
+// The common case of a bounded wait: the phase is already over.
+QL_DEV bool mbar_wait_fast(uint64_t* mbar, uint32_t parity) {
+  return mbar_try_wait(mbar, parity) || mbar_wait_bounded(mbar, parity);
+}
+// One box of a rank-3 tensor map (x = row in its 128-byte block, y = column, z = block).
+QL_DEV void tma_load_3d(void* dst, const CUtensorMap* tm, int x, int y, int z, uint64_t* mbar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+      "[%5];\n" ::"r"(smem_addr(dst)),
+      "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(z), "r"(smem_addr(mbar))
+      : "memory");
 }
 
-// The MMAs of one tile (control thread): d0 is the descriptor of plane 0, k-step 0.
+// The MMAs of one tile (whole warp, issued by the elected lane): d0 is the descriptor of
+// plane 0, k-step 0.
 template <int NC>
-QL_DEV void xg_issue_mmas(uint32_t tbase, uint64_t d0, uint32_t fresh) {
+QL_DEV void xg_issue_mmas(uint32_t leader, uint32_t tbase, uint64_t d0, uint32_t fresh) {
   using Sh = XgShape<NC>;
   constexpr uint64_t PL = Sh::PLANE >> 4;
 #pragma unroll 1
@@ -212,23 +244,23 @@ QL_DEV void xg_issue_mmas(uint32_t tbase, uint64_t d0, uint32_t fresh) {
     const uint64_t dk = d0 + (uint64_t)((kk * 2 * Sh::LBO) >> 4);
     const uint32_t first = (!fresh || kk > 0) ? 1u : 0u;
     if constexpr (NC == 8) {
-      umma_bf16(tbase, dk, dk, xg_idesc<64>(), first);
+      umma_bf16_if(leader, tbase, dk, dk, umma_idesc_bf16(128, 64), first);
     } else if constexpr (NC == 16) {
-      umma_bf16(tbase, dk, dk, xg_idesc<128>(), first);
+      umma_bf16_if(leader, tbase, dk, dk, umma_idesc_bf16(128, 128), first);
     } else if constexpr (NC == 32) {
-      umma_bf16(tbase, dk, dk, xg_idesc<256>(), first);
-      umma_bf16(tbase + 256, dk + 4 * PL, dk, xg_idesc<256>(), first);
+      umma_bf16_if(leader, tbase, dk, dk, umma_idesc_bf16(128, 256), first);
+      umma_bf16_if(leader, tbase + 256, dk + 4 * PL, dk, umma_idesc_bf16(128, 256), first);
     } else {
 #pragma unroll
       for (int b = 0; b < 8; ++b) {
-        uint32_t acc = first;
+        bool opened = false;
 #pragma unroll
         for (int p = -1; p <= 7; ++p) {
           const int q = 2 * b - p;
           if (q >= 0 && q <= 7) {
-            umma_bf16(tbase + (uint32_t)(b * 64), dk + (uint64_t)(int64_t)(p * (int64_t)PL), dk + (uint64_t)q * PL,
-                      xg_idesc<64>(), acc);
-            acc = 1u;
+            umma_bf16_if(leader, tbase + (uint32_t)(b * 64), dk + (uint64_t)(int64_t)(p * (int64_t)PL),
+                         dk + (uint64_t)q * PL, umma_idesc_bf16(128, 64), opened ? 1u : first);
+            opened = true;
           }
         }
       }
@@ -361,8 +393,8 @@ QL_DEV double wide_to_double(const Wide320& a, int e) {
 // operation and nothing to cancellation.  Integer multiplies run on the ALUs at full rate,
 // where FP64 (1/64 of the FP32 rate) or double-double would not: a double-double version of
 // the same factorisation needs about 0.9 M FP64 operations at n = 64, 0.2 ms on one SM.
-// 1 / sqrt(pivot) comes from FP64 with one double-double Newton step (relative 2^-103), by
-// one lane, while the other warps update the trailing rows.  A pivot below 2^-80 of its
+// 1 / sqrt(pivot) is formed in integers too, by one lane, while the other warps update the
+// trailing rows (a chain of dependent FP64 instructions took several times as long).  A pivot below 2^-80 of its
 // column (kappa above about 2^40), zero or negative stops the factorisation; a column that
 // is zero altogether gives a zero row of R.
 // ---------------------------------------------------------------------------------------
@@ -384,6 +416,8 @@ struct FxPivot {
   int x;
   int ok;  // 1: usable; 0: zero column; -1: pivot too small
 };
+// y ~ 1 / sqrt(f): single precision, one Newton step in 64-bit fixed point (2^-44), then one
+// third-order step y (1 + e / 2 + 3 e^2 / 8), e = 1 - f y^2, in 128 bits (2^-118).
 QL_DEV FxPivot fx_pivot(i128 d, bool zero_column) {
   FxPivot pv{0, 0, 0};
   if (zero_column) return pv;
@@ -394,20 +428,20 @@ QL_DEV FxPivot fx_pivot(i128 d, bool zero_column) {
   // d = 2^-2z f, f in [1/4, 1)
   const u64 hi = (u64)((u128)d >> 64);
   const int lead = hi ? __clzll((long long)hi) : 64 + __clzll((long long)(u64)d);  // of 128 bits
-  const int z = (lead - (128 - kFx)) >> 1;  // d < 2^(128 - lead - kFx)
+  const int z = (lead - (128 - kFx)) >> 1;
   const u128 f = (u128)d << (2 * z);
-  const u64 fh = (u64)(f >> 72);  // 53 bits at most: exact in a double
-  const double dh = (double)fh * 0x1p-53;
-  const double dl = (double)(u64)((f >> 19) & ((((u64)1) << 53) - 1)) * 0x1p-106;
-  const double r0 = rsqrt(dh);
-  const double th = r0 * r0, tl = fma(r0, r0, -th);
-  const double p = dh * th, pe = fma(dh, th, -p);
-  const double e = (1.0 - p) - (pe + fma(dh, tl, dl * th));
-  const double r1 = 0.5 * r0 * e;  // r0 in (1, 2]
-  // r / 2 in fixed point
-  i128 r = (i128)((u128)(u64)(r0 * 0x1p52) << (kFx - 53));
-  r += (i128)__double2ll_rn(r1 * 0x1p104) * ((i128)1 << (kFx - 105));
-  pv.r = r;
+  const u64 f64 = (u64)(f >> (kFx - 64));  // f 2^64
+  const float y0 = rsqrtf((float)(unsigned)(f64 >> 40) * 0x1p-24f);
+  const u64 y = (u64)(unsigned)(y0 * 0x1p23f) << 39;  // y 2^62
+  const long long e1 = (long long)((1ull << 60) - umul_hi(f64, umul_hi(y, y)));  // (1 - f y^2) 2^60
+  const u64 d1 = umul_hi(y, e1 < 0 ? (u64)-e1 : (u64)e1) << 3;                   // |y e / 2| 2^62
+  const u64 y1 = e1 < 0 ? y - d1 : y + d1;
+  const i128 t = (i128)(((u128)y1 * y1) >> 1);  // y^2 / 4
+  const i128 e = ((i128)1 << kFx) - fx_mul((i128)f, t) * 4;
+  const long long e64 = (long long)(e >> 20);   // e 2^105
+  const i128 e2 = (i128)(__mul64hi(e64, e64) >> 21);  // e^2
+  const i128 h = (i128)y1 << 62;                // y / 2
+  pv.r = h + fx_mul(h, (e >> 1) + (e2 * 3 >> 3));
   pv.x = z + 1;
   pv.ok = 1;
   return pv;
@@ -457,9 +491,6 @@ QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double
     for (int j = k + tid; j < n; j += T) {  // row k of R
       const i128 v = pv.ok ? fx_mul(get(k, j) << pv.x, pv.r) : (i128)0;
       put(k, j, v);
-      const u128 mag = v < 0 ? (u128)-v : (u128)v;
-      const double d = mag_to_double(mag, sj[j] - kFx + kXgUnitExp / 2);
-      Rout[k * LE + j] = v < 0 ? -d : d;
     }
     __syncthreads();
     if (warp == 0) {  // the next row, then its pivot
@@ -477,8 +508,16 @@ QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double
     }
     __syncthreads();
   }
-  for (int e = tid; e < n * n; e += T)
-    if (e / n > e % n) Rout[(e / n) * LE + e % n] = 0.0;
+  for (int i = warp; i < n; i += NW)
+    for (int j = lane; j < n; j += 32) {
+      double r = 0.0;
+      if (j >= i) {
+        const i128 v = get(i, j);
+        r = mag_to_double(v < 0 ? (u128)-v : (u128)v, sj[j] - kFx + kXgUnitExp / 2);
+        if (v < 0) r = -r;
+      }
+      Rout[i * LE + j] = r;
+    }
   __syncthreads();
   return 0;
 }
@@ -524,8 +563,7 @@ QL_DEV void xg_finish(const GramArgs<S>& a, unsigned char* smem, const int* colm
 // Row tiles [tiles bid / k, tiles (bid + 1) / k) of one problem; tensor memory at tbase and
 // barriers set up by xg_cta_begin, phases carried in bars (see gram_pipe_body).
 template <int NC, typename S>
-QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& bars, const CUtensorMap* tmA,
-                       const CUtensorMap* tmB) {
+QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& bars, const XgMaps* maps) {
   using Sh = XgShape<NC>;
   using Sm = XgSmem<NC, S>;
   constexpr int T = Sh::T, TS = Sh::TS, KT = Sh::KT, PLANE = Sh::PLANE, SBO = Sh::SBO, LBO = Sh::LBO, HALF = Sh::HALF,
@@ -533,9 +571,10 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
   extern __shared__ __align__(1024) unsigned char smem_umma[];
   unsigned char* smem = smem_umma;
   const int tid = threadIdx.x, n = a.n, lane = tid & 31, warp = tid >> 5;
-  const bool control = warp == TS / 32;
+  const bool control = warp >= TS / 32;  // copy warp, MMA warp
   auto digits = [&](int b) { return smem + Sh::PAD + (size_t)b * (Sh::DBUF + Sh::PAD); };
   unsigned char* raw0 = smem + Sm::kOffRaw;
+  unsigned char* rhs0 = smem + Sm::kOffB;
   int* scale = reinterpret_cast<int*>(smem + Sm::kOffScale);
   int* colmax = reinterpret_cast<int*>(smem + Sm::kOffColmax);
   int* misc = reinterpret_cast<int*>(smem + Sm::kOffMisc);
@@ -544,14 +583,14 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
   uint64_t* dbar = mbar + 4;                                          // [2] digits ready, per digit buffer
   uint64_t* rbar = mbar + 6;                                          // [2] stage read, per raw stage
   int* ngrp = reinterpret_cast<int*>(smem + Sm::kOffSlot + 4);        // [2] tile opens a new group
-  int* sfail = ngrp + 2;                                              // [2] where each role gave up
+  int* sfail = ngrp + 2;                                              // [3] where each role gave up
 
   a.tiles = (a.m + KT - 1) / KT;
   for (int i = tid; i < NC; i += T) {
     colmax[i] = 0;
     scale[i] = 0;
   }
-  if (tid < 2) sfail[tid] = 0;
+  if (tid < 3) sfail[tid] = 0;
   if constexpr (Sh::PAD > 0) {
     for (int z = 0; z < 3; ++z)
       for (int i = tid; i < Sh::PAD / 16; i += T)
@@ -579,21 +618,31 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
   const bool reader = !control && lg < LG;
   ulonglong2* acc = reinterpret_cast<ulonglong2*>(a.w.fbuf) + (size_t)bid * NC * 128;  // [column][lane]
 
-  if (control) {
-    // ---- control warp: copies two tiles ahead; per tile, once the slicers have read its
-    // stage, the copy two ahead into it; once its digits are ready, the MMAs
+  if (warp == TS / 32) {
+    // ---- copy warp: two tiles ahead; once the slicers have read a stage, the copy two ahead
+    // goes into it.  A full tile is one box of the rank-3 map; the last one of the matrix,
+    // whose rows end inside it, is copied by 128-byte row blocks (zeros past m).
     bool ok = true;
     uint32_t pend = 0u, ppar = 0u;  // bit b: a copy into stage b in flight, and its phase parity
+    const uint32_t leader = elect_one();
+    const bool has_b = a.src.nA < n;
     auto copy = [&](int64_t t, int b) {
       if (!bulk) return;
       unsigned char* stage = raw0 + (size_t)b * Sm::kRaw;
-      const int row0 = (int)(t * KT);
-      if (lane == 0) {
-        mbar_arrive_expect_tx(&lbar[b], (uint32_t)(NBOX * n * 128));
+      unsigned char* rhs = rhs0 + (size_t)b * Sm::kStageB;
+      const int64_t row0 = t * KT;
+      if (leader) {
+        if (maps->full && row0 + KT <= a.m) {
+          mbar_arrive_expect_tx(&lbar[b], (uint32_t)(Sm::kRaw + (has_b ? Sm::kStageB : 0)));
+          tma_load_3d(stage, &maps->tile, 0, 0, (int)(row0 / RPB), &lbar[b]);
+          if (has_b) bulk_g2s(rhs, a.src.b + row0, (uint32_t)Sm::kStageB, &lbar[b]);
+        } else {
+          mbar_arrive_expect_tx(&lbar[b], (uint32_t)(NBOX * n * 128));
 #pragma unroll 1
-        for (int kb = 0; kb < NBOX; ++kb) {
-          tma_load_2d(stage + (size_t)kb * NC * 128, tmA, row0 + kb * RPB, 0, &lbar[b]);
-          if (tmB) tma_load_2d(stage + (size_t)(kb * NC + a.src.nA) * 128, tmB, row0 + kb * RPB, 0, &lbar[b]);
+          for (int kb = 0; kb < NBOX; ++kb) {
+            tma_load_2d(stage + (size_t)kb * NC * 128, &maps->rows, (int)row0 + kb * RPB, 0, &lbar[b]);
+            if (has_b) tma_load_2d(rhs + (size_t)kb * 128, &maps->rhs, (int)row0 + kb * RPB, 0, &lbar[b]);
+          }
         }
       }
       __syncwarp();
@@ -605,29 +654,35 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
     if (t0 + 1 < t1) copy(t0 + 1, 1);
     for (int64_t t = t0; t < t1; ++t) {
       const int b = (int)((t - t0) & 1);
-      if (!__all_sync(0xffffffffu, mbar_wait_bounded(&rbar[b], (bars.mpar >> b) & 1u))) {
-        ok = false;
-        break;
-      }
-      pend &= ~(1u << b);
-      if (t + 2 < t1) copy(t + 2, b);
-      if (!__all_sync(0xffffffffu, mbar_wait_bounded(&dbar[b], (bars.mpar >> b) & 1u))) {
+      if (!__all_sync(0xffffffffu, mbar_wait_fast(&rbar[b], (bars.mpar >> b) & 1u))) {
         ok = false;
         break;
       }
       bars.mpar ^= 1u << b;
-      tc_fence_after();
-      if (lane == 0) {
-        // planes and k-steps add (byte offset >> 4) to the 14-bit address field, which stays
-        // below 2^14 (shared addresses < 256 KB); plane -1 is the zero plane before the buffer
-        xg_issue_mmas<NC>(tbase, umma_sdesc(smem_addr(digits(b)), LBO, SBO), (uint32_t)ngrp[b]);
-        umma_commit(&mbar[b]);
-      }
-      __syncwarp();
+      pend &= ~(1u << b);
+      if (t + 2 < t1) copy(t + 2, b);
     }
     for (int b = 0; b < 2; ++b)  // no copy may still be writing when the CTA moves on
       if (pend & (1u << b)) mbar_wait_bounded(&lbar[b], (ppar >> b) & 1u);
     if (!ok && lane == 0) sfail[1] = 2;
+  } else if (control) {
+    // ---- MMA warp: once a tile's digits are ready, its MMAs.  Planes and k-steps add (byte
+    // offset >> 4) to the 14-bit address field, which stays below 2^14 (shared addresses
+    // < 256 KB); plane -1 is the zero plane before the buffer.
+    const uint32_t leader = elect_one();
+    const uint64_t d0 = umma_sdesc(smem_addr(digits(0)), LBO, SBO);
+    for (int64_t t = t0; t < t1; ++t) {
+      const int b = (int)((t - t0) & 1);
+      if (!__all_sync(0xffffffffu, mbar_wait_fast(&dbar[b], (bars.mpar >> b) & 1u))) {
+        if (lane == 0) sfail[2] = 2;
+        break;
+      }
+      bars.mpar ^= 1u << b;
+      tc_fence_after();
+      xg_issue_mmas<NC>(leader, tbase, d0 + (uint64_t)b * ((Sh::DBUF + Sh::PAD) >> 4), (uint32_t)ngrp[b]);
+      umma_commit_if(leader, &mbar[b]);
+      __syncwarp();
+    }
   } else {
     // ---- slicer warps
     bool ok = true;
@@ -727,6 +782,12 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
       return slicer_and<TS>(mbar_wait_bounded(&mbar[last_b], (cpar >> last_b) & 1u));
     };
 
+    // where this unit lies in a staged tile: its 128-byte line and first 16-byte chunk, or the
+    // rows of the right-hand side
+    const bool rhs_unit = cu == a.src.nA;
+    const unsigned char* line0 = rhs_unit ? rhs0 + r0 * sizeof(S) : raw0 + (size_t)((r0 / RPB) * NC + cu) * 128;
+    const size_t line_step = rhs_unit ? Sm::kStageB : Sm::kRaw;
+    const int q0 = rhs_unit ? 0 : (r0 % RPB) * (int)sizeof(S) / 16, swz = rhs_unit ? 0 : (cu & 7);
     Rows8<S> v, ahead;
     auto load_global = [&](Rows8<S>& w, int64_t t) {
       const S* col = a.src.col(cu) + t * KT + r0;
@@ -740,7 +801,7 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
       const int i = (int)(t - t0), b = i & 1;
       bool landed = true;
       if (bulk) {
-        landed = mbar_wait_bounded(&lbar[b], (bars.lpar >> b) & 1u);
+        landed = mbar_wait_fast(&lbar[b], (bars.lpar >> b) & 1u);
         bars.lpar ^= 1u << b;
       }
       unsigned am = 0;
@@ -748,8 +809,7 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
       bool over = false;
       if (live) {
         if (bulk) {
-          const unsigned char* line = raw0 + (size_t)b * Sm::kRaw + (size_t)((r0 / RPB) * NC + cu) * 128;
-          const int q0 = (r0 % RPB) * (int)sizeof(S) / 16, swz = cu == a.src.nA ? 0 : (cu & 7);
+          const unsigned char* line = line0 + (size_t)b * line_step;
 #pragma unroll
           for (int q = 0; q < 8 * (int)sizeof(S) / 16; ++q)
             v.chunk(q, *reinterpret_cast<const uint4*>(line + (((q0 + q) ^ swz) << 4)));
@@ -762,12 +822,11 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
         es = Rows8<S>::exponent(am);
         over = es > scale[cu];
       }
-      // stage b is read: the control warp may copy the tile two ahead into it
-      fence_proxy_async_smem();
+      // stage b is read: the copy warp may copy the tile two ahead into it
       __syncwarp();
       if (lane == 0) mbar_arrive(&rbar[b]);
       // digit buffer b is free once the MMAs of tile t - 2 are done
-      const bool okw = i >= 2 ? mbar_wait_bounded(&mbar[b], (cpar >> b) & 1u) : true;
+      const bool okw = i >= 2 ? mbar_wait_fast(&mbar[b], (cpar >> b) & 1u) : true;
       const bool full = grp >= Sh::G;
       if (slicer_or<TS>(over || !okw || !landed) || full) {
         if (!slicer_and<TS>(landed)) {  // the copy engine did not deliver
@@ -846,7 +905,7 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
   }
   tc_fence_before();
   __syncthreads();
-  const int fw = sfail[0] ? sfail[0] : sfail[1];
+  const int fw = sfail[0] ? sfail[0] : (sfail[1] ? sfail[1] : sfail[2]);
   if (fw) {
     bars.ok = false;  // a late arrival may still complete a phase: the CTA takes no more work
     if (tid == 0) {   // the gated launches redo the call and report {QL_ERR_TIMEOUT, where}
@@ -877,12 +936,11 @@ QL_DEV uint32_t xg_cta_begin(unsigned char* smem) {
 
 template <int NC, typename S>
 __global__ void __launch_bounds__(XgShape<NC>::T, 1)
-    xgram_kernel(const __grid_constant__ GramArgs<S> a, const __grid_constant__ CUtensorMap tmA,
-                 const __grid_constant__ CUtensorMap tmB, int has_b) {
+    xgram_kernel(const __grid_constant__ GramArgs<S> a, const __grid_constant__ XgMaps maps) {
   extern __shared__ __align__(1024) unsigned char smem_umma[];
   const uint32_t tbase = xg_cta_begin<NC, S>(smem_umma);
   PipeBars bars;
-  xgram_body<NC, S>(a, blockIdx.x, gridDim.x, tbase, bars, &tmA, has_b ? &tmB : nullptr);
+  xgram_body<NC, S>(a, blockIdx.x, gridDim.x, tbase, bars, &maps);
   tc_fence_before();
   __syncthreads();
   if ((threadIdx.x >> 5) == 0) tmem_dealloc(tbase, XgShape<NC>::TCOLS);
@@ -927,15 +985,14 @@ ql_status xgram_launch_one(const GramCall& c, const GramWs& w) {
   a.resnorm = c.resnorm;
   a.Rext = c.Rext;
   a.info = c.info;
-  CUtensorMap tmA{}, tmB{};
-  const bool has_b = c.nA < c.n;
-  a.bulk = pipe_tensor_maps(&tmA, has_b ? &tmB : nullptr, c.A, c.b, std::is_same<S, double>::value ? QL_F64 : QL_F32,
-                            c.m, c.nA, c.lda)
+  XgMaps maps{};
+  a.bulk = xg_tensor_maps(&maps, NC, c.A, c.nA < c.n ? c.b : nullptr,
+                          std::is_same<S, double>::value ? QL_F64 : QL_F32, c.m, c.nA, c.lda)
                ? 1
                : 0;
   a.mround = NC >= 16 ? 2 : 1;  // how the next pass's kernel of this class reads M
   count_launch();
-  kern<<<(int)g, Sh::T, Sm::kBytes, c.stream>>>(a, tmA, tmB, has_b ? 1 : 0);
+  kern<<<(int)g, Sh::T, Sm::kBytes, c.stream>>>(a, maps);
   return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
