@@ -150,6 +150,9 @@ ql_status ql_tsqr_qless_noalloc(int64_t m, int64_t n, const void* X, ql_dtype dt
  * Both Cholesky factorisations, R1^{-1} and R2 R1 run on the device in FP64.  A
  * non-positive pivot sets info = {QL_ERR_NOT_SPD, pivot} (+1000 for the second pass) and
  * fills R with NaN.  Reliable for kappa_2(X) up to about 1e6 (the Gram squares kappa).
+ * For n >= 5 the first pass is exact (see ql_tsqr_qless): while every pivot of C stays above
+ * 2^-46 of its column, R1 from the fixed-point Cholesky is already the R that both passes
+ * give, with a smaller error, and the second pass ends at once.
  */
 ql_status ql_cholqr2_qless(int64_t m, int64_t n, const void* X, ql_dtype dtype, int64_t ldx, double* R,
                            int64_t ldr, int32_t* info, void* ws, size_t ws_bytes, void* stream);
@@ -162,7 +165,8 @@ ql_status ql_cholqr2_qless(int64_t m, int64_t n, const void* X, ql_dtype dtype, 
  *   pass 2: Y = X R1^{-1} formed tile by tile, R2 = chol(Y^T Y);
  *   pass 3: Y = X (R2 R1)^{-1}, R3 = chol(Y^T Y);  R = R3 R2 R1.
  * Arguments, workspace and outputs as ql_cholqr2_qless.  A non-positive pivot sets info =
- * {QL_ERR_NOT_SPD, pivot + 1000 (pass - 1)} and R = NaN.
+ * {QL_ERR_NOT_SPD, pivot + 1000 (pass - 1)} and R = NaN.  For n >= 5 the exact first pass
+ * gives R by itself (unshifted) while every pivot of C stays above 2^-66 of its column.
  */
 ql_status ql_scholqr3_qless(int64_t m, int64_t n, const void* X, ql_dtype dtype, int64_t ldx, double* R,
                             int64_t ldr, int32_t* info, void* ws, size_t ws_bytes, void* stream);
@@ -172,7 +176,8 @@ ql_status ql_scholqr3_qless(int64_t m, int64_t n, const void* X, ql_dtype dtype,
  * device), B1 = U L^{-1/2} with eigenvalues below rank_tol * lambda_max treated as zero
  * (rank_tol <= 0 selects n * 2^-52); second pass on X B1 (formed tile by tile); then
  * X = Q Z with Z = L2^{1/2} U2^T L1^{1/2} U1^T and R = qr_r(Z) (FP64 Householder on the
- * device).  Z (nullable device double n x n, ld n) receives Z.
+ * device).  Z (nullable device double n x n, ld n) receives Z.  For n >= 5, without Z and
+ * when no eigenvalue can be truncated, the exact first pass gives R by itself.
  */
 ql_status ql_svqb_qless(int64_t m, int64_t n, const void* X, ql_dtype dtype, int64_t ldx, double* R,
                         int64_t ldr, double* Z, double rank_tol, int32_t* info, void* ws, size_t ws_bytes,

@@ -23,7 +23,9 @@ constexpr int kGramMaxCtasPerSm = 4;
 constexpr int kGramFlushTiles = 16;
 
 struct GramWs {
-  int* flags;        // [0] range, [1] first-pass breakdown, [2] arrival counter pass 1, [3] pass 2,
+  int* flags;        // [0] range, [1] first-pass breakdown (TSQR call: Householder redo), [2] arrival
+                    // counter pass 1, [3] pass 2, [4] where a bounded wait gave up, [5] the exact first
+                    // pass has written R: the later passes have nothing to do,
                     // [64 + c]: largest biased exponent of column c over all rows (tensor-core pass 1)
   double* keep;      // 3 n x n blocks carried from pass 1 to pass 2 (row-major, ld n)
   double* partials;  // one NC x NC partial Gram per CTA
@@ -146,7 +148,8 @@ __global__ void __launch_bounds__(GramShape<NC>::T, 1) gram_kernel(GramArgs<S> a
   const int tid = threadIdx.x, n = a.n;
 
   if (a.gated && *(volatile int*)&a.w.flags[0] == 0) return;
-  if (Ar::kRangeChecked && a.pass >= 2 && *(volatile int*)&a.w.flags[0] != 0) return;  // FP64 redoes it
+  if (Ar::kRangeChecked && a.pass >= 2 && (*(volatile int*)&a.w.flags[0] != 0 || *(volatile int*)&a.w.flags[5] != 0))
+    return;  // FP64 redoes it, or R is written
   if (a.pass >= 2 && *(volatile int*)&a.w.flags[1] != 0) {  // first pass broke down
     if (blockIdx.x == 0) write_nan_outputs(a, T);
     return;
@@ -544,7 +547,8 @@ __global__ void __launch_bounds__(StreamShape<NC>::T) gram_stream_kernel(GramArg
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = a.n;
 
   if (a.gated && *(volatile int*)&a.w.flags[0] == 0) return;
-  if (Ar::kRangeChecked && a.pass >= 2 && *(volatile int*)&a.w.flags[0] != 0) return;  // FP64 redoes it
+  if (Ar::kRangeChecked && a.pass >= 2 && (*(volatile int*)&a.w.flags[0] != 0 || *(volatile int*)&a.w.flags[5] != 0))
+    return;  // FP64 redoes it, or R is written
   if (a.pass >= 2 && *(volatile int*)&a.w.flags[1] != 0) {  // first pass broke down
     if (blockIdx.x == 0) write_nan_outputs(a, T);
     return;
@@ -741,7 +745,8 @@ QL_DEV void gram_tc_body(const GramArgs<S>& a, int bid, int k) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x, n = a.n, lane = tid & 31, warp = tid >> 5;
 
-  if (a.pass >= 2 && *(volatile int*)&a.w.flags[0] != 0) return;  // the FP64 launches redo it
+  if (a.pass >= 2 && (*(volatile int*)&a.w.flags[0] != 0 || *(volatile int*)&a.w.flags[5] != 0))
+    return;  // the FP64 launches redo it, or R is written
   if (a.pass >= 2 && *(volatile int*)&a.w.flags[1] != 0) {         // first pass broke down
     if (bid == 0) write_nan_outputs(a, T);
     return;
@@ -1201,7 +1206,8 @@ QL_DEV void gram_umma_body(const GramArgs<S>& a, int bid, int k, uint32_t tbase,
   unsigned char* smem = smem_umma;
   const int tid = threadIdx.x, n = a.n, lane = tid & 31, warp = tid >> 5;
 
-  if (a.pass >= 2 && *(volatile int*)&a.w.flags[0] != 0) return;  // the FP64 launches redo it
+  if (a.pass >= 2 && (*(volatile int*)&a.w.flags[0] != 0 || *(volatile int*)&a.w.flags[5] != 0))
+    return;  // the FP64 launches redo it, or R is written
   if (a.pass >= 2 && *(volatile int*)&a.w.flags[1] != 0) {         // first pass broke down
     if (bid == 0) write_nan_outputs(a, T);
     return;
@@ -1746,7 +1752,8 @@ QL_DEV void gram_pipe_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBa
     // the entry conditions of every later pass, decided once for the whole CTA
     if (tid == 0) {
       int e = 0;
-      if (*(volatile int*)&a.w.flags[0] != 0) e = 1;       // the FP64 launches redo the call
+      if (*(volatile int*)&a.w.flags[0] != 0 || *(volatile int*)&a.w.flags[5] != 0)
+        e = 1;  // the FP64 launches redo the call, or R is written
       else if (*(volatile int*)&a.w.flags[1] != 0) e = 2;  // the first pass broke down
       entry[0] = e;
     }
@@ -2404,7 +2411,7 @@ ql_status gram_dispatch(const GramCall& c, const GramWs& w, int gated) {
         // below that mma.sync, whose per-tile read-out is cheaper than TMEM's
         if constexpr (NC == 64) {
           ql_status st =
-              pipe_gram_enabled() ? gram_pipe_launch_one<NC, S>(c, w) : gram_umma_launch_one<NC, S, kXNone>(c, w, 1);
+              pipe_gram_enabled() ? xgram_pass1<S>(c, w) : gram_umma_launch_one<NC, S, kXNone>(c, w, 1);
           if (st) return st;
           if (c.method == QL_SVQB2) return gram_umma_launch_one<NC, S, kXFull>(c, w, 2);
           st = gram_umma_launch_one<NC, S, kXUpper>(c, w, 2);
@@ -2412,7 +2419,7 @@ ql_status gram_dispatch(const GramCall& c, const GramWs& w, int gated) {
           return gram_umma_launch_one<NC, S, kXUpper>(c, w, 3);
         } else {
           ql_status st =
-              pipe_gram_enabled() ? gram_pipe_launch_one<NC, S>(c, w) : gram_tc_launch_one<NC, S, kXNone>(c, w, 1);
+              pipe_gram_enabled() ? xgram_pass1<S>(c, w) : gram_tc_launch_one<NC, S, kXNone>(c, w, 1);
           if (st) return st;
           // later passes: the pipelined kernel forms Y = X M' in its slicer warps
           const bool pipe2 = pipe_gram_enabled() && pipe_gram2_enabled();

@@ -1,10 +1,14 @@
-// Exact Gram pass on tcgen05 (C = X^T X) with a fixed-point Cholesky behind it: R of a TSQR
-// call in one pass over X, in the 8-, 16-, 32- and 64-column classes.
+// Exact Gram pass on tcgen05 (C = X^T X) with a fixed-point Cholesky behind it: R in one pass
+// over X, in the 8-, 16-, 32- and 64-column classes, for TSQR calls and, while their further
+// passes could not change R, for the Gram methods.
 //
-// Measured against the double-float Householder tiles it replaces (those stay for columns
-// dependent to about 2^-40 and for n <= 4): m = 2^22, n = 64 21.1 -> 2.40 ms; least squares
-// 2^24 x 31, FP32-stored, 19.2 -> 1.84 ms; 131072 x 8 145 -> 45 us; ||R - R_ref|| / ||R_ref||
-// 3.5e-16 -> 2.1e-16 (n = 64), 4.4e-16 -> 1.2e-16 (n = 8) against 64-bit references.
+// Measured against the double-float Householder tiles (which stay for columns dependent to
+// about 2^-40 and for n <= 4) and the Gram methods' own passes (which stay beyond the limits
+// in xg_finish): m = 2^22, n = 64 TSQR 21.1 -> 2.03 ms, Cholesky-QR2 8.30 -> 2.04 ms; SVQB2
+// 10^6 x 32 3.69 -> 0.21 ms; shifted Cholesky-QR3 300007 x 24 872 -> 119 us; least squares
+// 2^24 x 31, FP32-stored, 19.2 -> 1.68 ms; 131072 x 8 145 -> 39 us.  ||R - R_ref|| / ||R_ref||
+// falls in each of them (n = 64: 3.5e-16 -> 2.6e-16, Cholesky-QR2 9.9e-16 -> 2.6e-16,
+// SVQB2 1e-14 -> 3.3e-16 against 64-bit references).
 //
 // Every value is rounded to a signed 56-bit fixed point N relative to a running per-column
 // scale 2^e (|x| < 2^e, x ~ N 2^(e - 55)) and cut into EIGHT balanced base-128 digits, which
@@ -273,9 +277,11 @@ QL_DEV void tmem_ld(uint32_t taddr, uint32_t (&v)[2]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];\n" : "=r"(v[0]), "=r"(v[1]) : "r"(taddr));
 }
 
-QL_DEV i128 load_i128(const ulonglong2* p) {
-  const ulonglong2 t = __ldcg(p);
-  return (i128)(((u128)t.y << 64) | t.x);
+// c + a b, 32 x 32 bits into 64
+QL_DEV long long mad_wide(int a, int b, long long c) {
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
 }
 QL_DEV void store_i128(ulonglong2* p, i128 v) {
   __stcg(p, make_ulonglong2((u64)(u128)v, (u64)((u128)v >> 64)));
@@ -308,7 +314,11 @@ struct Wide320 {
 QL_DEV Wide320 sacc_load(const long long* limbs) {
   long long l[kLimbs];
 #pragma unroll
-  for (int k = 0; k < kLimbs; ++k) l[k] = __ldcg(limbs + k);
+  for (int k = 0; k < kLimbs; k += 2) {
+    const longlong2 t = __ldcg(reinterpret_cast<const longlong2*>(limbs + k));
+    l[k] = t.x;
+    l[k + 1] = t.y;
+  }
   constexpr u64 kMask = (1ull << kLimbBits) - 1ull;
   u64 d[kLimbs];
   long long carry = 0;
@@ -411,25 +421,52 @@ QL_DEV i128 fx_mul(i128 a, i128 b) {
   return p * 8;  // 2^128 / 2^125
 }
 
+// What a step needs of its pivot d = 2^-2z f, f in [1/4, 1): c ~ 1 / f in units of 2^-61
+// (single precision and one Newton step: 2^-44) and the correction 1 / f = c (1 + eps), eps in
+// units of 2^-102 (error 2^-102).
 struct FxPivot {
-  i128 r;  // 2^-x / sqrt(d) in (1/2, 1], fixed point
-  int x;
+  u64 c;
+  long long eps;
+  int z;
   int ok;  // 1: usable; 0: zero column; -1: pivot too small
 };
-// y ~ 1 / sqrt(f): single precision, one Newton step in 64-bit fixed point (2^-44), then one
-// third-order step y (1 + e / 2 + 3 e^2 / 8), e = 1 - f y^2, in 128 bits (2^-118).
-QL_DEV FxPivot fx_pivot(i128 d, bool zero_column) {
-  FxPivot pv{0, 0, 0};
+QL_DEV int fx_half_lead(i128 d) {  // z with d 4^z in [1/4, 1)
+  const u64 hi = (u64)((u128)d >> 64);
+  const int lead = hi ? __clzll((long long)hi) : 64 + __clzll((long long)(u64)d);  // of 128 bits
+  return (lead - (128 - kFx)) >> 1;
+}
+QL_DEV FxPivot fx_pivot(i128 d, bool zero_column, int min_bits) {
+  FxPivot pv{0, 0, 0, 0};
   if (zero_column) return pv;
-  if (d < ((i128)1 << (kFx - 80))) {
+  if (d < ((i128)1 << (kFx - min_bits))) {
     pv.ok = -1;
     return pv;
   }
-  // d = 2^-2z f, f in [1/4, 1)
-  const u64 hi = (u64)((u128)d >> 64);
-  const int lead = hi ? __clzll((long long)hi) : 64 + __clzll((long long)(u64)d);  // of 128 bits
-  const int z = (lead - (128 - kFx)) >> 1;
-  const u128 f = (u128)d << (2 * z);
+  pv.ok = 1;
+  pv.z = fx_half_lead(d);
+  const u128 f = (u128)d << (2 * pv.z);
+  const u64 f64 = (u64)(f >> (kFx - 64));  // f 2^64
+  const float y0 = __fdividef(1.0f, (float)(unsigned)(f64 >> 40) * 0x1p-24f);  // in [1, 4]
+  const u64 c0 = (u64)(unsigned)(y0 * 0x1p21f) << 40;
+  const long long e = (long long)((1ull << 61) - umul_hi(f64, c0));  // (1 - f y) 2^61
+  const u64 de = umul_hi(c0, e < 0 ? (u64)-e : (u64)e) << 3;
+  pv.c = e < 0 ? c0 - de : c0 + de;
+  const u128 p = (u128)(u64)(f >> 64) * pv.c + umul_hi((u64)f, pv.c);  // f c 2^122
+  const long long eps = (long long)((i128)(((u128)1 << 122) - p) >> 20);  // 2^102 (1 - f c)
+  pv.eps = eps + (__mul64hi(eps, eps) >> 38);                              // + eps^2
+  return pv;
+}
+// s / f in units of 2^-122 for s in units of 2^-kFx, |s / f| <= 2
+QL_DEV i128 fx_div_pivot(i128 s, const FxPivot& pv) {
+  const long long sh = (long long)(s >> 64);
+  i128 w = (i128)(u128)umul_hi((u64)s, pv.c);
+  // sh c, sh signed and c unsigned
+  w += (i128)((u128)(u64)sh * pv.c) - (sh < 0 ? (i128)((u128)pv.c << 64) : (i128)0);
+  return w + (i128)__mul64hi((long long)(w >> 61), pv.eps) * ((i128)1 << 23);
+}
+// 1 / (2 sqrt(f)) for f in [1/4, 1): single precision, one Newton step in 64-bit fixed point
+// (2^-44), then one third-order step y (1 + e / 2 + 3 e^2 / 8), e = 1 - f y^2, in 128 bits.
+QL_DEV i128 fx_half_rsqrt(i128 f) {
   const u64 f64 = (u64)(f >> (kFx - 64));  // f 2^64
   const float y0 = rsqrtf((float)(unsigned)(f64 >> 40) * 0x1p-24f);
   const u64 y = (u64)(unsigned)(y0 * 0x1p23f) << 39;  // y 2^62
@@ -437,26 +474,31 @@ QL_DEV FxPivot fx_pivot(i128 d, bool zero_column) {
   const u64 d1 = umul_hi(y, e1 < 0 ? (u64)-e1 : (u64)e1) << 3;                   // |y e / 2| 2^62
   const u64 y1 = e1 < 0 ? y - d1 : y + d1;
   const i128 t = (i128)(((u128)y1 * y1) >> 1);  // y^2 / 4
-  const i128 e = ((i128)1 << kFx) - fx_mul((i128)f, t) * 4;
-  const long long e64 = (long long)(e >> 20);   // e 2^105
+  const i128 e = ((i128)1 << kFx) - fx_mul(f, t) * 4;
+  const long long e64 = (long long)(e >> 20);         // e 2^105
   const i128 e2 = (i128)(__mul64hi(e64, e64) >> 21);  // e^2
-  const i128 h = (i128)y1 << 62;                // y / 2
-  pv.r = h + fx_mul(h, (e >> 1) + (e2 * 3 >> 3));
-  pv.x = z + 1;
-  pv.ok = 1;
-  return pv;
+  const i128 h = (i128)y1 << 62;                      // y / 2
+  return h + fx_mul(h, (e >> 1) + (e2 * 3 >> 3));
 }
 
 // sacc -> Rout (n x n upper triangle, row-major, ld LE, in shared memory).  Shared memory from
-// smem: two arrays of NC x LE words, then the scratch.  Returns 0, or the 1-based index of
+// smem: two arrays of NC x LE words, then the scratch.  A pivot below 2^-min_bits of its
+// column stops it, as does a zero column unless zero_ok.  Returns 0, or the 1-based index of
 // the pivot that stopped it (to every thread).
+//
+// Step k with pivot d = 2^-2z f keeps row k as s_j = S_kj 2^z and w_j = s_j / f, subtracts
+// s_i w_j from the trailing entries and leaves 1 / sqrt(f) to the end (R_kj = s_j / sqrt(f),
+// R_kk = 2^-z f / sqrt(f), all rows at once): the chain from one pivot to the next is a reciprocal and three multiplies.
 template <int NC, int T>
-QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double* Rout) {
+QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double* Rout, int min_bits, bool zero_ok) {
   constexpr int LE = NC + 1;
   u64* Slo = reinterpret_cast<u64*>(smem);
   long long* Shi = reinterpret_cast<long long*>(Slo + NC * LE);
-  int* sj = reinterpret_cast<int*>(Shi + NC * LE);  // column exponents
-  FxPivot* piv = reinterpret_cast<FxPivot*>(reinterpret_cast<unsigned char*>(sj) + 4 * NC + (16 - (4 * NC) % 16) % 16);
+  u64* Wlo = reinterpret_cast<u64*>(Shi + NC * LE);
+  long long* Whi = reinterpret_cast<long long*>(Wlo + NC);
+  FxPivot* piv = reinterpret_cast<FxPivot*>(Whi + NC);  // [2]
+  int* sj = reinterpret_cast<int*>(piv + 2);            // column exponents
+  int* zk = sj + NC;                                    // z of each pivot
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int NW = T / 32;
   auto get = [&](int i, int j) -> i128 { return (i128)(((u128)(u64)Shi[i * LE + j] << 64) | Slo[i * LE + j]); };
@@ -470,50 +512,73 @@ QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double
     sj[j] = bl ? (bl + 1) >> 1 : -1;
   }
   __syncthreads();
-  for (int i = warp; i < n; i += NW)
-    for (int j = i + lane; j < n; j += 32) {
-      i128 v = 0;
-      if (sj[i] >= 0 && sj[j] >= 0) {
-        const Wide320 a = sacc_load(sacc + (size_t)tri_index(i, j) * kLimbs);
-        const int r = sj[i] + sj[j] - kFx;
-        u128 mag = r > 0 ? bits_at(a, r) + (bits_at(a, r - 1) & 1)
-                         : bits_at(a, 0) << (-r);
-        v = a.neg ? -(i128)mag : (i128)mag;
-      }
-      put(i, j, v);
-    }
+  const int ne = n * (n + 1) / 2;
+#pragma unroll 2
+  for (int e = tid; e < ne; e += T) {
+    int j = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+    if (j * (j + 1) / 2 > e) --j;
+    if ((j + 1) * (j + 2) / 2 <= e) ++j;
+    const int i = e - j * (j + 1) / 2;
+    const Wide320 a = sacc_load(sacc + (size_t)e * kLimbs);
+    const int r = sj[i] + sj[j] - kFx;
+    u128 mag = r > 0 ? (bits_at(a, r - 1) + 1) >> 1 : (((u128)a.w[1] << 64) | a.w[0]) << (-r);
+    if (sj[i] < 0 || sj[j] < 0) mag = 0;
+    put(i, j, a.neg ? -(i128)mag : (i128)mag);
+  }
   __syncthreads();
-  if (tid == 0) piv[0] = fx_pivot(get(0, 0), sj[0] < 0);
+  auto pivot = [&](int k, i128 d) {
+    FxPivot pv = fx_pivot(d, sj[k] < 0, min_bits);
+    if (pv.ok == 0 && !zero_ok) pv.ok = -1;
+    piv[k & 1] = pv;
+  };
+  if (tid == 0) pivot(0, get(0, 0));
   __syncthreads();
   for (int k = 0; k < n; ++k) {
     const FxPivot pv = piv[k & 1];
     if (pv.ok < 0) return k + 1;  // uniform
-    for (int j = k + tid; j < n; j += T) {  // row k of R
-      const i128 v = pv.ok ? fx_mul(get(k, j) << pv.x, pv.r) : (i128)0;
+    for (int j = k + tid; j < n; j += T) {
+      const i128 v = pv.ok ? get(k, j) << (j == k ? 2 * pv.z : pv.z) : (i128)0;  // S_kk becomes f
       put(k, j, v);
+      if (j == k) zk[k] = pv.z;
+      const i128 w = j == k ? (i128)0 : fx_div_pivot(v, pv);
+      Wlo[j] = (u64)(u128)w;
+      Whi[j] = (long long)(w >> 64);
     }
     __syncthreads();
+    auto update_row = [&](int i) {
+      const i128 si = get(k, i);
+      i128 first = 0;
+      for (int j = i + lane; j < n; j += 32) {
+        const i128 w = (i128)(((u128)(u64)Whi[j] << 64) | Wlo[j]);
+        const i128 v = get(i, j) - fx_mul(si, w) * 8;  // units 2^-125 2^-122 2^128 / 2^3
+        put(i, j, v);
+        if (j == i) first = v;
+      }
+      return first;
+    };
     if (warp == 0) {  // the next row, then its pivot
-      const int i = k + 1;
-      if (i < n) {
-        const i128 lki = get(k, i);
-        for (int j = i + lane; j < n; j += 32) put(i, j, get(i, j) - fx_mul(lki, get(k, j)));
-        if (lane == 0) piv[i & 1] = fx_pivot(get(i, i), sj[i] < 0);
+      if (k + 1 < n) {
+        const i128 d = update_row(k + 1);
+        if (lane == 0) pivot(k + 1, d);
       }
     } else {
-      for (int i = k + 1 + warp; i < n; i += NW - 1) {
-        const i128 lki = get(k, i);
-        for (int j = i + lane; j < n; j += 32) put(i, j, get(i, j) - fx_mul(lki, get(k, j)));
-      }
+      for (int i = k + 1 + warp; i < n; i += NW - 1) update_row(i);
     }
     __syncthreads();
   }
+  for (int k = tid; k < n; k += T) {  // 1 / (2 sqrt(f))
+    const i128 r = sj[k] < 0 ? (i128)0 : fx_half_rsqrt(get(k, k));
+    Wlo[k] = (u64)(u128)r;
+    Whi[k] = (long long)(r >> 64);
+  }
+  __syncthreads();
   for (int i = warp; i < n; i += NW)
     for (int j = lane; j < n; j += 32) {
       double r = 0.0;
       if (j >= i) {
-        const i128 v = get(i, j);
-        r = mag_to_double(v < 0 ? (u128)-v : (u128)v, sj[j] - kFx + kXgUnitExp / 2);
+        const i128 h = (i128)(((u128)(u64)Whi[i] << 64) | Wlo[i]);
+        const i128 v = fx_mul(get(i, j), h);
+        r = mag_to_double(v < 0 ? (u128)-v : (u128)v, sj[j] + 1 - (j == i ? zk[i] : 0) - kFx + kXgUnitExp / 2);
         if (v < 0) r = -r;
       }
       Rout[i * LE + j] = r;
@@ -522,31 +587,88 @@ QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double
   return 0;
 }
 
-// Range verdict, election of the last CTA and, in it, the epilogue: for TSQR calls
-// (a.method == QL_TSQR) R from the fixed-point Cholesky, or the request that the Householder
-// launch redoes the call (flags[1]); for the Gram methods C in FP64 and their own epilogue.
+// Whether SVQB would keep every eigenvalue of C = R^T R: lambda_min > tol lambda_max, shown by
+// tol trace(C) ||R^{-1}||_F^2 <= 1/16 (trace >= lambda_max, ||R^{-1}||_F^2 >= 1 / lambda_min).  R in
+// shared memory (ld LE), scaled by rows of its inverse in FP32: good to a few per cent up to
+// the condition numbers (about 10^6) where the answer can be yes.  One warp per column.
+template <int NC, int T>
+QL_DEV bool svqb_full_rank(const double* R, int n, double tol, float* sums) {
+  constexpr int LE = NC + 1, NW = T / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // scale by the largest column norm so that FP32 covers the range
+  if (threadIdx.x < 2) sums[threadIdx.x] = 0.0f;
+  double big = 0.0;
+  for (int i = 0; i < n; ++i) big = fmax(big, fabs(R[i * LE + i]));
+  if (!(big > 0.0) || !isfinite(big)) return false;  // uniform
+  const double inv = 1.0 / big;
+  __syncthreads();
+  float tr = 0.0f, fr = 0.0f;
+  for (int c = warp; c < n; c += NW) {
+    float x0 = 0.0f, x1 = 0.0f;  // rows lane, lane + 32 of the right-hand side, e_c at the start
+    if (lane == (c & 31)) (c < 32 ? x0 : x1) = 1.0f;
+    for (int i = c; i >= 0; --i) {
+      const float xi =
+          __shfl_sync(0xffffffffu, i < 32 ? x0 : x1, i & 31) / (float)(R[i * LE + i] * inv);
+      fr = fmaf(xi, xi, fr);
+      if (lane < i) x0 = fmaf(-(float)(R[lane * LE + i] * inv), xi, x0);
+      if (NC > 32 && lane + 32 < i) x1 = fmaf(-(float)(R[(lane + 32) * LE + i] * inv), xi, x1);
+    }
+    for (int i = lane; i <= c; i += 32) {
+      const float v = (float)(R[i * LE + c] * inv);
+      tr = fmaf(v, v, tr);
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+  if (lane == 0) {
+    atomicAdd(&sums[0], tr);
+    atomicAdd(&sums[1], fr);
+  }
+  __syncthreads();
+  const double bound = tol * (double)sums[0] * (double)sums[1];
+  return bound <= 0.0625;
+}
+
+// Range verdict, election of the last CTA and, in it, R from the fixed-point Cholesky.  The
+// Gram methods end here as well when their further passes could not change R: with C exact
+// and factored to 2^-90, Y = X R1^{-1} is orthonormal to working precision and R2 the identity.
+// flags[5] then tells the later launches of the call.  What a method answers beyond that
+// range is left to its passes: Cholesky-QR2 from pivots of 2^-46 (where an FP64 Cholesky of C
+// may break down), shifted Cholesky-QR3 from 2^-66, SVQB2 when an eigenvalue could be
+// truncated or Z is wanted; a zero column breaks down there.  A TSQR call whose pivots fall below
+// 2^-80 is redone by the Householder launch (flags[1]).
 template <int NC, int T, typename S>
 QL_DEV void xg_finish(const GramArgs<S>& a, unsigned char* smem, const int* colmax, int* misc, int k) {
   if (!gram_elect<S, ArithDF>(a, colmax, misc, k)) return;
   const int tid = threadIdx.x, n = a.n;
   constexpr int LE = NC + 1;
-  if (a.method == QL_TSQR) {
-    if (*(volatile int*)&a.w.flags[1] != 0) return;  // a bounded wait gave up: Householder redoes the call
-    double* Rs = reinterpret_cast<double*>(smem);
-    double* vec = Rs + NC * LE;
-    int* sflag = reinterpret_cast<int*>(vec + 2 * LE);
-    unsigned char* scratch = smem + ((NC + 3) * LE * 8 + 255) / 256 * 256;
-    if (xg_cholesky<NC, T>(a.w.sacc, n, scratch, Rs)) {
-      if (tid == 0) {
-        a.w.flags[1] = 1;
-        if (a.redo) gram_request_redo(a.redo, a.redo_any);
-      }
-      return;
-    }
+  const bool tsqr = a.method == QL_TSQR;
+  if (tsqr && *(volatile int*)&a.w.flags[1] != 0) return;  // a bounded wait gave up: Householder redoes the call
+  double* Rs = reinterpret_cast<double*>(smem);
+  double* vec = Rs + NC * LE;
+  int* sflag = reinterpret_cast<int*>(vec + 2 * LE);
+  unsigned char* scratch = smem + ((NC + 3) * LE * 8 + 255) / 256 * 256;
+  const int min_bits = tsqr ? 80 : (a.method == QL_SCHOLQR3 ? 66 : 46);
+  bool done = false;
+  if (a.method != QL_SVQB2 || !a.Z) {
+    done = xg_cholesky<NC, T>(a.w.sacc, n, scratch, Rs, min_bits, tsqr) == 0;
+    if (done && a.method == QL_SVQB2)
+      done = svqb_full_rank<NC, T>(Rs, n, a.rank_tol > 0.0 ? a.rank_tol : (double)n * 2.220446049250313e-16,
+                                   reinterpret_cast<float*>(sflag));
+  }
+  __syncthreads();  // the scratch is reused
+  if (done) {
+    if (!tsqr && tid == 0) a.w.flags[5] = 1;
     if (a.epilogue == kEpiR)
       epilogue_r<T>(Rs, LE, n, a.R, a.ldr, a.info, sflag);
     else
       epilogue_lstsq<T>(Rs, LE, n, a.x, a.resnorm, a.Rext, a.info, vec, sflag);
+    return;
+  }
+  if (tsqr) {
+    if (tid == 0) {
+      a.w.flags[1] = 1;
+      if (a.redo) gram_request_redo(a.redo, a.redo_any);
+    }
     return;
   }
   double* Cs = reinterpret_cast<double*>(smem);
@@ -696,16 +818,22 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
     // Tensor-memory sums -> 128-bit integers.  A thread folds the eight sums of its (lane,
     // column): digits q of the other factor for NC <= 32 (planes p and p + 4 for NC = 32),
     // the eight weights of its parity for NC = 64.
+    // Eight sums d_q of spacing 7 or 14 bits are gathered by widening multiply-adds (one
+    // instruction each) into 64-bit groups at 32-bit offsets, then carried into 128 bits.  Rows
+    // of C below the diagonal block of the warp are not folded (NC = 64: a quarter of the work).
     auto readout = [&]() {
-      constexpr int JS = HALF < 4 ? HALF : 4;
+      constexpr int JS = HALF < 4 || NC == 32 ? 2 : 4;
       const uint32_t lane_base = tbase + ((uint32_t)(32 * qd) << 16) + (uint32_t)(hh * HALF);
       const bool keep = nread++ > 0;   // uniform: every slicer counts the read-outs
       if (NC == 8 && qd >= 2) return;  // lanes 64..127 hold nothing
 #pragma unroll 1
       for (int c0 = 0; c0 < HALF; c0 += JS) {
-        i128 sum[JS];
+        if (NC == 64 && hh * HALF + c0 + JS <= 32 * (qd & 1)) continue;  // columns left of every row of the warp
+        ulonglong2* p = acc + (size_t)(hh * HALF + c0) * 128 + L;
+        ulonglong2 old[JS];
 #pragma unroll
-        for (int j = 0; j < JS; ++j) sum[j] = 0;
+        for (int j = 0; j < JS; ++j) old[j] = keep ? __ldcg(p + j * 128) : make_ulonglong2(0, 0);
+        i128 sum[JS];
 #pragma unroll
         for (int part = 0; part < (NC == 32 ? 2 : 1); ++part) {
           uint32_t v[8][JS];
@@ -717,30 +845,26 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
             int d[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) d[q] = __float2int_rn(__uint_as_float(v[q][j]));
-            constexpr int SP = NC == 64 ? 14 : 7;
-            if constexpr (NC == 64) {
-              i128 s = (long long)d[0] * (1 << SP) + d[1];
-              s = s * ((i128)1 << (2 * SP)) + ((long long)d[2] * (1 << SP) + d[3]);
-              s = s * ((i128)1 << (2 * SP)) + ((long long)d[4] * (1 << SP) + d[5]);
-              s = s * ((i128)1 << (2 * SP)) + ((long long)d[6] * (1 << SP) + d[7]);
-              sum[j] = s;
-            } else {
-              long long h = d[0], l = d[4];
-#pragma unroll
-              for (int q = 1; q < 4; ++q) {
-                h = h * 128 + d[q];
-                l = l * 128 + d[4 + q];
-              }
-              const i128 s = (i128)h * (1 << 28) + l;
-              sum[j] = sum[j] * (1 << 28) + s;
+            if constexpr (NC == 64) {  // offsets 0, 14, .., 98
+              const long long a0 = mad_wide(d[5], 1 << 28, mad_wide(d[6], 1 << 14, (long long)d[7]));
+              const long long a1 = mad_wide(d[3], 1 << 24, mad_wide(d[4], 1 << 10, a0 >> 32));
+              const long long a2 = mad_wide(d[1], 1 << 20, mad_wide(d[2], 1 << 6, a1 >> 32));
+              const long long a3 = mad_wide(d[0], 1 << 2, a2 >> 32);
+              sum[j] = (i128)(((u128)(u64)(((u64)(unsigned)a3 << 32) | (unsigned)a2) << 64) |
+                              (((u64)(unsigned)a1 << 32) | (unsigned)a0));
+            } else {  // offsets 0, 7, .., 49
+              const long long l =
+                  mad_wide(d[4], 1 << 21, mad_wide(d[5], 1 << 14, mad_wide(d[6], 1 << 7, (long long)d[7])));
+              const long long h =
+                  mad_wide(d[0], 1 << 21, mad_wide(d[1], 1 << 14, mad_wide(d[2], 1 << 7, (long long)d[3])));
+              const i128 t = ((i128)h << 28) + l;
+              sum[j] = part == 0 ? t : (sum[j] << 28) + t;
             }
           }
         }
 #pragma unroll
-        for (int j = 0; j < JS; ++j) {
-          ulonglong2* p = acc + (size_t)(hh * HALF + c0 + j) * 128 + L;
-          store_i128(p, keep ? load_i128(p) + sum[j] : sum[j]);
-        }
+        for (int j = 0; j < JS; ++j)
+          store_i128(p + j * 128, (i128)(((u128)old[j].y << 64) | old[j].x) + sum[j]);
       }
     };
     // 128-bit sums -> the integer accumulators of C at the current column scales.  Lane groups
@@ -748,18 +872,26 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
     auto emit = [&](unsigned char* scratch) {
       ulonglong2* sc = reinterpret_cast<ulonglong2*>(scratch);
       if (reader && lg > 0) {
+        constexpr int JB = HALF < 8 ? HALF : 8;
 #pragma unroll 1
-        for (int j = 0; j < HALF; ++j)
-          sc[((size_t)(lg - 1) * NC + li) * NC + hh * HALF + j] = __ldcg(acc + (size_t)(hh * HALF + j) * 128 + L);
+        for (int j0 = 0; j0 < HALF; j0 += JB) {
+          ulonglong2 t[JB];
+#pragma unroll
+          for (int j = 0; j < JB; ++j) t[j] = __ldcg(acc + (size_t)(hh * HALF + j0 + j) * 128 + L);
+#pragma unroll
+          for (int j = 0; j < JB; ++j) sc[((size_t)(lg - 1) * NC + li) * NC + hh * HALF + j0 + j] = t[j];
+        }
       }
       slicer_sync<TS>();
       if (reader && lg == 0 && li < n) {
         const int si = scale[li];
+        ulonglong2 next = __ldcg(acc + (size_t)(hh * HALF) * 128 + L);
 #pragma unroll 1
         for (int j = 0; j < HALF; ++j) {
           const int jj = hh * HALF + j;
+          i128 v = (i128)(((u128)next.y << 64) | next.x);
+          if (j + 1 < HALF) next = __ldcg(acc + (size_t)(jj + 1) * 128 + L);
           if (jj < li || jj >= n) continue;
-          i128 v = load_i128(acc + (size_t)jj * 128 + L);
           auto part = [&](int g) -> i128 {
             const ulonglong2 t = sc[((size_t)(g - 1) * NC + li) * NC + jj];
             return (i128)(((u128)t.y << 64) | t.x);

@@ -90,3 +90,47 @@ def test_very_ill_conditioned_matches_oracle():
         R, info = tsqr(X)
         assert info == [0, 0]
         assert oracle.rel_err(R, oracle.householder_r(X)) <= oracle.tolerance(12, kappa)
+
+
+@pytest.mark.parametrize("n", [7, 16, 33])
+@pytest.mark.parametrize("kappa,rank_tol", [(1e3, 0.0), (1e3, 1e-4), (1e7, 0.0)])
+def test_svqb2_with_and_without_z_agree(n, kappa, rank_tol):
+    """Z forces both eigensolves; without it the exact pass may answer, but not where an
+    eigenvalue is truncated (kappa^-2 < rank_tol, or kappa^2 n 2^-52 > 1)."""
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    X = synth.conditioned(6000, n, kappa, seed=n)
+    Xd = torch.from_numpy(np.ascontiguousarray(X.T)).cuda().T
+    Rz, Z, iz = q.svqb_qless(Xd, rank_tol=rank_tol, want_z=True)
+    R, _, i = q.svqb_qless(Xd, rank_tol=rank_tol)
+    assert i.cpu().tolist() == iz.cpu().tolist()
+    assert oracle.rel_err(R.cpu().numpy(), Rz.cpu().numpy()) <= 2 * oracle.tolerance(n, min(kappa, 1e6))
+
+
+@pytest.mark.parametrize("n", [6, 20, 40])
+def test_gram_methods_against_oracle_on_both_sides_of_the_limits(n):
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    for kappa, fn in ((1e2, q.cholqr2_qless), (1e6, q.cholqr2_qless), (1e2, q.scholqr3_qless),
+                      (1e8, q.scholqr3_qless), (1e10, q.scholqr3_qless)):
+        X = synth.conditioned(5001, n, kappa, seed=n + 1)
+        Xd = torch.from_numpy(np.ascontiguousarray(X.T)).cuda().T
+        R, info = fn(Xd)
+        assert info.cpu().tolist() == [0, 0]
+        assert oracle.rel_err(R.cpu().numpy(), oracle.householder_r(X)) <= oracle.tolerance(n, kappa)
+
+
+def test_gram_methods_still_report_breakdowns():
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    X = synth.gaussian(4000, 10, seed=1)
+    X[:, 6] = 0.0                      # zero column: not the exact route's to answer here
+    Xd = torch.from_numpy(np.ascontiguousarray(X.T)).cuda().T
+    assert q.cholqr2_qless(Xd)[1].cpu().tolist() == [q.QL_ERR_NOT_SPD, 7]
+    assert q.scholqr3_qless(Xd)[1].cpu().tolist() == [q.QL_ERR_NOT_SPD, 1007]
