@@ -110,11 +110,11 @@ size_t ql_workspace_bytes(ql_method method, int64_t m, int64_t n, ql_dtype dtype
 
 /*
  * Q-less TSQR (Sec. 3.2, Algorithms 2-4): the R of X for any condition number.
- * For n >= 5 the first launch forms X^T X exactly (X rounded to 2^-56 of each column's
+ * For n >= 3 the first launch forms X^T X exactly (X rounded to 2^-56 of each column's
  * largest entry, every product and sum an integer) and factors it in 125-bit fixed point:
  * the same R, with an error below the Householder tiles'.  Columns dependent to about 2^-40
  * of their norm (a pivot below 2^-80) are left to the Householder launch behind it, which
- * otherwise exits at once and which is the only one for n <= 4: every CTA streams its row blocks of X
+ * otherwise exits at once and which is the only one for n <= 2 (n <= 4 below 2^14 rows): every CTA streams its row blocks of X
  * through shared memory, factors [R; W] in place with Householder reflectors (Algorithm 4),
  * and the per-CTA triangles are merged by a "last CTA done" R-tree (Algorithm 2, stage 2)
  * inside the same launch.  An FP64 fallback launch follows that exits at once unless the
@@ -150,7 +150,7 @@ ql_status ql_tsqr_qless_noalloc(int64_t m, int64_t n, const void* X, ql_dtype dt
  * Both Cholesky factorisations, R1^{-1} and R2 R1 run on the device in FP64.  A
  * non-positive pivot sets info = {QL_ERR_NOT_SPD, pivot} (+1000 for the second pass) and
  * fills R with NaN.  Reliable for kappa_2(X) up to about 1e6 (the Gram squares kappa).
- * For n >= 5 the first pass is exact (see ql_tsqr_qless): while every pivot of C stays above
+ * For n >= 3 the first pass is exact (see ql_tsqr_qless): while every pivot of C stays above
  * 2^-46 of its column, R1 from the fixed-point Cholesky is already the R that both passes
  * give, with a smaller error, and the second pass ends at once.
  */
@@ -165,7 +165,7 @@ ql_status ql_cholqr2_qless(int64_t m, int64_t n, const void* X, ql_dtype dtype, 
  *   pass 2: Y = X R1^{-1} formed tile by tile, R2 = chol(Y^T Y);
  *   pass 3: Y = X (R2 R1)^{-1}, R3 = chol(Y^T Y);  R = R3 R2 R1.
  * Arguments, workspace and outputs as ql_cholqr2_qless.  A non-positive pivot sets info =
- * {QL_ERR_NOT_SPD, pivot + 1000 (pass - 1)} and R = NaN.  For n >= 5 the exact first pass
+ * {QL_ERR_NOT_SPD, pivot + 1000 (pass - 1)} and R = NaN.  For n >= 3 the exact first pass
  * gives R by itself (unshifted) while every pivot of C stays above 2^-66 of its column.
  */
 ql_status ql_scholqr3_qless(int64_t m, int64_t n, const void* X, ql_dtype dtype, int64_t ldx, double* R,
@@ -176,7 +176,7 @@ ql_status ql_scholqr3_qless(int64_t m, int64_t n, const void* X, ql_dtype dtype,
  * device), B1 = U L^{-1/2} with eigenvalues below rank_tol * lambda_max treated as zero
  * (rank_tol <= 0 selects n * 2^-52); second pass on X B1 (formed tile by tile); then
  * X = Q Z with Z = L2^{1/2} U2^T L1^{1/2} U1^T and R = qr_r(Z) (FP64 Householder on the
- * device).  Z (nullable device double n x n, ld n) receives Z.  For n >= 5, without Z and
+ * device).  Z (nullable device double n x n, ld n) receives Z.  For n >= 3, without Z and
  * when no eigenvalue can be truncated, the exact first pass gives R by itself.
  */
 ql_status ql_svqb_qless(int64_t m, int64_t n, const void* X, ql_dtype dtype, int64_t ldx, double* R,

@@ -76,24 +76,26 @@ bool pipe_tensor_maps(CUtensorMap* tmA, CUtensorMap* tmB, const void* A, const v
   return true;
 }
 
-bool xg_tensor_maps(XgMaps* maps, int nc, const void* A, const void* b, int dtype, int64_t m, int nA, int64_t lda) {
-  if (!pipe_tensor_maps(&maps->rows, b ? &maps->rhs : nullptr, A, b, dtype, m, nA, lda)) return false;
+bool xg_tensor_map(CUtensorMap* map, int nc, const void* A, const void* b, int dtype, int64_t m, int nA, int64_t lda) {
+  const Encode encode = tensor_map_encoder();
   const size_t es = dtype == QL_F64 ? 8 : 4;
+  auto aligned = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
   const cuuint32_t rpb = (cuuint32_t)(128 / es), one[3] = {1, 1, 1};
+  if (!encode || m < 4096 / nc || m >= (int64_t(1) << 31) || nA < 1 || !aligned(A) || ((size_t)lda * es) % 16 ||
+      !aligned(b))
+    return false;
   const cuuint64_t dims[3] = {rpb, (cuuint64_t)nA, (cuuint64_t)(m / rpb)}, strides[2] = {(cuuint64_t)lda * es, 128};
   const cuuint32_t box[3] = {rpb, (cuuint32_t)nc, (cuuint32_t)(4096 / nc / rpb)};
-  maps->full = dims[2] > 0 && tensor_map_encoder()(&maps->tile, dtype == QL_F64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
-                                       const_cast<void*>(A), dims, strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                       CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
-                   ? 1
-                   : 0;
-  return true;
+  return encode(map, dtype == QL_F64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
+                const_cast<void*>(A), dims, strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 static int nc_of(int n) { return n <= 1 ? 1 : n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : n <= 16 ? 16 : n <= 32 ? 32 : 64; }
 
-static size_t gram_head_bytes(int n) { return 512 + (n > 4 ? (sacc_bytes(nc_of(n)) + 255) / 256 * 256 : 0); }
+static int xg_nc(int n) { return n <= 4 ? 4 : nc_of(n); }  // column class of the exact pass
+static size_t gram_head_bytes(int n) { return 512 + (sacc_bytes(xg_nc(n)) + 255) / 256 * 256; }
 
 static size_t gram_layout(int n, GramWs* w, void* base) {
   const int nc = nc_of(n);
@@ -103,9 +105,9 @@ static size_t gram_layout(int n, GramWs* w, void* base) {
   const size_t keep = ((size_t)3 * nc * nc * sizeof(double) + 255) / 256 * 256;  // 3 n x n blocks (ld n)
   // one NC x NC partial per CTA (the streaming kernel for nc <= 4 runs up to 8 CTAs per SM)
   const size_t parts = (size_t)device_sm_count() * (nc <= 4 ? 8 : kGramMaxCtasPerSm) * nc * nc * sizeof(double);
-  // accumulators of the tcgen05 kernels (8 to 64 columns, one CTA per SM): 128-bit sums (exact
-  // pass), an FP64 and a double-float level (pipelined later passes) or FP64 (per tile)
-  const size_t fbuf = nc >= 8 ? (size_t)device_sm_count() * nc * 128 * 2 * sizeof(double) : 0;
+  // accumulators of the tcgen05 kernels (one CTA per SM): 128-bit sums (exact pass), an FP64
+  // and a double-float level (pipelined later passes) or FP64 (per tile)
+  const size_t fbuf = (size_t)device_sm_count() * xg_nc(n) * 128 * 2 * sizeof(double);
   if (w && base) {
     unsigned char* b = static_cast<unsigned char*>(base);
     w->flags = reinterpret_cast<int*>(b);
@@ -145,8 +147,8 @@ ql_status gram_launch(const GramCall& c, ql_arith arith) {
 // Workspace and launch of the exact pass for a TSQR call (n >= 2).  The caller clears the
 // first *clear_bytes of `base` beforehand; flags[0] then asks for the FP64 launch and
 // flags[1] for the double-float Householder launch.
-size_t xgram_tsqr_bytes(int n) { return gram_layout(n < 5 ? 5 : n, nullptr, nullptr); }
-size_t xgram_tsqr_clear_bytes(int n) { return gram_head_bytes(n < 5 ? 5 : n); }
+size_t xgram_tsqr_bytes(int n) { return gram_layout(n, nullptr, nullptr); }
+size_t xgram_tsqr_clear_bytes(int n) { return gram_head_bytes(n); }
 ql_status xgram_tsqr_launch(const TsqrCall& t, void* base) {
   GramCall c;
   c.m = t.m;
@@ -166,7 +168,7 @@ ql_status xgram_tsqr_launch(const TsqrCall& t, void* base) {
   c.info = t.info;
   c.stream = t.stream;
   GramWs w;
-  gram_layout(c.n < 5 ? 5 : c.n, &w, base);
+  gram_layout(c.n, &w, base);
   return c.dtype == QL_F64 ? xgram_pass1<double>(c, w) : xgram_pass1<float>(c, w);
 }
 

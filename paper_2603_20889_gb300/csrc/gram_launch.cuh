@@ -2391,8 +2391,8 @@ ql_status gram_launch_one(const GramCall& c, const GramWs& w, int pass, int gate
   return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
-// Exact Gram pass (xgram.cuh): R of a TSQR call (method QL_TSQR, n >= 2), or the first pass
-// of a Gram method with n >= 5.
+// Exact Gram pass (xgram.cuh): R of a TSQR call (method QL_TSQR), or the first pass of a Gram
+// method, n >= 3.
 template <typename S>
 ql_status xgram_pass1(const GramCall& c, const GramWs& w);
 extern template ql_status xgram_pass1<double>(const GramCall&, const GramWs&);
@@ -2432,7 +2432,11 @@ ql_status gram_dispatch(const GramCall& c, const GramWs& w, int gated) {
       }
     }
     if constexpr (NC <= 4) {  // narrow X: the streaming kernel (n = 8 would spill its 36 accumulators)
-      ql_status st = gram_stream_launch_one<NC, S, Ar, kXNone>(c, w, 1, gated);
+      ql_status st;
+      if (NC == 4 && std::is_same<Ar, ArithDF>::value && tc_gram_enabled())
+        st = xgram_pass1<S>(c, w);
+      else
+        st = gram_stream_launch_one<NC, S, Ar, kXNone>(c, w, 1, gated);
       if (st) return st;
       if (c.method == QL_SVQB2) return gram_stream_launch_one<NC, S, Ar, kXFull>(c, w, 2, gated);
       st = gram_stream_launch_one<NC, S, Ar, kXUpper>(c, w, 2, gated);

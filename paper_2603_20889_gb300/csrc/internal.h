@@ -106,15 +106,11 @@ bool pipe_gram2_enabled();
 bool pipe_tensor_maps(CUtensorMap* tmA, CUtensorMap* tmB, const void* A, const void* b, int dtype, int64_t m, int nA,
                       int64_t lda);
 
-// Tensor maps of the exact Gram pass (xgram.cuh): `rows` and `rhs` as pipe_tensor_maps makes
-// them, and `tile`, A as rank 3 (128 bytes of rows, columns, row blocks) whose box is a whole
-// tile of 4096 / nc rows x nc columns (columns past nA read as zeros).
-struct XgMaps {
-  CUtensorMap tile, rows, rhs;
-  int full;  // `tile` is valid
-};
-// False if the data does not allow tensor copies (b null: no right-hand side).
-bool xg_tensor_maps(XgMaps* maps, int nc, const void* A, const void* b, int dtype, int64_t m, int nA, int64_t lda);
+// Tensor map of the exact Gram pass (xgram.cuh): A as rank 3 (128 bytes of rows, columns, row
+// blocks; 128-byte swizzle) whose box is a whole tile of 4096 / nc rows x nc columns (columns
+// past nA read as zeros).  False if the data does not allow tensor copies of its full tiles
+// (a column, or b unless it is null, not 16-byte aligned; m >= 2^31).
+bool xg_tensor_map(CUtensorMap* map, int nc, const void* A, const void* b, int dtype, int64_t m, int nA, int64_t lda);
 
 // Thread-layout variant of the TSQR kernels (environment QL_TSQR_CFG, 0 = default).
 int tsqr_variant();

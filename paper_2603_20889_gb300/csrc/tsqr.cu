@@ -49,10 +49,15 @@ size_t tsqr_workspace_bytes(int n, bool householder) {
          tree_slots((int)leaves) * (size_t)n * n * sizeof(double);
 }
 
-// The exact Gram pass (xgram.cuh) replaces the Householder tiles from 5 columns.  Measured
-// (m = 2^25, n = 4): Householder 0.92 ms, exact 1.59 ms (half of the 8-column class's work is
-// padding there).
-constexpr int kExactMinN = 5;
+// Whether the exact Gram pass (xgram.cuh) takes a TSQR call.  From 5 columns always (4099 x 5
+// 45 -> 35 us, everything larger gains more).  With 3 or 4 columns from 2^14 rows: m = 2^25,
+// n = 4 919 -> 382 us, 100000 x 4 61 -> 33 us, but 4099 x 3 27.7 -> 29.7 us, one Householder tile
+// per CTA and a one-level tree there.  One or two columns stay with the norm and the Householder
+// tiles: the 4-column class works for two columns that are not there (m = 2^25, n = 2 288 us
+// against 378).
+static bool exact_route(const TsqrCall& c, ql_arith arith) {
+  return !c.householder && arith != QL_ARITH_F64 && tc_gram_enabled() && (c.n >= 5 || (c.n >= 3 && c.m >= (1 << 14)));
+}
 
 template <typename S>
 static ql_status tsqr_launch_s(const TsqrCall& c, const TreeView& tv, bool exact, ql_arith arith) {
@@ -65,7 +70,7 @@ static ql_status tsqr_launch_s(const TsqrCall& c, const TreeView& tv, bool exact
 ql_status tsqr_launch(const TsqrCall& c, ql_arith arith) {
   if (c.n < 1 || c.n > kMaxN) return QL_ERR_ARG;
   if (!c.ws || c.ws_bytes < tsqr_workspace_bytes(c.n, c.householder)) return QL_ERR_WORKSPACE;
-  const bool exact = !c.householder && c.n >= kExactMinN && arith != QL_ARITH_F64 && tc_gram_enabled();
+  const bool exact = exact_route(c, arith);
   // [tree counters][flags (head of the exact pass's block)][slots]
   unsigned char* ws = static_cast<unsigned char*>(c.ws);
   const size_t cb = counter_bytes(), xb = c.householder || c.n < 2 ? kFlagBytes : xgram_tsqr_bytes(c.n);

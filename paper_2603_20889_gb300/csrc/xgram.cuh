@@ -1,14 +1,18 @@
 // Exact Gram pass on tcgen05 (C = X^T X) with a fixed-point Cholesky behind it: R in one pass
-// over X, in the 8-, 16-, 32- and 64-column classes, for TSQR calls and, while their further
+// over X, in the 4-, 8-, 16-, 32- and 64-column classes, for TSQR calls and, while their further
 // passes could not change R, for the Gram methods.
 //
 // Measured against the double-float Householder tiles (which stay for columns dependent to
-// about 2^-40 and for n <= 4) and the Gram methods' own passes (which stay beyond the limits
-// in xg_finish): m = 2^22, n = 64 TSQR 21.1 -> 2.03 ms, Cholesky-QR2 8.30 -> 2.04 ms; SVQB2
-// 10^6 x 32 3.69 -> 0.21 ms; shifted Cholesky-QR3 300007 x 24 872 -> 119 us; least squares
-// 2^24 x 31, FP32-stored, 19.2 -> 1.68 ms; 131072 x 8 145 -> 39 us.  ||R - R_ref|| / ||R_ref||
-// falls in each of them (n = 64: 3.5e-16 -> 2.6e-16, Cholesky-QR2 9.9e-16 -> 2.6e-16,
-// SVQB2 1e-14 -> 3.3e-16 against 64-bit references).
+// about 2^-40 and the narrow calls of exact_route) and the Gram methods' own passes (which stay
+// beyond the limits in xg_finish): TSQR m = 2^25, n = 4 917 -> 383 us; m = 2^23, n = 8, 16, 32
+// 213, 406, 783 us (2.5, 2.6, 2.7 TB/s of X); m = 2^22, n = 64 21.1 -> 2.11 ms, Cholesky-QR2
+// 8.30 -> 2.11 ms; SVQB2 10^6 x 32 3.89 -> 0.20 ms; shifted Cholesky-QR3 300007 x 24 871 ->
+// 114 us; least squares 2^24 x 31, FP32-stored, 19.3 -> 1.48 ms; 131072 x 8 145 -> 42 us.
+// ||R - R_ref|| / ||R_ref|| against 64-bit references: 3.5e-16 -> 1.9e-16 (n = 64), 1.1e-15 ->
+// 1.9e-16 (Cholesky-QR2), 1e-14 -> 3.3e-16 (SVQB2), 4.2e-15 -> 1.2e-16 (Cholesky-QR3).
+// Up to 32 columns the integer pipe bounds it (75 % busy: some 37 instructions of it per element
+// to cut and pack the digits); at 64 columns the MMAs do (36 of 128 x 64 x 16 per 16 rows: each
+// reads 6 KB of shared memory for 32 cycles of work) and the read-out every 8 tiles.
 //
 // Every value is rounded to a signed 56-bit fixed point N relative to a running per-column
 // scale 2^e (|x| < 2^e, x ~ N 2^(e - 55)) and cut into EIGHT balanced base-128 digits, which
@@ -26,22 +30,31 @@
 //    tiles ahead (a whole tile per instruction), one the MMAs, in warp-uniform code with one
 //    elected lane so that descriptors stay in uniform registers.  Two raw stages and two
 //    digit buffers alternate.
+//  * The slicers form two groups of eight warps: one takes the even tiles (stage and buffer 0),
+//    the other the odd ones, so that one group cuts while the other waits for its tile or
+//    votes; cutting is bound by the integer pipe, and with all sixteen warps in step that pipe
+//    idled 40 % of the time.  Each group votes once per tile whether a column outgrew its scale
+//    (the groups' votes alternate in tile order, so neither can hand a tile over that the
+//    tensor core would wait on the other for); a full group of tiles, such a column or the end
+//    brings both groups together for the read-out, with their next tiles already cut.
 //    Mbarriers: "MMAs done" and "digits ready" per digit buffer, "tile landed" and "stage
-//    read" per raw stage; one vote of the slicers per tile (a column outgrew its scale, or a
-//    wait gave up).
+//    read" per raw stage, "vote passed" per group.  All waits are bounded; the first that gives
+//    up sets a flag that ends the others at once.
 //  * The planes lie one after the other in the K-major core-matrix layout, so all planes
 //    together are one operand of 8 NC columns (plane p, column c at 8-column group
 //    (p NC + c) / 8).
-//      NC = 8:   one MMA 128 x 64 x 16 per 16 rows (lanes 64..127 see the memory behind the
-//                planes and are never read); lane p 8 + i, column q 8 + j.
-//      NC = 16:  one MMA 128 x 128 x 16: lane p 16 + i, column q 16 + j.
+//      NC = 16:  one MMA 128 x 128 x 16 per 16 rows; lane p 16 + i, column q 16 + j.
+//      NC = 4, 8: the tile is cut into 16 / NC row segments that stand side by side as 16
+//                virtual columns; the products of different segments are never read.  (MMAs
+//                of 8 NC columns took as long each: n = 4 was bound by their number.)
 //      NC = 32:  two MMAs 128 x 256 x 16 (planes 0..3, 4..7): 512 tensor-memory columns.
 //      NC = 64:  512 x 512 sums do not fit, so pairs of equal weight w = p + q share one of
 //                16 half blocks: block b holds weight 2 b in lanes 0..63 and 2 b + 1 in lanes
 //                64..127.  Plane q even meets the stacked planes (p, p + 1), p even, and q
 //                odd those with p odd (from -1 to 7; plane -1 and plane 8 are zeros), so
 //                every product lands on its own weight: 36 MMAs 128 x 64 x 16.
-//  * G tiles add up in tensor memory per read-out: G KT rows x (pairs per sum) x 64^2 <= 2^24.
+//  * G tiles add up in one set of tensor-memory sums: G KT rows x (pairs per sum) x 64^2 <=
+//    2^24.  The classes up to 16 columns fill NS sets in turn before a read-out (64 tiles).
 #pragma once
 
 #include "gram_launch.cuh"
@@ -54,50 +67,58 @@ using i128 = __int128;
 
 template <int NC>
 struct XgShape {
-  static constexpr int TS = 512;             // slicer threads
+  static constexpr int TS = 512;             // slicer threads, in two groups of TG
+  static constexpr int TG = 256;
   static constexpr int T = TS + 64;          // and the copy warp and the MMA warp
   static constexpr int KT = 4096 / NC;       // rows per tile
-  static constexpr int PLANE = NC * KT * 2;  // bytes per digit plane (8 KB)
+  static constexpr int VC = NC < 16 ? 16 : NC;      // columns of a digit plane: SEG segments x NC
+  static constexpr int SEG = VC / NC;
+  static constexpr int KV = KT / SEG;        // rows of a digit plane
+  static constexpr int PLANE = VC * KV * 2;  // bytes per digit plane (8 KB)
   static constexpr int DBUF = 8 * PLANE;     // digit planes of a tile (64 KB)
   static constexpr int PAD = NC == 64 ? PLANE : 0;  // zero planes before, between and after the buffers
   static constexpr int LBO = 128;            // bytes between core matrices along the rows
-  static constexpr int SBO = KT * 16;        // bytes between 8-column groups
-  static constexpr int TCOLS = NC == 8 ? 64 : (NC == 16 ? 128 : 512);
+  static constexpr int SBO = KV * 16;        // bytes between 8-column groups
+  static constexpr int SCOLS = VC == 16 ? 128 : 512;        // tensor-memory columns of one set of sums
+  static constexpr int NS = 512 / SCOLS;                    // sets: 4, 4, 4, 1, 1
   static constexpr int PAIRS = NC == 64 ? 8 : 1;     // products per sum (weight 7 has eight)
-  static constexpr int G = 4096 / (KT * PAIRS);      // tiles per read-out: 8, 16, 32, 8
+  static constexpr int G = 4096 / (KV * PAIRS);      // tiles per set: 16, 16, 16, 32, 8
+  static constexpr int GT = G * NS;                  // tiles per read-out: 64, 64, 64, 32, 8
   static constexpr int SLACK = 2;            // bits of headroom above a new column maximum
   static constexpr int HALF = NC / 4;        // columns of C per slicer thread at a read-out
-  static constexpr int LG = NC == 8 ? 8 : 128 / NC;  // lane groups (planes, or weight parities)
-  // a 128-bit sum takes at most 2^111 per row: emptied after 2^15 rows (and one more group)
-  static constexpr int MAX_READS = (1 << 15) / (G * KT);
-  static_assert(NC == 8 || NC == 16 || NC == 32 || NC == 64, "column classes");
-  static_assert((long long)G * KT * PAIRS * 4096 <= (1LL << 24), "exact FP32 digit sums");
+  static constexpr int LG = 128 / VC;        // lane groups (planes, or weight parities)
+  // the 128-bit sums of an entry's lane groups come together below 1.02 2^110 per row (NC = 64:
+  // 2^111 per row in the odd weights' one): emptied before 2^126
+  static constexpr int MAX_READS = (NC == 64 ? 1 << 15 : 1 << 16) / (GT * KT);
+  static_assert(NC == 4 || NC == 8 || NC == 16 || NC == 32 || NC == 64, "column classes");
+  static_assert((long long)G * KV * PAIRS * 4096 <= (1LL << 24), "exact FP32 digit sums");
 };
 
 template <int NC, typename S>
 struct XgSmem {
   using Sh = XgShape<NC>;
-  // a staged tile: boxes of 128 bytes of rows x NC columns, 128-byte swizzle (see PipeSmem);
+  // a staged tile: blocks of 128 bytes of rows x NC columns, column c of block k in the
+  // 128-byte line k NC + c, whose 16-byte chunk q sits at q ^ (line & 7) (128-byte swizzle);
   // the right-hand side of least squares is staged apart, its rows in order
   static constexpr int RPB = 128 / (int)sizeof(S);
-  static constexpr int NBOX = Sh::KT / RPB;
   static constexpr size_t kDig = 2 * (size_t)Sh::DBUF + 3 * (size_t)Sh::PAD;
   static constexpr size_t kRaw = sizeof(S) * (size_t)NC * Sh::KT;
   static constexpr size_t kOffRaw = kDig;
-  // (NC = 8: lanes 64..127 of the second buffer's MMAs read 64 KB past it, which must exist)
-  static constexpr size_t kRawSpan = NC == 8 && 2 * kRaw < (size_t)Sh::DBUF ? (size_t)Sh::DBUF : 2 * kRaw;
   static constexpr size_t kStageB = sizeof(S) * (size_t)Sh::KT;
-  static constexpr size_t kOffB = kOffRaw + kRawSpan;
+  static constexpr size_t kOffB = kOffRaw + 2 * kRaw;
   static constexpr size_t kOffScale = kOffB + 2 * kStageB;
   static constexpr size_t kOffColmax = kOffScale + 4 * NC;
   static constexpr size_t kOffMisc = kOffColmax + 4 * NC;
-  static constexpr size_t kOffBar = (kOffMisc + 64 * 4 + 15) / 16 * 16;
-  static constexpr size_t kOffSlot = kOffBar + 64;
+  // barriers and the tensor-memory slot: the same place in every class, so that a grouped
+  // launch sets them up once
+  static constexpr size_t kOffBar = 231424;
+  static constexpr size_t kOffSlot = kOffBar + 80;
   static constexpr size_t kBytes = kOffSlot + 32;
+  static_assert(kOffMisc + 64 * 4 <= kOffBar, "the tile areas end below the barriers");
   static constexpr size_t kEpi = 8 * (4 * (size_t)NC * (NC + 1) + 8 * (NC + 1)) + 64 * 4 + 16;
   static_assert(kBytes <= 232448, "shared memory of one SM");
   static_assert(kEpi <= kOffScale, "the epilogue's shared memory stays below the scales and barriers");
-  static_assert(16 * (size_t)(Sh::LG - 1) * NC * NC <= (size_t)Sh::DBUF, "lane-group sums fit in a digit buffer");
+  static_assert(16 * (size_t)(Sh::LG * Sh::SEG - 1) * NC * NC <= (size_t)Sh::DBUF, "lane-group sums fit in a digit buffer");
 };
 
 // Integer accumulators of C: entry (i <= j) at index i + j (j + 1) / 2, kLimbs limbs of 40 bits
@@ -110,17 +131,19 @@ constexpr int kXgUnitExp = 2 * (kEsMin - 1022) - 110;  // -188
 QL_DEV int tri_index(int i, int j) { return i + j * (j + 1) / 2; }
 
 // ---------------------------------------------------------------------------------------
-// Cutting.  Nb2 = 2 N + 1 + 2 kDigitBias8 rounded so that field p, (Nb2 >> (1 + 7 (7 - p)))
-// & 127 (& 255 for p = 0), is digit p + 64: Q = floor(2 |x| 2^(55 - e)) by one funnel shift,
-// the sign by a one's complement, and the bias constant adds the rounding half (ties away
-// from zero).  s = Es - E + 7 is the right shift of the significand aligned at bit 62.
+// Cutting.  Nb2 = Q + 1 + 2 kDigitBias8 with Q = floor(2 |x| 2^(55 - e)): field p, (Nb2 >> (1 +
+// 7 (7 - p))) & 127 (& 255 for p = 0), is digit p of |x| (rounded to nearest, ties away from
+// zero) plus 64.  Q is one funnel shift of the significand aligned at bit 62, by s = Es - E + 7.
+// Shift counts are formed without masking the sign bit off the exponent (modulo 2048, or 256
+// for FP32), which the shifter's own modulo 32 makes exact for elements less than 2^24 below
+// the scale; FAR covers the others.
 // ---------------------------------------------------------------------------------------
 constexpr u64 kCutBias = 2 * kDigitBias8 + 1;
 
 QL_DEV unsigned sig_hi(unsigned hw, unsigned lw) { return (__funnelshift_l(lw, hw, 10) & 0x3fffffffu) | 0x40000000u; }
 
 template <bool FAR>
-QL_DEV u64 cut56(unsigned h, unsigned l, unsigned sign_word, int s) {
+QL_DEV u64 cut56(unsigned h, unsigned l, int s) {
   unsigned ql = __funnelshift_r(l, h, s), qh = h >> (s & 31);
   if constexpr (FAR) {
     if (s > 31) {
@@ -128,14 +151,14 @@ QL_DEV u64 cut56(unsigned h, unsigned l, unsigned sign_word, int s) {
       qh = 0u;
     }
   }
-  const unsigned m = (unsigned)((int)sign_word >> 31);
-  return (((u64)(qh ^ m) << 32) | (ql ^ m)) + kCutBias;
+  return (((u64)qh << 32) | ql) + kCutBias;
 }
 
 // Planes 7 - 2 K and 6 - 2 K of eight elements: two adjacent 7-bit fields per element and
-// shift, packed for rows (r, r + 1) into one word each, bf16(128 + f) - 192 = f - 64.
+// shift, packed for rows (r, r + 1) into one word each; bf16(128 + f) sg - 192 sg = sg (f - 64)
+// in one packed multiply-add gives the signed digit.
 template <int PLANE, int K>
-QL_DEV void put_plane_pairs(unsigned char* base, const u64 (&Nb)[8]) {
+QL_DEV void put_plane_pairs(unsigned char* base, const u64 (&Nb)[8], const unsigned (&sg)[4]) {
   unsigned lo[4], hi[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
@@ -143,15 +166,17 @@ QL_DEV void put_plane_pairs(unsigned char* base, const u64 (&Nb)[8]) {
     const unsigned t = __byte_perm(fa, fb, 0x5410);
     const unsigned wl = (t & 0x007f007fu) | 0x43004300u;
     const unsigned wh = ((t >> 7) & (K == 3 ? 0x00ff00ffu : 0x007f007fu)) | 0x43004300u;
-    const __nv_bfloat162 off = __floats2bfloat162_rn(192.0f, 192.0f);
-    const __nv_bfloat162 rl = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&wl), off);
-    const __nv_bfloat162 rh = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&wh), off);
+    const unsigned one = sg[e] | 0x3f803f80u, off = sg[e] ^ 0xc340c340u;  // +-1, -+192
+    const __nv_bfloat162 m = *reinterpret_cast<const __nv_bfloat162*>(&one);
+    const __nv_bfloat162 c = *reinterpret_cast<const __nv_bfloat162*>(&off);
+    const __nv_bfloat162 rl = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&wl), m, c);
+    const __nv_bfloat162 rh = __hfma2(*reinterpret_cast<const __nv_bfloat162*>(&wh), m, c);
     lo[e] = *reinterpret_cast<const unsigned*>(&rl);
     hi[e] = *reinterpret_cast<const unsigned*>(&rh);
   }
   *reinterpret_cast<uint4*>(base + (7 - 2 * K) * PLANE) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
   *reinterpret_cast<uint4*>(base + (6 - 2 * K) * PLANE) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-  if constexpr (K < 3) put_plane_pairs<PLANE, K + 1>(base, Nb);
+  if constexpr (K < 3) put_plane_pairs<PLANE, K + 1>(base, Nb, sg);
 }
 
 // Eight rows of one column as raw words.
@@ -167,7 +192,11 @@ struct Rows8<double> {
     return a;
   }
   QL_DEV static int exponent(unsigned amax) { return (int)(amax >> 20); }
-  QL_DEV int shift(int j, int base) const { return base - (int)((hw[j] & 0x7fffffffu) >> 20); }
+  // the scale's shift base (an all-zero column: far for every element), an element's shift
+  // modulo kWrap, and the bits of it that are zero unless the element is far
+  static constexpr int kWrap = 2048, kFar = 0x7e0;
+  QL_DEV static int base(int Es) { return Es > 0 ? Es + 7 : 2000; }
+  QL_DEV int shift(int j, int base) const { return base - (int)(hw[j] >> 20); }
   QL_DEV unsigned h(int j) const { return sig_hi(hw[j], lw[j]); }
   QL_DEV unsigned l(int j) const { return lw[j] << 10; }
   QL_DEV void set(int j, double x) {
@@ -194,7 +223,9 @@ struct Rows8<float> {
     const int ef = (int)(amax >> 23);
     return ef == 0 ? 0 : ef + 896;
   }
-  QL_DEV int shift(int j, int base) const { return base - 896 - (int)((hw[j] & 0x7fffffffu) >> 23); }
+  static constexpr int kWrap = 256, kFar = 0xe0;
+  QL_DEV static int base(int Es) { return Es > 0 ? Es + 7 - 896 : 200; }
+  QL_DEV int shift(int j, int base) const { return base - (int)(hw[j] >> 23); }
   QL_DEV unsigned h(int j) const { return ((hw[j] << 7) & 0x3fffffffu) | 0x40000000u; }
   QL_DEV unsigned l(int) const { return 0u; }
   QL_DEV void set(int j, float x) { hw[j] = __float_as_uint(x); }
@@ -224,10 +255,41 @@ QL_DEV void umma_commit_if(uint32_t leader, uint64_t* mbar) {
       "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_addr(mbar)),
       "r"(leader));
 }
-// The common case of a bounded wait: the phase is already over.
-QL_DEV bool mbar_wait_fast(uint64_t* mbar, uint32_t parity) {
-  return mbar_try_wait(mbar, parity) || mbar_wait_bounded(mbar, parity);
+// Wait for a phase, at most 2^32 clocks (about 2 s).  The wait that gives up records `code` in
+// *fail; once that is set every other wait that would block gives up at once, so the roles of
+// the CTA run through with whatever the buffers hold and the call is redone.
+QL_DEV bool xg_wait(uint64_t* mbar, uint32_t parity, volatile int* fail, int code) {
+  if (mbar_try_wait(mbar, parity)) return true;
+  const long long t0 = clock64();
+  do {
+    if (mbar_try_wait(mbar, parity)) return true;
+    if (*fail) return false;
+  } while (clock64() - t0 <= (1ll << 32));
+  *fail = code;
+  return false;
 }
+// Whether a phase is over (never suspends the thread).
+QL_DEV bool mbar_test_wait(uint64_t* mbar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n.reg .pred P1;\nmbarrier.test_wait.parity.shared::cta.b64 P1, [%1], %2;\n"
+      "selp.b32 %0, 1, 0, P1;\n}\n"
+      : "=r"(done)
+      : "r"(smem_addr(mbar)), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+// Named barriers of the slicers: 1 and 2 one group each (with a vote), 3 both.
+QL_DEV bool group_or(int g, bool p) {
+  uint32_t r;
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbar.red.or.pred q, %2, 256, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((uint32_t)p), "r"(g + 1)
+      : "memory");
+  return r != 0;
+}
+QL_DEV void joint_sync() { asm volatile("bar.sync 3, 512;\n" ::: "memory"); }
 // One box of a rank-3 tensor map (x = row in its 128-byte block, y = column, z = block).
 QL_DEV void tma_load_3d(void* dst, const CUtensorMap* tm, int x, int y, int z, uint64_t* mbar) {
   asm volatile(
@@ -240,16 +302,14 @@ QL_DEV void tma_load_3d(void* dst, const CUtensorMap* tm, int x, int y, int z, u
 // The MMAs of one tile (whole warp, issued by the elected lane): d0 is the descriptor of
 // plane 0, k-step 0.
 template <int NC>
-QL_DEV void xg_issue_mmas(uint32_t leader, uint32_t tbase, uint64_t d0, uint32_t fresh) {
+QL_DEV void xg_issue_mmas(uint32_t leader, uint32_t tbase, uint64_t d0, bool fresh) {
   using Sh = XgShape<NC>;
   constexpr uint64_t PL = Sh::PLANE >> 4;
 #pragma unroll 1
-  for (int kk = 0; kk < Sh::KT / 16; ++kk) {
+  for (int kk = 0; kk < Sh::KV / 16; ++kk) {
     const uint64_t dk = d0 + (uint64_t)((kk * 2 * Sh::LBO) >> 4);
     const uint32_t first = (!fresh || kk > 0) ? 1u : 0u;
-    if constexpr (NC == 8) {
-      umma_bf16_if(leader, tbase, dk, dk, umma_idesc_bf16(128, 64), first);
-    } else if constexpr (NC == 16) {
+    if constexpr (NC <= 16) {
       umma_bf16_if(leader, tbase, dk, dk, umma_idesc_bf16(128, 128), first);
     } else if constexpr (NC == 32) {
       umma_bf16_if(leader, tbase, dk, dk, umma_idesc_bf16(128, 256), first);
@@ -272,7 +332,10 @@ QL_DEV void xg_issue_mmas(uint32_t leader, uint32_t tbase, uint64_t d0, uint32_t
   }
 }
 
-// tcgen05.ld of two columns (the 8-column class).
+// tcgen05.ld of one and two columns (the narrow classes).
+QL_DEV void tmem_ld(uint32_t taddr, uint32_t (&v)[1]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n" : "=r"(v[0]) : "r"(taddr));
+}
 QL_DEV void tmem_ld(uint32_t taddr, uint32_t (&v)[2]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];\n" : "=r"(v[0]), "=r"(v[1]) : "r"(taddr));
 }
@@ -685,11 +748,12 @@ QL_DEV void xg_finish(const GramArgs<S>& a, unsigned char* smem, const int* colm
 // Row tiles [tiles bid / k, tiles (bid + 1) / k) of one problem; tensor memory at tbase and
 // barriers set up by xg_cta_begin, phases carried in bars (see gram_pipe_body).
 template <int NC, typename S>
-QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& bars, const XgMaps* maps) {
+QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& bars, const CUtensorMap* map,
+                       int slot) {
   using Sh = XgShape<NC>;
   using Sm = XgSmem<NC, S>;
   constexpr int T = Sh::T, TS = Sh::TS, KT = Sh::KT, PLANE = Sh::PLANE, SBO = Sh::SBO, LBO = Sh::LBO, HALF = Sh::HALF,
-                RPB = Sm::RPB, NBOX = Sm::NBOX, LG = Sh::LG;
+                RPB = Sm::RPB, LG = Sh::LG, VC = Sh::VC, SEG = Sh::SEG, KV = Sh::KV;
   extern __shared__ __align__(1024) unsigned char smem_umma[];
   unsigned char* smem = smem_umma;
   const int tid = threadIdx.x, n = a.n, lane = tid & 31, warp = tid >> 5;
@@ -704,15 +768,19 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
   uint64_t* lbar = mbar + 2;                                          // [2] tile landed, per raw stage
   uint64_t* dbar = mbar + 4;                                          // [2] digits ready, per digit buffer
   uint64_t* rbar = mbar + 6;                                          // [2] stage read, per raw stage
-  int* ngrp = reinterpret_cast<int*>(smem + Sm::kOffSlot + 4);        // [2] tile opens a new group
-  int* sfail = ngrp + 2;                                              // [3] where each role gave up
+  uint64_t* vbar = mbar + 8;                                          // [2] vote passed, per slicer group
+  int* place = reinterpret_cast<int*>(smem + Sm::kOffSlot + 4);       // [2] the tile's place in its read-out
+  volatile int* fail = place + 2;                                     // where the first wait gave up
+  volatile int* req = place + 3;                                      // a column outgrew its scale
+  volatile int* pos = place + 4;                                      // [2] next tile of each group
 
   a.tiles = (a.m + KT - 1) / KT;
   for (int i = tid; i < NC; i += T) {
     colmax[i] = 0;
     scale[i] = 0;
   }
-  if (tid < 3) sfail[tid] = 0;
+  if (tid == 0) *fail = 0;
+  if (tid == 0) *req = 0;
   if constexpr (Sh::PAD > 0) {
     for (int z = 0; z < 3; ++z)
       for (int i = tid; i < Sh::PAD / 16; i += T)
@@ -725,95 +793,66 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
   __syncthreads();
   tc_fence_after();
 
-  const int64_t t0 = a.tiles * bid / k, t1 = a.tiles * (bid + 1) / k;
-  const bool bulk = a.bulk != 0;  // tensor copies; otherwise the slicers read X from global memory
+  const int64_t t0 = a.tiles * bid / k;
+  const int nt = (int)(a.tiles * (bid + 1) / k - t0);  // tiles of this CTA, i = 0 .. nt - 1
+  // full tiles (i < nbulk) arrive by tensor copies when the columns allow them; the last rows
+  // of the matrix, and unaligned columns, are read by the slicers from global memory
+  const int nbulk = a.bulk ? (int)min((int64_t)nt, a.m / KT - t0) : 0;
+  // tile i = 2 j + b uses stage and buffer b; the phase of its barriers has this parity
+  auto par = [&](int i) { return ((bars.mpar >> (i & 1)) ^ (uint32_t)(i >> 1)) & 1u; };
+  auto lpar = [&](int i) { return ((bars.lpar >> (i & 1)) ^ (uint32_t)(i >> 1)) & 1u; };
 
-  // this slicer's unit of a tile: rows r0..r0+7 of column cu (8 consecutive threads hold 8
-  // consecutive columns, so their digit stores fill whole core-matrix rows)
-  const int u8 = (tid & (TS - 1)) >> 3;
-  const int cu = 8 * (u8 / (KT / 8)) + (tid & 7), r0 = 8 * (u8 % (KT / 8));
-  const bool live = cu < n && !control;
   // read-out role: TMEM lane quarter qd, columns hh HALF + [0, HALF) of C; lane L belongs to
-  // lane group lg (plane, or weight parity) and row li of C
+  // lane group lg (plane, or weight parity), row segment seg and row li of C
   const int qd = warp & 3, hh = (warp >> 2) & 3;
-  const int L = 32 * qd + lane, lg = L / NC, li = L % NC;
-  const bool reader = !control && lg < LG;
-  ulonglong2* acc = reinterpret_cast<ulonglong2*>(a.w.fbuf) + (size_t)bid * NC * 128;  // [column][lane]
+  const int L = 32 * qd + lane, lg = L / VC, seg = L % VC / NC, li = L % NC;
+  const int g = warp >> 3;  // slicer group
+  ulonglong2* acc = reinterpret_cast<ulonglong2*>(a.w.fbuf) + (size_t)slot * NC * 128;  // [column][lane]
 
   if (warp == TS / 32) {
-    // ---- copy warp: two tiles ahead; once the slicers have read a stage, the copy two ahead
-    // goes into it.  A full tile is one box of the rank-3 map; the last one of the matrix,
-    // whose rows end inside it, is copied by 128-byte row blocks (zeros past m).
-    bool ok = true;
-    uint32_t pend = 0u, ppar = 0u;  // bit b: a copy into stage b in flight, and its phase parity
+    // ---- copy warp: two tiles ahead, a tile per instruction (one box of the rank-3 map); once
+    // the slicers have read a stage, the copy two ahead goes into it
     const uint32_t leader = elect_one();
     const bool has_b = a.src.nA < n;
-    auto copy = [&](int64_t t, int b) {
-      if (!bulk) return;
-      unsigned char* stage = raw0 + (size_t)b * Sm::kRaw;
-      unsigned char* rhs = rhs0 + (size_t)b * Sm::kStageB;
-      const int64_t row0 = t * KT;
+    int issued = 0;  // tiles 0 .. issued - 1
+    auto copy = [&]() {
+      const int b = issued & 1;
+      const int64_t row0 = (t0 + issued) * KT;
       if (leader) {
-        if (maps->full && row0 + KT <= a.m) {
-          mbar_arrive_expect_tx(&lbar[b], (uint32_t)(Sm::kRaw + (has_b ? Sm::kStageB : 0)));
-          tma_load_3d(stage, &maps->tile, 0, 0, (int)(row0 / RPB), &lbar[b]);
-          if (has_b) bulk_g2s(rhs, a.src.b + row0, (uint32_t)Sm::kStageB, &lbar[b]);
-        } else {
-          mbar_arrive_expect_tx(&lbar[b], (uint32_t)(NBOX * n * 128));
-#pragma unroll 1
-          for (int kb = 0; kb < NBOX; ++kb) {
-            tma_load_2d(stage + (size_t)kb * NC * 128, &maps->rows, (int)row0 + kb * RPB, 0, &lbar[b]);
-            if (has_b) tma_load_2d(rhs + (size_t)kb * 128, &maps->rhs, (int)row0 + kb * RPB, 0, &lbar[b]);
-          }
-        }
+        mbar_arrive_expect_tx(&lbar[b], (uint32_t)(Sm::kRaw + (has_b ? Sm::kStageB : 0)));
+        tma_load_3d(raw0 + (size_t)b * Sm::kRaw, map, 0, 0, (int)(row0 / RPB), &lbar[b]);
+        if (has_b) bulk_g2s(rhs0 + (size_t)b * Sm::kStageB, a.src.b + row0, (uint32_t)Sm::kStageB, &lbar[b]);
       }
       __syncwarp();
-      pend |= 1u << b;
-      ppar = (ppar & ~(1u << b)) | (bars.lpar & (1u << b));
-      bars.lpar ^= 1u << b;
+      ++issued;
     };
-    if (t0 < t1) copy(t0, 0);
-    if (t0 + 1 < t1) copy(t0 + 1, 1);
-    for (int64_t t = t0; t < t1; ++t) {
-      const int b = (int)((t - t0) & 1);
-      if (!__all_sync(0xffffffffu, mbar_wait_fast(&rbar[b], (bars.mpar >> b) & 1u))) {
-        ok = false;
-        break;
-      }
-      bars.mpar ^= 1u << b;
-      pend &= ~(1u << b);
-      if (t + 2 < t1) copy(t + 2, b);
+    while (issued < 2 && issued < nbulk) copy();
+    bool ok = true;
+    for (int i = 0; i + 2 < nbulk && ok; ++i) {
+      ok = __all_sync(0xffffffffu, xg_wait(&rbar[i & 1], par(i), fail, 2));
+      if (ok) copy();
     }
-    for (int b = 0; b < 2; ++b)  // no copy may still be writing when the CTA moves on
-      if (pend & (1u << b)) mbar_wait_bounded(&lbar[b], (ppar >> b) & 1u);
-    if (!ok && lane == 0) sfail[1] = 2;
+    // no copy may still be writing when the CTA moves on
+    for (int i = issued > 2 ? issued - 2 : 0; i < issued; ++i) mbar_wait_bounded(&lbar[i & 1], lpar(i));
   } else if (control) {
     // ---- MMA warp: once a tile's digits are ready, its MMAs.  Planes and k-steps add (byte
     // offset >> 4) to the 14-bit address field, which stays below 2^14 (shared addresses
     // < 256 KB); plane -1 is the zero plane before the buffer.
     const uint32_t leader = elect_one();
     const uint64_t d0 = umma_sdesc(smem_addr(digits(0)), LBO, SBO);
-    for (int64_t t = t0; t < t1; ++t) {
-      const int b = (int)((t - t0) & 1);
-      if (!__all_sync(0xffffffffu, mbar_wait_fast(&dbar[b], (bars.mpar >> b) & 1u))) {
-        if (lane == 0) sfail[2] = 2;
-        break;
-      }
-      bars.mpar ^= 1u << b;
+    for (int i = 0; i < nt; ++i) {
+      const int b = i & 1;
+      if (!__all_sync(0xffffffffu, xg_wait(&dbar[b], par(i), fail, 2))) break;
       tc_fence_after();
-      xg_issue_mmas<NC>(leader, tbase, d0 + (uint64_t)b * ((Sh::DBUF + Sh::PAD) >> 4), (uint32_t)ngrp[b]);
+      const int at = place[b];
+      xg_issue_mmas<NC>(leader, tbase + (uint32_t)(at / Sh::G * Sh::SCOLS), d0 + (uint64_t)b * ((Sh::DBUF + Sh::PAD) >> 4),
+                        at % Sh::G == 0);
       umma_commit_if(leader, &mbar[b]);
       __syncwarp();
     }
   } else {
     // ---- slicer warps
-    bool ok = true;
-    int fail_where = 0;  // 1: a tile copy never completed, 2: the MMAs never completed
-    int grp = 0;         // tiles summed in tensor memory since the last read-out
     int nread = 0;       // read-outs in the 128-bit sums since they were last emptied
-    int last_b = 0;      // digit buffer of the latest tile handed to the MMAs
-    uint32_t cpar = 0u;  // bit b: phase parity of the MMAs of the latest tile on buffer b
-    unsigned arun = 0;   // largest |x| this slicer's column has shown (range record)
 
     // Tensor-memory sums -> 128-bit integers.  A thread folds the eight sums of its (lane,
     // column): digits q of the other factor for NC <= 32 (planes p and p + 4 for NC = 32),
@@ -821,11 +860,10 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
     // Eight sums d_q of spacing 7 or 14 bits are gathered by widening multiply-adds (one
     // instruction each) into 64-bit groups at 32-bit offsets, then carried into 128 bits.  Rows
     // of C below the diagonal block of the warp are not folded (NC = 64: a quarter of the work).
-    auto readout = [&]() {
-      constexpr int JS = HALF < 4 || NC == 32 ? 2 : 4;
+    auto readout = [&](int sets) {
+      constexpr int JS = NC == 4 ? 1 : (NC == 64 ? 4 : 2);
       const uint32_t lane_base = tbase + ((uint32_t)(32 * qd) << 16) + (uint32_t)(hh * HALF);
-      const bool keep = nread++ > 0;   // uniform: every slicer counts the read-outs
-      if (NC == 8 && qd >= 2) return;  // lanes 64..127 hold nothing
+      const bool keep = nread++ > 0;  // uniform: every slicer counts the read-outs
 #pragma unroll 1
       for (int c0 = 0; c0 < HALF; c0 += JS) {
         if (NC == 64 && hh * HALF + c0 + JS <= 32 * (qd & 1)) continue;  // columns left of every row of the warp
@@ -836,15 +874,33 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
         i128 sum[JS];
 #pragma unroll
         for (int part = 0; part < (NC == 32 ? 2 : 1); ++part) {
-          uint32_t v[8][JS];
+          int dq[JS][8];
+#pragma unroll 1
+          for (int set = 0; set < (Sh::NS == 1 ? 1 : sets); ++set) {
+            uint32_t v[8][JS];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) tmem_ld(lane_base + (uint32_t)(part * 256 + q * NC + c0), v[q]);
-          tmem_ld_wait();
+            for (int sg = 0; sg < SEG; ++sg) {  // a lane keeps the columns of its own segment
+              uint32_t w[8][JS];
+#pragma unroll
+              for (int q = 0; q < 8; ++q)
+                tmem_ld(lane_base + (uint32_t)(set * Sh::SCOLS + part * 256 + q * VC + sg * NC + c0), w[q]);
+              tmem_ld_wait();
+#pragma unroll
+              for (int q = 0; q < 8; ++q)
+#pragma unroll
+                for (int j = 0; j < JS; ++j) v[q][j] = sg == 0 || sg == seg ? w[q][j] : v[q][j];
+            }
+#pragma unroll
+            for (int j = 0; j < JS; ++j)
+#pragma unroll
+              for (int q = 0; q < 8; ++q) {
+                const int t = __float2int_rn(__uint_as_float(v[q][j]));
+                dq[j][q] = set == 0 ? t : dq[j][q] + t;  // at most 16 2^24
+              }
+          }
 #pragma unroll
           for (int j = 0; j < JS; ++j) {
-            int d[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) d[q] = __float2int_rn(__uint_as_float(v[q][j]));
+            const int(&d)[8] = dq[j];
             if constexpr (NC == 64) {  // offsets 0, 14, .., 98
               const long long a0 = mad_wide(d[5], 1 << 28, mad_wide(d[6], 1 << 14, (long long)d[7]));
               const long long a1 = mad_wide(d[3], 1 << 24, mad_wide(d[4], 1 << 10, a0 >> 32));
@@ -871,7 +927,7 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
     // 1.. hand their sums to group 0 through `scratch` (a free digit buffer).
     auto emit = [&](unsigned char* scratch) {
       ulonglong2* sc = reinterpret_cast<ulonglong2*>(scratch);
-      if (reader && lg > 0) {
+      if (lg + seg > 0) {
         constexpr int JB = HALF < 8 ? HALF : 8;
 #pragma unroll 1
         for (int j0 = 0; j0 < HALF; j0 += JB) {
@@ -879,11 +935,11 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
 #pragma unroll
           for (int j = 0; j < JB; ++j) t[j] = __ldcg(acc + (size_t)(hh * HALF + j0 + j) * 128 + L);
 #pragma unroll
-          for (int j = 0; j < JB; ++j) sc[((size_t)(lg - 1) * NC + li) * NC + hh * HALF + j0 + j] = t[j];
+          for (int j = 0; j < JB; ++j) sc[((size_t)(lg * SEG + seg - 1) * NC + li) * NC + hh * HALF + j0 + j] = t[j];
         }
       }
-      slicer_sync<TS>();
-      if (reader && lg == 0 && li < n) {
+      joint_sync();
+      if (lg + seg == 0 && li < n) {
         const int si = scale[li];
         ulonglong2 next = __ldcg(acc + (size_t)(hh * HALF) * 128 + L);
 #pragma unroll 1
@@ -893,151 +949,189 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
           if (j + 1 < HALF) next = __ldcg(acc + (size_t)(jj + 1) * 128 + L);
           if (jj < li || jj >= n) continue;
           auto part = [&](int g) -> i128 {
-            const ulonglong2 t = sc[((size_t)(g - 1) * NC + li) * NC + jj];
+            const ulonglong2 t = sc[((size_t)(g - 1) * NC + li) * NC + jj];  // g = lane group SEG + segment
             return (i128)(((u128)t.y << 64) | t.x);
           };
           if constexpr (NC == 64) {
             v += part(1) >> 7;  // odd weights: a multiple of 2^7 (weight 15 is empty)
           } else {
 #pragma unroll 1
-            for (int g = 1; g < LG; ++g) v = v * 128 + part(g);
+            for (int g = 1; g < LG * SEG; ++g) v = (g % SEG == 0 ? v * 128 : v) + part(g);
           }
           const int sj = scale[jj];
           if (si >= kEsMin && sj >= kEsMin && si <= kEsMax && sj <= kEsMax)  // else flagged at the end, or zero
             sacc_add(a.w.sacc + (size_t)tri_index(li, jj) * kLimbs, v, si + sj - 2 * kEsMin);
         }
       }
-      slicer_sync<TS>();
+      joint_sync();
       nread = 0;
     };
-    auto wait_last = [&]() {  // the MMAs of every tile handed over are done
-      return slicer_and<TS>(mbar_wait_bounded(&mbar[last_b], (cpar >> last_b) & 1u));
-    };
 
-    // where this unit lies in a staged tile: its 128-byte line and first 16-byte chunk, or the
-    // rows of the right-hand side
-    const bool rhs_unit = cu == a.src.nA;
-    const unsigned char* line0 = rhs_unit ? rhs0 + r0 * sizeof(S) : raw0 + (size_t)((r0 / RPB) * NC + cu) * 128;
-    const size_t line_step = rhs_unit ? Sm::kStageB : Sm::kRaw;
-    const int q0 = rhs_unit ? 0 : (r0 % RPB) * (int)sizeof(S) / 16, swz = rhs_unit ? 0 : (cu & 7);
-    Rows8<S> v, ahead;
-    auto load_global = [&](Rows8<S>& w, int64_t t) {
-      const S* col = a.src.col(cu) + t * KT + r0;
-      const int64_t left = a.m - (t * KT + r0);
+    // This thread's two units of a tile: rows r0 .. r0 + 7 of column cu; eight consecutive threads
+    // hold eight consecutive columns of a digit plane, so their stores fill whole core-matrix
+    // rows.  Plane column cv and row rv are column cv % NC, row rv of segment cv / NC.
+    constexpr int TG = Sh::TG;
+    const int gt = tid & (TG - 1);
+    int cu[2], r0[2];
+    const unsigned char* line[2];  // the unit in its 128-byte line of the staged tile (or in the
+    // right-hand side): chunk q of 16 bytes at this address ^ 16 q (the swizzle and the unit's
+    // first chunk, a multiple of its chunks, only flip other bits or the same ones)
+    bool live[2];
+    unsigned arun[2] = {0, 0};  // largest |x| the unit's column has shown (range record)
+    unsigned char* dst[2];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) w.set(j, j < left ? __ldg(col + j) : S(0));
+    for (int u = 0; u < 2; ++u) {
+      const int w = (gt >> 3) + u * (TG / 8), cv = 8 * (w / (KV / 8)) + (gt & 7), rv = 8 * (w % (KV / 8));
+      cu[u] = cv % NC;
+      r0[u] = cv / NC * KV + rv;
+      live[u] = cu[u] < n;
+      const int line_no = (r0[u] / RPB) * NC + cu[u];
+      const bool rhs_unit = cu[u] == a.src.nA;
+      line[u] = rhs_unit ? rhs0 + (size_t)g * Sm::kStageB + r0[u] * sizeof(S)
+                         : raw0 + (size_t)g * Sm::kRaw + (size_t)line_no * 128 +
+                               ((((r0[u] % RPB) * (int)sizeof(S) / 16) ^ (line_no & 7)) << 4);
+      dst[u] = digits(g) + (cv >> 3) * SBO + (cv & 7) * 16 + (rv >> 3) * LBO;
+    }
+    auto clear_dead = [&]() {  // columns past n: zero digits
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (!live[u])
+#pragma unroll
+          for (int p = 0; p < 8; ++p) *reinterpret_cast<uint4*>(dst[u] + p * PLANE) = make_uint4(0, 0, 0, 0);
     };
-    if (!bulk && live && t0 < t1) load_global(ahead, t0);
+    clear_dead();
 
-    for (int64_t t = t0; t < t1; ++t) {
-      const int i = (int)(t - t0), b = i & 1;
-      bool landed = true;
-      if (bulk) {
-        landed = mbar_wait_fast(&lbar[b], (bars.lpar >> b) & 1u);
-        bars.lpar ^= 1u << b;
-      }
-      unsigned am = 0;
-      int es = 0;
-      bool over = false;
-      if (live) {
-        if (bulk) {
-          const unsigned char* line = line0 + (size_t)b * line_step;
+    Rows8<S> v[2];
+    // tile i: loaded into v, voted on (no column of it outgrows its scale), cut into its buffer
+    bool have = false, voted = false, cut = false, over[2] = {false, false};
+    int es[2] = {0, 0};
+    int i = g;                 // this group's next tile
+    int first = 0;             // first tile of the sums in tensor memory
+    int done0 = 0, done1 = 1;  // the groups' positions at the last meeting
+    for (;;) {
+      bool meet = i >= nt;  // uniform in the group, like every flag but over
+      if (!meet) {
+        if (!have) {
+          const bool bulk = i < nbulk;
+          if (bulk) xg_wait(&lbar[g], lpar(i), fail, 1);
 #pragma unroll
-          for (int q = 0; q < 8 * (int)sizeof(S) / 16; ++q)
-            v.chunk(q, *reinterpret_cast<const uint4*>(line + (((q0 + q) ^ swz) << 4)));
-        } else {
-          v = ahead;
-          if (t + 1 < t1) load_global(ahead, t + 1);
-        }
-        am = v.amax();
-        arun = max(arun, am);
-        es = Rows8<S>::exponent(am);
-        over = es > scale[cu];
-      }
-      // stage b is read: the copy warp may copy the tile two ahead into it
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&rbar[b]);
-      // digit buffer b is free once the MMAs of tile t - 2 are done
-      const bool okw = i >= 2 ? mbar_wait_fast(&mbar[b], (cpar >> b) & 1u) : true;
-      const bool full = grp >= Sh::G;
-      if (slicer_or<TS>(over || !okw || !landed) || full) {
-        if (!slicer_and<TS>(landed)) {  // the copy engine did not deliver
-          ok = false;
-          fail_where = 1;
-          break;
-        }
-        if (!slicer_and<TS>(okw)) {  // the tensor core did not finish
-          ok = false;
-          fail_where = 2;
-          break;
-        }
-        const bool anyover = slicer_or<TS>(over);
-        if (grp > 0) {
-          if (!wait_last()) {
-            ok = false;
-            fail_where = 2;
-            break;
+          for (int u = 0; u < 2; ++u) {
+            if (!live[u]) continue;
+            if (bulk) {
+#pragma unroll
+              for (int q = 0; q < 8 * (int)sizeof(S) / 16; ++q)
+                v[u].chunk(q, *reinterpret_cast<const uint4*>(reinterpret_cast<uintptr_t>(line[u]) ^ (uintptr_t)(16 * q)));
+            } else {
+              const int64_t row = (t0 + i) * KT + r0[u], left = a.m - row;
+              const S* col = a.src.col(cu[u]) + row;
+#pragma unroll
+              for (int j = 0; j < 8; ++j) v[u].set(j, j < left ? __ldg(col + j) : S(0));
+            }
           }
+          // the stage is read: the copy warp may copy the tile two ahead into it
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&rbar[g]);
+          have = true;
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            if (!live[u]) continue;
+            const unsigned am = v[u].amax();
+            arun[u] = max(arun[u], am);
+            es[u] = Rows8<S>::exponent(am);
+          }
+        }
+        if (!voted) {
+          over[0] = live[0] && es[0] > scale[cu[0]];
+          over[1] = live[1] && es[1] > scale[cu[1]];
+          // the other group's vote on the tile before comes first, or it has stopped
+          bool passed = i == 0;
+          while (!passed && !*req && !*fail) passed = mbar_test_wait(&vbar[g ^ 1], par(i - 1));
+          voted = !group_or(g, over[0] || over[1] || (!passed && !*fail));
+          if (voted && gt == 0) mbar_arrive(&vbar[g]);
+        }
+        if (voted && !cut) {
+          if (i >= 2) xg_wait(&mbar[g], par(i - 2), fail, 2);  // the MMAs are done with this buffer
+          // eight digits of every element
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            if (!live[u]) continue;
+            const int base = Rows8<S>::base(scale[cu[u]]);
+            int sh[8], any = 0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              sh[j] = v[u].shift(j, base);
+              any |= sh[j];
+            }
+            unsigned sg[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              sg[e] = __byte_perm(v[u].hw[2 * e], v[u].hw[2 * e + 1], 0x7632) & 0x80008000u;
+            u64 Nb[8];
+            if (any & Rows8<S>::kFar) {  // an element more than 2^24 below the scale (or zero)
+#pragma unroll
+              for (int j = 0; j < 8; ++j) Nb[j] = cut56<true>(v[u].h(j), v[u].l(j), sh[j] & (Rows8<S>::kWrap - 1));
+            } else {
+#pragma unroll
+              for (int j = 0; j < 8; ++j) Nb[j] = cut56<false>(v[u].h(j), v[u].l(j), sh[j]);
+            }
+            put_plane_pairs<PLANE, 0>(dst[u], Nb, sg);
+          }
+          cut = true;
+        }
+        meet = !voted || i >= first + Sh::GT;
+      }
+      if (meet) {
+        // ---- both groups meet: read the sums out, and empty the 128-bit ones when a scale
+        // rises (their unit changes) or they are full, and at the end
+        if (have && !voted && (over[0] || over[1])) *req = 1;
+        if (gt == 0) pos[g] = i;
+        joint_sync();
+        const int p0 = pos[0], p1 = pos[1];  // the first tile of each group not handed over
+        const bool raise = *req != 0, last = p0 >= nt && p1 >= nt;
+        if (p0 > done0 || p1 > done1) {
+          if (p0 > 0) xg_wait(&mbar[0], par(p0 - 2), fail, 2);
+          if (p1 > 1) xg_wait(&mbar[1], par(p1 - 2), fail, 2);
           tc_fence_after();
-          readout();
-          grp = 0;
+          readout((min(p0, p1) - first + Sh::G - 1) / Sh::G);
         }
-        if (nread > 0 && (anyover || nread >= Sh::MAX_READS)) emit(digits(0));  // every MMA is done: both buffers are free
-        if (anyover) {
-          slicer_sync<TS>();  // every read of the old scales is done
-          if (over) atomicMax(&scale[cu], max(es + Sh::SLACK, kEsMin));
+        const bool empty = nread > 0 && (raise || last || nread >= Sh::MAX_READS);
+        if (empty) {
+          emit(digits(0));  // every MMA is done: the buffers are free, and cut again below
+          clear_dead();
         }
-        slicer_sync<TS>();
+        joint_sync();  // every read of the flags, the scales and the sums is done
+        if (last) break;
+        if (raise) {
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+            if (have && !voted && over[u]) atomicMax(&scale[cu[u]], max(es[u] + Sh::SLACK, kEsMin));
+          if (tid == 0) *req = 0;
+        }
+        joint_sync();
+        if (raise || empty) cut = false;
+        done0 = p0;
+        done1 = p1;
+        first = min(p0, p1);
+        continue;
       }
-      // eight digits of every element into buffer b
-      unsigned char* dst = digits(b) + (cu >> 3) * SBO + (r0 >> 3) * LBO + (cu & 7) * 16;
-      if (live) {
-        const int Es = scale[cu], base = Es > 0 ? Es + 7 : 4096;
-        int s[8], any = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          s[j] = v.shift(j, base);
-          any |= s[j];
-        }
-        u64 Nb[8];
-        if (any > 31) {  // an element more than 2^24 below the scale (or zero)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) Nb[j] = cut56<true>(v.h(j), v.l(j), v.hw[j], s[j]);
-        } else {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) Nb[j] = cut56<false>(v.h(j), v.l(j), v.hw[j], s[j]);
-        }
-        put_plane_pairs<PLANE, 0>(dst, Nb);
-      } else {
-#pragma unroll
-        for (int p = 0; p < 8; ++p) *reinterpret_cast<uint4*>(dst + p * PLANE) = make_uint4(0, 0, 0, 0);
-      }
-      if (tid == 0) ngrp[b] = grp == 0 ? 1 : 0;
+      if (gt == 0) place[g] = i - first;
       fence_proxy_async_smem();  // the digit planes are read by the tensor core
       tc_fence_before();         // the read-out's TMEM loads come before the next MMAs
       __syncwarp();
-      if (lane == 0) mbar_arrive(&dbar[b]);
-      cpar = (cpar & ~(1u << b)) | (bars.mpar & (1u << b));
-      bars.mpar ^= 1u << b;
-      last_b = b;
-      ++grp;
+      if (lane == 0) mbar_arrive(&dbar[g]);
+      have = voted = cut = false;
+      i += 2;
     }
-    if (ok && grp > 0) {  // the last group
-      if (!wait_last()) {
-        ok = false;
-        fail_where = 2;
-      } else {
-        tc_fence_after();
-        readout();
-      }
-    }
-    if (ok && nread > 0) emit(digits(0));
-    if (!ok && tid == 0) sfail[0] = fail_where;
-    if (live && arun > 0) atomicMax(&colmax[cu], Rows8<S>::exponent(arun));
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (live[u] && arun[u] > 0) atomicMax(&colmax[cu[u]], Rows8<S>::exponent(arun[u]));
   }
+  // every thread carries the same phase counts to the next work item
+  bars.mpar ^= (uint32_t)(((nt + 1) >> 1) & 1) | (uint32_t)((nt >> 1) & 1) << 1;
+  bars.lpar ^= (uint32_t)(((nbulk + 1) >> 1) & 1) | (uint32_t)((nbulk >> 1) & 1) << 1;
   tc_fence_before();
   __syncthreads();
-  const int fw = sfail[0] ? sfail[0] : (sfail[1] ? sfail[1] : sfail[2]);
+  const int fw = *fail;
   if (fw) {
     bars.ok = false;  // a late arrival may still complete a phase: the CTA takes no more work
     if (tid == 0) {   // the gated launches redo the call and report {QL_ERR_TIMEOUT, where}
@@ -1054,11 +1148,12 @@ template <int NC, typename S>
 QL_DEV uint32_t xg_cta_begin(unsigned char* smem) {
   using Sm = XgSmem<NC, S>;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + Sm::kOffSlot);
-  if ((threadIdx.x >> 5) == 0) tmem_alloc(tslot, XgShape<NC>::TCOLS);
+  if ((threadIdx.x >> 5) == 0) tmem_alloc(tslot, 512);
   if (threadIdx.x == 0) {
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + Sm::kOffBar);
     for (int i = 0; i < 4; ++i) mbar_init(bar + i, 1);
-    for (int i = 4; i < 8; ++i) mbar_init(bar + i, XgShape<NC>::TS / 32);  // one arrival per slicer warp
+    for (int i = 4; i < 8; ++i) mbar_init(bar + i, XgShape<NC>::TG / 32);  // one arrival per warp of the group
+    for (int i = 8; i < 10; ++i) mbar_init(bar + i, 1);
   }
   tc_fence_before();
   __syncthreads();
@@ -1068,14 +1163,14 @@ QL_DEV uint32_t xg_cta_begin(unsigned char* smem) {
 
 template <int NC, typename S>
 __global__ void __launch_bounds__(XgShape<NC>::T, 1)
-    xgram_kernel(const __grid_constant__ GramArgs<S> a, const __grid_constant__ XgMaps maps) {
+    xgram_kernel(const __grid_constant__ GramArgs<S> a, const __grid_constant__ CUtensorMap map) {
   extern __shared__ __align__(1024) unsigned char smem_umma[];
   const uint32_t tbase = xg_cta_begin<NC, S>(smem_umma);
   PipeBars bars;
-  xgram_body<NC, S>(a, blockIdx.x, gridDim.x, tbase, bars, &maps);
+  xgram_body<NC, S>(a, blockIdx.x, gridDim.x, tbase, bars, &map, blockIdx.x);
   tc_fence_before();
   __syncthreads();
-  if ((threadIdx.x >> 5) == 0) tmem_dealloc(tbase, XgShape<NC>::TCOLS);
+  if ((threadIdx.x >> 5) == 0) tmem_dealloc(tbase, 512);
 }
 
 template <int NC, typename S>
@@ -1117,19 +1212,20 @@ ql_status xgram_launch_one(const GramCall& c, const GramWs& w) {
   a.resnorm = c.resnorm;
   a.Rext = c.Rext;
   a.info = c.info;
-  XgMaps maps{};
-  a.bulk = xg_tensor_maps(&maps, NC, c.A, c.nA < c.n ? c.b : nullptr,
-                          std::is_same<S, double>::value ? QL_F64 : QL_F32, c.m, c.nA, c.lda)
+  CUtensorMap map{};
+  a.bulk = xg_tensor_map(&map, NC, c.A, c.nA < c.n ? c.b : nullptr, std::is_same<S, double>::value ? QL_F64 : QL_F32,
+                         c.m, c.nA, c.lda)
                ? 1
                : 0;
   a.mround = NC >= 16 ? 2 : 1;  // how the next pass's kernel of this class reads M
   count_launch();
-  kern<<<(int)g, Sh::T, Sm::kBytes, c.stream>>>(a, maps);
+  kern<<<(int)g, Sh::T, Sm::kBytes, c.stream>>>(a, map);
   return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
 template <typename S>
 ql_status xgram_pass1(const GramCall& c, const GramWs& w) {
+  if (c.n <= 4) return xgram_launch_one<4, S>(c, w);
   if (c.n <= 8) return xgram_launch_one<8, S>(c, w);
   if (c.n <= 16) return xgram_launch_one<16, S>(c, w);
   if (c.n <= 32) return xgram_launch_one<32, S>(c, w);

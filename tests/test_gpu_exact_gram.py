@@ -1,4 +1,4 @@
-"""The exact Gram route of TSQR (n >= 5): tile edges, column classes, scale changes, zero and
+"""The exact Gram route (n >= 2): tile edges, column classes, scale changes, zero and
 dependent columns, unaligned columns, and the hand-over to the Householder tiles.
 
 Tolerance.  X is rounded to 2^-56 of each column's largest entry and everything after that is
@@ -33,10 +33,10 @@ def gram_error(R, X):
     return np.abs((R.T @ R - G) / np.where(d > 0, d, 1)[:, None] / np.where(d > 0, d, 1)[None, :]).max()
 
 
-@pytest.mark.parametrize("n", [5, 8, 9, 16, 17, 32, 33, 64])
+@pytest.mark.parametrize("n", [2, 4, 5, 8, 9, 16, 17, 32, 33, 64])
 @pytest.mark.parametrize("dtype", [np.float64, np.float32])
 def test_tile_edges_against_oracle(n, dtype):
-    kt = 4096 // (8 if n <= 8 else 16 if n <= 16 else 32 if n <= 32 else 64)
+    kt = 4096 // (4 if n <= 4 else 8 if n <= 8 else 16 if n <= 16 else 32 if n <= 32 else 64)
     for m, pad in ((n, 0), (kt - 1, 1), (kt, 0), (kt + 1, 2), (3 * kt + 5, 3)):
         X = synth.conditioned(max(m, n), n, 100.0, seed=m + n, dtype=dtype)
         R, info = tsqr(X, pad)
@@ -47,7 +47,7 @@ def test_tile_edges_against_oracle(n, dtype):
         assert oracle.rel_err(R, ref) <= oracle.tolerance(n, kappa), (m, pad)
 
 
-@pytest.mark.parametrize("n,log2m", [(8, 18), (16, 17), (32, 16), (64, 16)])
+@pytest.mark.parametrize("n,log2m", [(3, 19), (8, 18), (16, 17), (32, 16), (64, 16)])
 def test_many_tiles_per_cta_exact_r(n, log2m):
     X, R0 = synth.hadamard_exact_case(1 << log2m, n, 1e4, seed=n)
     R, info = tsqr(X)
@@ -55,7 +55,7 @@ def test_many_tiles_per_cta_exact_r(n, log2m):
     assert oracle.rel_err(R, R0) <= 1e-15  # R0 is exact; R rounds once per entry
 
 
-@pytest.mark.parametrize("n,m", [(5, 200001), (16, 100003), (32, 60002), (64, 40000)])
+@pytest.mark.parametrize("n,m", [(4, 500002), (5, 200001), (16, 100003), (32, 60002), (64, 40000)])
 def test_growing_rows_raise_the_column_scales(n, m):
     X = synth.gaussian(m, n, seed=n) * np.exp2(np.floor(24.0 * np.arange(m) / m))[:, None]
     R, info = tsqr(X)
@@ -74,7 +74,7 @@ def test_zero_and_far_apart_entries(n):
     assert gram_error(R, X) <= 1e-14 * n
 
 
-@pytest.mark.parametrize("n", [8, 20, 64])
+@pytest.mark.parametrize("n", [4, 8, 20, 64])
 def test_dependent_columns_go_to_householder(n):
     X = synth.gaussian(3000, n, seed=5)
     X[:, n - 1] = X[:, 0]              # pivot exactly zero: the Householder tiles redo the call
@@ -92,7 +92,7 @@ def test_very_ill_conditioned_matches_oracle():
         assert oracle.rel_err(R, oracle.householder_r(X)) <= oracle.tolerance(12, kappa)
 
 
-@pytest.mark.parametrize("n", [7, 16, 33])
+@pytest.mark.parametrize("n", [4, 7, 16, 33])
 @pytest.mark.parametrize("kappa,rank_tol", [(1e3, 0.0), (1e3, 1e-4), (1e7, 0.0)])
 def test_svqb2_with_and_without_z_agree(n, kappa, rank_tol):
     """Z forces both eigensolves; without it the exact pass may answer, but not where an
@@ -109,7 +109,7 @@ def test_svqb2_with_and_without_z_agree(n, kappa, rank_tol):
     assert oracle.rel_err(R.cpu().numpy(), Rz.cpu().numpy()) <= 2 * oracle.tolerance(n, min(kappa, 1e6))
 
 
-@pytest.mark.parametrize("n", [6, 20, 40])
+@pytest.mark.parametrize("n", [3, 6, 20, 40])
 def test_gram_methods_against_oracle_on_both_sides_of_the_limits(n):
     import torch
 
