@@ -261,11 +261,12 @@ typedef struct {
  * of a problem is its method_hint, or for QL_AUTO the autotune table entry of its
  * (m, n, dtype, kappa) class (ql_autotune), else Cholesky-QR2 from 24 columns when
  * 0 < kappa_hint <= 1e6 and TSQR otherwise; the Gram method needs n (+1 for least squares)
- * >= 9, narrower problems always run TSQR.  All TSQR problems run in ONE persistent launch
- * (work list of row-tile chunks, per-problem R-trees); the Cholesky-QR2 problems run as
- * work items of one persistent launch per (column class, storage, pass) of the
- * tensor-core Gram kernels.  A problem that leaves the double-float range, or (QL_AUTO)
- * whose Cholesky breaks down, is redone by a final gated FP64 TSQR launch.  The plan lives
+ * >= 9, narrower problems always run TSQR.  All problems run as work items (row-tile chunks)
+ * of ONE persistent launch of the exact Gram pass (see ql_tsqr_qless); Cholesky-QR2 problems
+ * asked for by method_hint keep a second pass per (column class, storage), which ends at once
+ * unless a pivot fell below the method's limit.  A problem that leaves the double-float
+ * range, or whose pivots fall below the limit of a TSQR call (QL_TSQR, QL_AUTO), is redone by
+ * a final gated Householder launch with per-problem R-trees.  The plan lives
  * in `ws` (ql_batch_workspace_bytes) and is rebuilt on every call.  Equivalent, problem by
  * problem, to the single-call entry points up to rounding order.
  */

@@ -6,18 +6,17 @@
 // TSQR otherwise).  The Gram method covers n >= 9 (tensor-core kernels); narrower problems
 // always run TSQR.
 //
-// TSQR problems run in ONE persistent launch.  The host plan splits every problem into
-// chunks of row tiles (the leaves of that problem's R-tree) and orders the problems by
-// decreasing work.  A fixed grid of persistent CTAs claims chunks through one atomic
-// counter; a CTA factors its chunk with the single-problem tile machinery (tsqr.cuh) of
-// the problem's column class, stores the leaf triangle and climbs that problem's tree;
-// whoever completes a root writes R (or the least-squares solution).
+// In double-float mode every problem, of either method, is a run of work items of ONE grouped
+// exact Gram launch (xgram_group.cu; chunks of row tiles, the problems by decreasing work).  A
+// TSQR problem, or an automatically chosen Cholesky-QR2 one, that the exact route cannot answer
+// (a pivot below its limit, data outside the range) is redone by the batch's last launch with
+// Householder tiles; the host plan splits every problem into chunks for it as well (the leaves
+// of that problem's R-tree).  Cholesky-QR2 problems asked for by method_hint keep their second
+// passes (batch_gram.cu), which end at once unless a pivot fell below the method's limit.
 //
-// Cholesky-QR2 problems run as work items of grouped persistent Gram launches, one per
-// (column class, storage, pass) (batch_gram.cu).  Stream order: the Gram first passes, the
-// TSQR launch, the Gram second passes, then a gated FP64 TSQR launch that redoes every
-// flagged problem -- TSQR problems whose data leave the double-float range, and Gram
-// problems that left it or (method chosen automatically) whose Cholesky broke down.
+// Stream order: the exact launch, the second Gram passes if there are any, then the gated
+// Householder launch: double-float for kRedoDF, FP64 for kRedoF64 (range, or an explicit
+// Cholesky-QR2 that left it).  In FP64 mode the persistent TSQR kernel takes every problem.
 #include <algorithm>
 #include <cstddef>
 #include <cstring>
@@ -80,17 +79,25 @@ struct BatchItem {
 
 constexpr int kMaxGramGroups = 6;  // column classes 16, 32, 64 x storage F64, F32
 struct BatchHeader {
-  int work_counter[2];  // [0] double-float launch, [1] gated FP64 launch
+  int work_counter[3];  // [0] persistent TSQR launch, [1] gated launch, [2] exact launch
   int count;
-  int pad;
   int64_t total_work;     // chunks of every problem (the gated FP64 launch)
   int64_t total_work_df;  // chunks of the TSQR problems, which come first
   int gram_counter[2 * kMaxGramGroups];  // per group and pass
 };
 
+// The outputs of one problem from its triangle Ra (shared memory, ld nc).
+QL_DEV void batch_write(const BatchItem& it, double* Ra, int nc, double* sd, int* s_flag, int tmo) {
+  if (it.kind == 0)
+    epilogue_r<kBatchT>(Ra, nc, it.n, it.R, it.n, it.info, s_flag, tmo);
+  else
+    epilogue_lstsq<kBatchT>(Ra, nc, it.n, it.x, it.x + (it.n - 1), it.R, it.info, sd, s_flag, tmo);
+  __syncthreads();
+}
+
 template <int NC, typename S, typename Ar>
 QL_DEV void batch_chunk(const BatchItem& it, int64_t chunk, unsigned char* smem, double* slots, int* counters,
-                        int* flags) {
+                        int* flags, bool in_redo) {
   constexpr int TC = BatchCls<NC>::TC, RPT = BatchCls<NC>::RPT, T = kBatchT;
   using Cta = TsqrCta<NC, TC, RPT, T, S, Ar>;
   Cta cta;
@@ -111,7 +118,7 @@ QL_DEV void batch_chunk(const BatchItem& it, int64_t chunk, unsigned char* smem,
   cta.run(p, 0, t0, t1);
   const int n = it.n;
   if (threadIdx.x == 0 && cta.out_of_range(n, it.m)) {
-    atomicOr(&flags[it.flag_idx], 1);
+    atomicOr(&flags[it.flag_idx], in_redo ? kRedoDFRange : kRedoF64);
     atomicOr(&flags[-1], 1);  // any_flag lives just before the per-problem flags
   }
   TreeView tv;
@@ -127,37 +134,53 @@ QL_DEV void batch_chunk(const BatchItem& it, int64_t chunk, unsigned char* smem,
   double* Ra = cta.arena;
   if (!climb_tree<NC, T>(tv, (int)chunk, n, cta.arena, cta.sd, &cta.misc[1], tree_arity<NC>())) return;
   __threadfence();
-  if (Ar::kRangeChecked && *(volatile int*)&flags[it.flag_idx] != 0) return;
+  const int flag = *(volatile int*)&flags[it.flag_idx];
+  if constexpr (Ar::kRangeChecked) {
+    if (in_redo && (flag & kRedoDFRange)) {
+      // columns both dependent and, in some row block, out of the double-float range (which the
+      // exact launch's own chunks did not show): the root's CTA refactors the problem in FP64
+      __syncthreads();
+      using Cta64 = TsqrCta<NC, TC, RPT, T, S, ArithF64>;
+      Cta64 whole;
+      whole.init(smem);
+      whole.reset_r();
+      __syncthreads();
+      whole.run(p, 0, 0, it.tiles);
+      __syncthreads();
+      for (int i = threadIdx.x; i < NC * NC; i += T) whole.arena[i] = (i / NC <= i % NC) ? whole.R[i] : 0.0;
+      __syncthreads();
+      batch_write(it, whole.arena, NC, whole.sd, &whole.misc[2], (flag >> 8) & 0xff);
+      return;
+    }
+    if (flag != 0 && !in_redo) return;
+  }
   // a Gram pass whose bounded wait gave up put the place into bits 8.. of the redo flag
-  const int tmo = Ar::kRangeChecked ? 0 : (*(volatile int*)&flags[it.flag_idx] >> 8) & 0xff;
-  if (it.kind == 0)
-    epilogue_r<T>(Ra, NC, n, it.R, n, it.info, &cta.misc[2], tmo);
-  else
-    epilogue_lstsq<T>(Ra, NC, n, it.x, it.x + (n - 1), it.R, it.info, cta.sd, &cta.misc[2], tmo);
-  __syncthreads();
+  batch_write(it, Ra, NC, cta.sd, &cta.misc[2], (flag >> 8) & 0xff);
 }
 
 template <typename S, typename Ar>
 QL_DEV void batch_dispatch(const BatchItem& it, int64_t chunk, unsigned char* smem, double* slots, int* counters,
-                           int* flags) {
+                           int* flags, bool in_redo) {
   switch (it.nc) {
-    case 4: batch_chunk<4, S, Ar>(it, chunk, smem, slots, counters, flags); break;
-    case 8: batch_chunk<8, S, Ar>(it, chunk, smem, slots, counters, flags); break;
-    case 16: batch_chunk<16, S, Ar>(it, chunk, smem, slots, counters, flags); break;
-    case 32: batch_chunk<32, S, Ar>(it, chunk, smem, slots, counters, flags); break;
-    default: batch_chunk<64, S, Ar>(it, chunk, smem, slots, counters, flags); break;
+    case 4: batch_chunk<4, S, Ar>(it, chunk, smem, slots, counters, flags, in_redo); break;
+    case 8: batch_chunk<8, S, Ar>(it, chunk, smem, slots, counters, flags, in_redo); break;
+    case 16: batch_chunk<16, S, Ar>(it, chunk, smem, slots, counters, flags, in_redo); break;
+    case 32: batch_chunk<32, S, Ar>(it, chunk, smem, slots, counters, flags, in_redo); break;
+    default: batch_chunk<64, S, Ar>(it, chunk, smem, slots, counters, flags, in_redo); break;
   }
 }
 
-template <typename Ar>
+// MODE 0: every problem in FP64.  1: the TSQR problems in double-float.  2: the gated launch behind
+// either: problems flagged kRedoF64 in FP64, those flagged kRedoDF in double-float.
+template <int MODE>
 __global__ void __launch_bounds__(kBatchT, 1)
-    batch_kernel(BatchHeader* hdr, const BatchItem* items, int count, double* slots, int* counters, int* flags,
-                 int gated) {
+    batch_kernel(BatchHeader* hdr, const BatchItem* items, int count, double* slots, int* counters, int* flags) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int64_t s_work;
   __shared__ int s_item;
-  if (gated && *(volatile int*)&flags[-1] == 0) return;  // no problem left the range
-  const int64_t total = gated ? hdr->total_work : hdr->total_work_df;
+  constexpr bool gated = MODE == 2;
+  if (gated && *(volatile int*)&flags[-1] == 0) return;  // nothing to redo
+  const int64_t total = MODE == 1 ? hdr->total_work_df : hdr->total_work;
   for (;;) {
     if (threadIdx.x == 0) {
       s_work = atomicAdd(&hdr->work_counter[gated ? 1 : 0], 1);
@@ -176,12 +199,25 @@ __global__ void __launch_bounds__(kBatchT, 1)
     __syncthreads();
     if (w >= total) break;
     const BatchItem it = items[idx];
-    if (gated && *(volatile int*)&flags[it.flag_idx] == 0) continue;
+    const int flag = gated ? *(volatile int*)&flags[it.flag_idx] : 0;
+    if (gated && (flag & (kRedoF64 | kRedoDF)) == 0) continue;
     const int64_t chunk = w - it.work_begin;
-    if (it.dtype == QL_F64)
-      batch_dispatch<double, Ar>(it, chunk, smem, slots, counters, flags);
-    else
-      batch_dispatch<float, Ar>(it, chunk, smem, slots, counters, flags);
+    const bool f64 = MODE == 0 || (gated && (flag & kRedoF64));
+    if (f64) {
+      if constexpr (MODE != 1) {
+        if (it.dtype == QL_F64)
+          batch_dispatch<double, ArithF64>(it, chunk, smem, slots, counters, flags, false);
+        else
+          batch_dispatch<float, ArithF64>(it, chunk, smem, slots, counters, flags, false);
+      }
+    } else {
+      if constexpr (MODE != 0) {
+        if (it.dtype == QL_F64)
+          batch_dispatch<double, ArithDF>(it, chunk, smem, slots, counters, flags, gated);
+        else
+          batch_dispatch<float, ArithDF>(it, chunk, smem, slots, counters, flags, gated);
+      }
+    }
     __syncthreads();
   }
 }
@@ -191,13 +227,18 @@ static size_t cls_smem() {
   return TsqrSmem<NC, BatchCls<NC>::TC, BatchCls<NC>::RPT, kBatchT, S, Ar>::kBytes;
 }
 template <typename Ar>
-static size_t batch_smem_bytes() {
+static size_t arith_smem_bytes() {
   size_t b = 0;
   b = std::max({b, cls_smem<4, float, Ar>(), cls_smem<8, float, Ar>(), cls_smem<16, float, Ar>(),
                 cls_smem<32, float, Ar>(), cls_smem<64, float, Ar>()});
   b = std::max({b, cls_smem<4, double, Ar>(), cls_smem<8, double, Ar>(), cls_smem<16, double, Ar>(),
                 cls_smem<32, double, Ar>(), cls_smem<64, double, Ar>()});
   return b;
+}
+
+static size_t batch_smem_bytes(int mode) {
+  const size_t d = arith_smem_bytes<ArithDF>(), f = arith_smem_bytes<ArithF64>();
+  return mode == 0 ? f : (mode == 1 ? d : std::max(d, f));
 }
 
 // ---------------------------------------------------------------------------------------
@@ -215,16 +256,20 @@ struct BatchPlan {
   std::vector<BatchItem> items;        // TSQR plan of every problem, TSQR problems first
   std::vector<int32_t> method;         // chosen method per problem, in the caller's order
   std::vector<GramGroupPlan> groups;   // Cholesky-QR2 problems by (column class, storage)
+  bool exact = false;                  // the exact launch takes every problem (its items below)
+  std::vector<XgItem> xg;
+  int64_t xg_total = 0;
+  int xg_max_nc = 4;
   size_t off_items = 0, off_flags = 0, off_counters = 0, off_gflags = 0, off_slots = 0, off_gram = 0,
-         off_groups = 0, bytes = 0;
+         off_acc = 0, off_groups = 0, off_xg = 0, bytes = 0;
   int64_t total_work = 0, total_work_df = 0;
-  size_t gram_flag_blocks = 0;  // Gram problems (512-byte flag block each, zeroed per launch)
 };
 
 // Tiles per chunk: aim for chunks of about kTargetRows rows (fewer, longer chunks for
 // wide problems keep their FP64 tree merges cheap), overridable by the tuner.
 static int64_t g_target_rows = 1 << 15;
 
+static int xg_class_of(int ncols) { return ncols <= 4 ? 4 : ncols <= 8 ? 8 : ncols <= 16 ? 16 : ncols <= 32 ? 32 : 64; }
 static int gram_class_of(int ncols) { return ncols <= 8 ? 0 : ncols <= 16 ? 16 : ncols <= 32 ? 32 : 64; }
 
 // The method of one problem (see the file comment).
@@ -312,17 +357,33 @@ static bool make_plan(int32_t count, const ql_problem* probs, BatchPlan& P, unsi
   // Gram problems: flag blocks (cleared with the counters), then carried blocks, partials
   // and FP64 accumulator blocks, then the group item arrays
   P.off_gflags = off;
+  P.exact = current_arith() != QL_ARITH_F64 && tc_gram_enabled() && pipe_gram_enabled();
+  auto explicit_gram = [&](int k) {
+    return P.items[k].method == QL_CHOLQR2 && probs[order[k]].method_hint == QL_CHOLQR2;
+  };
   std::vector<int> gram_probs;
   for (int k = 0; k < count; ++k)
-    if (P.items[k].method == QL_CHOLQR2) gram_probs.push_back(k);
-  P.gram_flag_blocks = gram_probs.size();
-  off += gram_probs.size() * 512;
+    if (P.items[k].method == QL_CHOLQR2 && (!P.exact || explicit_gram(k))) gram_probs.push_back(k);
+  // flag block of each problem that has one: 512 bytes, then the exact pass's accumulators
+  std::vector<size_t> flag_off(count, 0);
+  if (P.exact) {
+    for (int k = 0; k < count; ++k) {
+      flag_off[k] = off;
+      off += 512 + (sacc_bytes(xg_class_of(P.items[k].n)) + 255) / 256 * 256;
+    }
+  } else {
+    for (int k : gram_probs) {
+      flag_off[k] = off;
+      off += 512;
+    }
+  }
   P.off_slots = off;
   off += ((size_t)slots * sizeof(double) + 255) / 256 * 256;
   P.off_gram = off;
+  auto at = [&](size_t o) { return ws ? ws + o : nullptr; };
+  std::vector<size_t> keep_at(count, 0);  // the carried blocks of a Cholesky-QR2 problem
   int gidx[3][2];
   for (auto& r : gidx) r[0] = r[1] = -1;
-  int fb = 0;
   for (int k : gram_probs) {
     const BatchItem& it = P.items[k];
     const int nc = gram_class_of(it.n), ci = nc == 16 ? 0 : (nc == 32 ? 1 : 2), di = it.dtype == QL_F64 ? 0 : 1;
@@ -342,11 +403,9 @@ static bool make_plan(int32_t count, const ql_problem* probs, BatchPlan& P, unsi
     const size_t keep_b = ((size_t)3 * nc * nc * sizeof(double) + 255) / 256 * 256;
     const size_t part_b = (size_t)nch * nc * nc * sizeof(double);
     const size_t fbuf_b = (size_t)nch * nc * 128 * 2 * sizeof(double);  // accumulator levels of the tcgen05 kernels
-    const size_t flags_off = P.off_gflags + (size_t)fb * 512, keep_off = off, part_off = off + keep_b,
-                 fbuf_off = off + keep_b + part_b;
+    const size_t keep_off = off, part_off = off + keep_b, fbuf_off = off + keep_b + part_b;
     off += keep_b + part_b + fbuf_b;
-    ++fb;
-    auto at = [&](size_t o) { return ws ? ws + o : nullptr; };
+    keep_at[k] = keep_off;
     a.src.A = static_cast<const double*>(it.A);
     a.src.lda = it.lda;
     a.src.b = static_cast<const double*>(it.b);
@@ -358,7 +417,7 @@ static bool make_plan(int32_t count, const ql_problem* probs, BatchPlan& P, unsi
     a.method = QL_CHOLQR2;
     a.gated = 0;
     a.epilogue = it.kind == 1 ? kEpiLstsq : kEpiR;
-    a.w.flags = reinterpret_cast<int*>(at(flags_off));
+    a.w.flags = reinterpret_cast<int*>(at(flag_off[k]));
     a.w.keep = reinterpret_cast<double*>(at(keep_off));
     a.w.partials = reinterpret_cast<double*>(at(part_off));
     a.w.fbuf = reinterpret_cast<double*>(at(fbuf_off));
@@ -390,25 +449,87 @@ static bool make_plan(int32_t count, const ql_problem* probs, BatchPlan& P, unsi
     G.total += nch;
     G.items.push_back(gi);
   }
+  if (P.exact) {
+    // Work items of the exact launch: a tile of the 64-column class takes 4.3 us, of the others
+    // 1.8 us (measured at m = 2^22..2^23), and a chunk 4 to 15 us beside its tiles (set-up,
+    // emptying its sums), so chunks of about a quarter of a CTA's share, but of 16 tiles at least.
+    auto tiles_of = [&](int k) {
+      const int64_t kt = 4096 / xg_class_of(P.items[k].n);
+      return (P.items[k].m + kt - 1) / kt;
+    };
+    auto tile_cost = [&](int k) { return xg_class_of(P.items[k].n) == 64 ? 5 : 2; };
+    int64_t cost = 0;
+    std::vector<int> by_cost(count);
+    for (int k = 0; k < count; ++k) {
+      by_cost[k] = k;
+      cost += tiles_of(k) * tile_cost(k);
+    }
+    std::stable_sort(by_cost.begin(), by_cost.end(),
+                     [&](int x, int y) { return tiles_of(x) * tile_cost(x) > tiles_of(y) * tile_cost(y); });
+    const int64_t share = std::max<int64_t>(32, cost / (4 * ctas));
+    for (int k : by_cost) {
+      const BatchItem& it = P.items[k];
+      XgItem x{};
+      x.nc = xg_class_of(it.n);
+      x.dtype = it.dtype;
+      P.xg_max_nc = std::max(P.xg_max_nc, x.nc);
+      const int64_t tiles = tiles_of(k), tpc = std::max<int64_t>(1, share / tile_cost(k));
+      x.nchunks = (int)std::max<int64_t>(1, std::min<int64_t>(4096, (tiles + tpc - 1) / tpc));
+      GramArgs<double>& a = x.args;
+      a.src.A = static_cast<const double*>(it.A);
+      a.src.lda = it.lda;
+      a.src.b = static_cast<const double*>(it.b);
+      a.src.nA = it.nA;
+      a.m = it.m;
+      a.n = it.n;
+      a.tiles = tiles;
+      a.pass = 1;
+      a.method = explicit_gram(k) ? QL_CHOLQR2 : QL_TSQR;
+      a.epilogue = it.kind == 1 ? kEpiLstsq : kEpiR;
+      a.w.flags = reinterpret_cast<int*>(at(flag_off[k]));
+      a.w.sacc = reinterpret_cast<long long*>(at(flag_off[k] + 512));
+      a.w.keep = reinterpret_cast<double*>(at(keep_at[k]));
+      if (it.kind == 1) {  // R_ext into R (ld n + 1), x and the residual norm into x
+        a.x = it.x;
+        a.resnorm = it.x + (it.n - 1);
+        a.Rext = it.R;
+      } else {
+        a.R = it.R;
+        a.ldr = it.n;
+      }
+      a.info = it.info;
+      a.mround = 2;
+      a.redo = reinterpret_cast<int*>(at(P.off_flags)) + 1 + k;
+      a.redo_any = reinterpret_cast<int*>(at(P.off_flags));
+      a.bulk = xg_tensor_map(&x.map, x.nc, it.A, it.kind == 1 ? it.b : nullptr, it.dtype, it.m, it.nA, it.lda) ? 1 : 0;
+      x.work_begin = P.xg_total;
+      P.xg_total += x.nchunks;
+      P.xg.push_back(x);
+    }
+    P.off_acc = off = (off + 255) / 256 * 256;
+    off += (size_t)std::min<int64_t>(P.xg_total, ctas) * xg_acc_bytes(P.xg_max_nc);
+  }
   P.off_groups = off = (off + 255) / 256 * 256;
   for (auto& G : P.groups) {
     G.off_items = off;
     off += (G.items.size() * sizeof(GramGroupItem) + 255) / 256 * 256;
   }
+  P.off_xg = off;
+  off += (P.xg.size() * sizeof(XgItem) + 255) / 256 * 256;
   P.bytes = off;
   return true;
 }
 
-template <typename Ar>
-static ql_status launch_batch(unsigned char* ws, const BatchPlan& P, int count, cudaStream_t stream, int gated) {
+template <int MODE>
+static ql_status launch_batch(unsigned char* ws, const BatchPlan& P, int count, cudaStream_t stream) {
   static int occ = 0;
   static size_t smem = 0;
   static std::mutex mu;
-  auto kern = batch_kernel<Ar>;
+  auto kern = batch_kernel<MODE>;
   {
     std::lock_guard<std::mutex> lk(mu);
     if (occ == 0) {
-      smem = batch_smem_bytes<Ar>();
+      smem = batch_smem_bytes(MODE);
       if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return QL_ERR_CUDA;
       int o = 0;
@@ -423,7 +544,7 @@ static ql_status launch_batch(unsigned char* ws, const BatchPlan& P, int count, 
                                          reinterpret_cast<const BatchItem*>(ws + P.off_items), count,
                                          reinterpret_cast<double*>(ws + P.off_slots),
                                          reinterpret_cast<int*>(ws + P.off_counters),
-                                         reinterpret_cast<int*>(ws + P.off_flags) + 1, gated);
+                                         reinterpret_cast<int*>(ws + P.off_flags) + 1);
   return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
@@ -456,7 +577,7 @@ void set_batch_target_rows(int64_t rows) { g_target_rows = rows < 256 ? 256 : ro
 int64_t batch_target_rows() { return g_target_rows; }
 
 // The host image of what the device needs of a plan: [header, TSQR items] (uploaded to
-// offset 0) followed by the Gram group item arrays (uploaded to off_groups).
+// offset 0) followed by the Gram group and exact item arrays (uploaded to off_groups).
 static size_t upload_bytes(const BatchPlan& P) { return P.off_flags + (P.bytes - P.off_groups); }
 static void fill_upload(const BatchPlan& P, int32_t count, unsigned char* dst) {
   BatchHeader h{};
@@ -468,6 +589,8 @@ static void fill_upload(const BatchPlan& P, int32_t count, unsigned char* dst) {
   std::memcpy(dst + P.off_items, P.items.data(), P.items.size() * sizeof(BatchItem));
   for (const auto& G : P.groups)
     std::memcpy(dst + P.off_flags + (G.off_items - P.off_groups), G.items.data(), G.items.size() * sizeof(GramGroupItem));
+  if (!P.xg.empty())
+    std::memcpy(dst + P.off_flags + (P.off_xg - P.off_groups), P.xg.data(), P.xg.size() * sizeof(XgItem));
 }
 
 // Asynchronous plan upload through a caller-owned pinned staging buffer (the serving
@@ -534,14 +657,14 @@ ql_status ql_batch_launch(void* ws, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   unsigned char* w = static_cast<unsigned char*>(ws);
   const int count = (int)P.items.size();
-  // work counters, tree counters and every flag (TSQR and Gram) start at zero on every launch
+  // work counters, tree counters, flags and the exact pass's accumulators start at zero on every launch
   if (cudaMemsetAsync(w, 0, offsetof(BatchHeader, count), st) != cudaSuccess) return QL_ERR_CUDA;
   if (cudaMemsetAsync(w + offsetof(BatchHeader, gram_counter), 0, sizeof(int) * 2 * kMaxGramGroups, st) !=
       cudaSuccess)
     return QL_ERR_CUDA;
   if (cudaMemsetAsync(w + P.off_flags, 0, P.off_slots - P.off_flags, st) != cudaSuccess) return QL_ERR_CUDA;
   BatchHeader* hdr = reinterpret_cast<BatchHeader*>(w);
-  const bool f64 = current_arith() == QL_ARITH_F64;  // then every problem runs TSQR (the plan chose so)
+  if (current_arith() == QL_ARITH_F64) return launch_batch<0>(w, P, count, st);  // Householder tiles for every problem
   ql_status s = QL_OK;
   auto gram_pass = [&](int pass) {
     for (size_t g = 0; g < P.groups.size() && s == QL_OK; ++g) {
@@ -550,11 +673,16 @@ ql_status ql_batch_launch(void* ws, void* stream) {
                             reinterpret_cast<const GramGroupItem*>(w + G.off_items), (int)G.items.size(), G.total, st);
     }
   };
-  gram_pass(1);
-  if (s == QL_OK) s = f64 ? launch_batch<ArithF64>(w, P, count, st, 0) : launch_batch<ArithDF>(w, P, count, st, 0);
+  if (P.exact) {
+    const int grid = (int)std::min<int64_t>(P.xg_total, device_sm_count());
+    s = xgram_group_launch(&hdr->work_counter[2], reinterpret_cast<const XgItem*>(w + P.off_xg), count, P.xg_total, grid,
+                           reinterpret_cast<double*>(w + P.off_acc), P.xg_max_nc, st);
+  } else {  // the comparison kernels: per-tile first Gram passes, Householder tiles
+    gram_pass(1);
+    if (s == QL_OK) s = launch_batch<1>(w, P, count, st);
+  }
   if (s == QL_OK) gram_pass(2);
-  if (s != QL_OK || f64) return s;
-  return launch_batch<ArithF64>(w, P, count, st, 1);  // flagged problems, any method
+  return s == QL_OK ? launch_batch<2>(w, P, count, st) : s;  // flagged problems, any method
 }
 
 ql_status ql_batch_methods(void* ws, int32_t* methods, int32_t count) {

@@ -69,10 +69,12 @@ struct GramArgs {
   int redo_on_breakdown;
 };
 
-// Ask the batched FP64 TSQR launch to redo this problem.  Bits 8.. of the flag carry where a
-// bounded wait gave up (0: none), which that launch reports as {QL_ERR_TIMEOUT, where}.
-QL_DEV void gram_request_redo(int* redo, int* redo_any, int timeout_where = 0) {
-  atomicOr(redo, 1 | (timeout_where << 8));
+// Ask the batch's last launch to redo this problem with Householder tiles, in FP64 or in
+// double-float.  Bits 8.. of the flag carry where a bounded wait gave up (0: none), which that
+// launch reports as {QL_ERR_TIMEOUT, where}.
+constexpr int kRedoF64 = 1, kRedoDF = 2, kRedoDFRange = 4;  // the last: the double-float redo left its range
+QL_DEV void gram_request_redo(int* redo, int* redo_any, int timeout_where = 0, int kind = kRedoF64) {
+  atomicOr(redo, kind | (timeout_where << 8));
   atomicOr(redo_any, 1);
 }
 

@@ -705,7 +705,10 @@ QL_DEV void xg_finish(const GramArgs<S>& a, unsigned char* smem, const int* colm
   const int tid = threadIdx.x, n = a.n;
   constexpr int LE = NC + 1;
   const bool tsqr = a.method == QL_TSQR;
-  if (tsqr && *(volatile int*)&a.w.flags[1] != 0) return;  // a bounded wait gave up: Householder redoes the call
+  if (tsqr && *(volatile int*)&a.w.flags[1] != 0) {  // a bounded wait gave up: Householder redoes the call
+    if (a.redo && tid == 0) gram_request_redo(a.redo, a.redo_any, *(volatile int*)&a.w.flags[4], kRedoDF);
+    return;
+  }
   double* Rs = reinterpret_cast<double*>(smem);
   double* vec = Rs + NC * LE;
   int* sflag = reinterpret_cast<int*>(vec + 2 * LE);
@@ -730,7 +733,7 @@ QL_DEV void xg_finish(const GramArgs<S>& a, unsigned char* smem, const int* colm
   if (tsqr) {
     if (tid == 0) {
       a.w.flags[1] = 1;
-      if (a.redo) gram_request_redo(a.redo, a.redo_any);
+      if (a.redo) gram_request_redo(a.redo, a.redo_any, 0, kRedoDF);
     }
     return;
   }

@@ -134,3 +134,44 @@ def test_gram_methods_still_report_breakdowns():
     Xd = torch.from_numpy(np.ascontiguousarray(X.T)).cuda().T
     assert q.cholqr2_qless(Xd)[1].cpu().tolist() == [q.QL_ERR_NOT_SPD, 7]
     assert q.scholqr3_qless(Xd)[1].cpu().tolist() == [q.QL_ERR_NOT_SPD, 1007]
+
+
+@pytest.mark.parametrize("hint", ["tsqr", "auto", "cholqr2"])
+def test_batch_of_every_class_and_every_way_out(hint):
+    """One batch: every column class and both storages on the exact launch, and problems that
+    its last launch redoes (dependent columns, data out of the double-float range)."""
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    mats, keep, probs = [], [], []
+    for k, n in enumerate([1, 2, 3, 4, 6, 8, 13, 16, 20, 32, 40, 64, 9, 30]):
+        m = [3001, 40000, 2048][k % 3]
+        X = synth.conditioned(m, n, 10.0 ** (k % 4), seed=k, dtype=np.float32 if k % 3 == 2 else np.float64)
+        if n == 13 and hint != "cholqr2":
+            X[:, 7] = X[:, 2]                      # pivot zero
+        if n == 20:
+            X = X * 2.0 ** 70                      # beyond the range check
+        if n == 9:
+            X[:, 4] *= 0.0 if hint != "cholqr2" else 1.0
+        if n == 30:
+            X = synth.conditioned(m, n, 1e8, seed=k)   # beyond Cholesky-QR2's pivot limit
+        mats.append(X)
+        d = torch.from_numpy(np.ascontiguousarray(X.T)).cuda()
+        R = torch.zeros((n, n), dtype=torch.float64, device="cuda")
+        info = torch.full((2,), -1, dtype=torch.int32, device="cuda")
+        keep.append((d, R, info))
+        probs.append(q.Problem(m=m, n=n, ld=m, X=d.data_ptr(), dtype=q.QL_F64 if X.dtype == np.float64 else q.QL_F32,
+                               kind=0, b=None, R=R.data_ptr(), x=None, info=info.data_ptr(),
+                               method_hint={"tsqr": q.QL_TSQR, "auto": q.QL_AUTO, "cholqr2": q.QL_CHOLQR2}[hint],
+                               kappa_hint=1e4))
+    q.batch_qless(probs)
+    torch.cuda.synchronize()
+    for X, (_, R, info) in zip(mats, keep):
+        n = X.shape[1]
+        R = R.cpu().numpy().T
+        assert info.cpu().tolist() == [0, 0], n
+        assert np.all(np.diag(R) >= 0.0) and gram_error(R, X) <= 1e-13 * n, n
+        if n not in (9, 13):
+            kappa = 1e8 if n == 30 else 1e3
+            assert oracle.rel_err(R, oracle.householder_r(X.astype(np.float64))) <= oracle.tolerance(n, kappa), n
