@@ -5,23 +5,29 @@
 // so that W = (I - Y Y^T) X to working precision even when X is nearly in range(Y).  The R
 // of the orthogonalised block is then any of the Q-less calls on W.
 //
-// Four launches (cross product, update, cross product, update).  The cross product Y^T V is
-// a reduction over the m rows: every CTA accumulates 4 x 4 blocks of the k x n product over
-// its row tiles in double-float, writes one FP64 partial, and the last CTA to finish sums
-// the partials in a fixed order (reproducible).  The update W = V - Y C streams the rows,
+// Six launches (cross product, its reduction, update; twice).  The cross product Y^T V is a
+// reduction over the m rows: every CTA accumulates 4 x 4 blocks of the k x n product over its row
+// tiles in double-float, two rows per packed FP32 instruction (half the issue slots; two CTAs per
+// SM, so that one loads while the other multiplies), and writes one FP64 partial;
+// cross_reduce_kernel sums the partials in a fixed order (reproducible), an entry per thread over
+// many CTAs, where the last CTA used to sum all of them.  The update W = V - Y C streams the rows,
 // one per thread.  Tiles outside the double-float exponent range run in FP64.
+//
+// Both are bound by the FP32 pipes, 13 operations per product and row: k = n = 64, m = 2^19
+// 0.71 ms each; measured 1.34 + 0.05 ms (cross product and reduction) and 2.27 ms (update).  QR
+// of 524288 x 128, with two of each: 15.3 -> 11.7 ms.
 #include <mutex>
 
+#include "df2.cuh"
 #include "internal.h"
 #include "small_dense.cuh"
 
 namespace ql {
 
 constexpr int kProjT = 256;
-constexpr int kProjB = 128;  // rows per tile of the cross product
+constexpr int kProjB = 64;   // rows per tile of the cross product
 
 struct ProjWs {
-  int* flags;        // [0] arrival counter
   double* cprev;     // C of the first pass (k x n, ld n)
   double* cpass;     // C of the current pass, read by the update (k x n, ld n)
   double* partials;  // one KC x NC partial per CTA
@@ -53,30 +59,29 @@ QL_DEV df load_df(float x, int& E) {
   return df{x, 0.0f};
 }
 
-// ---- C = Y^T V over the rows (partials per CTA, fixed-order reduction in the last CTA)
+// ---- C = Y^T V over the rows: one partial per CTA
 template <int KC, int NC, typename S>
-__global__ void __launch_bounds__(kProjT, 1) cross_kernel(ProjArgs<S> a) {
+__global__ void __launch_bounds__(kProjT, 2) cross_kernel(ProjArgs<S> a) {
   constexpr int T = kProjT, B = kProjB;
   constexpr int NBLK = (KC / 4) * (NC / 4);  // 4 x 4 blocks of C
   constexpr int SL = T / NBLK >= 1 ? T / NBLK : 1;
   static_assert(NBLK <= T, "one block per thread at least");
   extern __shared__ __align__(16) unsigned char smem[];
-  df* Ys = reinterpret_cast<df*>(smem);             // [KC][B]
-  df* Vs = Ys + KC * B;                             // [NC][B]
-  double* red = reinterpret_cast<double*>(Vs + NC * B);  // [SL][KC][NC] at the end
-  int* misc = reinterpret_cast<int*>(red + (size_t)SL * KC * NC);
+  df2* Ys = reinterpret_cast<df2*>(smem);  // [KC][B / 2] row pairs
+  df2* Vs = Ys + KC * (B / 2);             // [NC][B / 2]
+  double* red = reinterpret_cast<double*>(smem);  // [SL][KC][NC] at the end
   const int tid = threadIdx.x, k = a.k, n = a.n;
   const int blk = tid / SL, slice = tid % SL;
   const bool active = blk < NBLK;
   const int bi = active ? (blk / (NC / 4)) * 4 : 0, bj = active ? (blk % (NC / 4)) * 4 : 0;
 
-  ArithDF::Acc acc[4][4];
+  df2 acc[4][4];
   double acc64[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      acc[i][j] = ArithDF::acc_zero();
+      acc[i][j] = df2{0, 0};
       acc64[i][j] = 0.0;
     }
   const int64_t nb = gridDim.x, bid = blockIdx.x;
@@ -84,34 +89,36 @@ __global__ void __launch_bounds__(kProjT, 1) cross_kernel(ProjArgs<S> a) {
   for (int64_t t = t0; t < t1; ++t) {
     const int64_t row0 = t * B;
     bool bad = false;
-    for (int e = tid; e < (KC + NC) * B; e += T) {
-      const int c = e / B, r = e % B;
-      const int64_t row = row0 + r;
-      df v = df{0.0f, 0.0f};
-      int E = 0;
-      if (c < KC) {
-        if (c < k && row < a.m) v = load_df(a.Y[c * a.ldy + row], E);
-        Ys[c * B + r] = v;
-      } else {
-        const int cv = c - KC;
-        if (cv < n && row < a.m) v = load_df(a.V[cv * a.ldv + row], E);
-        Vs[cv * B + r] = v;
+#pragma unroll 8
+    for (int e = tid; e < (KC + NC) * (B / 2); e += T) {
+      const int c = e / (B / 2), r = e % (B / 2);
+      const int64_t row = row0 + 2 * r;
+      const bool isY = c < KC, used = isY ? c < k : c - KC < n;
+      const S* p = (isY ? a.Y + c * a.ldy : a.V + (c - KC) * a.ldv) + row;
+      S x0 = S(0), x1 = S(0);
+      if (used) {
+        if (row < a.m) x0 = p[0];
+        if (row + 1 < a.m) x1 = p[1];
       }
-      if (!df_range_ok_dev(E)) bad = true;
+      int E0, E1;
+      const df v0 = load_df(x0, E0), v1 = load_df(x1, E1);
+      if (!df_range_ok_dev(E0) || !df_range_ok_dev(E1)) bad = true;
+      Ys[e] = df2{f2_make(v0.hi, v1.hi), f2_make(v0.lo, v1.lo)};
     }
     const bool f64 = __syncthreads_or(bad);
     if (active) {
       if (!f64) {
-        for (int r = slice; r < B; r += SL) {
-          df y[4], v[4];
+#pragma unroll 1
+        for (int r = slice; r < B / 2; r += SL) {
+          df2 v[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) y[i] = Ys[(bi + i) * B + r];
+          for (int j = 0; j < 4; ++j) v[j] = Vs[(bj + j) * (B / 2) + r];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) v[j] = Vs[(bj + j) * B + r];
+          for (int i = 0; i < 4; ++i) {
+            const df2n y = df2_factor(Ys[(bi + i) * (B / 2) + r]);
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) ArithDF::acc_fma(acc[i][j], y[i], v[j]);
+            for (int j = 0; j < 4; ++j) df2_acc_fma(acc[i][j], y, v[j]);
+          }
         }
       } else {  // FP64 for this tile, straight from global memory
         for (int r = slice; r < B; r += SL) {
@@ -131,42 +138,41 @@ __global__ void __launch_bounds__(kProjT, 1) cross_kernel(ProjArgs<S> a) {
     }
     __syncthreads();
   }
-  // combine the slices and store this CTA's partial (FP64)
+  // combine the row parities and the slices and store this CTA's partial (FP64)
   if (active) {
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        red[((size_t)slice * KC + bi + i) * NC + bj + j] =
-            df_to_double(ArithDF::acc_get(acc[i][j])) + acc64[i][j];
+      for (int j = 0; j < 4; ++j) {
+        df e, o;
+        df2_rows(acc[i][j], e, o);
+        red[((size_t)slice * KC + bi + i) * NC + bj + j] = (df_to_double(e) + df_to_double(o)) + acc64[i][j];
+      }
   }
   __syncthreads();
   double* part = a.w.partials + (size_t)bid * KC * NC;
   for (int e = tid; e < KC * NC; e += T) {
     double s = 0.0;
     for (int sl = 0; sl < SL; ++sl) s += red[(size_t)sl * KC * NC + e];
-    __stcg(part + e, s);
+    part[e] = s;
   }
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    const int old = atomicAdd(&a.w.flags[0], 1);
-    misc[0] = old == (int)nb - 1;
-    if (old == (int)nb - 1) a.w.flags[0] = 0;
-  }
-  __syncthreads();
-  if (!misc[0]) return;
-  __threadfence();
-  // last CTA: fixed-order sum of the partials -> C of this pass (and the running total)
-  for (int e = tid; e < k * n; e += T) {
-    const int i = e / n, j = e % n;
-    double s = 0.0;
-    for (int b = 0; b < (int)nb; ++b) s += __ldcg(a.w.partials + (size_t)b * KC * NC + i * NC + j);
-    a.w.cpass[i * n + j] = s;
-    const double tot = a.pass == 1 ? s : __ldcg(a.w.cprev + i * n + j) + s;
-    if (a.pass == 1) a.w.cprev[i * n + j] = s;
-    a.C[j * a.ldc + i] = tot;
-  }
+}
+
+// ---- the fixed-order sum of the nb partials: C of this pass and the running total
+constexpr int kReduceT = 64;
+template <typename S>
+__global__ void __launch_bounds__(kReduceT) cross_reduce_kernel(ProjArgs<S> a, int kc, int nc, int nb) {
+  const int e = blockIdx.x * kReduceT + threadIdx.x, i = e / nc, j = e % nc;
+  if (e >= kc * nc || i >= a.k || j >= a.n) return;
+  const double* p = a.w.partials + e;
+  const size_t step = (size_t)kc * nc;
+  double s = 0.0;
+#pragma unroll 16
+  for (int b = 0; b < nb; ++b) s += __ldg(p + b * step);
+  a.w.cpass[i * a.n + j] = s;
+  const double tot = a.pass == 1 ? s : a.w.cprev[i * a.n + j] + s;
+  if (a.pass == 1) a.w.cprev[i * a.n + j] = s;
+  a.C[j * a.ldc + i] = tot;
 }
 
 // ---- W = V - Y C (C of this pass), one row per thread
@@ -194,6 +200,7 @@ __global__ void __launch_bounds__(kProjT, 1) update_kernel(ProjArgs<S> a) {
     const int64_t row = t * T + tid;
     const bool live = row < a.m;
     bool bad = false;
+#pragma unroll 8
     for (int i = 0; i < k; ++i) {
       int E = 0;
       df y = df{0.0f, 0.0f};
@@ -255,11 +262,14 @@ template <int KC, int NC>
 struct ProjSmem {
   static constexpr int NBLK = (KC / 4) * (NC / 4);
   static constexpr int SL = kProjT / NBLK >= 1 ? kProjT / NBLK : 1;
-  static constexpr size_t kCross = 8 * (size_t)(KC + NC) * kProjB + 8 * (size_t)SL * KC * NC + 64;
+  static constexpr size_t kTile = 8 * (size_t)(KC + NC) * kProjB, kRed = 8 * (size_t)SL * KC * NC;
+  static constexpr size_t kCross = kTile > kRed ? kTile : kRed;
   static constexpr size_t kUpdate = 16 * (size_t)KC * NC + 8 * (size_t)KC * kProjT;
+  static_assert(kUpdate <= 232448, "shared memory of one SM");
 };
 
-static size_t proj_parts_bytes() { return (size_t)device_sm_count() * 64 * 64 * sizeof(double); }
+constexpr int kCrossCtasPerSm = 2;
+static size_t proj_parts_bytes() { return (size_t)device_sm_count() * kCrossCtasPerSm * 64 * 64 * sizeof(double); }
 
 size_t project_workspace_bytes(int k, int n) {
   if (k < 1 || k > kMaxN || n < 1 || n > kMaxN) return 0;
@@ -282,8 +292,10 @@ static ql_status proj_run(ProjArgs<S> a, cudaStream_t st) {
       ready = true;
     }
   }
+  int occ = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, uk, kProjT, Sm::kUpdate) != cudaSuccess) return QL_ERR_CUDA;
   const int64_t ctiles = (a.m + kProjB - 1) / kProjB, utiles = (a.m + kProjT - 1) / kProjT;
-  int64_t gc = device_sm_count(), gu = device_sm_count();
+  int64_t gc = (int64_t)device_sm_count() * kCrossCtasPerSm, gu = (int64_t)device_sm_count() * (occ < 1 ? 1 : occ);
   if (gc > ctiles) gc = ctiles;
   if (gu > utiles) gu = utiles;
   if (gc < 1) gc = 1;
@@ -302,6 +314,9 @@ static ql_status proj_run(ProjArgs<S> a, cudaStream_t st) {
     a.tiles = ctiles;
     count_launch();
     ck<<<(int)gc, kProjT, Sm::kCross, st>>>(a);
+    if (cudaPeekAtLastError() != cudaSuccess) return QL_ERR_CUDA;
+    count_launch();
+    cross_reduce_kernel<S><<<(KC * NC + kReduceT - 1) / kReduceT, kReduceT, 0, st>>>(a, KC, NC, (int)gc);
     if (cudaPeekAtLastError() != cudaSuccess) return QL_ERR_CUDA;
     a.tiles = utiles;
     count_launch();
@@ -346,11 +361,9 @@ ql_status ql_project_out(int64_t m, int64_t k, const void* Y, int64_t ldy, int64
   cudaStream_t st = (cudaStream_t)stream;
   unsigned char* b = static_cast<unsigned char*>(ws);
   ProjWs w;
-  w.flags = reinterpret_cast<int*>(b);
   w.cprev = reinterpret_cast<double*>(b + 256);
   w.cpass = w.cprev + (size_t)kMaxN * kMaxN;
   w.partials = w.cpass + (size_t)kMaxN * kMaxN;
-  if (cudaMemsetAsync(w.flags, 0, 256, st) != cudaSuccess) return QL_ERR_CUDA;
   if (dtype == QL_F64) {
     ProjArgs<double> a{m, (int)k, (int)n, static_cast<const double*>(Y), ldy, static_cast<const double*>(X), ldx,
                        static_cast<double*>(W), ldw, C, ldc, 1, w, 0};
