@@ -132,8 +132,8 @@ ql_status gram_launch(const GramCall& c, ql_arith arith) {
   if (!c.ws || c.ws_bytes < gram_layout(c.n, nullptr, nullptr)) return QL_ERR_WORKSPACE;
   GramWs w;
   gram_layout(c.n, &w, c.ws);
-  if (cudaMemsetAsync(w.flags, 0, gram_head_bytes(c.n), c.stream) != cudaSuccess) return QL_ERR_CUDA;
   ql_status st;
+  if ((st = clear_async(w.flags, gram_head_bytes(c.n), c.stream))) return st;
   if (c.dtype == QL_F64) {
     if (arith == QL_ARITH_F64) return gram_dispatch<double, ArithF64>(c, w, 0);
     if ((st = gram_dispatch<double, ArithDF>(c, w, 0))) return st;

@@ -149,6 +149,8 @@ __global__ void __launch_bounds__(GramShape<NC>::T, 1) gram_kernel(GramArgs<S> a
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x, n = a.n;
 
+  pdl_release();
+  pdl_wait();
   if (a.gated && *(volatile int*)&a.w.flags[0] == 0) return;
   if (Ar::kRangeChecked && a.pass >= 2 && (*(volatile int*)&a.w.flags[0] != 0 || *(volatile int*)&a.w.flags[5] != 0))
     return;  // FP64 redoes it, or R is written
@@ -548,6 +550,8 @@ __global__ void __launch_bounds__(StreamShape<NC>::T) gram_stream_kernel(GramArg
   extern __shared__ __align__(16) unsigned char smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = a.n;
 
+  pdl_release();
+  pdl_wait();
   if (a.gated && *(volatile int*)&a.w.flags[0] == 0) return;
   if (Ar::kRangeChecked && a.pass >= 2 && (*(volatile int*)&a.w.flags[0] != 0 || *(volatile int*)&a.w.flags[5] != 0))
     return;  // FP64 redoes it, or R is written
@@ -725,8 +729,7 @@ ql_status gram_stream_launch_one(const GramCall& c, const GramWs& w, int pass, i
   }
   a.mround = std::is_same<Ar, ArithDF>::value ? 1 : 0;
   count_launch();
-  kern<<<(int)g, Sh::T, Sm::kBytes, c.stream>>>(a);
-  return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+  return launch_dependent(kern, (int)g, Sh::T, Sm::kBytes, c.stream, a) == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
 // Tensor-core Gram pass (double-float policy only): see gram_tc.cuh.  The body handles the
@@ -1103,6 +1106,8 @@ QL_DEV void gram_tc_body(const GramArgs<S>& a, int bid, int k) {
 
 template <int NC, typename S, int XF>
 __global__ void __launch_bounds__(256, 1) gram_tc_kernel(GramArgs<S> a) {
+  pdl_release();
+  pdl_wait();
   gram_tc_body<NC, S, XF>(a, blockIdx.x, gridDim.x);
 }
 
@@ -1151,8 +1156,7 @@ ql_status gram_tc_launch_one(const GramCall& c, const GramWs& w, int pass) {
   a.info = c.info;
   a.mround = 2;
   count_launch();
-  kern<<<(int)g, Sh::T, Sm::kBytes, c.stream>>>(a);
-  return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+  return launch_dependent(kern, (int)g, Sh::T, Sm::kBytes, c.stream, a) == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
 // Tensor-core Gram pass on tcgen05 (double-float policy only): see gram_umma.cuh.  The
@@ -1606,6 +1610,8 @@ __global__ void __launch_bounds__(umma_threads<XF>(), 1) gram_umma_kernel(GramAr
   extern __shared__ __align__(1024) unsigned char smem_umma[];
   unsigned char* smem = smem_umma;
   uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + Sm::kOffBar + 16);
+  pdl_release();
+  pdl_wait();
   const uint32_t tbase = umma_cta_begin<NC, S>(smem, tslot);
   UmmaBars bars;
   gram_umma_body<NC, S, XF>(a, blockIdx.x, gridDim.x, tbase, bars);
@@ -1663,8 +1669,7 @@ ql_status gram_umma_launch_one(const GramCall& c, const GramWs& w, int pass) {
   }
   a.mround = 2;
   count_launch();
-  kern<<<(int)g, umma_threads<XF>(), Sm::kBytes, c.stream>>>(a);
-  return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+  return launch_dependent(kern, (int)g, umma_threads<XF>(), Sm::kBytes, c.stream, a) == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -2282,6 +2287,8 @@ __global__ void __launch_bounds__(PipeShape<NC>::T, 1)
     gram_pipe_kernel(const __grid_constant__ GramArgs<S> a, const __grid_constant__ CUtensorMap tmA,
                      const __grid_constant__ CUtensorMap tmB, int has_b) {
   extern __shared__ __align__(1024) unsigned char smem_umma[];
+  pdl_release();
+  pdl_wait();
   const uint32_t tbase = pipe_cta_begin<NC, S>(smem_umma);
   PipeBars bars;
   gram_pipe_body<NC, S, XF>(a, blockIdx.x, gridDim.x, tbase, bars, &tmA, has_b ? &tmB : nullptr);
@@ -2340,8 +2347,8 @@ ql_status gram_pipe_launch_one(const GramCall& c, const GramWs& w, int pass = 1)
                : 0;
   a.mround = 2;
   count_launch();
-  kern<<<(int)g, Sh::T, Sm::kBytes, c.stream>>>(a, tmA, tmB, has_b ? 1 : 0);
-  return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+  return launch_dependent(kern, (int)g, Sh::T, Sm::kBytes, c.stream, a, tmA, tmB, has_b ? 1 : 0) == cudaSuccess ? QL_OK
+                                                                                                                : QL_ERR_CUDA;
 }
 
 template <int NC, typename S, typename Ar, int XF>
@@ -2389,8 +2396,7 @@ ql_status gram_launch_one(const GramCall& c, const GramWs& w, int pass, int gate
   a.info = c.info;
   a.mround = std::is_same<Ar, ArithDF>::value ? 1 : 0;
   count_launch();
-  kern<<<(int)g, Sh::T, Sm::kBytes, c.stream>>>(a);
-  return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+  return launch_dependent(kern, (int)g, Sh::T, Sm::kBytes, c.stream, a) == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
 // Exact Gram pass (xgram.cuh): R of a TSQR call (method QL_TSQR), or the first pass of a Gram

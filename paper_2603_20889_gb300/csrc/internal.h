@@ -115,6 +115,26 @@ bool xg_tensor_map(CUtensorMap* map, int nc, const void* A, const void* b, int d
 // Thread-layout variant of the TSQR kernels (environment QL_TSQR_CFG, 0 = default).
 int tsqr_variant();
 
+// Launch a kernel that may start while its predecessor in the stream still runs; it calls
+// pdl_wait (common.cuh) before it touches anything the predecessor writes.
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kern)(P...), int grid, int block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+// Zero `bytes` (a multiple of 16, at a 16-byte boundary) on the stream, by a kernel that lets
+// the next one start early.
+ql_status clear_async(void* p, size_t bytes, cudaStream_t st);
+
 // Counts every kernel this library launches (reported by ql_launch_count()).
 void count_launch();
 // dst = the first nonzero {status, index} pair among src[0 .. count) (one tiny launch).

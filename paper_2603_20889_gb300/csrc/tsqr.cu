@@ -33,6 +33,18 @@ int device_sm_count() {
   return v;
 }
 
+static __global__ void __launch_bounds__(256) clear_kernel(uint4* p, unsigned n) {
+  pdl_release();
+  const unsigned i = blockIdx.x * 256 + threadIdx.x;
+  if (i < n) p[i] = make_uint4(0, 0, 0, 0);
+}
+ql_status clear_async(void* p, size_t bytes, cudaStream_t st) {
+  const unsigned n = (unsigned)(bytes / 16);
+  count_launch();
+  clear_kernel<<<(n + 255) / 256, 256, 0, st>>>(static_cast<uint4*>(p), n);
+  return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+}
+
 // Workspace: the exact Gram pass's block (its head, the flags, is shared by every launch of
 // the call) unless the call is Householder only, then the tree's counters and slots.
 constexpr size_t kFlagBytes = 512;
@@ -79,11 +91,12 @@ ql_status tsqr_launch(const TsqrCall& c, ql_arith arith) {
   tv.flags = reinterpret_cast<int*>(ws + cb);
   tv.slots = reinterpret_cast<double*>(ws + cb + xb);
   tv.leaves = 0;
-  if (cudaMemsetAsync(ws, 0, cb + (exact ? xgram_tsqr_clear_bytes(c.n) : kFlagBytes), c.stream) != cudaSuccess)
-    return QL_ERR_CUDA;
   if (exact) {
-    ql_status st = xgram_tsqr_launch(c, ws + cb);
+    ql_status st = clear_async(ws, cb + xgram_tsqr_clear_bytes(c.n), c.stream);
+    if (st == QL_OK) st = xgram_tsqr_launch(c, ws + cb);
     if (st != QL_OK) return st;
+  } else if (cudaMemsetAsync(ws, 0, cb + kFlagBytes, c.stream) != cudaSuccess) {
+    return QL_ERR_CUDA;
   }
   return c.dtype == QL_F64 ? tsqr_launch_s<double>(c, tv, exact, arith) : tsqr_launch_s<float>(c, tv, exact, arith);
 }

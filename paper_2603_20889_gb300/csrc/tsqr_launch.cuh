@@ -34,6 +34,8 @@ template <int NC, int TC, int RPT, int T, typename S, typename Ar>
 __global__ void __launch_bounds__(T, 1) tsqr_kernel(TsqrArgs<S> a) {
   extern __shared__ __align__(16) unsigned char smem[];
   using Cta = TsqrCta<NC, TC, RPT, T, S, Ar>;
+  pdl_release();
+  pdl_wait();
   if (a.gated) {  // flags[0]: range, flags[1]: Householder redo (see TsqrArgs)
     if (*(volatile int*)&a.tv.flags[a.gated - 1] == 0) return;
   }
@@ -116,6 +118,7 @@ ql_status launch_one(const TsqrCall& c, const TreeView& tv_in, int gated) {
   a.Rext = c.Rext;
   a.info = c.info;
   count_launch();
+  if (gated) return launch_dependent(kern, (int)g, T, Sm::kBytes, c.stream, a) == cudaSuccess ? QL_OK : QL_ERR_CUDA;
   kern<<<(int)g, T, Sm::kBytes, c.stream>>>(a);
   return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }

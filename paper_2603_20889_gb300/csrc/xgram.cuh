@@ -929,6 +929,7 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
     // 128-bit sums -> the integer accumulators of C at the current column scales.  Lane groups
     // 1.. hand their sums to group 0 through `scratch` (a free digit buffer).
     auto emit = [&](unsigned char* scratch) {
+      pdl_wait();  // the accumulators have been cleared
       ulonglong2* sc = reinterpret_cast<ulonglong2*>(scratch);
       if (lg + seg > 0) {
         constexpr int JB = HALF < 8 ? HALF : 8;
@@ -1135,6 +1136,7 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
   tc_fence_before();
   __syncthreads();
   const int fw = *fail;
+  pdl_wait();  // before the first use of the flags
   if (fw) {
     bars.ok = false;  // a late arrival may still complete a phase: the CTA takes no more work
     if (tid == 0) {   // the gated launches redo the call and report {QL_ERR_TIMEOUT, where}
@@ -1168,6 +1170,9 @@ template <int NC, typename S>
 __global__ void __launch_bounds__(XgShape<NC>::T, 1)
     xgram_kernel(const __grid_constant__ GramArgs<S> a, const __grid_constant__ CUtensorMap map) {
   extern __shared__ __align__(1024) unsigned char smem_umma[];
+  // The workspace is cleared by the kernel before this one, which this one may overlap (X itself
+  // was complete before that kernel started): nothing in it is read or added to before pdl_wait.
+  pdl_release();
   const uint32_t tbase = xg_cta_begin<NC, S>(smem_umma);
   PipeBars bars;
   xgram_body<NC, S>(a, blockIdx.x, gridDim.x, tbase, bars, &map, blockIdx.x);
@@ -1222,8 +1227,7 @@ ql_status xgram_launch_one(const GramCall& c, const GramWs& w) {
                : 0;
   a.mround = NC >= 16 ? 2 : 1;  // how the next pass's kernel of this class reads M
   count_launch();
-  kern<<<(int)g, Sh::T, Sm::kBytes, c.stream>>>(a, map);
-  return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+  return launch_dependent(kern, (int)g, Sh::T, Sm::kBytes, c.stream, a, map) == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
 template <typename S>
