@@ -1,6 +1,6 @@
 // Two double-floats at a time on the packed FP32 instructions (add / mul / fma .rn.f32x2): the
-// values of two rows side by side.  Every operation rounds like its scalar form in common.cuh,
-// so results are the same bits; one instruction slot serves both rows (the FP32 pipes give the
+// two values (rows or columns) side by side.  Every operation rounds like its scalar form in common.cuh,
+// so results are the same bits; one instruction slot serves both (the FP32 pipes give the
 // packed form no more flops, but half the issue slots, and kernels with few warps are bound by
 // issue and latency).
 #pragma once
@@ -9,7 +9,7 @@
 
 namespace ql {
 
-using f2 = unsigned long long;  // two floats: row 0 in the low word
+using f2 = unsigned long long;  // two floats, the first in the low word
 struct df2 {
   f2 hi, lo;
 };
@@ -46,7 +46,7 @@ struct df2n {
 };
 QL_DEV df2n df2_factor(df2 a) { return df2n{a.hi, a.lo, f2_neg(a.hi), f2_neg(a.lo)}; }
 
-// acc += a b (as ArithDF::acc_fma in each row).
+// acc += a b (as ArithDF::acc_fma in each half).
 QL_DEV void df2_acc_fma(df2& acc, const df2n& a, const df2& b) {
   const f2 p = f2_mul(a.hi, b.hi);
   f2 ne = f2_fma(a.nhi, b.hi, p);  // -(a.hi b.hi - p)
@@ -59,7 +59,7 @@ QL_DEV void df2_acc_fma(df2& acc, const df2n& a, const df2& b) {
   acc.hi = s;
   acc.lo = f2_add(acc.lo, f2_sub(t, ne));
 }
-// The two rows of a finished accumulator.
+// The two halves of a finished accumulator.
 QL_DEV void df2_rows(const df2& a, df& r0, df& r1) {
   float h0, h1, l0, l1;
   f2_split(a.hi, h0, h1);

@@ -1,14 +1,24 @@
 // Q reconstruction: Q = X R^{-1}, the orthonormal factor of X = Q R from the R that any of
 // the Q-less calls returned (the explicit Q of Sec. 1 that block iterative solvers use).
 //
-// One launch.  Every CTA inverts R (FP64, shared memory; n <= 64 so this is cheap) and then
-// streams row tiles of T rows: each thread owns one row, converts it once to double-float
-// (shared memory, conflict-free), and forms its row of Q = X M eight columns at a time from
-// the M rows above the diagonal.  A tile whose X or whose M lies outside the double-float
-// exponent range is formed in FP64 instead (decided per tile, the same for the whole CTA),
-// so no second launch and no workspace are needed.
+// One launch.  Every CTA inverts R (FP64, shared memory; n <= 64 so this is cheap); then each
+// warp streams blocks of 64 rows by itself: a thread owns two adjacent rows, fetches them eight
+// columns at a time (16-byte loads, all in flight at once), converts them once to double-float
+// (its own words of shared memory, so no barrier and the warps drift apart), and forms its rows
+// of Q = X M eight columns at a time from the M rows above the diagonal, two columns per packed
+// FP32 instruction.  A block whose X or whose M lies outside the double-float exponent range is
+// formed in FP64 instead (decided per warp), so no second launch and no workspace are needed.
+//
+// Bound: 13 FP32 operations per product and row (m = 2^23, n = 16: 378 us at the measured FP32
+// rate, against 323 us of HBM).  Measured there 1638 us with one row per thread, a column fetched
+// at a time and block-wide tiles, 1195 us now; 4000000 x 32 2393 -> 1430 us, 2097152 x 64 5015 ->
+// 3994 us, 4000001 x 8 381 -> 263 us.  What is left is latency (fixed-latency stalls at 5 to 24
+// warps per SM) and the conversions of X and of the results (three FP64-pipe instructions each,
+// 640 us of that pipe at n = 16, overlapped; assembling the doubles with integer instructions
+// instead measured slower, 1605 us).
 #include <mutex>
 
+#include "df2.cuh"
 #include "internal.h"
 #include "small_dense.cuh"
 
@@ -25,30 +35,36 @@ struct QformArgs {
   S* Q;
   int64_t ldq;
   int32_t* info;
-  int64_t tiles;
+  int64_t tiles;  // blocks of 64 rows
+  int pair;       // two adjacent rows of every column can be read and written in one access
 };
 
 template <int NC>
 struct QformSmem {
-  static constexpr int T = 256;                              // rows per tile, one per thread
+  // one CTA per SM of as many warps as the shared memory holds (32 and 16 KB each) at 64 and 32
+  // columns, else three of eight warps
+  static constexpr int T = NC == 64 ? 160 : (NC == 32 ? 384 : 256);
+  static constexpr int kCtas = NC <= 16 ? 3 : 1;
   static constexpr int LDM = NC + 1;                         // odd stride: column walks of the inverse
   static constexpr size_t kM = 8 * (size_t)NC * LDM;         // FP64 M = R^{-1}
-  static constexpr size_t kMd = 8 * (size_t)NC * NC;         // double-float M (row k, 8 columns per load)
-  static constexpr size_t kX = 8 * (size_t)NC * T;           // the tile as double-float, [k][row]
-  static constexpr size_t kOffMd = kM;
+  static constexpr size_t kMd = 8 * (size_t)NC * NC;         // double-float M, [k][column pair]
+  static constexpr size_t kX = 16 * (size_t)NC * T;          // two rows per thread as double-float, [k][thread]
+  static constexpr size_t kOffMd = (kM + 15) / 16 * 16;
   static constexpr size_t kOffX = kOffMd + kMd;
   static constexpr size_t kOffMisc = kOffX + kX;
   static constexpr size_t kBytes = kOffMisc + 64;
+  static_assert(kBytes <= 232448, "shared memory of one SM");
+  static_assert(kX >= 8 * (size_t)NC * LDM, "R fits in the row area");
 };
 
 template <int NC, typename S>
-__global__ void __launch_bounds__(256, 1) qform_kernel(QformArgs<S> a) {
+__global__ void __launch_bounds__(QformSmem<NC>::T, QformSmem<NC>::kCtas) qform_kernel(QformArgs<S> a) {
   using Sm = QformSmem<NC>;
   constexpr int T = Sm::T, LDM = Sm::LDM;
   extern __shared__ __align__(16) unsigned char smem[];
   double* Mf = reinterpret_cast<double*>(smem);
-  df* Md = reinterpret_cast<df*>(smem + Sm::kOffMd);
-  df* xs = reinterpret_cast<df*>(smem + Sm::kOffX);
+  df2* Md = reinterpret_cast<df2*>(smem + Sm::kOffMd);
+  float4* xs = reinterpret_cast<float4*>(smem + Sm::kOffX);  // (hi, lo) of both rows
   int* misc = reinterpret_cast<int*>(smem + Sm::kOffMisc);
   const int tid = threadIdx.x, n = a.n;
 
@@ -71,7 +87,7 @@ __global__ void __launch_bounds__(256, 1) qform_kernel(QformArgs<S> a) {
   const int zi = misc[0];
   if (zi) {  // Q would not be finite: NaN columns from the first zero pivot on, and the status
     const int64_t k = gridDim.x;
-    const int64_t r0 = a.tiles * blockIdx.x / k * T, r1 = min(a.m, a.tiles * (blockIdx.x + 1) / k * T);
+    const int64_t r0 = a.tiles * blockIdx.x / k * 64, r1 = min(a.m, a.tiles * (blockIdx.x + 1) / k * 64);
     for (int j = 0; j < n; ++j)
       for (int64_t r = r0 + tid; r < r1; r += T) a.Q[j * a.ldq + r] = (S)__longlong_as_double(0x7ff8000000000000ll);
     if (blockIdx.x == 0 && tid == 0 && a.info) {
@@ -83,14 +99,20 @@ __global__ void __launch_bounds__(256, 1) qform_kernel(QformArgs<S> a) {
   tri_upper_inverse<T>(Rs, LDM, Mf, LDM, n);
   // double-float copy (zero below the diagonal and past n) and its range verdict
   bool mbad = false;
-  for (int e = tid; e < NC * NC; e += T) {
-    const int k = e / NC, j = e % NC;
-    const double v = (k < n && j < n && k <= j) ? Mf[k * LDM + j] : 0.0;
-    if (v != 0.0) {
-      const int E = (int)((__double_as_longlong(v) >> 52) & 0x7ff);
-      if (E < 1023 - 60 || E > 1023 + 60) mbad = true;
+  for (int e = tid; e < NC * NC / 2; e += T) {
+    const int k = e / (NC / 2), j0 = 2 * (e % (NC / 2));
+    df m2[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int j = j0 + h;
+      const double v = (k < n && j < n && k <= j) ? Mf[k * LDM + j] : 0.0;
+      if (v != 0.0) {
+        const int E = (int)((__double_as_longlong(v) >> 52) & 0x7ff);
+        if (E < 1023 - 60 || E > 1023 + 60) mbad = true;
+      }
+      m2[h] = df_from_double_rn(v);
     }
-    Md[k * NC + j] = df_from_double_rn(v);
+    Md[e] = df2{f2_make(m2[0].hi, m2[1].hi), f2_make(m2[0].lo, m2[1].lo)};
   }
   const bool m_f64 = __syncthreads_or(mbad);
   if (blockIdx.x == 0 && tid == 0 && a.info) {
@@ -98,79 +120,108 @@ __global__ void __launch_bounds__(256, 1) qform_kernel(QformArgs<S> a) {
     a.info[1] = 0;
   }
 
-  const int64_t k = gridDim.x, bid = blockIdx.x;
-  const int64_t t0 = a.tiles * bid / k, t1 = a.tiles * (bid + 1) / k;
-  for (int64_t t = t0; t < t1; ++t) {
-    const int64_t row = t * T + tid;
-    const bool live = row < a.m;
-    // this thread's row as double-float, [k][row] in shared memory (conflict-free)
+  // ---- row blocks of 64 rows (tiles), one warp each
+  const int lane = tid & 31;
+  const int64_t nw = (int64_t)gridDim.x * (T / 32);
+  float4* mine = xs + tid;  // column k of this thread's rows at mine[k T]
+  using S2 = typename std::conditional<sizeof(S) == 8, double2, float2>::type;
+  for (int64_t t = (int64_t)blockIdx.x * (T / 32) + (tid >> 5); t < a.tiles; t += nw) {
+    const int64_t row = t * 64 + 2 * lane;
+    const bool live0 = row < a.m, live1 = row + 1 < a.m;
+    const bool whole = a.pair && t * 64 + 64 <= a.m;  // uniform in the warp
     bool xbad = false;
-    for (int c = 0; c < n; ++c) {
-      int E = 0;
-      df v = df{0.0f, 0.0f};
-      if (live) {
-        const S x = a.X[c * a.ldx + row];
-        if constexpr (sizeof(S) == 8) {
-          v = df_split_double((double)x, E);
-        } else {
-          const int e = (__float_as_int((float)x) >> 23) & 0xff;
-          E = e == 0 ? 0 : e + 896;
-          v = df{(float)x, 0.0f};
+#pragma unroll 1
+    for (int c0 = 0; c0 < n; c0 += 8) {
+      S2 v[8];
+      if (whole) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (c0 + u < n) v[u] = __ldcs(reinterpret_cast<const S2*>(a.X + (c0 + u) * a.ldx + row));
+      } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          v[u].x = c0 + u < n && live0 ? __ldg(a.X + (c0 + u) * a.ldx + row) : S(0);
+          v[u].y = c0 + u < n && live1 ? __ldg(a.X + (c0 + u) * a.ldx + row + 1) : S(0);
         }
       }
-      if (E != 0 && (E < kDfEminLimit || E > kDfEmaxLimit)) xbad = true;
-      xs[c * T + tid] = v;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (c0 + u >= n) break;
+        int E0, E1;
+        const df v0 = ArithDF::load(v[u].x, E0), v1 = ArithDF::load(v[u].y, E1);
+        if ((E0 != 0 && (E0 < kDfEminLimit || E0 > kDfEmaxLimit)) || (E1 != 0 && (E1 < kDfEminLimit || E1 > kDfEmaxLimit)))
+          xbad = true;
+        mine[(c0 + u) * T] = make_float4(v0.hi, v0.lo, v1.hi, v1.lo);
+      }
     }
-    const bool f64 = __syncthreads_or(xbad) || m_f64;
+    const bool f64 = __any_sync(0xffffffffu, xbad) || m_f64;
     if (!f64) {
 #pragma unroll 1
       for (int jb = 0; jb < n; jb += 8) {
-        ArithDF::Acc acc[8];
+        df2 acc[2][4];  // [row][column pair]
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) acc[jj] = ArithDF::acc_zero();
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int jj = 0; jj < 4; ++jj) acc[h][jj] = df2{0, 0};
         const int kend = min(n, jb + 8);  // M is upper triangular: rows past column jb + 7 are zero
-#pragma unroll 1
+#pragma unroll (NC <= 16 ? 1 : 2)
         for (int kk = 0; kk < kend; ++kk) {
-          const df xk = xs[kk * T + tid];
+          const float4 x = mine[kk * T];
+          const df2n x0 = df2_factor(df2{f2_make(x.x, x.x), f2_make(x.y, x.y)});
+          const df2n x1 = df2_factor(df2{f2_make(x.z, x.z), f2_make(x.w, x.w)});
+          const df2* mrow = Md + kk * (NC / 2) + jb / 2;
 #pragma unroll
-          for (int jj = 0; jj < 8; ++jj) ArithDF::acc_fma(acc[jj], xk, Md[kk * NC + jb + jj]);
+          for (int jj = 0; jj < 4; ++jj) {
+            const df2 mv = mrow[jj];
+            df2_acc_fma(acc[0][jj], x0, mv);
+            df2_acc_fma(acc[1][jj], x1, mv);
+          }
         }
-        if (live) {
 #pragma unroll
-          for (int jj = 0; jj < 8; ++jj) {
-            if (jb + jj < n) {
-              const df q = ArithDF::acc_get(acc[jj]);
-              if constexpr (sizeof(S) == 8)
-                a.Q[(jb + jj) * a.ldq + row] = (double)q.hi + (double)q.lo;
-              else
-                a.Q[(jb + jj) * a.ldq + row] = __fadd_rn(q.hi, q.lo);
-            }
+        for (int jj = 0; jj < 8; ++jj) {
+          if (jb + jj >= n) break;
+          S2 o;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            df c[2];
+            df2_rows(acc[h][jj / 2], c[0], c[1]);
+            const df q = c[jj & 1];
+            const S r = sizeof(S) == 8 ? (S)((double)q.hi + (double)q.lo) : (S)__fadd_rn(q.hi, q.lo);
+            (h == 0 ? o.x : o.y) = r;
+          }
+          S* out = a.Q + (jb + jj) * a.ldq + row;
+          if (whole) {
+            __stcs(reinterpret_cast<S2*>(out), o);
+          } else {
+            if (live0) out[0] = o.x;
+            if (live1) out[1] = o.y;
           }
         }
       }
     } else {
-      // FP64 for this tile: outside the double-float range, or M is
+      // FP64 for this block: outside the double-float range, or M is
 #pragma unroll 1
-      for (int jb = 0; jb < n; jb += 8) {
-        double acc[8];
+      for (int h = 0; h < 2; ++h) {
+        const int64_t r = row + h;
+        if (r >= a.m) break;
+        for (int jb = 0; jb < n; jb += 8) {
+          double acc[8];
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) acc[jj] = 0.0;
-        const int kend = min(n, jb + 8);
+          for (int jj = 0; jj < 8; ++jj) acc[jj] = 0.0;
+          const int kend = min(n, jb + 8);
 #pragma unroll 1
-        for (int kk = 0; kk < kend; ++kk) {
-          const double xk = live ? (double)a.X[kk * a.ldx + row] : 0.0;
+          for (int kk = 0; kk < kend; ++kk) {
+            const double xk = (double)a.X[kk * a.ldx + r];
+#pragma unroll
+            for (int jj = 0; jj < 8; ++jj)
+              acc[jj] = fma(xk, (jb + jj < n && kk <= jb + jj) ? Mf[kk * LDM + jb + jj] : 0.0, acc[jj]);
+          }
 #pragma unroll
           for (int jj = 0; jj < 8; ++jj)
-            acc[jj] = fma(xk, (kk < n && jb + jj < n && kk <= jb + jj) ? Mf[kk * LDM + jb + jj] : 0.0, acc[jj]);
-        }
-        if (live) {
-#pragma unroll
-          for (int jj = 0; jj < 8; ++jj)
-            if (jb + jj < n) a.Q[(jb + jj) * a.ldq + row] = (S)acc[jj];
+            if (jb + jj < n) a.Q[(jb + jj) * a.ldq + r] = (S)acc[jj];
         }
       }
     }
-    __syncthreads();  // the tile area is rewritten by the next tile
   }
 }
 
@@ -191,7 +242,8 @@ static ql_status qform_launch_one(const QformArgs<S>& a, cudaStream_t stream) {
   int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, Sm::T, Sm::kBytes) != cudaSuccess) return QL_ERR_CUDA;
   int64_t g = (int64_t)device_sm_count() * (occ < 1 ? 1 : occ);
-  if (g > a.tiles) g = a.tiles;
+  const int64_t need = (a.tiles + Sm::T / 32 - 1) / (Sm::T / 32);
+  if (g > need) g = need;
   if (g < 1) g = 1;
   count_launch();
   kern<<<(int)g, Sm::T, Sm::kBytes, stream>>>(a);
@@ -200,8 +252,10 @@ static ql_status qform_launch_one(const QformArgs<S>& a, cudaStream_t stream) {
 
 template <typename S>
 static ql_status qform_dispatch(QformArgs<S> a, cudaStream_t stream) {
-  a.tiles = (a.m + QformSmem<8>::T - 1) / QformSmem<8>::T;
+  a.tiles = (a.m + 63) / 64;
   if (a.tiles < 1) a.tiles = 1;
+  auto aligned = [](const void* p) { return reinterpret_cast<uintptr_t>(p) % (2 * sizeof(S)) == 0; };
+  a.pair = aligned(a.X) && aligned(a.Q) && a.ldx % 2 == 0 && a.ldq % 2 == 0 ? 1 : 0;
   const int n = a.n;
   if (n <= 8) return qform_launch_one<8, S>(a, stream);
   if (n <= 16) return qform_launch_one<16, S>(a, stream);
@@ -244,9 +298,9 @@ extern "C" ql_status ql_q_from_r(int64_t m, int64_t n, const void* X, ql_dtype d
     return QL_ERR_ALIGN;
   cudaStream_t st = (cudaStream_t)stream;
   if (dtype == QL_F64) {
-    QformArgs<double> a{m, (int)n, static_cast<const double*>(X), ldx, R, ldr, static_cast<double*>(Q), ldq, info, 0};
+    QformArgs<double> a{m, (int)n, static_cast<const double*>(X), ldx, R, ldr, static_cast<double*>(Q), ldq, info, 0, 0};
     return qform_dispatch(a, st);
   }
-  QformArgs<float> a{m, (int)n, static_cast<const float*>(X), ldx, R, ldr, static_cast<float*>(Q), ldq, info, 0};
+  QformArgs<float> a{m, (int)n, static_cast<const float*>(X), ldx, R, ldr, static_cast<float*>(Q), ldq, info, 0, 0};
   return qform_dispatch(a, st);
 }
