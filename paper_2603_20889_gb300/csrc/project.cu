@@ -175,84 +175,119 @@ __global__ void __launch_bounds__(kReduceT) cross_reduce_kernel(ProjArgs<S> a, i
   a.C[j * a.ldc + i] = tot;
 }
 
-// ---- W = V - Y C (C of this pass), one row per thread
+// ---- W = V - Y C (C of this pass): blocks of 64 rows, a warp each, two adjacent rows per thread
+// and two columns per packed instruction (as qform_kernel)
+template <int KC>
+__host__ __device__ constexpr int update_threads() {
+  return KC == 64 ? 160 : 256;
+}
 template <int KC, int NC, typename S>
-__global__ void __launch_bounds__(kProjT, 1) update_kernel(ProjArgs<S> a) {
-  constexpr int T = kProjT;
+__global__ void __launch_bounds__(update_threads<KC>(), 1) update_kernel(ProjArgs<S> a) {
+  constexpr int T = update_threads<KC>();
   extern __shared__ __align__(16) unsigned char smem[];
-  double* Cf = reinterpret_cast<double*>(smem);     // [KC][NC]
-  df* Cd = reinterpret_cast<df*>(Cf + KC * NC);      // [KC][NC]
-  df* ys = Cd + KC * NC;                             // [KC][T]
-  const int tid = threadIdx.x, k = a.k, n = a.n;
+  df2* Cd = reinterpret_cast<df2*>(smem);                                        // [KC][NC / 2] column pairs
+  float4* mine = reinterpret_cast<float4*>(Cd + KC * NC / 2) + threadIdx.x;     // column i of this thread's rows at mine[i T]
+  const int tid = threadIdx.x, lane = tid & 31, k = a.k, n = a.n;
   bool cbad = false;
-  for (int e = tid; e < KC * NC; e += T) {
-    const int i = e / NC, j = e % NC;
-    const double c = (i < k && j < n) ? __ldcg(a.w.cpass + i * n + j) : 0.0;
-    Cf[e] = c;
-    const int E = (int)((__double_as_longlong(c) >> 52) & 0x7ff);
-    if (c != 0.0 && (E < 1023 - 80 || E > 1023 + 80)) cbad = true;  // products with Y stay normal floats
-    Cd[e] = df_from_double_rn(c);
+  for (int e = tid; e < KC * NC / 2; e += T) {
+    const int i = e / (NC / 2), j0 = 2 * (e % (NC / 2));
+    df c2[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const double c = (i < k && j0 + h < n) ? __ldcg(a.w.cpass + i * n + j0 + h) : 0.0;
+      const int E = (int)((__double_as_longlong(c) >> 52) & 0x7ff);
+      if (c != 0.0 && (E < 1023 - 80 || E > 1023 + 80)) cbad = true;  // products with Y stay normal floats
+      c2[h] = df_from_double_rn(c);
+    }
+    Cd[e] = df2{f2_make(c2[0].hi, c2[1].hi), f2_make(c2[0].lo, c2[1].lo)};
   }
   const bool c64 = __syncthreads_or(cbad);
-  const int64_t nb = gridDim.x, bid = blockIdx.x;
-  const int64_t t0 = a.tiles * bid / nb, t1 = a.tiles * (bid + 1) / nb;
-  for (int64_t t = t0; t < t1; ++t) {
-    const int64_t row = t * T + tid;
-    const bool live = row < a.m;
+  auto fp64_entry = [&](int64_t row, int j) {
+    double s = (double)a.V[j * a.ldv + row];
+    for (int i = 0; i < k; ++i) s = fma(-(double)a.Y[i * a.ldy + row], __ldcg(a.w.cpass + i * n + j), s);
+    a.W[j * a.ldw + row] = (S)s;
+  };
+  const int64_t nw = (int64_t)gridDim.x * (T / 32);
+  for (int64_t t = (int64_t)blockIdx.x * (T / 32) + (tid >> 5); t < a.tiles; t += nw) {
+    const int64_t row = t * 64 + 2 * lane;
+    const bool live0 = row < a.m, live1 = row + 1 < a.m;
     bool bad = false;
-#pragma unroll 8
-    for (int i = 0; i < k; ++i) {
-      int E = 0;
-      df y = df{0.0f, 0.0f};
-      if (live) y = load_df(a.Y[i * a.ldy + row], E);
-      if (!df_range_ok_dev(E)) bad = true;
-      ys[i * T + tid] = y;
+#pragma unroll 1
+    for (int i0 = 0; i0 < k; i0 += 8) {
+      S x[8][2];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const S* p = a.Y + (i0 + u) * a.ldy + row;
+        x[u][0] = i0 + u < k && live0 ? __ldg(p) : S(0);
+        x[u][1] = i0 + u < k && live1 ? __ldg(p + 1) : S(0);
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (i0 + u >= k) break;
+        int E0, E1;
+        const df y0 = load_df(x[u][0], E0), y1 = load_df(x[u][1], E1);
+        if (!df_range_ok_dev(E0) || !df_range_ok_dev(E1)) bad = true;
+        mine[(i0 + u) * T] = make_float4(y0.hi, y0.lo, y1.hi, y1.lo);
+      }
     }
-    const bool f64 = __syncthreads_or(bad) || c64;
+    const bool f64 = __any_sync(0xffffffffu, bad) || c64;
 #pragma unroll 1
     for (int jb = 0; jb < n; jb += 8) {
       if (!f64) {
-        ArithDF::Acc acc[8];
+        // V's entries first: their fetch hides behind the products (W may be V itself)
+        S v[2][8];
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) acc[jj] = ArithDF::acc_zero();
-#pragma unroll 1
-        for (int i = 0; i < k; ++i) {
-          const df y = ys[i * T + tid];
-#pragma unroll
-          for (int jj = 0; jj < 8; ++jj) ArithDF::acc_fma(acc[jj], y, Cd[i * NC + jb + jj]);
+        for (int jj = 0; jj < 8; ++jj) {
+          v[0][jj] = jb + jj < n && live0 ? a.V[(jb + jj) * a.ldv + row] : S(0);
+          v[1][jj] = jb + jj < n && live1 ? a.V[(jb + jj) * a.ldv + row + 1] : S(0);
         }
-        if (live) {
+        df2 acc[2][4];  // [row][column pair]
 #pragma unroll
-          for (int jj = 0; jj < 8; ++jj) {
-            const int j = jb + jj;
-            if (j < n) {
-              int E;
-              const df v = load_df(a.V[j * a.ldv + row], E);
-              bool vbad = !df_range_ok_dev(E);
-              if (!vbad) {
-                const df w = df_sub(v, ArithDF::acc_get(acc[jj]));
-                if constexpr (sizeof(S) == 8)
-                  a.W[j * a.ldw + row] = (double)w.hi + (double)w.lo;
-                else
-                  a.W[j * a.ldw + row] = __fadd_rn(w.hi, w.lo);
-              } else {  // this entry alone is out of range: FP64
-                double s = (double)a.V[j * a.ldv + row];
-                for (int i = 0; i < k; ++i) s = fma(-(double)a.Y[i * a.ldy + row], Cf[i * NC + j], s);
-                a.W[j * a.ldw + row] = (S)s;
-              }
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int jj = 0; jj < 4; ++jj) acc[h][jj] = df2{0, 0};
+#pragma unroll 2
+        for (int i = 0; i < k; ++i) {
+          const float4 x = mine[i * T];
+          const df2n y0 = df2_factor(df2{f2_make(x.x, x.x), f2_make(x.y, x.y)});
+          const df2n y1 = df2_factor(df2{f2_make(x.z, x.z), f2_make(x.w, x.w)});
+          const df2* crow = Cd + i * (NC / 2) + jb / 2;
+#pragma unroll
+          for (int jj = 0; jj < 4; ++jj) {
+            const df2 c = crow[jj];
+            df2_acc_fma(acc[0][jj], y0, c);
+            df2_acc_fma(acc[1][jj], y1, c);
+          }
+        }
+#pragma unroll
+        for (int jj = 0; jj < 8; ++jj) {
+          const int j = jb + jj;
+          if (j >= n) break;
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (h == 0 ? !live0 : !live1) continue;
+            df c[2];
+            df2_rows(acc[h][jj / 2], c[0], c[1]);
+            int E;
+            const df vv = load_df(v[h][jj], E);
+            if (df_range_ok_dev(E)) {
+              const df w = df_sub(vv, c[jj & 1]);
+              if constexpr (sizeof(S) == 8)
+                a.W[j * a.ldw + row + h] = (double)w.hi + (double)w.lo;
+              else
+                a.W[j * a.ldw + row + h] = __fadd_rn(w.hi, w.lo);
+            } else {  // this entry alone is out of range: FP64
+              fp64_entry(row + h, j);
             }
           }
         }
-      } else if (live) {
+      } else {
         for (int jj = 0; jj < 8 && jb + jj < n; ++jj) {
-          const int j = jb + jj;
-          double s = (double)a.V[j * a.ldv + row];
-          for (int i = 0; i < k; ++i) s = fma(-(double)a.Y[i * a.ldy + row], Cf[i * NC + j], s);
-          a.W[j * a.ldw + row] = (S)s;
+          if (live0) fp64_entry(row, jb + jj);
+          if (live1) fp64_entry(row + 1, jb + jj);
         }
       }
     }
-    __syncthreads();  // ys is rewritten by the next tile
   }
 }
 
@@ -264,7 +299,7 @@ struct ProjSmem {
   static constexpr int SL = kProjT / NBLK >= 1 ? kProjT / NBLK : 1;
   static constexpr size_t kTile = 8 * (size_t)(KC + NC) * kProjB, kRed = 8 * (size_t)SL * KC * NC;
   static constexpr size_t kCross = kTile > kRed ? kTile : kRed;
-  static constexpr size_t kUpdate = 16 * (size_t)KC * NC + 8 * (size_t)KC * kProjT;
+  static constexpr size_t kUpdate = 8 * (size_t)KC * NC + 16 * (size_t)KC * update_threads<KC>();
   static_assert(kUpdate <= 232448, "shared memory of one SM");
 };
 
@@ -292,12 +327,14 @@ static ql_status proj_run(ProjArgs<S> a, cudaStream_t st) {
       ready = true;
     }
   }
+  constexpr int UT = update_threads<KC>();
   int occ = 1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, uk, kProjT, Sm::kUpdate) != cudaSuccess) return QL_ERR_CUDA;
-  const int64_t ctiles = (a.m + kProjB - 1) / kProjB, utiles = (a.m + kProjT - 1) / kProjT;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, uk, UT, Sm::kUpdate) != cudaSuccess) return QL_ERR_CUDA;
+  const int64_t ctiles = (a.m + kProjB - 1) / kProjB, utiles = (a.m + 63) / 64;
   int64_t gc = (int64_t)device_sm_count() * kCrossCtasPerSm, gu = (int64_t)device_sm_count() * (occ < 1 ? 1 : occ);
   if (gc > ctiles) gc = ctiles;
-  if (gu > utiles) gu = utiles;
+  const int64_t uneed = (utiles + UT / 32 - 1) / (UT / 32);
+  if (gu > uneed) gu = uneed;
   if (gc < 1) gc = 1;
   if (gu < 1) gu = 1;
   const S* X = a.V;
@@ -320,7 +357,7 @@ static ql_status proj_run(ProjArgs<S> a, cudaStream_t st) {
     if (cudaPeekAtLastError() != cudaSuccess) return QL_ERR_CUDA;
     a.tiles = utiles;
     count_launch();
-    uk<<<(int)gu, kProjT, Sm::kUpdate, st>>>(a);
+    uk<<<(int)gu, UT, Sm::kUpdate, st>>>(a);
     if (cudaPeekAtLastError() != cudaSuccess) return QL_ERR_CUDA;
   }
   return QL_OK;
