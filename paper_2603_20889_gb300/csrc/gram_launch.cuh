@@ -1673,7 +1673,7 @@ ql_status gram_umma_launch_one(const GramCall& c, const GramWs& w, int pass) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Pipelined first Gram pass on tcgen05 (see gram_pipe.cuh).  The body handles the row tiles
+// Pipelined later Gram pass on tcgen05 (see gram_pipe.cuh).  The body handles the row tiles
 // [tiles bid / k, tiles (bid + 1) / k) of one problem as partial `bid` of `k`, with the
 // tensor memory at tbase and the barriers that pipe_cta_begin set up; bars carries their
 // phase counts from one work item to the next.
@@ -1689,17 +1689,6 @@ QL_DEV void put_planes7(unsigned char* base, const unsigned long long (&Nb)[8]) 
   if constexpr (P + 1 < 7) put_planes7<PLANE, P + 1>(base, Nb);
 }
 
-template <int NC, int PLANE, int P = 0>
-QL_DEV void put_planes8(unsigned char* base, const unsigned long long (&Nb)[8]) {
-  uint4 w;
-  w.x = digit_word<P>(Nb[0], Nb[1]);
-  w.y = digit_word<P>(Nb[2], Nb[3]);
-  w.z = digit_word<P>(Nb[4], Nb[5]);
-  w.w = digit_word<P>(Nb[6], Nb[7]);
-  *reinterpret_cast<uint4*>(base + P * PLANE) = w;
-  if constexpr (P + 1 < 8) put_planes8<NC, PLANE, P + 1>(base, Nb);
-}
-
 // Digits P.. of one element (biased fixed point Nb, see biased_fixed56) into their planes,
 // one 2-byte store per plane.
 template <int PLANE, int P = 0>
@@ -1708,20 +1697,18 @@ QL_DEV void put_digits8_one(unsigned char* p0, unsigned long long Nb) {
   if constexpr (P + 1 < 8) put_digits8_one<PLANE, P + 1>(p0, Nb);
 }
 
-// XF = kXNone: the first pass (C = X^T X).  XF = kXUpper / kXFull (n <= 32): a later pass of
-// Cholesky-QR2 / shifted Cholesky-QR3 (M = R1^{-1}, upper triangular) or SVQB2 (M = B1):
-// C = Y^T Y with Y = X M formed tile by tile and never stored.  The slicer warps then cut X
-// into seven digits at the whole matrix's column scale (the first pass recorded it), form
-// Y = X M' (M' = diag(2^e_k) M) on mma.sync from those digits and the M' digits (B
-// fragments in shared memory), fold the seven weights of each element into a double-float
-// and cut Y into the eight digits of the Gram, as the first pass cuts X; the control warp,
-// the copies and the tensor-memory sums are the first pass's.
-template <int NC, typename S, int XF = kXNone>
+// A later pass of Cholesky-QR2 / shifted Cholesky-QR3 (XF = kXUpper, M = R1^{-1}) or SVQB2
+// (kXFull, M = B1), n <= 32: C = Y^T Y with Y = X M formed tile by tile and never stored.  The
+// slicer warps cut X into seven digits at the whole matrix's column scale (the first pass
+// recorded it), form Y = X M' (M' = diag(2^e_k) M) on mma.sync from those digits and the M'
+// digits (B fragments in shared memory), fold the seven weights of each element into a
+// double-float and cut Y into eight digits for the Gram, whose sums stay in tensor memory.
+template <int NC, typename S, int XF>
 QL_DEV void gram_pipe_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& bars, const CUtensorMap* tmA,
                            const CUtensorMap* tmB) {
   using Sh = PipeShape<NC>;
-  using Sm = PipeSmem<NC, S, XF>;
-  static_assert(XF == kXNone || NC <= 32, "later passes: the M' fragments of n <= 32 columns");
+  using Sm = PipeSmem<NC, S>;
+  static_assert(XF != kXNone && NC <= 32, "the M' fragments of n <= 32 columns");
   constexpr int T = Sh::T, TS = Sh::TS, UPT = Sh::UPT, KT = Sh::KT, SP = Sh::SP, PLANE = Sh::PLANE,
                 SBO = Sh::SBO, LBO = Sh::LBO, HALF = Sh::HALF, G = Sh::G, RPB = Sm::RPB, NBOX = Sm::NBOX;
   constexpr uint32_t IDESC = umma_idesc_bf16(128, 128);
@@ -1751,7 +1738,7 @@ QL_DEV void gram_pipe_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBa
   }
   if (tid < 2) sfail[tid] = 0;
   bool skip_tiles = false;
-  if constexpr (XF != kXNone) {
+  {
     int* gexp = reinterpret_cast<int*>(smem + Sm::kOffGexp);  // X's column exponents (whole matrix)
     int* fexp = reinterpret_cast<int*>(smem + Sm::kOffFexp);  // M''s column exponents
     int* entry = reinterpret_cast<int*>(smem + Sm::kOffEntry);
@@ -1842,9 +1829,6 @@ QL_DEV void gram_pipe_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBa
   // block: the FP64 level, then the double-float sums (each slicer touches only its own)
   double* fb = a.w.fbuf + (size_t)bid * NC * 128 * 2;
   float2* fd = reinterpret_cast<float2*>(fb + (size_t)NC * 128);
-  int erun[UPT];  // largest exponent each unit's column has shown this slicer (range record)
-#pragma unroll
-  for (int uu = 0; uu < UPT; ++uu) erun[uu] = 0;
 
   if (control) {
     // ---- control warp: copies two tiles ahead, then per tile: once the slicers have read
@@ -1978,262 +1962,170 @@ QL_DEV void gram_pipe_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBa
         fail_where = 1;
         break;
       }
-      if constexpr (XF == kXNone) {
-        S v[UPT][8];
-        int e[UPT];
-        bool over = false;
-  #pragma unroll
-        for (int uu = 0; uu < UPT; ++uu) {
-          e[uu] = 0;
-          if (live_[uu]) {
-            if (bulk) {
-              load8_swz<NC, S>(v[uu], raw0 + (size_t)b * Sm::kRaw, c_[uu], r0_[uu],
-                               c_[uu] == a.src.nA ? 0 : (c_[uu] & 7));
-            } else {
-              const S* col = a.src.col(c_[uu]);
-              const int64_t row0 = t * KT + r0_[uu];
-  #pragma unroll
-              for (int j = 0; j < 8; ++j) v[uu][j] = row0 + j < a.m ? __ldg(col + row0 + j) : S(0);
-            }
-  #pragma unroll
-            for (int j = 0; j < 8; ++j) e[uu] = max(e[uu], elem_exponent(v[uu][j]));
-            erun[uu] = max(erun[uu], e[uu]);
-            over = over || e[uu] > scale[c_[uu]];
+      // ---- later pass: Y = X M' for this tile, then Y's digits
+      const int* gexp = reinterpret_cast<const int*>(smem + Sm::kOffGexp);
+      const int* fexp = reinterpret_cast<const int*>(smem + Sm::kOffFexp);
+      const uint2* bqs = reinterpret_cast<const uint2*>(smem + Sm::kOffBq);
+      constexpr int NCB = Sm::NCB, KSTEPS = Sm::KSTEPS;
+      static_assert(NCB * (KT / 16) == 2 * (TS / 32), "two 16 x 8 blocks of Y per slicer warp");
+      // buffer b takes X's digits first: the MMAs of tile t - 2 must be done with it
+      const bool okw = i >= 2 ? mbar_wait_bounded(&mbar[b], (cpar >> b) & 1u) : true;
+      if (!slicer_and<TS>(okw)) {  // the tensor core did not finish: FP64 redoes the call
+        ok = false;
+        fail_where = 2;
+        break;
+      }
+      // seven balanced digits of X at the whole matrix's column scale, 8 rows of one
+      // column per unit (the core-matrix layout of the Gram digits)
+#pragma unroll
+      for (int uu = 0; uu < UPT; ++uu) {
+        const int cu = c_[uu], em = live_[uu] ? gexp[cu] : 0;
+        S xv[8];
+        if (live_[uu]) {
+          if (bulk) {
+            load8_swz<NC, S>(xv, raw0 + (size_t)b * Sm::kRaw, cu, r0_[uu], cu == a.src.nA ? 0 : (cu & 7));
           } else {
-  #pragma unroll
-            for (int j = 0; j < 8; ++j) v[uu][j] = S(0);
+            const S* col = a.src.col(cu);
+            const int64_t row0 = t * KT + r0_[uu];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) xv[j] = row0 + j < a.m ? __ldg(col + row0 + j) : S(0);
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) xv[j] = S(0);
+        }
+        unsigned long long Nb[8];  // N + kDigitBias + kDigitTop7 >= 0 (see digit_word7)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          long long N;
+          if constexpr (sizeof(S) == 8) {
+            N = em > 0 ? fixed48_of_double((double)xv[j], em) : 0ll;
+          } else {
+            N = em > 0 ? fixed48_of_float((float)xv[j], em - 896) : 0ll;
+          }
+          Nb[j] = (unsigned long long)(N + kDigitBias) + kDigitTop7;
+        }
+        put_planes7<PLANE>(dig + (cu >> 3) * SBO + (r0_[uu] >> 3) * LBO + (cu & 7) * 16, Nb);
+      }
+      // stage b is read: the control warp may copy the tile two ahead into it
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&rbar[b]);
+      slicer_sync<TS>();  // X's digits are in place
+      // Y = X M' on mma.sync: this warp's 8-column block cb and two 16-row blocks; per
+      // block the 28 digit pairs (p + q <= 6) accumulate exactly in FP32 per weight
+      const int g = lane >> 2, t4 = lane & 3, cb = warp % NCB;
+      const int ksw = XF == kXUpper ? (cb >> 1) + 1 : KSTEPS;  // M' upper triangular: k <= j
+      df y[2][4];
+#pragma unroll
+      for (int bi = 0; bi < 2; ++bi) {
+        const int rb = warp / NCB + bi * (16 / NCB);
+        float ac[7][4];
+#pragma unroll
+        for (int d = 0; d < 7; ++d)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) ac[d][e] = 0.0f;
+#pragma unroll
+        for (int ks = 0; ks < KSTEPS; ++ks) {
+          if (ks < ksw) {
+            uint2 bw[7];
+#pragma unroll
+            for (int q = 0; q < 7; ++q) bw[q] = bqs[((cb * KSTEPS + ks) * 7 + q) * 32 + lane];
+            // ldmatrix .trans of core matrix (column group 2 ks + K, row group 2 rb + R)
+            const unsigned char* ap =
+                dig + (2 * ks + (lane >> 4)) * SBO + (2 * rb + ((lane >> 3) & 1)) * LBO + (lane & 7) * 16;
+#pragma unroll
+            for (int p = 0; p < 7; ++p) {
+              unsigned a0, a1, a2, a3;
+              ldsm_x4_t(a0, a1, a2, a3, ap + p * PLANE);
+#pragma unroll
+              for (int q = 0; q + p < 7; ++q) mma_bf16(ac[p + q], a0, a1, a2, a3, bw[q].x, bw[q].y);
+            }
           }
         }
-        // stage b is read: the control warp may copy the tile two ahead into it
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&rbar[b]);
-        // digit buffer b is free once the MMAs of tile t - 2 are done; a column whose tile
-        // maximum exceeds its scale, or a full group, needs a read-out first (rare)
-        const bool okw = i >= 2 ? mbar_wait_bounded(&mbar[b], (cpar >> b) & 1u) : true;
-        const bool full = grp >= G;
-        if (slicer_or<TS>(over || !okw) || full) {
-          if (!slicer_and<TS>(okw)) {  // the tensor core did not finish: FP64 redoes the call
+        // fold the seven weights (smallest first) into one double-float per element;
+        // weight d of column j weighs 2^(f_j - 12 - 7 d), f_j = fexp[j] - 1022
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int F = fexp[cb * 8 + 2 * t4 + (e & 1)], f = F - 1022;
+          float hi = ac[6][e] * __int_as_float((f - kDigitScaleLog2 - 42 + 127) << 23), lo = 0.0f;
+#pragma unroll
+          for (int d = 5; d >= 0; --d) {
+            float s2, e2;
+            two_sum(hi, ac[d][e] * __int_as_float((f - kDigitScaleLog2 - 7 * d + 127) << 23), s2, e2);
+            hi = s2;
+            lo = __fadd_rn(lo, e2);
+          }
+          y[bi][e] = F > 0 ? df_make(hi, lo) : df{0.0f, 0.0f};
+        }
+      }
+      slicer_sync<TS>();  // every read of X's digits is done: buffer b takes Y's digits next
+      // Y against the running column scales (this lane holds columns c0 and c0 + 1); the
+      // exponent of the high part bounds the double-float's (no FP64 instruction here: the
+      // FP64 pipe runs at 1/64 of the FP32 rate)
+      const int c0 = cb * 8 + 2 * t4;
+      int ey[2] = {0, 0};
+#pragma unroll
+      for (int bi = 0; bi < 2; ++bi)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) ey[e & 1] = max(ey[e & 1], elem_exponent(y[bi][e].hi));
+      const bool over = ey[0] > scale[c0] || ey[1] > scale[c0 + 1];
+      const bool full = grp >= G;
+      if (slicer_or<TS>(over) || full) {
+        if (grp > 0) {  // read the sums out before their scale changes or they could round
+          if (!slicer_and<TS>(mbar_wait_bounded(&mbar[last_b], (cpar >> last_b) & 1u))) {
             ok = false;
             fail_where = 2;
             break;
           }
-          const bool anyover = slicer_or<TS>(over);
-          if ((anyover || full) && grp > 0) {  // read the sums out before their scale changes or they could round
-            if (!slicer_and<TS>(mbar_wait_bounded(&mbar[last_b], (cpar >> last_b) & 1u))) {
-              ok = false;
-              fail_where = 2;
-              break;
-            }
-            tc_fence_after();
-            readout();
-            grp = 0;
-            if (++nread == Sh::DF_FLUSH) {  // double-float sums -> FP64
-  #pragma unroll 4
-              for (int j = 0; j < HALF; ++j) {
-                double* f = fb + (size_t)(hh * HALF + j) * 128 + L;
-                float2* g = fd + (size_t)(hh * HALF + j) * 128 + L;
-                const float2 d2 = __ldcg(g);
-                __stcg(f, __ldcg(f) + df_to_double(df{d2.x, d2.y}));
-                __stcg(g, make_float2(0.0f, 0.0f));
-              }
-              nread = 0;
-            }
-            slicer_sync<TS>();  // every read of the blocks and of the old scales is done
-          }
-  #pragma unroll
-          for (int uu = 0; uu < UPT; ++uu)
-            if (live_[uu] && e[uu] > scale[c_[uu]]) atomicMax(&scale[c_[uu]], e[uu] + Sh::SLACK);
-          slicer_sync<TS>();
-          for (int cc = tid; cc < NC; cc += TS) {
-            const int s = scale[cc];
-            pow2c[cc] = s > 0 ? __int_as_float(max(1, min(254, s - 895)) << 23) : 0.0f;  // 2^(s - 1022)
-          }
-        }
-        // eight digits of every element into the core-matrix layout of buffer b
-  #pragma unroll
-        for (int uu = 0; uu < UPT; ++uu) {
-          const int cu = c_[uu], Es = live_[uu] ? scale[cu] : 0;
-          unsigned long long Nb[8];
-  #pragma unroll
-          for (int j = 0; j < 8; ++j) Nb[j] = biased_fixed56<S>(v[uu][j], Es);  // dead columns hold zeros
-          put_planes8<NC, PLANE>(dig + (cu >> 3) * SBO + (r0_[uu] >> 3) * LBO + (cu & 7) * 16, Nb);
-        }
-        if (tid == 0) ngrp[b] = grp == 0 ? 1 : 0;
-        fence_proxy_async_smem();  // the digit planes are read by the tensor core
-        tc_fence_before();         // the read-out's TMEM loads come before the next MMAs
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&dbar[b]);
-        cpar = (cpar & ~(1u << b)) | (bars.mpar & (1u << b));
-        bars.mpar ^= 1u << b;
-        last_b = b;
-        ++grp;
-      } else {
-        // ---- later pass: Y = X M' for this tile, then Y's digits
-        const int* gexp = reinterpret_cast<const int*>(smem + Sm::kOffGexp);
-        const int* fexp = reinterpret_cast<const int*>(smem + Sm::kOffFexp);
-        const uint2* bqs = reinterpret_cast<const uint2*>(smem + Sm::kOffBq);
-        constexpr int NCB = Sm::NCB, KSTEPS = Sm::KSTEPS;
-        static_assert(NCB * (KT / 16) == 2 * (TS / 32), "two 16 x 8 blocks of Y per slicer warp");
-        // buffer b takes X's digits first: the MMAs of tile t - 2 must be done with it
-        const bool okw = i >= 2 ? mbar_wait_bounded(&mbar[b], (cpar >> b) & 1u) : true;
-        if (!slicer_and<TS>(okw)) {  // the tensor core did not finish: FP64 redoes the call
-          ok = false;
-          fail_where = 2;
-          break;
-        }
-        // seven balanced digits of X at the whole matrix's column scale, 8 rows of one
-        // column per unit (the core-matrix layout of the Gram digits)
-#pragma unroll
-        for (int uu = 0; uu < UPT; ++uu) {
-          const int cu = c_[uu], em = live_[uu] ? gexp[cu] : 0;
-          S xv[8];
-          if (live_[uu]) {
-            if (bulk) {
-              load8_swz<NC, S>(xv, raw0 + (size_t)b * Sm::kRaw, cu, r0_[uu], cu == a.src.nA ? 0 : (cu & 7));
-            } else {
-              const S* col = a.src.col(cu);
-              const int64_t row0 = t * KT + r0_[uu];
-#pragma unroll
-              for (int j = 0; j < 8; ++j) xv[j] = row0 + j < a.m ? __ldg(col + row0 + j) : S(0);
-            }
-          } else {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) xv[j] = S(0);
-          }
-          unsigned long long Nb[8];  // N + kDigitBias + kDigitTop7 >= 0 (see digit_word7)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            long long N;
-            if constexpr (sizeof(S) == 8) {
-              N = em > 0 ? fixed48_of_double((double)xv[j], em) : 0ll;
-            } else {
-              N = em > 0 ? fixed48_of_float((float)xv[j], em - 896) : 0ll;
-            }
-            Nb[j] = (unsigned long long)(N + kDigitBias) + kDigitTop7;
-          }
-          put_planes7<PLANE>(dig + (cu >> 3) * SBO + (r0_[uu] >> 3) * LBO + (cu & 7) * 16, Nb);
-        }
-        // stage b is read: the control warp may copy the tile two ahead into it
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&rbar[b]);
-        slicer_sync<TS>();  // X's digits are in place
-        // Y = X M' on mma.sync: this warp's 8-column block cb and two 16-row blocks; per
-        // block the 28 digit pairs (p + q <= 6) accumulate exactly in FP32 per weight
-        const int g = lane >> 2, t4 = lane & 3, cb = warp % NCB;
-        const int ksw = XF == kXUpper ? (cb >> 1) + 1 : KSTEPS;  // M' upper triangular: k <= j
-        df y[2][4];
-#pragma unroll
-        for (int bi = 0; bi < 2; ++bi) {
-          const int rb = warp / NCB + bi * (16 / NCB);
-          float ac[7][4];
-#pragma unroll
-          for (int d = 0; d < 7; ++d)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) ac[d][e] = 0.0f;
-#pragma unroll
-          for (int ks = 0; ks < KSTEPS; ++ks) {
-            if (ks < ksw) {
-              uint2 bw[7];
-#pragma unroll
-              for (int q = 0; q < 7; ++q) bw[q] = bqs[((cb * KSTEPS + ks) * 7 + q) * 32 + lane];
-              // ldmatrix .trans of core matrix (column group 2 ks + K, row group 2 rb + R)
-              const unsigned char* ap =
-                  dig + (2 * ks + (lane >> 4)) * SBO + (2 * rb + ((lane >> 3) & 1)) * LBO + (lane & 7) * 16;
-#pragma unroll
-              for (int p = 0; p < 7; ++p) {
-                unsigned a0, a1, a2, a3;
-                ldsm_x4_t(a0, a1, a2, a3, ap + p * PLANE);
-#pragma unroll
-                for (int q = 0; q + p < 7; ++q) mma_bf16(ac[p + q], a0, a1, a2, a3, bw[q].x, bw[q].y);
-              }
-            }
-          }
-          // fold the seven weights (smallest first) into one double-float per element;
-          // weight d of column j weighs 2^(f_j - 12 - 7 d), f_j = fexp[j] - 1022
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int F = fexp[cb * 8 + 2 * t4 + (e & 1)], f = F - 1022;
-            float hi = ac[6][e] * __int_as_float((f - kDigitScaleLog2 - 42 + 127) << 23), lo = 0.0f;
-#pragma unroll
-            for (int d = 5; d >= 0; --d) {
-              float s2, e2;
-              two_sum(hi, ac[d][e] * __int_as_float((f - kDigitScaleLog2 - 7 * d + 127) << 23), s2, e2);
-              hi = s2;
-              lo = __fadd_rn(lo, e2);
-            }
-            y[bi][e] = F > 0 ? df_make(hi, lo) : df{0.0f, 0.0f};
-          }
-        }
-        slicer_sync<TS>();  // every read of X's digits is done: buffer b takes Y's digits next
-        // Y against the running column scales (this lane holds columns c0 and c0 + 1); the
-        // exponent of the high part bounds the double-float's (no FP64 instruction here: the
-        // FP64 pipe runs at 1/64 of the FP32 rate)
-        const int c0 = cb * 8 + 2 * t4;
-        int ey[2] = {0, 0};
-#pragma unroll
-        for (int bi = 0; bi < 2; ++bi)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) ey[e & 1] = max(ey[e & 1], elem_exponent(y[bi][e].hi));
-        const bool over = ey[0] > scale[c0] || ey[1] > scale[c0 + 1];
-        const bool full = grp >= G;
-        if (slicer_or<TS>(over) || full) {
-          if (grp > 0) {  // read the sums out before their scale changes or they could round
-            if (!slicer_and<TS>(mbar_wait_bounded(&mbar[last_b], (cpar >> last_b) & 1u))) {
-              ok = false;
-              fail_where = 2;
-              break;
-            }
-            tc_fence_after();
-            readout();
-            grp = 0;
-            if (++nread == Sh::DF_FLUSH) {  // double-float sums -> FP64
+          tc_fence_after();
+          readout();
+          grp = 0;
+          if (++nread == Sh::DF_FLUSH) {  // double-float sums -> FP64
 #pragma unroll 4
-              for (int j = 0; j < HALF; ++j) {
-                double* f = fb + (size_t)(hh * HALF + j) * 128 + L;
-                float2* gd = fd + (size_t)(hh * HALF + j) * 128 + L;
-                const float2 d2 = __ldcg(gd);
-                __stcg(f, __ldcg(f) + df_to_double(df{d2.x, d2.y}));
-                __stcg(gd, make_float2(0.0f, 0.0f));
-              }
-              nread = 0;
+            for (int j = 0; j < HALF; ++j) {
+              double* f = fb + (size_t)(hh * HALF + j) * 128 + L;
+              float2* gd = fd + (size_t)(hh * HALF + j) * 128 + L;
+              const float2 d2 = __ldcg(gd);
+              __stcg(f, __ldcg(f) + df_to_double(df{d2.x, d2.y}));
+              __stcg(gd, make_float2(0.0f, 0.0f));
             }
-            slicer_sync<TS>();  // every read of the blocks and of the old scales is done
+            nread = 0;
           }
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-            if (ey[h] > scale[c0 + h]) atomicMax(&scale[c0 + h], ey[h] + Sh::SLACK);
-          slicer_sync<TS>();
-          for (int cc = tid; cc < NC; cc += TS) {
-            const int sc = scale[cc];
-            pow2c[cc] = sc > 0 ? __int_as_float(max(1, min(254, sc - 895)) << 23) : 0.0f;  // 2^(s - 1022)
-          }
+          slicer_sync<TS>();  // every read of the blocks and of the old scales is done
         }
-        // eight digits of every Y element into buffer b (rows g, g + 8 of each 16-row block)
 #pragma unroll
-        for (int bi = 0; bi < 2; ++bi) {
-          const int rb = warp / NCB + bi * (16 / NCB);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int c = c0 + (e & 1), r = 16 * rb + g + 8 * (e >> 1);
-            // fixed point of hi + lo: the two parts rounded separately (hi is exact unless the
-            // element lies 2^32 below its column's scale), one bias removed
-            const unsigned long long Nb = biased_fixed56<float>(y[bi][e].hi, scale[c]) +
-                                          biased_fixed56<float>(y[bi][e].lo, scale[c]) - kDigitBias8;
-            put_digits8_one<PLANE>(dig + (c >> 3) * SBO + (r >> 3) * LBO + (c & 7) * 16 + (r & 7) * 2, Nb);
-          }
+        for (int h = 0; h < 2; ++h)
+          if (ey[h] > scale[c0 + h]) atomicMax(&scale[c0 + h], ey[h] + Sh::SLACK);
+        slicer_sync<TS>();
+        for (int cc = tid; cc < NC; cc += TS) {
+          const int sc = scale[cc];
+          pow2c[cc] = sc > 0 ? __int_as_float(max(1, min(254, sc - 895)) << 23) : 0.0f;  // 2^(s - 1022)
         }
-        if (tid == 0) ngrp[b] = grp == 0 ? 1 : 0;
-        fence_proxy_async_smem();  // the digit planes are read by the tensor core
-        tc_fence_before();         // the read-out's TMEM loads come before the next MMAs
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&dbar[b]);
-        cpar = (cpar & ~(1u << b)) | (bars.mpar & (1u << b));
-        bars.mpar ^= 1u << b;
-        last_b = b;
-        ++grp;
       }
+      // eight digits of every Y element into buffer b (rows g, g + 8 of each 16-row block)
+#pragma unroll
+      for (int bi = 0; bi < 2; ++bi) {
+        const int rb = warp / NCB + bi * (16 / NCB);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int c = c0 + (e & 1), r = 16 * rb + g + 8 * (e >> 1);
+          // fixed point of hi + lo: the two parts rounded separately (hi is exact unless the
+          // element lies 2^32 below its column's scale), one bias removed
+          const unsigned long long Nb = biased_fixed56<float>(y[bi][e].hi, scale[c]) +
+                                        biased_fixed56<float>(y[bi][e].lo, scale[c]) - kDigitBias8;
+          put_digits8_one<PLANE>(dig + (c >> 3) * SBO + (r >> 3) * LBO + (c & 7) * 16 + (r & 7) * 2, Nb);
+        }
+      }
+      if (tid == 0) ngrp[b] = grp == 0 ? 1 : 0;
+      fence_proxy_async_smem();  // the digit planes are read by the tensor core
+      tc_fence_before();         // the read-out's TMEM loads come before the next MMAs
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&dbar[b]);
+      cpar = (cpar & ~(1u << b)) | (bars.mpar & (1u << b));
+      bars.mpar ^= 1u << b;
+      last_b = b;
+      ++grp;
     }
     if (ok && grp > 0) {  // the last group
       if (!slicer_and<TS>(mbar_wait_bounded(&mbar[last_b], (cpar >> last_b) & 1u))) {
@@ -2245,9 +2137,6 @@ QL_DEV void gram_pipe_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBa
       }
     }
     if (!ok && tid == 0) sfail[0] = fail_where;
-#pragma unroll
-    for (int uu = 0; uu < UPT; ++uu)
-      if (live_[uu] && erun[uu] > 0) atomicMax(&colmax[c_[uu]], erun[uu]);
   }
   tc_fence_before();
   __syncthreads();
@@ -2282,7 +2171,7 @@ QL_DEV void gram_pipe_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBa
   gram_finish<NC, T, S, ArithDF>(a, smem, colmax, misc, k);
 }
 
-template <int NC, typename S, int XF = kXNone>
+template <int NC, typename S, int XF>
 __global__ void __launch_bounds__(PipeShape<NC>::T, 1)
     gram_pipe_kernel(const __grid_constant__ GramArgs<S> a, const __grid_constant__ CUtensorMap tmA,
                      const __grid_constant__ CUtensorMap tmB, int has_b) {
@@ -2297,11 +2186,11 @@ __global__ void __launch_bounds__(PipeShape<NC>::T, 1)
   if ((threadIdx.x >> 5) == 0) tmem_dealloc(tbase, PipeShape<NC>::TCOLS);
 }
 
-// pass 1 (XF = kXNone) or a later pass (XF = kXUpper / kXFull, pass 2 or 3)
-template <int NC, typename S, int XF = kXNone>
-ql_status gram_pipe_launch_one(const GramCall& c, const GramWs& w, int pass = 1) {
+// a later pass (2 or 3)
+template <int NC, typename S, int XF>
+ql_status gram_pipe_launch_one(const GramCall& c, const GramWs& w, int pass) {
   using Sh = PipeShape<NC>;
-  using Sm = PipeSmem<NC, S, XF>;
+  using Sm = PipeSmem<NC, S>;
   auto kern = gram_pipe_kernel<NC, S, XF>;
   static bool ready = false;
   static std::mutex mu;
@@ -2414,9 +2303,8 @@ ql_status gram_dispatch(const GramCall& c, const GramWs& w, int gated) {
     constexpr int NC = decltype(nc_tag)::value;
     if constexpr (NC >= 16 && std::is_same<Ar, ArithDF>::value) {
       if (tc_gram_enabled()) {
-        // first pass: the pipelined tcgen05 kernel (its read-outs are rare, so stacking
-        // 128 / NC planes costs little).  Later passes: tcgen05 per tile for 64 columns;
-        // below that mma.sync, whose per-tile read-out is cheaper than TMEM's
+        // first pass: the exact kernel, which also ends the call where it can (xg_finish).
+        // Later passes, beyond that: tcgen05 per tile for 64 columns, the pipelined kernel below
         if constexpr (NC == 64) {
           ql_status st =
               pipe_gram_enabled() ? xgram_pass1<S>(c, w) : gram_umma_launch_one<NC, S, kXNone>(c, w, 1);

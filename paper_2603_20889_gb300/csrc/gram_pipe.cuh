@@ -1,5 +1,6 @@
-// Pipelined first Gram pass on tcgen05 (C = X^T X, paper Sec. 3.1, Algorithm 1 step 1, and
-// the first pass of SVQB2) for the 16-, 32- and 64-column classes.
+// Pipelined later Gram pass on tcgen05 (C = Y^T Y, Y = X M, paper Sec. 3.1, Algorithm 1 step 3,
+// and the second pass of SVQB2) for the 16- and 32-column classes, and the tile and digit
+// helpers that the exact first pass (xgram.cuh) shares.  Below "a value" is an element of Y.
 //
 // The products are the exact bf16 digit products of gram_umma.cuh, arranged so that the
 // tensor core, the CUDA cores and the copy engine work on different tiles at once:
@@ -65,7 +66,7 @@ struct PipeShape {
   static_assert((long long)G * KT * PAIRS_MAX * 4096 <= (1LL << 24), "exact FP32 digit sums");
 };
 
-template <int NC, typename S, int XF = kXNone>
+template <int NC, typename S>
 struct PipeSmem {
   using Sh = PipeShape<NC>;
   // a staged tile is KT / RPB boxes of RPB rows (128 bytes) x NC columns, written by the
@@ -93,11 +94,11 @@ struct PipeSmem {
   // decision
   static constexpr int NCB = NC / 8, KSTEPS = NC / 16;
   static constexpr size_t kOffBq = (kMain + 15) / 16 * 16;
-  static constexpr size_t kBq = XF == kXNone ? 0 : sizeof(uint2) * NCB * KSTEPS * 7 * 32;
+  static constexpr size_t kBq = sizeof(uint2) * NCB * KSTEPS * 7 * 32;
   static constexpr size_t kOffGexp = kOffBq + kBq;
   static constexpr size_t kOffFexp = kOffGexp + 4 * NC;
   static constexpr size_t kOffEntry = kOffFexp + 4 * NC;
-  static constexpr size_t kBytes = XF == kXNone ? kMain : kOffEntry + 16;
+  static constexpr size_t kBytes = kOffEntry + 16;
   static_assert(kEpi <= kOffPow, "the epilogue's shared memory stays below the scales and barriers");
   static_assert(kRed <= 2 * (size_t)Sh::DBUF, "per-lane sums fit in the digit buffers");
 };
