@@ -6,8 +6,7 @@ Cholesky-QR2 and SVQB2.  Inputs are device-resident before the timed region and 
 larger than the 129 MB L2 (>= 268 MB), so no L2 flush is needed between steps.
 
 metric: effective GB/s = sum over calls of 8 m n bytes / sum of the calls' time (the
-paper's "effective bandwidth", counted once per call even though the Gram methods read X
-twice).  Per-call breakdown, the roofline of the dominant kernel, the oracle on the host
+paper's "effective bandwidth", counted once per call however often a method reads X).  Per-call breakdown, the roofline of the dominant kernel, the oracle on the host
 cores, the host-buffer end-to-end number and the SM clocks seen during the timed region
 are attached.
 
@@ -36,21 +35,16 @@ NS = [1, 2, 4, 8, 16, 32, 64]
 LS_M, LS_N = 1 << 24, 31  # least-squares [A b] workload
 KAPPA = 1e4
 METHODS = ["tsqr", "cholqr2", "svqb2"]
-PASSES = {"tsqr": 1, "cholqr2": 2, "svqb2": 2}
 # DRAM bytes (read + write) per row of X per launch, from one ncu capture of the same kernel
 # on a smaller m (dram__bytes_read.sum + dram__bytes_write.sum of that launch / its m); the
 # roofline's "traffic" is this times m for the dominant call, null where no capture of the
 # current kernel exists.
 MEASURED_TRAFFIC_PER_ROW = {
-    ("tsqr", 64): (1.074413e9 + 3.693568e6) / 2 ** 21,       # tsqr_kernel<64, 16, 16, 256>, m = 2^21
-    ("tsqr", 4): (536.98944e6 + 3.195648e6) / 2 ** 24,       # tsqr_kernel<4, 1, 8, 128>, m = 2^24
-    ("cholqr2", 64): (2.256619e9 + 174.161664e6) / 2 ** 22,  # gram_pipe_kernel<64> (first pass), m = 2^22
+    ("tsqr", 64): (1.085169e9 + 25.390080e6) / 2 ** 21,   # xgram_kernel<64>, m = 2^21
+    ("cholqr2", 64): (1.085169e9 + 25.390080e6) / 2 ** 21,
+    ("svqb2", 64): (1.085169e9 + 25.390080e6) / 2 ** 21,
+    ("tsqr", 4): (1.074413e9 + 10.586368e6) / 2 ** 25,    # xgram_kernel<4>, m = 2^25
 }
-
-
-# FP32 instructions of one double-float (dot, update) pair of the Householder column step:
-# an accumulating product (13, lo * lo kept) and a product subtracted with renormalisation (15)
-DF_INSTR_PER_PAIR = 28
 
 
 def rel_err(R, R_ref) -> float:
@@ -90,9 +84,16 @@ def lapack_r(X):
 
 
 def kernel_name(meth: str, n: int) -> str:
-    if meth == "tsqr":
-        return "tsqr_kernel"
-    return "gram_umma_kernel" if n > 32 else ("gram_tc_kernel" if n > 8 else "gram_kernel")
+    if n >= 3:
+        return "xgram_kernel"  # the exact Gram pass answers every method at this kappa
+    return "tsqr_kernel" if meth == "tsqr" and n > 1 else "gram_stream_kernel"
+
+
+def passes(meth: str, n: int) -> int:
+    """Passes over X that the call makes: one where the exact Gram pass answers it."""
+    return 1 if n >= 3 or meth == "tsqr" else 2
+
+
 METRIC = "Q-less QR effective GB/s (8mn B/time)"
 WORKLOAD = ("Q-less QR condition sweep: X = G S, m = 2^25 rows, n in {1,2,4,8,16,32,64}, kappa = 1e4, "
             "FP64 storage; TSQR + Cholesky-QR2 + SVQB2 per n; plus least squares via the QR of [A b], "
@@ -330,12 +331,12 @@ def run_ours(args, rank, world, local_rank):
     for i, (meth, n) in enumerate(calls):
         ms = per_call[i] / args.steps
         sweep.append({"method": meth, "n": n, "ms": round(ms, 4), "eff_gbs": round(nbytes(meth, n) / ms / 1e6, 1),
-                      "alg_gbs": round(PASSES.get(meth, 1) * nbytes(meth, n) / ms / 1e6, 1)})
+                      "alg_gbs": round(passes(meth, n) * nbytes(meth, n) / ms / 1e6, 1)})
     dom = max(range(len(calls)), key=lambda i: per_call[i])
     dmeth, dn = calls[dom]
     dms = per_call[dom] / args.steps
     # the timed share of the dominant kernel: one pass = one launch reading its bytes
-    kern_ms = dms / PASSES.get(dmeth, 1)
+    kern_ms = dms / passes(dmeth, dn)
     achieved = nbytes(dmeth, dn) / kern_ms / 1e6
     per_row = MEASURED_TRAFFIC_PER_ROW.get((dmeth, dn))
     traffic = int(per_row * M) if per_row else None
@@ -343,41 +344,14 @@ def run_ours(args, rank, world, local_rank):
                 "frac": round(achieved / peak, 4), "peak_source": peak_kind}
     kname = f"{kernel_name(dmeth, dn)} ({dmeth}, n={dn}, m=2^25)"
     # measured compute-pipe peaks of this GPU (FP32 / FP64 FMA, FP64 MMA, the library's
-    # double-float multiply-accumulate), the denominators of the arithmetic-bound rooflines
+    # double-float multiply-accumulate)
     try:
         peaks = {k: round(v, 3) for k, v in q.measure_peaks(stream).items()}
         peaks["unit"] = "TFLOP/s"
     except Exception as exc:
         peaks = {"error": repr(exc)[:200]}
-    if dmeth == "tsqr" and dn > 1:
-        # the double-float Householder is bound by the FP32 pipes: 2 m n^2 FP64-equivalent
-        # flops per launch against the measured FP32 FMA instruction rate at 27 FP32
-        # instructions per (dot, update) pair of 4 flops
-        flops = 2.0 * M * dn * dn
-        ach = flops / (kern_ms / 1e3) / 1e12
-        if "fp32_fma" in peaks:
-            alu_peak = peaks["fp32_fma"] / 2.0 * 4.0 / DF_INSTR_PER_PAIR
-            src = "measured"
-            deriv = (f"measured FP32 FMA rate {peaks['fp32_fma']} TFLOP/s = {peaks['fp32_fma'] / 2:.2f} T instr/s, "
-                     f"x 4 FP64-equivalent flops per {DF_INSTR_PER_PAIR} FP32 instructions (one dot + update pair)")
-        else:
-            sms = torch.cuda.get_device_properties(dev).multi_processor_count
-            clk_hz = float(clk.get("sm_max_mhz") or 2070.0) * 1e6
-            alu_peak = sms * 128 * clk_hz / (DF_INSTR_PER_PAIR / 4.0) / 1e12
-            src = "derived"
-            deriv = (f"{sms} SMs x 128 FP32 lanes x {clk_hz / 1e6:.0f} MHz / "
-                     f"({DF_INSTR_PER_PAIR} FP32 instructions per 4 FP64-equivalent flops)")
-        roofline = {"bound": "alu", "achieved": round(ach, 3), "peak": round(alu_peak, 3), "unit": "TFLOP/s",
-                    "frac": round(ach / alu_peak, 4), "traffic": traffic, "peak_source": src,
-                    "peak_derivation": deriv,
-                    "kernel": kname, "algorithmic_flops_per_launch": int(flops),
-                    "algorithmic_bytes_per_launch": int(nbytes(dmeth, dn)), "hbm": hbm_view,
-                    "note": "per-launch time from CUDA events around the call on its stream"}
-    else:
-        roofline = dict(hbm_view, traffic=traffic, kernel=kname,
-                        algorithmic_bytes_per_launch=int(nbytes(dmeth, dn)),
-                        note="per-launch time from CUDA events around the call on its stream; Gram methods: "
-                             "call time / 2 passes")
+    roofline = dict(hbm_view, traffic=traffic, kernel=kname, algorithmic_bytes_per_launch=int(nbytes(dmeth, dn)),
+                    note="per-launch time from CUDA events around the call on its stream, its n x n work included")
 
     e2e = run_e2e(args, q, lib, torch, dev, Xs, ws, wsb, stream, ls, world) if args.e2e_steps > 0 else None
     accuracy = None
@@ -439,7 +413,9 @@ def run_ours(args, rank, world, local_rank):
         "metric": METRIC, "value": round(value, 2), "unit": "GB/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": round(ms_step, 3), "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "f32x2", "data": "synthetic",
-        "config": {"workload": WORKLOAD, "storage": "f64", "arith": "double-float (f32x2) m-loops, FP64 n x n",
+        "config": {"workload": WORKLOAD, "storage": "f64",
+                   "arith": "exact integer Gram of 56-bit digits (bf16 tensor cores), 125-bit fixed-point Cholesky; "
+                            "double-float for n <= 2",
                    "m": M, "n": NS, "kappa": KAPPA, "methods": METHODS, "parallelism": f"replicas x{world}",
                    "l2": "every input > L2 (>= 268 MB); no flush needed"},
         "roofline": roofline, "clocks": clk, "gpu_launches": int(launches),
