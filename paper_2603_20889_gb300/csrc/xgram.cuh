@@ -800,7 +800,7 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
   const int nt = (int)(a.tiles * (bid + 1) / k - t0);  // tiles of this CTA, i = 0 .. nt - 1
   // full tiles (i < nbulk) arrive by tensor copies when the columns allow them; the last rows
   // of the matrix, and unaligned columns, are read by the slicers from global memory
-  const int nbulk = a.bulk ? (int)min((int64_t)nt, a.m / KT - t0) : 0;
+  const int nbulk = a.bulk ? (int)max((int64_t)0, min((int64_t)nt, a.m / KT - t0)) : 0;
   // tile i = 2 j + b uses stage and buffer b; the phase of its barriers has this parity
   auto par = [&](int i) { return ((bars.mpar >> (i & 1)) ^ (uint32_t)(i >> 1)) & 1u; };
   auto lpar = [&](int i) { return ((bars.lpar >> (i & 1)) ^ (uint32_t)(i >> 1)) & 1u; };
@@ -1007,7 +1007,8 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
 
     Rows8<S> v[2];
     // tile i: loaded into v, voted on (no column of it outgrows its scale), cut into its buffer
-    bool have = false, voted = false, cut = false, over[2] = {false, false};
+    // (freed: its stage has been given back)
+    bool have = false, freed = false, voted = false, cut = false, over[2] = {false, false};
     int es[2] = {0, 0};
     int i = g;                 // this group's next tile
     int first = 0;             // first tile of the sums in tensor memory
@@ -1032,9 +1033,6 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
               for (int j = 0; j < 8; ++j) v[u].set(j, j < left ? __ldg(col + j) : S(0));
             }
           }
-          // the stage is read: the copy warp may copy the tile two ahead into it
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&rbar[g]);
           have = true;
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
@@ -1045,12 +1043,20 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
           }
         }
         if (!voted) {
-          over[0] = live[0] && es[0] > scale[cu[0]];
-          over[1] = live[1] && es[1] > scale[cu[1]];
+          const int above0 = live[0] ? es[0] - scale[cu[0]] : 0, above1 = live[1] ? es[1] - scale[cu[1]] : 0;
+          const bool above = max(above0, above1) > 0;  // needs every element of both units
+          over[0] = above0 > 0;
+          over[1] = above1 > 0;
           // the other group's vote on the tile before comes first, or it has stopped
           bool passed = i == 0;
           while (!passed && !*req && !*fail) passed = mbar_test_wait(&vbar[g ^ 1], par(i - 1));
-          voted = !group_or(g, over[0] || over[1] || (!passed && !*fail));
+          voted = !group_or(g, above | (!passed & !*fail));
+          // The copy warp may refill the stage only now: the vote took every element of every
+          // thread, so all loads have returned.  An arrival right after the loads does not wait
+          // for them (the copy of the tile two ahead overtook loads in flight, seen with the
+          // right-hand side of a 4-column class in L2).
+          if (gt == 0 && !freed) mbar_arrive(&rbar[g]);
+          freed = true;
           if (voted && gt == 0) mbar_arrive(&vbar[g]);
         }
         if (voted && !cut) {
@@ -1123,7 +1129,7 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
       tc_fence_before();         // the read-out's TMEM loads come before the next MMAs
       __syncwarp();
       if (lane == 0) mbar_arrive(&dbar[g]);
-      have = voted = cut = false;
+      have = freed = voted = cut = false;
       i += 2;
     }
 #pragma unroll
@@ -1157,8 +1163,8 @@ QL_DEV uint32_t xg_cta_begin(unsigned char* smem) {
   if (threadIdx.x == 0) {
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + Sm::kOffBar);
     for (int i = 0; i < 4; ++i) mbar_init(bar + i, 1);
-    for (int i = 4; i < 8; ++i) mbar_init(bar + i, XgShape<NC>::TG / 32);  // one arrival per warp of the group
-    for (int i = 8; i < 10; ++i) mbar_init(bar + i, 1);
+    for (int i = 4; i < 6; ++i) mbar_init(bar + i, XgShape<NC>::TG / 32);  // one arrival per warp of the group
+    for (int i = 6; i < 10; ++i) mbar_init(bar + i, 1);
   }
   tc_fence_before();
   __syncthreads();

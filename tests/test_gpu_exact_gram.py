@@ -175,3 +175,22 @@ def test_batch_of_every_class_and_every_way_out(hint):
         if n not in (9, 13):
             kappa = 1e8 if n == 30 else 1e3
             assert oracle.rel_err(R, oracle.householder_r(X.astype(np.float64))) <= oracle.tolerance(n, kappa), n
+
+
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+@pytest.mark.parametrize("n,m", [(1, 4099), (2, 700000), (3, 4099), (3, 700000), (3, 700003), (7, 350000), (15, 150000)])
+def test_right_hand_side_rows_stay_with_their_rows(n, m, dtype):
+    # repeated on data that stays in L2, where a copy into a stage follows its release soonest: one
+    # 16-byte piece of a column read from another tile changes the Gram matrix by about 2 / m
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    X = synth.gaussian(m, n + 1, seed=m + n).astype(dtype)
+    A = torch.from_numpy(np.ascontiguousarray(X[:, :n].T)).cuda().T
+    b = torch.from_numpy(np.ascontiguousarray(X[:, n])).cuda()
+    for _ in range(12):
+        x, rn, R, info = q.lstsq_qless(A, b, want_rext=True)
+        assert info.cpu().tolist() == [0, 0]
+        assert gram_error(R.cpu().numpy(), X) <= 1e-14 * (n + 1)
+        assert rn.item() == R[n, n].item()
