@@ -25,7 +25,8 @@ constexpr int kGramFlushTiles = 16;
 struct GramWs {
   int* flags;        // [0] range, [1] first-pass breakdown (TSQR call: Householder redo), [2] arrival
                     // counter pass 1, [3] pass 2, [4] where a bounded wait gave up, [5] the exact first
-                    // pass has written R: the later passes have nothing to do,
+                    // pass has written R: the later passes have nothing to do, [6], [7] columns with
+                    // light entries (exact pass, a bit each),
                     // [64 + c]: largest biased exponent of column c over all rows (tensor-core pass 1)
   double* keep;      // 3 n x n blocks carried from pass 1 to pass 2 (row-major, ld n)
   double* partials;  // one NC x NC partial Gram per CTA

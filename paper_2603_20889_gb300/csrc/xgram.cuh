@@ -108,7 +108,9 @@ struct XgSmem {
   static constexpr size_t kOffB = kOffRaw + 2 * kRaw;
   static constexpr size_t kOffScale = kOffB + 2 * kStageB;
   static constexpr size_t kOffColmax = kOffScale + 4 * NC;
-  static constexpr size_t kOffMisc = kOffColmax + 4 * NC;
+  static constexpr size_t kOffBal = kOffColmax + 4 * NC;  // per column: light entries less the others,
+  static constexpr size_t kOffLit = kOffBal + 4 * NC;     // whether a unit of eight rows was light
+  static constexpr size_t kOffMisc = kOffLit + 4 * NC;
   // barriers and the tensor-memory slot: the same place in every class, so that a grouped
   // launch sets them up once
   static constexpr size_t kOffBar = 231424;
@@ -691,6 +693,36 @@ QL_DEV bool svqb_full_rank(const double* R, int n, double tol, float* sums) {
   return bound <= 0.0625;
 }
 
+// Whether the fixed point has lost rows that R depends on.  An entry is held to 2^-54 to 2^-53 of
+// the largest entry that its CTA has met in the column, not to 48 bits of its own as in the
+// Householder tiles and the SIMT Gram passes.  That matters where a few heavy rows (weighted or
+// constraint rows of a least-squares problem) stand above light ones and do not determine every
+// column: then R_kk, made of light rows, is small against the column's largest entry, and its
+// error of about 2^-56 of that entry is not (m = 2^14, n = 3, first row 2^30 times the others: R was
+// 3e-11 off, the Householder tiles 2e-15).  So: column k has light entries (kLightBits below its
+// scale in a CTA's last two tiles, for eight rows together or for most of the rows), and R_kk is below four times its
+// largest entry.  Neither alone would do: Gaussian columns of any condition number show no light
+// units, and light rows beside a large R_kk change nothing.
+constexpr int kLightBits = 8;
+// E: largest exponent of column k, mask: the word of flags[6], [7] with its bit.
+QL_DEV double light_floor(int E, int mask, int k) {  // R_kk below it: lost (0: column k has no light entries)
+  return E > 0 && ((mask >> (k & 31)) & 1) ? __longlong_as_double((long long)(E + 2) << 52) : 0.0;
+}
+
+// One unit of a column: with bal, its nonzero entries below the light limit count 1 and the others
+// -1; a unit that is light in all eight rows sets *lit.
+template <typename S>
+QL_DEV void count_light(const Rows8<S>& v, int limit, int* bal, int* lit) {
+  int below = 0, above = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const unsigned ax = v.hw[j] & 0x7fffffffu;
+    if (ax) ++(Rows8<S>::exponent(ax) < limit ? below : above);
+  }
+  if (bal && below != above) atomicAdd(bal, below - above);
+  if (below == 8) *lit = 1;
+}
+
 // Range verdict, election of the last CTA and, in it, R from the fixed-point Cholesky.  The
 // Gram methods end here as well when their further passes could not change R: with C exact
 // and factored to 2^-90, Y = X R1^{-1} is orthonormal to working precision and R2 the identity.
@@ -698,7 +730,9 @@ QL_DEV bool svqb_full_rank(const double* R, int n, double tol, float* sums) {
 // range is left to its passes: Cholesky-QR2 from pivots of 2^-46 (where an FP64 Cholesky of C
 // may break down), shifted Cholesky-QR3 from 2^-66, SVQB2 when an eigenvalue could be
 // truncated or Z is wanted; a zero column breaks down there.  A TSQR call whose pivots fall below
-// 2^-80 is redone by the Householder launch (flags[1]).
+// 2^-80 is redone by the Householder launch (flags[1]), as is one that has lost light rows; so are
+// Gram calls of up to 8 columns by their passes (of 48-bit entries; those of 9 columns and more hold
+// X in fixed point themselves).
 template <int NC, int T, typename S>
 QL_DEV void xg_finish(const GramArgs<S>& a, unsigned char* smem, const int* colmax, int* misc, int k) {
   if (!gram_elect<S, ArithDF>(a, colmax, misc, k)) return;
@@ -714,6 +748,8 @@ QL_DEV void xg_finish(const GramArgs<S>& a, unsigned char* smem, const int* colm
   int* sflag = reinterpret_cast<int*>(vec + 2 * LE);
   unsigned char* scratch = smem + ((NC + 3) * LE * 8 + 255) / 256 * 256;
   const int min_bits = tsqr ? 80 : (a.method == QL_SCHOLQR3 ? 66 : 46);
+  const bool check_light = tid < n && (tsqr || NC <= 8);
+  const int E = check_light ? __ldcg(&a.w.flags[64 + tid]) : 0, mask = check_light ? __ldcg(&a.w.flags[6 + (tid >> 5)]) : 0;
   bool done = false;
   if (a.method != QL_SVQB2 || !a.Z) {
     done = xg_cholesky<NC, T>(a.w.sacc, n, scratch, Rs, min_bits, tsqr) == 0;
@@ -721,7 +757,8 @@ QL_DEV void xg_finish(const GramArgs<S>& a, unsigned char* smem, const int* colm
       done = svqb_full_rank<NC, T>(Rs, n, a.rank_tol > 0.0 ? a.rank_tol : (double)n * 2.220446049250313e-16,
                                    reinterpret_cast<float*>(sflag));
   }
-  __syncthreads();  // the scratch is reused
+  // (the barrier: the scratch is reused)
+  if (__syncthreads_or(done && check_light && fabs(Rs[tid * LE + tid]) < light_floor(E, mask, tid))) done = false;
   if (done) {
     if (!tsqr && tid == 0) a.w.flags[5] = 1;
     if (a.epilogue == kEpiR)
@@ -766,6 +803,8 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
   unsigned char* rhs0 = smem + Sm::kOffB;
   int* scale = reinterpret_cast<int*>(smem + Sm::kOffScale);
   int* colmax = reinterpret_cast<int*>(smem + Sm::kOffColmax);
+  int* bal = reinterpret_cast<int*>(smem + Sm::kOffBal);
+  int* lit = reinterpret_cast<int*>(smem + Sm::kOffLit);
   int* misc = reinterpret_cast<int*>(smem + Sm::kOffMisc);
   uint64_t* mbar = reinterpret_cast<uint64_t*>(smem + Sm::kOffBar);  // [2] MMAs done, per digit buffer
   uint64_t* lbar = mbar + 2;                                          // [2] tile landed, per raw stage
@@ -781,6 +820,8 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
   for (int i = tid; i < NC; i += T) {
     colmax[i] = 0;
     scale[i] = 0;
+    bal[i] = 0;
+    lit[i] = 0;
   }
   if (tid == 0) *fail = 0;
   if (tid == 0) *req = 0;
@@ -1132,9 +1173,15 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
       have = freed = voted = cut = false;
       i += 2;
     }
+    // Light data (see light_floor) is looked for in each group's last tile, which v still holds,
+    // against the final scales: all units, the single entries of a column's first 32 rows.  (In the
+    // loop, where it holds registers, the look took 2 to 4 %, in sampled tiles as well.)
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
-      if (live[u] && arun[u] > 0) atomicMax(&colmax[cu[u]], Rows8<S>::exponent(arun[u]));
+    for (int u = 0; u < 2; ++u) {
+      if (!live[u]) continue;
+      if (arun[u] > 0) atomicMax(&colmax[cu[u]], Rows8<S>::exponent(arun[u]));
+      if (i > g) count_light(v[u], scale[cu[u]] - kLightBits, r0[u] % KV < 32 ? bal + cu[u] : nullptr, lit + cu[u]);
+    }
   }
   // every thread carries the same phase counts to the next work item
   bars.mpar ^= (uint32_t)(((nt + 1) >> 1) & 1) | (uint32_t)((nt >> 1) & 1) << 1;
@@ -1150,8 +1197,11 @@ QL_DEV void xgram_body(GramArgs<S> a, int bid, int k, uint32_t tbase, PipeBars& 
       atomicOr(&a.w.flags[a.method == QL_TSQR ? 1 : 0], 2);
     }
   }
-  for (int cc = tid; cc < n; cc += T)  // column exponents of the whole matrix, for the later passes
+  for (int cc = tid; cc < n; cc += T) {  // column exponents of the whole matrix, for the later passes
     if (colmax[cc] > 0) atomicMax(&a.w.flags[64 + cc], colmax[cc]);
+    if (lit[cc] || bal[cc] >= 4)  // four: a ragged tile may hold few rows of a column
+      atomicOr(&a.w.flags[6 + (cc >> 5)], 1 << (cc & 31));
+  }
   xg_finish<NC, T, S>(a, smem, colmax, misc, k);
 }
 

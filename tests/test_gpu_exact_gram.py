@@ -194,3 +194,65 @@ def test_right_hand_side_rows_stay_with_their_rows(n, m, dtype):
         assert info.cpu().tolist() == [0, 0]
         assert gram_error(R.cpu().numpy(), X) <= 1e-14 * (n + 1)
         assert rn.item() == R[n, n].item()
+
+
+def r_of_integers(X):
+    """R of X with integer entries: the Gram matrix in integers, Cholesky in 400-bit fixed point."""
+    from math import isqrt
+
+    n, bits = X.shape[1], 400
+    cols = [[int(v) for v in X[:, j].tolist()] for j in range(n)]
+    S = [[sum(a * b for a, b in zip(cols[i], cols[j])) << bits if j >= i else 0 for j in range(n)] for i in range(n)]
+    R = np.zeros((n, n))
+    for k in range(n):
+        r = [isqrt(S[k][k] << bits)] * (k + 1) + [0] * (n - k - 1)
+        for j in range(k + 1, n):
+            r[j] = (S[k][j] << bits) // r[k]
+        for i in range(k + 1, n):
+            for j in range(i, n):
+                S[i][j] -= r[i] * r[j] >> bits
+        R[k, k:] = [v / (1 << bits) for v in r[k:]]
+    return R
+
+
+def row_error(R, ref):
+    return (np.abs(R - ref).max(axis=1) / np.abs(ref).max(axis=1)).max()
+
+
+def heavy_rows(m, n, where, log2w):
+    """Rows of N(0,1) (integers up to 2^53) under a few rows 2^log2w times as large."""
+    X = np.rint(np.random.default_rng(m + n).standard_normal((m, n)) * 2.0 ** 50)
+    if where == "parallel":  # every fourth row along one direction, in half of the columns
+        X[::4] = 0.0
+        X[::4, : (n + 1) // 2] = np.rint(np.linspace(1.0, 2.0, (n + 1) // 2) * 2.0 ** 30) * 2.0 ** (20 + log2w)
+        return X
+    X[{"first": [0, 1], "last": [m - 1], "spread": list(range(5, m, m // 2))}[where]] *= 2.0 ** log2w
+    return X
+
+
+@pytest.mark.parametrize("where", ["first", "last", "spread", "parallel"])
+@pytest.mark.parametrize("m,n,log2w", [(16384, 3, 30), (16385, 3, 24), (16384, 8, 30), (4096, 14, 24), (70000, 14, 30)])
+def test_light_rows_under_heavy_ones(m, n, log2w, where):
+    """R row by row, against exact integers: no further off than the Householder tiles (the
+    workspace-free entry) by more than a factor of two, or than 2^-44 n: 48-bit entries, a few
+    roundings of that size per column.  Gram calls of up to 8 columns: 2^-44 n."""
+    import ctypes
+
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    X = heavy_rows(m, n, where, log2w) * 2.0 ** -50
+    ref = r_of_integers(X * 2.0 ** 50) * 2.0 ** -50
+    Xd = torch.from_numpy(np.ascontiguousarray(X.T)).cuda().T
+    Rh = torch.zeros((n, n), dtype=torch.float64, device="cuda").T
+    info = torch.zeros(2, dtype=torch.int32, device="cuda")
+    L = q.load_library()
+    assert L.ql_tsqr_qless_noalloc(m, n, Xd.data_ptr(), q.QL_F64, m, Rh.data_ptr(), n, info.data_ptr(),
+                                   ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)) == q.QL_OK
+    bound = max(n * 2.0 ** -44, 2.0 * row_error(Rh.cpu().numpy(), ref))
+    R, info = q.tsqr_qless(Xd)
+    assert info.cpu().tolist() == [0, 0] and row_error(R.cpu().numpy(), ref) <= bound
+    if n == 3 and where != "parallel":  # kappa of the others is beyond the Gram methods
+        R, info = q.cholqr2_qless(Xd)
+        assert info.cpu().tolist() == [0, 0] and row_error(R.cpu().numpy(), ref) <= n * 2.0 ** -44
