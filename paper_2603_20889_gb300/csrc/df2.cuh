@@ -9,6 +9,15 @@
 
 namespace ql {
 
+// One stored element and its biased double exponent (0 for zeros and subnormals); FP32 subnormals
+// keep their value, unlike in ArithDF::load, whose sums of squares could not hold them.
+QL_DEV df load_df(double x, int& E) { return df_split_double(x, E); }
+QL_DEV df load_df(float x, int& E) {
+  const int e = (__float_as_int(x) >> 23) & 0xff;
+  E = e == 0 ? 0 : e + 896;
+  return df{x, 0.0f};
+}
+
 using f2 = unsigned long long;  // two floats, the first in the low word
 struct df2 {
   f2 hi, lo;

@@ -52,12 +52,6 @@ struct ProjArgs {
 
 QL_DEV bool df_range_ok_dev(int E) { return E == 0 || (E >= kDfEminLimit && E <= kDfEmaxLimit); }
 
-QL_DEV df load_df(double x, int& E) { return df_split_double(x, E); }
-QL_DEV df load_df(float x, int& E) {
-  const int e = (__float_as_int(x) >> 23) & 0xff;
-  E = e == 0 ? 0 : e + 896;
-  return df{x, 0.0f};
-}
 
 // ---- C = Y^T V over the rows: one partial per CTA
 template <int KC, int NC, typename S>

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(QformSmem<NC>::T, QformSmem<NC>::kCtas) qform_
       for (int u = 0; u < 8; ++u) {
         if (c0 + u >= n) break;
         int E0, E1;
-        const df v0 = ArithDF::load(v[u].x, E0), v1 = ArithDF::load(v[u].y, E1);
+        const df v0 = load_df(v[u].x, E0), v1 = load_df(v[u].y, E1);
         if ((E0 != 0 && (E0 < kDfEminLimit || E0 > kDfEmaxLimit)) || (E1 != 0 && (E1 < kDfEminLimit || E1 > kDfEmaxLimit)))
           xbad = true;
         mine[(c0 + u) * T] = make_float4(v0.hi, v0.lo, v1.hi, v1.lo);
