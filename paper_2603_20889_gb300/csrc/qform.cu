@@ -36,19 +36,20 @@ struct QformArgs {
   int64_t ldq;
   int32_t* info;
   int64_t tiles;  // blocks of 64 rows
+  int spread;     // fewer blocks than warps: adjacent blocks go to different CTAs
   int pair;       // two adjacent rows of every column can be read and written in one access
 };
 
-template <int NC>
+template <int NC, typename S>
 struct QformSmem {
-  // one CTA per SM of as many warps as the shared memory holds (32 and 16 KB each) at 64 and 32
-  // columns, else three of eight warps
-  static constexpr int T = NC == 64 ? 160 : (NC == 32 ? 384 : 256);
+  // one CTA per SM of as many warps as the shared memory holds (32 and 16 KB each for FP64) at 64
+  // and 32 columns, else three of eight warps
+  static constexpr int T = NC == 64 ? (sizeof(S) == 8 ? 160 : 320) : (NC == 32 ? 384 : 256);
   static constexpr int kCtas = NC <= 16 ? 3 : 1;
   static constexpr int LDM = NC + 1;                         // odd stride: column walks of the inverse
   static constexpr size_t kM = 8 * (size_t)NC * LDM;         // FP64 M = R^{-1}
   static constexpr size_t kMd = 8 * (size_t)NC * NC;         // double-float M, [k][column pair]
-  static constexpr size_t kX = 16 * (size_t)NC * T;          // two rows per thread as double-float, [k][thread]
+  static constexpr size_t kX = 2 * sizeof(S) * (size_t)NC * T;  // two rows per thread, [k][thread]: (hi, lo) or FP32
   static constexpr size_t kOffMd = (kM + 15) / 16 * 16;
   static constexpr size_t kOffX = kOffMd + kMd;
   static constexpr size_t kOffMisc = kOffX + kX;
@@ -58,34 +59,30 @@ struct QformSmem {
 };
 
 template <int NC, typename S>
-__global__ void __launch_bounds__(QformSmem<NC>::T, QformSmem<NC>::kCtas) qform_kernel(QformArgs<S> a) {
-  using Sm = QformSmem<NC>;
+__global__ void __launch_bounds__(QformSmem<NC, S>::T, QformSmem<NC, S>::kCtas) qform_kernel(QformArgs<S> a) {
+  using Sm = QformSmem<NC, S>;
   constexpr int T = Sm::T, LDM = Sm::LDM;
   extern __shared__ __align__(16) unsigned char smem[];
   double* Mf = reinterpret_cast<double*>(smem);
   df2* Md = reinterpret_cast<df2*>(smem + Sm::kOffMd);
-  float4* xs = reinterpret_cast<float4*>(smem + Sm::kOffX);  // (hi, lo) of both rows
+  using X2 = typename std::conditional<sizeof(S) == 8, float4, float2>::type;  // both rows: (hi, lo) each, or FP32
+  X2* xs = reinterpret_cast<X2*>(smem + Sm::kOffX);
   int* misc = reinterpret_cast<int*>(smem + Sm::kOffMisc);
   const int tid = threadIdx.x, n = a.n;
 
   // ---- M = R^{-1} (FP64).  A zero diagonal entry (rank-deficient R) gives no inverse.
   double* Rs = reinterpret_cast<double*>(smem + Sm::kOffX);  // the tile area is free here
+  if (tid == 0) misc[0] = NC + 1;
+  __syncthreads();
   for (int e = tid; e < n * n; e += T) {
     const int i = e % n, j = e / n;
-    Rs[i * LDM + j] = i <= j ? __ldcg(a.R + (int64_t)j * a.ldr + i) : 0.0;
-  }
-  if (tid == 0) {
-    int zi = 0;
-    for (int i = 0; i < n; ++i)
-      if (!(__ldcg(a.R + (int64_t)i * a.ldr + i) != 0.0)) {
-        zi = i + 1;
-        break;
-      }
-    misc[0] = zi;
+    const double r = i <= j ? __ldcg(a.R + (int64_t)j * a.ldr + i) : 0.0;
+    Rs[i * LDM + j] = r;
+    if (i == j && !(r != 0.0)) atomicMin(&misc[0], i + 1);
   }
   __syncthreads();
   const int zi = misc[0];
-  if (zi) {  // Q would not be finite: NaN columns from the first zero pivot on, and the status
+  if (zi <= n) {  // Q would not be finite: NaN columns from the first zero pivot on, and the status
     const int64_t k = gridDim.x;
     const int64_t r0 = a.tiles * blockIdx.x / k * 64, r1 = min(a.m, a.tiles * (blockIdx.x + 1) / k * 64);
     for (int j = 0; j < n; ++j)
@@ -123,9 +120,11 @@ __global__ void __launch_bounds__(QformSmem<NC>::T, QformSmem<NC>::kCtas) qform_
   // ---- row blocks of 64 rows (tiles), one warp each
   const int lane = tid & 31;
   const int64_t nw = (int64_t)gridDim.x * (T / 32);
-  float4* mine = xs + tid;  // column k of this thread's rows at mine[k T]
+  X2* mine = xs + tid;  // column k of this thread's rows at mine[k T]
   using S2 = typename std::conditional<sizeof(S) == 8, double2, float2>::type;
-  for (int64_t t = (int64_t)blockIdx.x * (T / 32) + (tid >> 5); t < a.tiles; t += nw) {
+  const int warp = tid >> 5;
+  for (int64_t t = a.spread ? blockIdx.x + (int64_t)warp * gridDim.x : (int64_t)blockIdx.x * (T / 32) + warp; t < a.tiles;
+       t += nw) {
     const int64_t row = t * 64 + 2 * lane;
     const bool live0 = row < a.m, live1 = row + 1 < a.m;
     const bool whole = a.pair && t * 64 + 64 <= a.m;  // uniform in the warp
@@ -151,7 +150,10 @@ __global__ void __launch_bounds__(QformSmem<NC>::T, QformSmem<NC>::kCtas) qform_
         const df v0 = load_df(v[u].x, E0), v1 = load_df(v[u].y, E1);
         if ((E0 != 0 && (E0 < kDfEminLimit || E0 > kDfEmaxLimit)) || (E1 != 0 && (E1 < kDfEminLimit || E1 > kDfEmaxLimit)))
           xbad = true;
-        mine[(c0 + u) * T] = make_float4(v0.hi, v0.lo, v1.hi, v1.lo);
+        if constexpr (sizeof(S) == 8)
+          mine[(c0 + u) * T] = make_float4(v0.hi, v0.lo, v1.hi, v1.lo);
+        else
+          mine[(c0 + u) * T] = make_float2(v0.hi, v1.hi);
       }
     }
     const bool f64 = __any_sync(0xffffffffu, xbad) || m_f64;
@@ -166,9 +168,15 @@ __global__ void __launch_bounds__(QformSmem<NC>::T, QformSmem<NC>::kCtas) qform_
         const int kend = min(n, jb + 8);  // M is upper triangular: rows past column jb + 7 are zero
 #pragma unroll (NC <= 16 ? 1 : 2)
         for (int kk = 0; kk < kend; ++kk) {
-          const float4 x = mine[kk * T];
-          const df2n x0 = df2_factor(df2{f2_make(x.x, x.x), f2_make(x.y, x.y)});
-          const df2n x1 = df2_factor(df2{f2_make(x.z, x.z), f2_make(x.w, x.w)});
+          const X2 x = mine[kk * T];
+          df2n x0, x1;
+          if constexpr (sizeof(S) == 8) {
+            x0 = df2_factor(df2{f2_make(x.x, x.x), f2_make(x.y, x.y)});
+            x1 = df2_factor(df2{f2_make(x.z, x.z), f2_make(x.w, x.w)});
+          } else {
+            x0 = df2_factor(df2{f2_make(x.x, x.x), 0});
+            x1 = df2_factor(df2{f2_make(x.y, x.y), 0});
+          }
           const df2* mrow = Md + kk * (NC / 2) + jb / 2;
 #pragma unroll
           for (int jj = 0; jj < 4; ++jj) {
@@ -226,8 +234,8 @@ __global__ void __launch_bounds__(QformSmem<NC>::T, QformSmem<NC>::kCtas) qform_
 }
 
 template <int NC, typename S>
-static ql_status qform_launch_one(const QformArgs<S>& a, cudaStream_t stream) {
-  using Sm = QformSmem<NC>;
+static ql_status qform_launch_one(QformArgs<S> a, cudaStream_t stream) {
+  using Sm = QformSmem<NC, S>;
   auto kern = qform_kernel<NC, S>;
   static bool ready = false;
   static std::mutex mu;
@@ -241,9 +249,15 @@ static ql_status qform_launch_one(const QformArgs<S>& a, cudaStream_t stream) {
   }
   int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, Sm::T, Sm::kBytes) != cudaSuccess) return QL_ERR_CUDA;
-  int64_t g = (int64_t)device_sm_count() * (occ < 1 ? 1 : occ);
-  const int64_t need = (a.tiles + Sm::T / 32 - 1) / (Sm::T / 32);
-  if (g > need) g = need;
+  // A block of rows costs its SM's FP64 pipe 3 n conversions each way per row, so with fewer blocks
+  // than warps they are spread over the SMs, a warp or a few in each CTA, instead of filling the
+  // warps of a few CTAs
+  // (and, while one CTA per SM has the warps, one copy of R^{-1} is formed per SM)
+  const int64_t sms = device_sm_count();
+  int64_t g = sms * (occ < 1 ? 1 : occ);
+  a.spread = a.tiles < g * (Sm::T / 32) ? 1 : 0;
+  if (a.tiles <= sms * (Sm::T / 32)) g = sms;
+  if (g > a.tiles) g = a.tiles;
   if (g < 1) g = 1;
   count_launch();
   kern<<<(int)g, Sm::T, Sm::kBytes, stream>>>(a);
@@ -298,9 +312,9 @@ extern "C" ql_status ql_q_from_r(int64_t m, int64_t n, const void* X, ql_dtype d
     return QL_ERR_ALIGN;
   cudaStream_t st = (cudaStream_t)stream;
   if (dtype == QL_F64) {
-    QformArgs<double> a{m, (int)n, static_cast<const double*>(X), ldx, R, ldr, static_cast<double*>(Q), ldq, info, 0, 0};
+    QformArgs<double> a{m, (int)n, static_cast<const double*>(X), ldx, R, ldr, static_cast<double*>(Q), ldq, info, 0, 0, 0};
     return qform_dispatch(a, st);
   }
-  QformArgs<float> a{m, (int)n, static_cast<const float*>(X), ldx, R, ldr, static_cast<float*>(Q), ldq, info, 0, 0};
+  QformArgs<float> a{m, (int)n, static_cast<const float*>(X), ldx, R, ldr, static_cast<float*>(Q), ldq, info, 0, 0, 0};
   return qform_dispatch(a, st);
 }

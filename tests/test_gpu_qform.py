@@ -30,3 +30,36 @@ def test_fp32_subnormals_keep_their_value(m, n, ld):
     Q, info = q.q_from_r(Xd, torch.eye(n, dtype=torch.float64, device="cuda").T)
     assert info.cpu().tolist() == [0, 0]
     assert np.array_equal(Q.cpu().numpy().view(np.int32), X.view(np.int32))
+
+
+@pytest.mark.parametrize("n", [1, 8, 16, 33, 64])
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_few_rows_spread_over_the_sms(n, dtype):
+    """Row counts on both sides of a block and of a warp per CTA.  Entries and products hold 48 bits
+    (FP32 results 24), so |Q - X M| <= (n 2^-44 + u) |X| |M| with M = R^-1 in FP64."""
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    rng = np.random.default_rng(n)
+    R = np.triu(rng.standard_normal((n, n)) / n) + 2.0 * np.eye(n)
+    M = np.linalg.inv(R)
+    u = 2.0 ** -24 if dtype == np.float32 else 2.0 ** -53
+    for m, ld in ((1, 1), (63, 64), (65, 65), (1000, 1000), (9729, 9731), (30002, 30002)):
+        X = rng.standard_normal((m, n)).astype(dtype)
+        Q, info = q.q_from_r(col_major(X, ld), torch.from_numpy(np.ascontiguousarray(R.T)).cuda().T)
+        assert info.cpu().tolist() == [0, 0]
+        X = X.astype(np.float64)
+        assert np.all(np.abs(Q.cpu().numpy() - X @ M) <= (n * 2.0 ** -44 + u) * (np.abs(X) @ np.abs(M))), m
+
+
+@pytest.mark.parametrize("n,bad", [(1, 1), (8, 8), (40, 17)])
+def test_first_zero_pivot_is_reported(n, bad):
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    R = np.eye(n)
+    R[bad - 1:, bad - 1:] = 0.0
+    Q, info = q.q_from_r(col_major(np.ones((200, n)), 200), torch.from_numpy(np.ascontiguousarray(R.T)).cuda().T)
+    assert info.cpu().tolist() == [q.QL_ERR_NOT_SPD, bad] and bool(torch.isnan(Q).all())
