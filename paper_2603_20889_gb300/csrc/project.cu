@@ -48,6 +48,7 @@ struct ProjArgs {
   int pass;
   ProjWs w;
   int64_t tiles;
+  int spread;  // update: fewer blocks than warps, adjacent blocks go to different CTAs
 };
 
 QL_DEV bool df_range_ok_dev(int E) { return E == 0 || (E >= kDfEminLimit && E <= kDfEmaxLimit); }
@@ -65,6 +66,8 @@ __global__ void __launch_bounds__(kProjT, 2) cross_kernel(ProjArgs<S> a) {
   df2* Vs = Ys + KC * (B / 2);             // [NC][B / 2]
   double* red = reinterpret_cast<double*>(smem);  // [SL][KC][NC] at the end
   const int tid = threadIdx.x, k = a.k, n = a.n;
+  pdl_release();
+  pdl_wait();
   const int blk = tid / SL, slice = tid % SL;
   const bool active = blk < NBLK;
   const int bi = active ? (blk / (NC / 4)) * 4 : 0, bj = active ? (blk % (NC / 4)) * 4 : 0;
@@ -156,6 +159,8 @@ __global__ void __launch_bounds__(kProjT, 2) cross_kernel(ProjArgs<S> a) {
 constexpr int kReduceT = 64;
 template <typename S>
 __global__ void __launch_bounds__(kReduceT) cross_reduce_kernel(ProjArgs<S> a, int kc, int nc, int nb) {
+  pdl_release();
+  pdl_wait();
   const int e = blockIdx.x * kReduceT + threadIdx.x, i = e / nc, j = e % nc;
   if (e >= kc * nc || i >= a.k || j >= a.n) return;
   const double* p = a.w.partials + e;
@@ -181,7 +186,9 @@ __global__ void __launch_bounds__(update_threads<KC>(), 1) update_kernel(ProjArg
   extern __shared__ __align__(16) unsigned char smem[];
   df2* Cd = reinterpret_cast<df2*>(smem);                                        // [KC][NC / 2] column pairs
   float4* mine = reinterpret_cast<float4*>(Cd + KC * NC / 2) + threadIdx.x;     // column i of this thread's rows at mine[i T]
-  const int tid = threadIdx.x, lane = tid & 31, k = a.k, n = a.n;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = a.k, n = a.n;
+  pdl_release();
+  pdl_wait();
   bool cbad = false;
   for (int e = tid; e < KC * NC / 2; e += T) {
     const int i = e / (NC / 2), j0 = 2 * (e % (NC / 2));
@@ -202,7 +209,8 @@ __global__ void __launch_bounds__(update_threads<KC>(), 1) update_kernel(ProjArg
     a.W[j * a.ldw + row] = (S)s;
   };
   const int64_t nw = (int64_t)gridDim.x * (T / 32);
-  for (int64_t t = (int64_t)blockIdx.x * (T / 32) + (tid >> 5); t < a.tiles; t += nw) {
+  for (int64_t t = a.spread ? blockIdx.x + (int64_t)warp * gridDim.x : (int64_t)blockIdx.x * (T / 32) + warp; t < a.tiles;
+       t += nw) {
     const int64_t row = t * 64 + 2 * lane;
     const bool live0 = row < a.m, live1 = row + 1 < a.m;
     bool bad = false;
@@ -327,8 +335,8 @@ static ql_status proj_run(ProjArgs<S> a, cudaStream_t st) {
   const int64_t ctiles = (a.m + kProjB - 1) / kProjB, utiles = (a.m + 63) / 64;
   int64_t gc = (int64_t)device_sm_count() * kCrossCtasPerSm, gu = (int64_t)device_sm_count() * (occ < 1 ? 1 : occ);
   if (gc > ctiles) gc = ctiles;
-  const int64_t uneed = (utiles + UT / 32 - 1) / (UT / 32);
-  if (gu > uneed) gu = uneed;
+  a.spread = utiles < gu * (UT / 32) ? 1 : 0;  // as in qform.cu: the conversions' FP64 pipes
+  if (gu > utiles) gu = utiles;
   if (gc < 1) gc = 1;
   if (gu < 1) gu = 1;
   const S* X = a.V;
@@ -344,15 +352,21 @@ static ql_status proj_run(ProjArgs<S> a, cudaStream_t st) {
     }
     a.tiles = ctiles;
     count_launch();
-    ck<<<(int)gc, kProjT, Sm::kCross, st>>>(a);
-    if (cudaPeekAtLastError() != cudaSuccess) return QL_ERR_CUDA;
+    // The first kernel is an ordinary launch (its inputs are the caller's); the others start while
+    // their predecessor runs and wait for its end before they touch memory.
+    if (pass == 1) {
+      ck<<<(int)gc, kProjT, Sm::kCross, st>>>(a);
+      if (cudaPeekAtLastError() != cudaSuccess) return QL_ERR_CUDA;
+    } else if (launch_dependent(ck, (int)gc, kProjT, Sm::kCross, st, a) != cudaSuccess) {
+      return QL_ERR_CUDA;
+    }
     count_launch();
-    cross_reduce_kernel<S><<<(KC * NC + kReduceT - 1) / kReduceT, kReduceT, 0, st>>>(a, KC, NC, (int)gc);
-    if (cudaPeekAtLastError() != cudaSuccess) return QL_ERR_CUDA;
+    if (launch_dependent(cross_reduce_kernel<S>, (KC * NC + kReduceT - 1) / kReduceT, kReduceT, 0, st, a, KC, NC, (int)gc) !=
+        cudaSuccess)
+      return QL_ERR_CUDA;
     a.tiles = utiles;
     count_launch();
-    uk<<<(int)gu, UT, Sm::kUpdate, st>>>(a);
-    if (cudaPeekAtLastError() != cudaSuccess) return QL_ERR_CUDA;
+    if (launch_dependent(uk, (int)gu, UT, Sm::kUpdate, st, a) != cudaSuccess) return QL_ERR_CUDA;
   }
   return QL_OK;
 }
@@ -397,11 +411,11 @@ ql_status ql_project_out(int64_t m, int64_t k, const void* Y, int64_t ldy, int64
   w.partials = w.cpass + (size_t)kMaxN * kMaxN;
   if (dtype == QL_F64) {
     ProjArgs<double> a{m, (int)k, (int)n, static_cast<const double*>(Y), ldy, static_cast<const double*>(X), ldx,
-                       static_cast<double*>(W), ldw, C, ldc, 1, w, 0};
+                       static_cast<double*>(W), ldw, C, ldc, 1, w, 0, 0};
     return proj_dispatch(a, st);
   }
   ProjArgs<float> a{m, (int)k, (int)n, static_cast<const float*>(Y), ldy, static_cast<const float*>(X), ldx,
-                    static_cast<float*>(W), ldw, C, ldc, 1, w, 0};
+                    static_cast<float*>(W), ldw, C, ldc, 1, w, 0, 0};
   return proj_dispatch(a, st);
 }
 

@@ -63,3 +63,32 @@ def test_first_zero_pivot_is_reported(n, bad):
     R[bad - 1:, bad - 1:] = 0.0
     Q, info = q.q_from_r(col_major(np.ones((200, n)), 200), torch.from_numpy(np.ascontiguousarray(R.T)).cuda().T)
     assert info.cpu().tolist() == [q.QL_ERR_NOT_SPD, bad] and bool(torch.isnan(Q).all())
+
+
+@pytest.mark.parametrize("k,n", [(1, 1), (8, 9), (64, 3), (33, 64)])
+@pytest.mark.parametrize("dtype", [np.float64, np.float32])
+def test_projection_of_few_rows(k, n, dtype):
+    """Row counts on both sides of the tiles, out of place and in place.  W and C to 48-bit products
+    and the storage's rounding: |C - Y^T X| and |W - (X - Y Y^T X)| <= 8 k (m 2^-47 + u) max|X|."""
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    rng = np.random.default_rng(k + n)
+    u = 2.0 ** -24 if dtype == np.float32 else 2.0 ** -53
+    for m, ld in ((k, k), (65, 65), (129, 131), (1000, 1000), (9729, 9730)):
+        if m < k:
+            continue
+        Y = np.linalg.qr(rng.standard_normal((m, k)))[0].astype(dtype)
+        X = rng.standard_normal((m, n)).astype(dtype)
+        Yd, Xd = col_major(Y, ld), col_major(X, ld)
+        W, C = q.project_out(Yd, Xd)
+        Wi, Ci = q.project_out(Yd, Xd, W=Xd)
+        assert torch.equal(W, Wi) and torch.equal(C, Ci)
+        Y, X = Y.astype(np.float64), X.astype(np.float64)
+        C0 = Y.T @ X
+        W0 = X - Y @ C0
+        C1 = Y.T @ W0  # Y is orthonormal to its storage's rounding only
+        tol = 8 * k * (m * 2.0 ** -47 + u) * np.abs(X).max()
+        assert np.abs(C.cpu().numpy() - (C0 + C1)).max() <= tol, m
+        assert np.abs(W.cpu().numpy() - (W0 - Y @ C1)).max() <= tol, m
