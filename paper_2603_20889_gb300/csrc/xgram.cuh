@@ -492,6 +492,8 @@ QL_DEV i128 fx_mul(i128 a, i128 b) {
 struct FxPivot {
   u64 c;
   long long eps;
+  u64 flo;  // f in units of 2^-kFx
+  long long fhi;
   int z;
   int ok;  // 1: usable; 0: zero column; -1: pivot too small
 };
@@ -501,7 +503,7 @@ QL_DEV int fx_half_lead(i128 d) {  // z with d 4^z in [1/4, 1)
   return (lead - (128 - kFx)) >> 1;
 }
 QL_DEV FxPivot fx_pivot(i128 d, bool zero_column, int min_bits) {
-  FxPivot pv{0, 0, 0, 0};
+  FxPivot pv{0, 0, 0, 0, 0, 0};
   if (zero_column) return pv;
   if (d < ((i128)1 << (kFx - min_bits))) {
     pv.ok = -1;
@@ -510,6 +512,8 @@ QL_DEV FxPivot fx_pivot(i128 d, bool zero_column, int min_bits) {
   pv.ok = 1;
   pv.z = fx_half_lead(d);
   const u128 f = (u128)d << (2 * pv.z);
+  pv.flo = (u64)f;
+  pv.fhi = (long long)(u64)(f >> 64);
   const u64 f64 = (u64)(f >> (kFx - 64));  // f 2^64
   const float y0 = __fdividef(1.0f, (float)(unsigned)(f64 >> 40) * 0x1p-24f);  // in [1, 4]
   const u64 c0 = (u64)(unsigned)(y0 * 0x1p21f) << 40;
@@ -528,6 +532,12 @@ QL_DEV i128 fx_div_pivot(i128 s, const FxPivot& pv) {
   // sh c, sh signed and c unsigned
   w += (i128)((u128)(u64)sh * pv.c) - (sh < 0 ? (i128)((u128)pv.c << 64) : (i128)0);
   return w + (i128)__mul64hi((long long)(w >> 61), pv.eps) * ((i128)1 << 23);
+}
+// w = s / f of fx_div_pivot with its residual divided once more: 2^-99 -> 2^-117.
+QL_DEV i128 fx_div_refine(i128 w, i128 s, const FxPivot& pv) {
+  const i128 f = (i128)(((u128)(u64)pv.fhi << 64) | pv.flo);
+  const long long r = (long long)((s >> 3) - fx_mul(f, w));  // units of 2^-122, below 2^-97
+  return w + (((i128)r * (i128)(u128)pv.c) >> 61);
 }
 // 1 / (2 sqrt(f)) for f in [1/4, 1): single precision, one Newton step in 64-bit fixed point
 // (2^-44), then one third-order step y (1 + e / 2 + 3 e^2 / 8), e = 1 - f y^2, in 128 bits.
@@ -551,11 +561,20 @@ QL_DEV i128 fx_half_rsqrt(i128 f) {
 // column stops it, as does a zero column unless zero_ok.  Returns 0, or the 1-based index of
 // the pivot that stopped it (to every thread).
 //
+// dependent: the second attempt of a TSQR call that a small pivot has stopped.  The divisions are
+// refined, which leaves Schur complements good to n 2^-117 (2^-99 otherwise), and a pivot below
+// kDependentBits, half of what the Householder tiles' 48 bits could tell from zero, is the zero that
+// they make of it: R_kk and its row vanish.  lstsq: a pivot of A between the limits (not the last
+// one, the squared residual norm) stops the attempt, since the tiles may answer such a call or
+// report it, depending on the order of the rows.
+//
 // Step k with pivot d = 2^-2z f keeps row k as s_j = S_kj 2^z and w_j = s_j / f, subtracts
 // s_i w_j from the trailing entries and leaves 1 / sqrt(f) to the end (R_kj = s_j / sqrt(f),
 // R_kk = 2^-z f / sqrt(f), all rows at once): the chain from one pivot to the next is a reciprocal and three multiplies.
+constexpr int kDependentBits = 96;
 template <int NC, int T>
-QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double* Rout, int min_bits, bool zero_ok) {
+QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double* Rout, int min_bits, bool zero_ok,
+                       bool dependent = false, bool lstsq = false) {
   constexpr int LE = NC + 1;
   u64* Slo = reinterpret_cast<u64*>(smem);
   long long* Shi = reinterpret_cast<long long*>(Slo + NC * LE);
@@ -592,7 +611,13 @@ QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double
   }
   __syncthreads();
   auto pivot = [&](int k, i128 d) {
-    FxPivot pv = fx_pivot(d, sj[k] < 0, min_bits);
+    int limit = min_bits;
+    bool zero = sj[k] < 0;
+    if (dependent) {
+      zero |= d < ((i128)1 << (kFx - kDependentBits));
+      if (!lstsq || k == n - 1) limit = kFx;
+    }
+    FxPivot pv = fx_pivot(d, zero, limit);
     if (pv.ok == 0 && !zero_ok) pv.ok = -1;
     piv[k & 1] = pv;
   };
@@ -605,7 +630,8 @@ QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double
       const i128 v = pv.ok ? get(k, j) << (j == k ? 2 * pv.z : pv.z) : (i128)0;  // S_kk becomes f
       put(k, j, v);
       if (j == k) zk[k] = pv.z;
-      const i128 w = j == k ? (i128)0 : fx_div_pivot(v, pv);
+      i128 w = j == k ? (i128)0 : fx_div_pivot(v, pv);
+      if (dependent && j != k && pv.ok) w = fx_div_refine(w, v, pv);
       Wlo[j] = (u64)(u128)w;
       Whi[j] = (long long)(w >> 64);
     }
@@ -632,7 +658,7 @@ QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double
     __syncthreads();
   }
   for (int k = tid; k < n; k += T) {  // 1 / (2 sqrt(f))
-    const i128 r = sj[k] < 0 ? (i128)0 : fx_half_rsqrt(get(k, k));
+    const i128 f = get(k, k), r = f == 0 ? (i128)0 : fx_half_rsqrt(f);
     Wlo[k] = (u64)(u128)r;
     Whi[k] = (long long)(r >> 64);
   }
@@ -730,7 +756,8 @@ QL_DEV void count_light(const Rows8<S>& v, int limit, int* bal, int* lit) {
 // range is left to its passes: Cholesky-QR2 from pivots of 2^-46 (where an FP64 Cholesky of C
 // may break down), shifted Cholesky-QR3 from 2^-66, SVQB2 when an eigenvalue could be
 // truncated or Z is wanted; a zero column breaks down there.  A TSQR call whose pivots fall below
-// 2^-80 is redone by the Householder launch (flags[1]), as is one that has lost light rows; so are
+// 2^-80 is factored again as dependent (see xg_cholesky).  One that this does not answer is redone
+// by the Householder launch (flags[1]), as is one that has lost light rows; so are
 // Gram calls of up to 8 columns by their passes (of 48-bit entries; those of 9 columns and more hold
 // X in fixed point themselves).
 template <int NC, int T, typename S>
@@ -753,6 +780,10 @@ QL_DEV void xg_finish(const GramArgs<S>& a, unsigned char* smem, const int* colm
   bool done = false;
   if (a.method != QL_SVQB2 || !a.Z) {
     done = xg_cholesky<NC, T>(a.w.sacc, n, scratch, Rs, min_bits, tsqr) == 0;
+    if (tsqr && !done) {
+      __syncthreads();  // the scratch is written again
+      done = xg_cholesky<NC, T>(a.w.sacc, n, scratch, Rs, min_bits, true, true, a.epilogue == kEpiLstsq) == 0;
+    }
     if (done && a.method == QL_SVQB2)
       done = svqb_full_rank<NC, T>(Rs, n, a.rank_tol > 0.0 ? a.rank_tol : (double)n * 2.220446049250313e-16,
                                    reinterpret_cast<float*>(sflag));

@@ -256,3 +256,45 @@ def test_light_rows_under_heavy_ones(m, n, log2w, where):
     if n == 3 and where != "parallel":  # kappa of the others is beyond the Gram methods
         R, info = q.cholqr2_qless(Xd)
         assert info.cpu().tolist() == [0, 0] and row_error(R.cpu().numpy(), ref) <= n * 2.0 ** -44
+
+
+@pytest.mark.parametrize("m,n", [(20000, 3), (3001, 5), (5000, 8), (2000, 16), (1500, 33), (900, 64)])
+def test_numerically_dependent_columns(m, n):
+    """A pivot below 2^-96 of its column gives a zero row, as the Householder tiles give; one of about
+    2^-86 is resolved where X itself is exact in the fixed point (integers below 2^47: an error of
+    n 2^-117 in the Schur complement, 2^-25 of that pivot at 64 columns)."""
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    X = np.random.default_rng(n).integers(-7, 8, (m, n)).astype(np.float64)
+    k = n // 2 + 1
+    Xs = X.copy()
+    Xs[:, k] = 0.3 * X[:, 0] + X[:, k - 1] / 3.0  # rounded sums: dependent to 2^-53
+    R, info = tsqr(Xs)
+    assert info == [0, 0] and np.all(R[k, k:] == 0.0)
+    assert gram_error(R, Xs) <= 1e-13 * n
+    X[:, k] += X[:, 0] * 2.0 ** 43
+    ref = r_of_integers(X)
+    R, info = tsqr(X)
+    assert info == [0, 0] and row_error(R, ref) <= 2.0 ** -24
+    if n < 64:
+        A = torch.from_numpy(np.ascontiguousarray(Xs.T)).cuda().T
+        b = torch.from_numpy(np.random.default_rng(1).standard_normal(m)).cuda()
+        x, rn, _, info = q.lstsq_qless(A, b)
+        assert info.cpu().tolist() == [q.QL_ERR_NOT_SPD, k + 1] and bool(torch.isnan(x).all())
+
+
+@pytest.mark.parametrize("m,n", [(20000, 2), (3000, 7), (2000, 20), (1000, 63), (6, 6), (40, 40)])
+def test_consistent_least_squares(m, n):
+    """b = A 1 up to the rounding of its entries: x to kappa 2^-50, the residual norm to 2^-52 ||b||."""
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    A = synth.conditioned(m, n, 10.0, seed=n) if m > n else np.eye(n) + 0.25 * np.triu(np.ones((n, n))) / n
+    b = A @ np.ones(n)
+    x, rn, _, info = q.lstsq_qless(torch.from_numpy(np.ascontiguousarray(A.T)).cuda().T, torch.from_numpy(b).cuda())
+    assert info.cpu().tolist() == [0, 0]
+    assert np.abs(x.cpu().numpy() - 1.0).max() <= 100 * n * 2.0 ** -50
+    assert 0.0 <= rn.item() <= 4 * n * 2.0 ** -52 * np.linalg.norm(b)
