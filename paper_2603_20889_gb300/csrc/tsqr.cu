@@ -61,14 +61,22 @@ size_t tsqr_workspace_bytes(int n, bool householder) {
          tree_slots((int)leaves) * (size_t)n * n * sizeof(double);
 }
 
-// Whether the exact Gram pass (xgram.cuh) takes a TSQR call.  From 5 columns always (4099 x 5
-// 45 -> 35 us, everything larger gains more).  With 3 or 4 columns from 2^14 rows: m = 2^25,
-// n = 4 919 -> 382 us, 100000 x 4 61 -> 33 us, but 4099 x 3 27.7 -> 29.7 us, one Householder tile
-// per CTA and a one-level tree there.  One or two columns stay with the norm and the Householder
-// tiles: the 4-column class works for two columns that are not there (m = 2^25, n = 2 288 us
-// against 378).
+// Whether the exact Gram pass (xgram.cuh) takes a TSQR call.  Below the line one Householder tile
+// per CTA and a one-level tree are the shorter chain.  Measured, Householder and exact, us:
+//   R:             3 columns 2048 rows 22.7, 24;  4096 24.7, 24;  8192 27.1, 25;  16384 35, 25
+//                  4 columns 2048 rows 25.6, 25;  4096 28.3, 25;  16384 45, 25
+//                  5 columns  100 rows 28.8, 27;  2048 39, 28
+//   least squares: 3 columns 4096 rows 27, 30;    8192 32, 30;    16384 39, 30
+//                  4 columns 4096 rows 32, 31;    8192 35, 31
+//                  5 columns 1024 rows 30, 36;    2048 40, 34
+//                  6 columns 1024 rows 33, 38;    2048 44, 37;    9 columns 100 rows 48, 45
+// One or two columns stay with the norm and the Householder tiles: the 4-column class works for two
+// columns that are not there (m = 2^25, n = 2 288 us against 378).  With fewer rows than columns the
+// exact pass would factor twice (dependent columns), where a single tile is quick.
 static bool exact_route(const TsqrCall& c, ql_arith arith) {
-  return !c.householder && arith != QL_ARITH_F64 && tc_gram_enabled() && (c.n >= 5 || (c.n >= 3 && c.m >= (1 << 14)));
+  if (c.householder || arith == QL_ARITH_F64 || !tc_gram_enabled() || c.n < 3 || c.m < c.n) return false;
+  if (c.epilogue == kEpiR) return c.n >= 5 || c.m >= (1 << 12);
+  return c.n >= 7 || c.m >= (c.n >= 5 ? 1 << 11 : 1 << 13);
 }
 
 template <typename S>

@@ -298,3 +298,30 @@ def test_consistent_least_squares(m, n):
     assert info.cpu().tolist() == [0, 0]
     assert np.abs(x.cpu().numpy() - 1.0).max() <= 100 * n * 2.0 ** -50
     assert 0.0 <= rn.item() <= 4 * n * 2.0 ** -52 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("n,rows", [(3, 4096), (4, 4096), (5, 5), (40, 40)])
+def test_both_sides_of_the_routes_line(n, rows):
+    """One row below the line the Householder tiles answer, at the line the exact pass; with fewer
+    rows than columns the rows of R past the last one are zero."""
+    for m in (rows - 1, rows, rows + 1):
+        X = synth.gaussian(m, n, seed=m)
+        R, info = tsqr(X)
+        assert info == [0, 0] and gram_error(R, X) <= 1e-13 * n
+        assert np.all(R[m:] == 0.0)
+
+
+@pytest.mark.parametrize("n,rows", [(2, 8192), (3, 8192), (4, 2048), (5, 2048), (7, 8)])
+def test_both_sides_of_the_routes_line_least_squares(n, rows):
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    for m in (rows - 1, rows, rows + 1):
+        A, b, _ = synth.lstsq_case(m, n, 10.0, seed=m)
+        x_ref, rho_ref, _, _ = oracle.lstsq(A, b)
+        x, rn, _, info = q.lstsq_qless(torch.from_numpy(np.ascontiguousarray(A.T)).cuda().T, torch.from_numpy(b).cuda())
+        assert info.cpu().tolist() == [0, 0]
+        kappa = max(10.0, np.linalg.cond(A))
+        assert np.linalg.norm(x.cpu().numpy() - x_ref) <= oracle.tolerance(n, kappa) * kappa * np.linalg.norm(x_ref)
+        assert abs(rn.item() - rho_ref) <= oracle.tolerance(n, kappa) * np.linalg.norm(b)
