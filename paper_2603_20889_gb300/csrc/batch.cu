@@ -6,16 +6,18 @@
 // TSQR otherwise).  The Gram method covers n >= 9 (tensor-core kernels); narrower problems
 // always run TSQR.
 //
-// In double-float mode every problem, of either method, is a run of work items of ONE grouped
-// exact Gram launch (xgram_group.cu; chunks of row tiles, the problems by decreasing work).  A
+// In double-float mode the problems, of either method, are runs of work items of ONE grouped
+// exact Gram launch (xgram_group.cu; chunks of row tiles, the problems by decreasing work).  A batch
+// of TSQR problems of one or two columns or few rows only (tiles_are_quicker), and many rows of
+// single columns in a mixed one, run on the persistent Householder launch instead.  A
 // TSQR problem, or an automatically chosen Cholesky-QR2 one, that the exact route cannot answer
 // (a pivot below its limit, data outside the range) is redone by the batch's last launch with
 // Householder tiles; the host plan splits every problem into chunks for it as well (the leaves
 // of that problem's R-tree).  Cholesky-QR2 problems asked for by method_hint keep their second
 // passes (batch_gram.cu), which end at once unless a pivot fell below the method's limit.
 //
-// Stream order: the exact launch, the second Gram passes if there are any, then the gated
-// Householder launch: double-float for kRedoDF, FP64 for kRedoF64 (range, or an explicit
+// Stream order: the exact launch, the persistent Householder launch and the second Gram passes if
+// there are any, then the gated Householder launch: double-float for kRedoDF, FP64 for kRedoF64 (range, or an explicit
 // Cholesky-QR2 that left it).  In FP64 mode the persistent TSQR kernel takes every problem.
 #include <algorithm>
 #include <cstddef>
@@ -82,7 +84,7 @@ struct BatchHeader {
   int work_counter[3];  // [0] persistent TSQR launch, [1] gated launch, [2] exact launch
   int count;
   int64_t total_work;     // chunks of every problem (the gated FP64 launch)
-  int64_t total_work_df;  // chunks of the TSQR problems, which come first
+  int64_t total_work_df;  // chunks of the persistent launch's problems, which come first
   int gram_counter[2 * kMaxGramGroups];  // per group and pass
 };
 
@@ -179,6 +181,9 @@ __global__ void __launch_bounds__(kBatchT, 1)
   __shared__ int64_t s_work;
   __shared__ int s_item;
   constexpr bool gated = MODE == 2;
+  // the gated launch may start behind its predecessor's last CTAs; it reads nothing before their end
+  pdl_release();
+  if (gated) pdl_wait();
   if (gated && *(volatile int*)&flags[-1] == 0) return;  // nothing to redo
   const int64_t total = MODE == 1 ? hdr->total_work_df : hdr->total_work;
   for (;;) {
@@ -253,10 +258,10 @@ struct GramGroupPlan {
 };
 
 struct BatchPlan {
-  std::vector<BatchItem> items;        // TSQR plan of every problem, TSQR problems first
+  std::vector<BatchItem> items;        // TSQR plan of every problem, the persistent launch's first
   std::vector<int32_t> method;         // chosen method per problem, in the caller's order
   std::vector<GramGroupPlan> groups;   // Cholesky-QR2 problems by (column class, storage)
-  bool exact = false;                  // the exact launch takes every problem (its items below)
+  bool exact = false;                  // the exact launch takes the other problems
   std::vector<XgItem> xg;
   int64_t xg_total = 0;
   int xg_max_nc = 4;
@@ -283,6 +288,15 @@ static int choose_method(const ql_problem& pr, int ncols) {
   return (pr.kappa_hint > 0.0 && pr.kappa_hint <= 1e6 && ncols >= 24) ? QL_CHOLQR2 : QL_TSQR;
 }
 
+// Whether a TSQR problem of a batch is quicker on the persistent Householder launch than on the exact
+// one: one or two columns, and small problems, whose single chunk costs the exact launch its set-up
+// and a Cholesky.  Measured, Householder and exact, us: 64 problems of 4096 x 1 43, 64;
+// 100000 x 1 156, 212; 4096 x 4 49, 65; 100000 x 3 282, 247; 4096 x 8 73, 78; 1000 x 16 77, 79;
+// 256 of 300 x 8 94, 146; 300 x 16 134, 177; 300 x 32 630, 203.
+static bool tiles_are_quicker(int64_t m, int ncols) {
+  return ncols <= 2 || (ncols <= 4 && m < (1 << 14)) || (ncols <= 8 && m <= (1 << 12)) || (ncols <= 16 && m < (1 << 10));
+}
+
 // Build the plan; with `ws` non-null the Gram items' device pointers point into it.
 static bool make_plan(int32_t count, const ql_problem* probs, BatchPlan& P, unsigned char* ws = nullptr) {
   P = BatchPlan();
@@ -294,13 +308,26 @@ static bool make_plan(int32_t count, const ql_problem* probs, BatchPlan& P, unsi
     if (!pr.R || (pr.kind == 1 && (!pr.x || !pr.b)) || (pr.m > 0 && !pr.X)) return false;
     P.method[i] = choose_method(pr, (int)pr.n + (pr.kind == 1 ? 1 : 0));
   }
+  P.exact = current_arith() != QL_ARITH_F64 && tc_gram_enabled() && pipe_gram_enabled();
+  // The problems of the persistent Householder launch.  In double-float mode a batch whose problems
+  // are all quicker there runs on it alone; a mixed one has single columns of 2^21 rows together
+  // (some 20 us less than on the exact launch) on a launch of their own, else one launch for all.
+  std::vector<char> tiles_only(count);
+  bool all = true;
+  int64_t rows1 = 0;
+  for (int i = 0; i < count; ++i) {
+    const int nc = (int)probs[i].n + (probs[i].kind == 1 ? 1 : 0);
+    tiles_only[i] = P.method[i] == QL_TSQR && (!P.exact || tiles_are_quicker(probs[i].m, nc));
+    all = all && tiles_only[i];
+    if (tiles_only[i] && nc == 1) rows1 += probs[i].m;
+  }
+  if (P.exact && !all && rows1 < (1 << 21)) std::fill(tiles_only.begin(), tiles_only.end(), (char)0);
   std::vector<int> order(count);
   for (int i = 0; i < count; ++i) order[i] = i;
   auto work = [&](int i) { return (double)probs[i].m * probs[i].n * probs[i].n; };
-  // TSQR problems first (the double-float TSQR launch covers a prefix of the work list),
-  // each part by decreasing work
+  // the persistent launch covers a prefix of the work list, each part by decreasing work
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
-    const bool ta = P.method[a] == QL_TSQR, tb = P.method[b] == QL_TSQR;
+    const bool ta = tiles_only[a] != 0, tb = tiles_only[b] != 0;
     if (ta != tb) return ta;
     return work(a) > work(b);
   });
@@ -334,7 +361,7 @@ static bool make_plan(int32_t count, const ql_problem* probs, BatchPlan& P, unsi
     it.tiles_per_chunk = tpc;
     it.work_begin = wb;
     wb += it.chunks;
-    if (P.method[order[k]] == QL_TSQR) P.total_work_df = wb;
+    if (tiles_only[order[k]]) P.total_work_df = wb;
     it.slot_off = slots;
     slots += (int64_t)tree_slots(it.chunks) * it.n * it.n;
     it.cnt_off = cnts;
@@ -357,7 +384,6 @@ static bool make_plan(int32_t count, const ql_problem* probs, BatchPlan& P, unsi
   // Gram problems: flag blocks (cleared with the counters), then carried blocks, partials
   // and FP64 accumulator blocks, then the group item arrays
   P.off_gflags = off;
-  P.exact = current_arith() != QL_ARITH_F64 && tc_gram_enabled() && pipe_gram_enabled();
   auto explicit_gram = [&](int k) {
     return P.items[k].method == QL_CHOLQR2 && probs[order[k]].method_hint == QL_CHOLQR2;
   };
@@ -368,6 +394,7 @@ static bool make_plan(int32_t count, const ql_problem* probs, BatchPlan& P, unsi
   std::vector<size_t> flag_off(count, 0);
   if (P.exact) {
     for (int k = 0; k < count; ++k) {
+      if (tiles_only[order[k]]) continue;
       flag_off[k] = off;
       off += 512 + (sacc_bytes(xg_class_of(P.items[k].n)) + 255) / 256 * 256;
     }
@@ -459,9 +486,10 @@ static bool make_plan(int32_t count, const ql_problem* probs, BatchPlan& P, unsi
     };
     auto tile_cost = [&](int k) { return xg_class_of(P.items[k].n) == 64 ? 5 : 2; };
     int64_t cost = 0;
-    std::vector<int> by_cost(count);
+    std::vector<int> by_cost;
     for (int k = 0; k < count; ++k) {
-      by_cost[k] = k;
+      if (tiles_only[order[k]]) continue;
+      by_cost.push_back(k);
       cost += tiles_of(k) * tile_cost(k);
     }
     std::stable_sort(by_cost.begin(), by_cost.end(),
@@ -540,11 +568,16 @@ static ql_status launch_batch(unsigned char* ws, const BatchPlan& P, int count, 
   int grid = device_sm_count() * occ;
   if (P.total_work < grid) grid = (int)std::max<int64_t>(1, P.total_work);
   count_launch();
-  kern<<<grid, kBatchT, smem, stream>>>(reinterpret_cast<BatchHeader*>(ws),
-                                         reinterpret_cast<const BatchItem*>(ws + P.off_items), count,
-                                         reinterpret_cast<double*>(ws + P.off_slots),
-                                         reinterpret_cast<int*>(ws + P.off_counters),
-                                         reinterpret_cast<int*>(ws + P.off_flags) + 1);
+  BatchHeader* hdr = reinterpret_cast<BatchHeader*>(ws);
+  const BatchItem* items = reinterpret_cast<const BatchItem*>(ws + P.off_items);
+  double* slots = reinterpret_cast<double*>(ws + P.off_slots);
+  int* counters = reinterpret_cast<int*>(ws + P.off_counters);
+  int* flags = reinterpret_cast<int*>(ws + P.off_flags) + 1;
+  if (MODE == 2)
+    return launch_dependent(kern, grid, kBatchT, smem, stream, hdr, items, count, slots, counters, flags) == cudaSuccess
+               ? QL_OK
+               : QL_ERR_CUDA;
+  kern<<<grid, kBatchT, smem, stream>>>(hdr, items, count, slots, counters, flags);
   return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
@@ -675,12 +708,12 @@ ql_status ql_batch_launch(void* ws, void* stream) {
   };
   if (P.exact) {
     const int grid = (int)std::min<int64_t>(P.xg_total, device_sm_count());
-    s = xgram_group_launch(&hdr->work_counter[2], reinterpret_cast<const XgItem*>(w + P.off_xg), count, P.xg_total, grid,
-                           reinterpret_cast<double*>(w + P.off_acc), P.xg_max_nc, st);
-  } else {  // the comparison kernels: per-tile first Gram passes, Householder tiles
+    s = xgram_group_launch(&hdr->work_counter[2], reinterpret_cast<const XgItem*>(w + P.off_xg), (int)P.xg.size(), P.xg_total,
+                           grid, reinterpret_cast<double*>(w + P.off_acc), P.xg_max_nc, st);
+  } else {  // the comparison kernels: per-tile first Gram passes
     gram_pass(1);
-    if (s == QL_OK) s = launch_batch<1>(w, P, count, st);
   }
+  if (s == QL_OK && (P.total_work_df > 0 || !P.exact)) s = launch_batch<1>(w, P, count, st);
   if (s == QL_OK) gram_pass(2);
   return s == QL_OK ? launch_batch<2>(w, P, count, st) : s;  // flagged problems, any method
 }

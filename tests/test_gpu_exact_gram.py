@@ -325,3 +325,38 @@ def test_both_sides_of_the_routes_line_least_squares(n, rows):
         kappa = max(10.0, np.linalg.cond(A))
         assert np.linalg.norm(x.cpu().numpy() - x_ref) <= oracle.tolerance(n, kappa) * kappa * np.linalg.norm(x_ref)
         assert abs(rn.item() - rho_ref) <= oracle.tolerance(n, kappa) * np.linalg.norm(b)
+
+
+def test_batch_across_the_tiles_line():
+    """Both sides of the batch's line between Householder tiles and the exact launch, in one call
+    and with every problem on one side; least squares among them."""
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    small = [(3001, 1), (70000, 1), (50000, 2), (16383, 4), (4096, 8), (1023, 16), (5, 9), (300, 3), (0, 4)]
+    large = [(16384, 3), (4097, 8), (4097, 5), (1024, 16), (200, 17), (3000, 40)]
+    for shapes in (small, large, small + large, small + large + [(1 << 21, 1)]):
+        probs, keep = [], []
+        for k, (m, n) in enumerate(shapes):
+            X = synth.gaussian(max(m, 1), n, seed=k)[:m]
+            ls = k % 3 == 1 and m > n + 1
+            Xd = torch.from_numpy(np.ascontiguousarray(X.T)).cuda()
+            b = torch.from_numpy(synth.gaussian(max(m, 1), 1, seed=k + 50)[:, 0].copy()).cuda()
+            R = torch.zeros((n + ls, n + ls), dtype=torch.float64, device="cuda")
+            x = torch.zeros(n + 1, dtype=torch.float64, device="cuda")
+            info = torch.full((2,), -1, dtype=torch.int32, device="cuda")
+            keep.append((X, b, ls, Xd, R, x, info))
+            probs.append(q.Problem(m=m, n=n, ld=max(m, 1), X=Xd.data_ptr(), dtype=q.QL_F64, kind=int(ls),
+                                   b=b.data_ptr() if ls else None, R=R.data_ptr(), x=x.data_ptr() if ls else None,
+                                   info=info.data_ptr(), method_hint=q.QL_AUTO, kappa_hint=0.0))
+        q.batch_qless(probs)
+        torch.cuda.synchronize()
+        for X, b, ls, _, R, x, info in keep:
+            m, n = X.shape
+            full = np.column_stack([X, b.cpu().numpy()[:m]]) if ls else X
+            R = R.cpu().numpy().T
+            assert info.cpu().tolist() == [0, 0], (m, n)
+            assert gram_error(R, full) <= 1e-13 * (n + 1), (m, n)
+            if ls:
+                assert x[n].item() == R[n, n]
