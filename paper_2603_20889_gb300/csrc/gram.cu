@@ -133,7 +133,11 @@ ql_status gram_launch(const GramCall& c, ql_arith arith) {
   GramWs w;
   gram_layout(c.n, &w, c.ws);
   ql_status st;
-  if ((st = clear_async(w.flags, gram_head_bytes(c.n), c.stream))) return st;
+  if (c.n <= 2) {  // no exact pass, nothing for it to overlap with
+    if (cudaMemsetAsync(w.flags, 0, 512, c.stream) != cudaSuccess) return QL_ERR_CUDA;
+  } else if ((st = clear_async(w.flags, gram_head_bytes(c.n), c.stream))) {
+    return st;
+  }
   if (c.dtype == QL_F64) {
     if (arith == QL_ARITH_F64) return gram_dispatch<double, ArithF64>(c, w, 0);
     if ((st = gram_dispatch<double, ArithDF>(c, w, 0))) return st;

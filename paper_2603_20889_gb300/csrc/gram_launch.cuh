@@ -730,6 +730,12 @@ ql_status gram_stream_launch_one(const GramCall& c, const GramWs& w, int pass, i
   }
   a.mround = std::is_same<Ar, ArithDF>::value ? 1 : 0;
   count_launch();
+  if ((NC <= 2 || (c.method == QL_SVQB2 && c.Z)) && !gated) {
+    // both passes read X here: CTAs of the second that start beside the first's last ones cost more
+    // than the launch (m = 2^25, n = 1 157 us, 164 as a dependent launch)
+    kern<<<(int)g, Sh::T, Sm::kBytes, c.stream>>>(a);
+    return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
+  }
   return launch_dependent(kern, (int)g, Sh::T, Sm::kBytes, c.stream, a) == cudaSuccess ? QL_OK : QL_ERR_CUDA;
 }
 
@@ -2330,7 +2336,8 @@ ql_status gram_dispatch(const GramCall& c, const GramWs& w, int gated) {
     }
     if constexpr (NC <= 4) {  // narrow X: the streaming kernel (n = 8 would spill its 36 accumulators)
       ql_status st;
-      if (NC == 4 && std::is_same<Ar, ArithDF>::value && tc_gram_enabled())
+      // (SVQB2 with Z wanted needs its second pass anyway: the streaming first one is quicker)
+      if (NC == 4 && std::is_same<Ar, ArithDF>::value && tc_gram_enabled() && !(c.method == QL_SVQB2 && c.Z))
         st = xgram_pass1<S>(c, w);
       else
         st = gram_stream_launch_one<NC, S, Ar, kXNone>(c, w, 1, gated);
