@@ -1,14 +1,15 @@
 // Project autotuner: for an (m, n, dtype, kappa) class it times the candidate
 // configurations on the current GPU and records the fastest in a process-wide table that
 // the single-call entry points, ql_autotune_choose() and the batched form consult:
-//   * TSQR: CTAs per SM (1, 2, and 4 for n <= 4 -- it sets the R-tree leaves and the rows
+//   * Householder tiles (TSQR calls that the exact Gram pass does not take, and the workspace-free
+//     entry point, up to 16 columns, for those that it takes): CTAs per SM (1, 2, and 4 for n <= 4 -- it sets the R-tree leaves and the rows
 //     per CTA; a request above what registers and shared memory allow is clamped), the
 //     row-block height (for n > 8 three thread layouts of the tile kernel: 16 rows x 4
 //     columns per thread at 256 threads, 8 rows x 4 columns at 256 threads, 8 rows x 8
 //     columns at 128 threads, i.e. tiles of 256/128/128 rows at n = 64) and the R-tree
 //     arity (binary, or the wide default of narrow X);
-//   * Cholesky-QR2, when the condition hint allows it (kappa <= 1e6, where the Gram method
-//     stays within the accuracy bound).
+//   * Cholesky-QR2 against TSQR, when the condition hint allows it (kappa <= 1e6, where the Gram
+//     method stays within the accuracy bound) and the two are not the same exact pass anyway.
 // The table persists as a small JSON text file.
 #include <chrono>
 #include <cmath>
@@ -114,15 +115,21 @@ ql_status ql_autotune(int64_t m, int64_t n, ql_dtype dtype, double kappa_hint, v
   std::vector<Cand> cands;
   const int ctas_opts[3] = {1, 2, 4};
   const int nvar = (n > 8 && dtype == QL_F64) ? 3 : 1;
-  for (int ci = 0; ci < (n <= 4 ? 3 : 2); ++ci)
-    for (int v = 0; v < nvar; ++v)
-      for (int ar : {0, 2}) cands.push_back(Cand{QL_TSQR, ctas_opts[ci], v, ar});
-  if (kappa_hint <= 1e6 && n > 1) cands.push_back(Cand{QL_CHOLQR2, 0, 0, 0});
+  // on the exact route the tiles are timed by themselves, for the workspace-free entry point, and the
+  // call once; beyond that entry point's columns there is nothing to choose
+  const bool exact = tsqr_exact_route(m, (int)n);
+  if (!exact || n <= kNoAllocMaxN)
+    for (int ci = 0; ci < (n <= 4 ? 3 : 2); ++ci)
+      for (int v = 0; v < nvar; ++v)
+        for (int ar : {0, 2}) cands.push_back(Cand{QL_TSQR, ctas_opts[ci], v, ar});
+  if (exact) cands.push_back(Cand{QL_AUTO, 0, 0, 0});
+  if (!exact && kappa_hint <= 1e6 && n > 1) cands.push_back(Cand{QL_CHOLQR2, 0, 0, 0});
   TuneVal best{QL_TSQR, 0, 0, 0, 1e30};
   for (size_t ci = 0; ci < cands.size(); ++ci) {
     auto run = [&]() -> ql_status {
-      if (cands[ci].method == QL_TSQR) {
+      if (cands[ci].method != QL_CHOLQR2) {
         TsqrCall c;
+        c.householder = exact && cands[ci].method == QL_TSQR;
         c.m = m;
         c.n = (int)n;
         c.nA = (int)n;
@@ -155,7 +162,9 @@ ql_status ql_autotune(int64_t m, int64_t n, ql_dtype dtype, double kappa_hint, v
       cudaEventElapsedTime(&ms, e0, e1);
       if (ms < best_ms) best_ms = ms;
     }
-    if (best_ms < best.ms)
+    if (cands[ci].method == QL_AUTO)  // the call itself: the tiles' settings stay
+      best.ms = best_ms;
+    else if (best_ms < best.ms)
       best = TuneVal{cands[ci].method, cands[ci].ctas, cands[ci].variant, cands[ci].arity, best_ms};
   }
   cudaEventDestroy(e0);

@@ -47,6 +47,10 @@ size_t tsqr_workspace_bytes(int n, bool householder = false);
 size_t xgram_tsqr_bytes(int n);
 size_t xgram_tsqr_clear_bytes(int n);
 ql_status xgram_tsqr_launch(const TsqrCall& c, void* base);
+// Whether ql_tsqr_qless of m rows and n columns starts with that pass.
+bool tsqr_exact_route(int64_t m, int n);
+// Columns of the workspace-free entry point (tsqr_noalloc.cu), always on Householder tiles.
+constexpr int kNoAllocMaxN = 16;
 // Launch the double-float TSQR (or FP64 when arith == QL_ARITH_F64) and, after a
 // double-float launch, the gated FP64 fallback.
 ql_status tsqr_launch(const TsqrCall& c, ql_arith arith);

@@ -79,6 +79,13 @@ static bool exact_route(const TsqrCall& c, ql_arith arith) {
   return c.n >= 7 || c.m >= (c.n >= 5 ? 1 << 11 : 1 << 13);
 }
 
+bool tsqr_exact_route(int64_t m, int n) {
+  TsqrCall c;
+  c.m = m;
+  c.n = n;
+  return exact_route(c, current_arith());
+}
+
 template <typename S>
 static ql_status tsqr_launch_s(const TsqrCall& c, const TreeView& tv, bool exact, ql_arith arith) {
   if (arith == QL_ARITH_F64) return dispatch<S, ArithF64>(c, tv, 0);

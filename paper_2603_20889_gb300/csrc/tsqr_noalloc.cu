@@ -17,7 +17,6 @@ namespace ql {
 // Scratch capacity: enough for the R-tree of up to kMaxCtasPerSm CTAs per SM on 152 SMs
 // with n <= 16 columns (1216 triangle slots of 16 x 16 doubles plus counters and flags).
 constexpr size_t kNoAllocScratchBytes = 4u << 20;  // 4 MiB
-constexpr int kNoAllocMaxN = 16;
 
 static __device__ __align__(256) unsigned char g_tsqr_scratch[kNoAllocScratchBytes];
 
