@@ -561,7 +561,8 @@ QL_DEV i128 fx_half_rsqrt(i128 f) {
 // column stops it, as does a zero column unless zero_ok.  Returns 0, or the 1-based index of
 // the pivot that stopped it (to every thread).
 //
-// dependent: the second attempt of a TSQR call that a small pivot has stopped.  The divisions are
+// dependent: the second attempt of a call that a small pivot has stopped (of Cholesky-QR2 only if
+// its own Cholesky would have answered).  The divisions are
 // refined, which leaves Schur complements good to n 2^-117 (2^-99 otherwise), and a pivot below
 // kDependentBits, half of what the Householder tiles' 48 bits could tell from zero, is the zero that
 // they make of it: R_kk and its row vanish.  lstsq: a pivot of A between the limits (not the last
@@ -572,9 +573,9 @@ QL_DEV i128 fx_half_rsqrt(i128 f) {
 // s_i w_j from the trailing entries and leaves 1 / sqrt(f) to the end (R_kj = s_j / sqrt(f),
 // R_kk = 2^-z f / sqrt(f), all rows at once): the chain from one pivot to the next is a reciprocal and three multiplies.
 constexpr int kDependentBits = 96;
-template <int NC, int T>
+template <int NC, int T, bool dependent>
 QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double* Rout, int min_bits, bool zero_ok,
-                       bool dependent = false, bool lstsq = false) {
+                       bool lstsq) {
   constexpr int LE = NC + 1;
   u64* Slo = reinterpret_cast<u64*>(smem);
   long long* Shi = reinterpret_cast<long long*>(Slo + NC * LE);
@@ -631,7 +632,7 @@ QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double
       put(k, j, v);
       if (j == k) zk[k] = pv.z;
       i128 w = j == k ? (i128)0 : fx_div_pivot(v, pv);
-      if (dependent && j != k && pv.ok) w = fx_div_refine(w, v, pv);
+      if (dependent && j != k && pv.ok != 0) w = fx_div_refine(w, v, pv);
       Wlo[j] = (u64)(u128)w;
       Whi[j] = (long long)(w >> 64);
     }
@@ -676,6 +677,14 @@ QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double
     }
   __syncthreads();
   return 0;
+}
+
+// The second attempt, apart from the kernel's code: small calls feel its instruction cache.  (One
+// copy with a switch at run time took 2 us of 35 at 131072 x 8.)
+template <int NC, int T>
+__device__ __noinline__ bool xg_cholesky_dependent(const long long* sacc, int n, unsigned char* smem, double* Rout, int min_bits,
+                                                   bool zero_ok, bool lstsq) {
+  return xg_cholesky<NC, T, true>(sacc, n, smem, Rout, min_bits, zero_ok, lstsq) == 0;
 }
 
 // Whether SVQB would keep every eigenvalue of C = R^T R: lambda_min > tol lambda_max, shown by
@@ -753,8 +762,8 @@ QL_DEV void count_light(const Rows8<S>& v, int limit, int* bal, int* lit) {
 // Gram methods end here as well when their further passes could not change R: with C exact
 // and factored to 2^-90, Y = X R1^{-1} is orthonormal to working precision and R2 the identity.
 // flags[5] then tells the later launches of the call.  What a method answers beyond that
-// range is left to its passes: Cholesky-QR2 from pivots of 2^-46 (where an FP64 Cholesky of C
-// may break down), shifted Cholesky-QR3 from 2^-66, SVQB2 when an eigenvalue could be
+// range is left to its passes: Cholesky-QR2 where its first Cholesky, FP64 of C, breaks down (asked
+// below pivots of 2^-46; the R it accepts is then factored again in fixed point), shifted Cholesky-QR3 from 2^-66, SVQB2 when an eigenvalue could be
 // truncated or Z is wanted; a zero column breaks down there.  A TSQR call whose pivots fall below
 // 2^-80 is factored again as dependent (see xg_cholesky).  One that this does not answer is redone
 // by the Householder launch (flags[1]), as is one that has lost light rows; so are
@@ -777,12 +786,28 @@ QL_DEV void xg_finish(const GramArgs<S>& a, unsigned char* smem, const int* colm
   const int min_bits = tsqr ? 80 : (a.method == QL_SCHOLQR3 ? 66 : 46);
   const bool check_light = tid < n && (tsqr || NC <= 8);
   const int E = check_light ? __ldcg(&a.w.flags[64 + tid]) : 0, mask = check_light ? __ldcg(&a.w.flags[6 + (tid >> 5)]) : 0;
+  auto load_c = [&]() {  // C in FP64 (Rs)
+    __syncthreads();
+    for (int i = tid >> 5; i < n; i += T / 32)
+      for (int j = i + (tid & 31); j < n; j += 32) {
+        const double v = wide_to_double(sacc_load(a.w.sacc + (size_t)tri_index(i, j) * kLimbs), kXgUnitExp);
+        Rs[i * LE + j] = v;
+        Rs[j * LE + i] = v;
+      }
+    __syncthreads();
+  };
   bool done = false;
   if (a.method != QL_SVQB2 || !a.Z) {
-    done = xg_cholesky<NC, T>(a.w.sacc, n, scratch, Rs, min_bits, tsqr) == 0;
-    if (tsqr && !done) {
+    done = xg_cholesky<NC, T, false>(a.w.sacc, n, scratch, Rs, min_bits, tsqr, false) == 0;
+    if (!done && (tsqr || a.method == QL_CHOLQR2)) {
       __syncthreads();  // the scratch is written again
-      done = xg_cholesky<NC, T>(a.w.sacc, n, scratch, Rs, min_bits, true, true, a.epilogue == kEpiLstsq) == 0;
+      bool again = true;
+      if (!tsqr) {  // would its own first Cholesky answer?
+        load_c();
+        again = chol_upper_inplace<T>(Rs, LE, n, sflag) == 0;
+        __syncthreads();
+      }
+      if (again) done = xg_cholesky_dependent<NC, T>(a.w.sacc, n, scratch, Rs, min_bits, tsqr, tsqr && a.epilogue == kEpiLstsq);
     }
     if (done && a.method == QL_SVQB2)
       done = svqb_full_rank<NC, T>(Rs, n, a.rank_tol > 0.0 ? a.rank_tol : (double)n * 2.220446049250313e-16,
@@ -805,14 +830,7 @@ QL_DEV void xg_finish(const GramArgs<S>& a, unsigned char* smem, const int* colm
     }
     return;
   }
-  double* Cs = reinterpret_cast<double*>(smem);
-  for (int i = tid >> 5; i < n; i += T / 32)
-    for (int j = i + (tid & 31); j < n; j += 32) {
-      const double v = wide_to_double(sacc_load(a.w.sacc + (size_t)tri_index(i, j) * kLimbs), kXgUnitExp);
-      Cs[i * LE + j] = v;
-      Cs[j * LE + i] = v;
-    }
-  __syncthreads();
+  load_c();
   gram_epilogue<NC, T, S, ArithDF>(a, smem);
 }
 

@@ -360,3 +360,21 @@ def test_batch_across_the_tiles_line():
             assert gram_error(R, full) <= 1e-13 * (n + 1), (m, n)
             if ls:
                 assert x[n].item() == R[n, n]
+
+
+@pytest.mark.parametrize("n,m", [(3, 20000), (8, 4097), (20, 5000), (64, 3000)])
+def test_cholqr2_between_its_limits_and_a_breakdown(n, m):
+    """kappa = 3e7 (pivots of about 2^-50): FP64 Cholesky of C answers, and R comes from the fixed-point
+    factorisation of the same C as TSQR's, 2^-99 / 2^-50 off.  A dependent column still breaks down
+    or is answered by the passes."""
+    import torch
+
+    import paper_2603_20889_gb300 as q
+
+    Xd = torch.from_numpy(np.ascontiguousarray(synth.conditioned(m, n, 3e7, seed=n).T)).cuda().T
+    R, info = q.cholqr2_qless(Xd)
+    Rt, _ = q.tsqr_qless(Xd)
+    assert info.cpu().tolist() == [0, 0]
+    assert row_error(R.cpu().numpy(), Rt.cpu().numpy()) <= 2.0 ** -46
+    Xd[:, n - 1] = 0.0
+    assert q.cholqr2_qless(Xd)[1].cpu().tolist() == [q.QL_ERR_NOT_SPD, n]
