@@ -28,6 +28,19 @@ QL_DEV void xg_dispatch(const XgItem& it, int chunk, uint32_t tbase, PipeBars& b
 constexpr size_t kGroupBytes = (XgSmem<64, double>::kBytes + 15) / 16 * 16 + 32;
 static_assert(kGroupBytes <= 232448, "shared memory of one SM");
 
+// Last item whose work_begin <= v (items ordered by work_begin).
+QL_DEV int item_of(const XgItem* items, int count, int64_t v) {
+  int lo = 0, hi = count - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (items[mid].work_begin <= v)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  return lo;
+}
+
 __global__ void __launch_bounds__(XgShape<64>::T, 1)
     xgram_group_kernel(int* counter, const XgItem* items, int count, int64_t total, double* acc, int max_nc) {
   extern __shared__ __align__(1024) unsigned char smem_umma[];
@@ -40,16 +53,8 @@ __global__ void __launch_bounds__(XgShape<64>::T, 1)
   while (bars.ok) {  // a CTA whose bounded wait gave up takes no more work
     if (threadIdx.x == 0) {
       const int64_t v = atomicAdd(counter, 1);
-      int lo = 0, hi = count - 1;
-      while (lo < hi) {  // last item whose work_begin <= v (items ordered by work_begin)
-        const int mid = (lo + hi + 1) >> 1;
-        if (items[mid].work_begin <= v)
-          lo = mid;
-        else
-          hi = mid - 1;
-      }
       *s_work = v;
-      *s_item = lo;
+      *s_item = item_of(items, count, v);
     }
     __syncthreads();
     const int64_t w = *s_work;
@@ -64,6 +69,14 @@ __global__ void __launch_bounds__(XgShape<64>::T, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+  }
+  if (!bars.ok && threadIdx.x == 0) {
+    // Should every CTA give up, nobody would claim the rest and its problems would have neither an
+    // answer nor a redo: hand what is left to the gated launch.
+    for (int64_t v = atomicAdd(counter, 1); v < total; v = atomicAdd(counter, 1)) {
+      const GramArgs<double>& a = items[item_of(items, count, v)].args;
+      gram_request_redo(a.redo, a.redo_any, 1, a.method == QL_TSQR ? kRedoDF : kRedoF64);
+    }
   }
   tc_fence_before();
   __syncthreads();
