@@ -550,7 +550,8 @@ static bool make_plan(int32_t count, const ql_problem* probs, BatchPlan& P, unsi
 
 template <int MODE>
 static ql_status launch_batch(unsigned char* ws, const BatchPlan& P, int count, cudaStream_t stream) {
-  static int occ = 0;
+  static int occ_of[kMaxDevices] = {};
+  int& occ = occ_of[device_slot()];
   static size_t smem = 0;
   static std::mutex mu;
   auto kern = batch_kernel<MODE>;

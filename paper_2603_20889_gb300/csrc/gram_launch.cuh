@@ -682,7 +682,8 @@ ql_status gram_stream_launch_one(const GramCall& c, const GramWs& w, int pass, i
   using Sh = StreamShape<NC>;
   using Sm = StreamSmem<NC, S, Ar>;
   auto kern = gram_stream_kernel<NC, S, Ar, XF>;
-  static int occ = 0;
+  static int occ_of[kMaxDevices] = {};
+  int& occ = occ_of[device_slot()];
   static std::mutex mu;
   {
     std::lock_guard<std::mutex> lk(mu);
@@ -1123,7 +1124,8 @@ ql_status gram_tc_launch_one(const GramCall& c, const GramWs& w, int pass) {
   using Sh = TcShape<NC>;
   using Sm = TcSmem<NC, S>;
   auto kern = gram_tc_kernel<NC, S, XF>;
-  static int occ = 0;
+  static int occ_of[kMaxDevices] = {};
+  int& occ = occ_of[device_slot()];
   static std::mutex mu;
   {
     std::lock_guard<std::mutex> lk(mu);
@@ -1632,7 +1634,8 @@ ql_status gram_umma_launch_one(const GramCall& c, const GramWs& w, int pass) {
   using Sh = UmmaShape<NC>;
   using Sm = UmmaSmem<NC, S>;
   auto kern = gram_umma_kernel<NC, S, XF>;
-  static bool ready = false;
+  static bool ready_on[kMaxDevices] = {};
+  bool& ready = ready_on[device_slot()];
   static std::mutex mu;
   {
     std::lock_guard<std::mutex> lk(mu);
@@ -2199,7 +2202,8 @@ ql_status gram_pipe_launch_one(const GramCall& c, const GramWs& w, int pass) {
   using Sh = PipeShape<NC>;
   using Sm = PipeSmem<NC, S>;
   auto kern = gram_pipe_kernel<NC, S, XF>;
-  static bool ready = false;
+  static bool ready_on[kMaxDevices] = {};
+  bool& ready = ready_on[device_slot()];
   static std::mutex mu;
   {
     std::lock_guard<std::mutex> lk(mu);
@@ -2252,7 +2256,8 @@ ql_status gram_launch_one(const GramCall& c, const GramWs& w, int pass, int gate
   using Sh = GramShape<NC>;
   using Sm = GramSmem<NC, S, Ar>;
   auto kern = gram_kernel<NC, S, Ar, XF>;
-  static int occ = 0;
+  static int occ_of[kMaxDevices] = {};
+  int& occ = occ_of[device_slot()];
   static std::mutex mu;
   {
     std::lock_guard<std::mutex> lk(mu);

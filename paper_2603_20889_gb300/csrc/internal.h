@@ -82,6 +82,10 @@ ql_status gram_launch(const GramCall& c, ql_arith arith);
 
 // SM count of the current device (cached per device).
 int device_sm_count();
+// The current device's index below kMaxDevices, for what is set up or cached once per device (a
+// kernel's shared-memory limit and occupancy hold for the device that was current).
+constexpr int kMaxDevices = 64;
+int device_slot();
 ql_arith current_arith();
 
 // Largest n any entry point accepts.

@@ -318,7 +318,8 @@ static ql_status proj_run(ProjArgs<S> a, cudaStream_t st) {
   using Sm = ProjSmem<KC, NC>;
   auto ck = cross_kernel<KC, NC, S>;
   auto uk = update_kernel<KC, NC, S>;
-  static bool ready = false;
+  static bool ready_on[kMaxDevices] = {};
+  bool& ready = ready_on[device_slot()];
   static std::mutex mu;
   {
     std::lock_guard<std::mutex> lk(mu);

@@ -237,7 +237,8 @@ template <int NC, typename S>
 static ql_status qform_launch_one(QformArgs<S> a, cudaStream_t stream) {
   using Sm = QformSmem<NC, S>;
   auto kern = qform_kernel<NC, S>;
-  static bool ready = false;
+  static bool ready_on[kMaxDevices] = {};
+  bool& ready = ready_on[device_slot()];
   static std::mutex mu;
   {
     std::lock_guard<std::mutex> lk(mu);

@@ -20,12 +20,15 @@ int tsqr_variant() {
   return v;
 }
 
+int device_slot() {
+  int dev = 0;
+  return cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices ? 0 : dev;
+}
+
 int device_sm_count() {
   // cached per device: a process may drive GPUs with different SM counts
-  constexpr int kMaxDev = 64;
-  static std::atomic<int> sms[kMaxDev] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) dev = 0;
+  static std::atomic<int> sms[kMaxDevices] = {};
+  const int dev = device_slot();
   int v = sms[dev].load(std::memory_order_relaxed);
   if (v > 0) return v;
   if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) v = 1;

@@ -75,7 +75,8 @@ ql_status launch_one(const TsqrCall& c, const TreeView& tv_in, int gated) {
   using Sm = TsqrSmem<NC, TC, RPT, T, S, Ar>;
   using Sh = TsqrShape<NC, TC, RPT, T>;
   auto kern = tsqr_kernel<NC, TC, RPT, T, S, Ar>;
-  static int occ = 0;  // CTAs per SM at this configuration's registers and shared memory
+  static int occ_of[kMaxDevices] = {};
+  int& occ = occ_of[device_slot()];  // CTAs per SM at this configuration's registers and shared memory
   static std::mutex mu;
   {
     std::lock_guard<std::mutex> lk(mu);

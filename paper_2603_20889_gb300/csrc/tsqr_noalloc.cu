@@ -22,7 +22,6 @@ static __device__ __align__(256) unsigned char g_tsqr_scratch[kNoAllocScratchByt
 
 // Device address of the scratch array, looked up once per device with that device current.
 // In host code the array's name is only a host-side stand-in, never a device address.
-static constexpr int kMaxDevices = 64;
 static void* g_scratch_addr[kMaxDevices] = {};
 static std::mutex g_scratch_mu;
 

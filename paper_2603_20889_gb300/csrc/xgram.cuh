@@ -492,8 +492,6 @@ QL_DEV i128 fx_mul(i128 a, i128 b) {
 struct FxPivot {
   u64 c;
   long long eps;
-  u64 flo;  // f in units of 2^-kFx
-  long long fhi;
   int z;
   int ok;  // 1: usable; 0: zero column; -1: pivot too small
 };
@@ -503,7 +501,7 @@ QL_DEV int fx_half_lead(i128 d) {  // z with d 4^z in [1/4, 1)
   return (lead - (128 - kFx)) >> 1;
 }
 QL_DEV FxPivot fx_pivot(i128 d, bool zero_column, int min_bits) {
-  FxPivot pv{0, 0, 0, 0, 0, 0};
+  FxPivot pv{0, 0, 0, 0};
   if (zero_column) return pv;
   if (d < ((i128)1 << (kFx - min_bits))) {
     pv.ok = -1;
@@ -512,8 +510,6 @@ QL_DEV FxPivot fx_pivot(i128 d, bool zero_column, int min_bits) {
   pv.ok = 1;
   pv.z = fx_half_lead(d);
   const u128 f = (u128)d << (2 * pv.z);
-  pv.flo = (u64)f;
-  pv.fhi = (long long)(u64)(f >> 64);
   const u64 f64 = (u64)(f >> (kFx - 64));  // f 2^64
   const float y0 = __fdividef(1.0f, (float)(unsigned)(f64 >> 40) * 0x1p-24f);  // in [1, 4]
   const u64 c0 = (u64)(unsigned)(y0 * 0x1p21f) << 40;
@@ -534,8 +530,7 @@ QL_DEV i128 fx_div_pivot(i128 s, const FxPivot& pv) {
   return w + (i128)__mul64hi((long long)(w >> 61), pv.eps) * ((i128)1 << 23);
 }
 // w = s / f of fx_div_pivot with its residual divided once more: 2^-99 -> 2^-117.
-QL_DEV i128 fx_div_refine(i128 w, i128 s, const FxPivot& pv) {
-  const i128 f = (i128)(((u128)(u64)pv.fhi << 64) | pv.flo);
+QL_DEV i128 fx_div_refine(i128 w, i128 s, i128 f, const FxPivot& pv) {
   const long long r = (long long)((s >> 3) - fx_mul(f, w));  // units of 2^-122, below 2^-97
   return w + (((i128)r * (i128)(u128)pv.c) >> 61);
 }
@@ -584,6 +579,7 @@ QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double
   FxPivot* piv = reinterpret_cast<FxPivot*>(Whi + NC);  // [2]
   int* sj = reinterpret_cast<int*>(piv + 2);            // column exponents
   int* zk = sj + NC;                                    // z of each pivot
+  u64* fk = reinterpret_cast<u64*>(zk + NC);            // [2] f of the pivot, low and high word (dependent)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int NW = T / 32;
   auto get = [&](int i, int j) -> i128 { return (i128)(((u128)(u64)Shi[i * LE + j] << 64) | Slo[i * LE + j]); };
@@ -621,6 +617,11 @@ QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double
     FxPivot pv = fx_pivot(d, zero, limit);
     if (pv.ok == 0 && !zero_ok) pv.ok = -1;
     piv[k & 1] = pv;
+    if (dependent) {
+      const u128 f = (u128)d << (2 * pv.z);
+      fk[2 * (k & 1)] = (u64)f;
+      fk[2 * (k & 1) + 1] = (u64)(f >> 64);
+    }
   };
   if (tid == 0) pivot(0, get(0, 0));
   __syncthreads();
@@ -632,7 +633,10 @@ QL_DEV int xg_cholesky(const long long* sacc, int n, unsigned char* smem, double
       put(k, j, v);
       if (j == k) zk[k] = pv.z;
       i128 w = j == k ? (i128)0 : fx_div_pivot(v, pv);
-      if (dependent && j != k && pv.ok != 0) w = fx_div_refine(w, v, pv);
+      if (dependent && j != k && pv.ok != 0) {
+        const i128 f = (i128)(((u128)fk[2 * (k & 1) + 1] << 64) | fk[2 * (k & 1)]);
+        w = fx_div_refine(w, v, f, pv);
+      }
       Wlo[j] = (u64)(u128)w;
       Whi[j] = (long long)(w >> 64);
     }
@@ -1291,7 +1295,8 @@ ql_status xgram_launch_one(const GramCall& c, const GramWs& w) {
   using Sh = XgShape<NC>;
   using Sm = XgSmem<NC, S>;
   auto kern = xgram_kernel<NC, S>;
-  static bool ready = false;
+  static bool ready_on[kMaxDevices] = {};
+  bool& ready = ready_on[device_slot()];
   static std::mutex mu;
   {
     std::lock_guard<std::mutex> lk(mu);
