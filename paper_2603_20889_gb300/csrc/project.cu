@@ -10,12 +10,15 @@
 // tiles in double-float, two rows per packed FP32 instruction (half the issue slots; two CTAs per
 // SM, so that one loads while the other multiplies), and writes one FP64 partial;
 // cross_reduce_kernel sums the partials in a fixed order (reproducible), an entry per thread over
-// many CTAs, where the last CTA used to sum all of them.  The update W = V - Y C streams the rows,
-// one per thread.  Tiles outside the double-float exponent range run in FP64.
+// many CTAs, where the last CTA used to sum all of them.  The update W = V - Y C streams blocks of
+// 64 rows, a warp each, two adjacent rows per thread and two columns per packed instruction; few
+// blocks are spread over the SMs (see qform.cu).  Tiles outside the double-float exponent range run
+// in FP64.  With few rows the later launches wait on the device for their predecessors (programmatic
+// dependent launches): 1000 rows, k = 8, n = 1 57 -> 44 us.
 //
 // Both are bound by the FP32 pipes, 13 operations per product and row: k = n = 64, m = 2^19
-// 0.71 ms each; measured 1.34 + 0.05 ms (cross product and reduction) and 2.27 ms (update).  QR
-// of 524288 x 128, with two of each: 15.3 -> 11.7 ms.
+// 0.71 ms each; measured 1.34 + 0.05 ms (cross product and reduction) and 1.67 ms (update).  QR
+// of 524288 x 128, with two of each: 15.3 -> 9.8 ms.
 #include <mutex>
 
 #include "df2.cuh"
@@ -48,7 +51,7 @@ struct ProjArgs {
   int pass;
   ProjWs w;
   int64_t tiles;
-  int spread;  // update: fewer blocks than warps, adjacent blocks go to different CTAs
+  int cta_step, warp_step;  // update: first block of a warp = CTA x cta_step + warp x warp_step
 };
 
 QL_DEV bool df_range_ok_dev(int E) { return E == 0 || (E >= kDfEminLimit && E <= kDfEmaxLimit); }
@@ -186,7 +189,7 @@ __global__ void __launch_bounds__(update_threads<KC>(), 1) update_kernel(ProjArg
   extern __shared__ __align__(16) unsigned char smem[];
   df2* Cd = reinterpret_cast<df2*>(smem);                                        // [KC][NC / 2] column pairs
   float4* mine = reinterpret_cast<float4*>(Cd + KC * NC / 2) + threadIdx.x;     // column i of this thread's rows at mine[i T]
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = a.k, n = a.n;
+  const int tid = threadIdx.x, lane = tid & 31, k = a.k, n = a.n;
   pdl_release();
   pdl_wait();
   bool cbad = false;
@@ -209,8 +212,7 @@ __global__ void __launch_bounds__(update_threads<KC>(), 1) update_kernel(ProjArg
     a.W[j * a.ldw + row] = (S)s;
   };
   const int64_t nw = (int64_t)gridDim.x * (T / 32);
-  for (int64_t t = a.spread ? blockIdx.x + (int64_t)warp * gridDim.x : (int64_t)blockIdx.x * (T / 32) + warp; t < a.tiles;
-       t += nw) {
+  for (int64_t t = (int64_t)blockIdx.x * a.cta_step + (tid >> 5) * a.warp_step; t < a.tiles; t += nw) {
     const int64_t row = t * 64 + 2 * lane;
     const bool live0 = row < a.m, live1 = row + 1 < a.m;
     bool bad = false;
@@ -336,8 +338,11 @@ static ql_status proj_run(ProjArgs<S> a, cudaStream_t st) {
   const int64_t ctiles = (a.m + kProjB - 1) / kProjB, utiles = (a.m + 63) / 64;
   int64_t gc = (int64_t)device_sm_count() * kCrossCtasPerSm, gu = (int64_t)device_sm_count() * (occ < 1 ? 1 : occ);
   if (gc > ctiles) gc = ctiles;
-  a.spread = utiles < gu * (UT / 32) ? 1 : 0;  // as in qform.cu: the conversions' FP64 pipes
+  const bool spread = utiles < gu * (UT / 32);  // as in qform.cu: the conversions' FP64 pipes
   if (gu > utiles) gu = utiles;
+  // (a choice between the two orders inside the kernel slowed its loop: 6.1 -> 6.36 ms)
+  a.cta_step = spread ? 1 : UT / 32;
+  a.warp_step = spread ? (int)gu : 1;
   if (gc < 1) gc = 1;
   if (gu < 1) gu = 1;
   const S* X = a.V;
@@ -353,21 +358,31 @@ static ql_status proj_run(ProjArgs<S> a, cudaStream_t st) {
     }
     a.tiles = ctiles;
     count_launch();
-    // The first kernel is an ordinary launch (its inputs are the caller's); the others start while
-    // their predecessor runs and wait for its end before they touch memory.
-    if (pass == 1) {
+    // The first kernel is an ordinary launch (its inputs are the caller's).  With few rows the others
+    // start while their predecessor runs and wait for its end before they touch memory; with many
+    // they are ordinary launches too (as dependent ones k = n = 64, m = 2^19 took 6.5 instead of 6.1 ms).
+    if (pass == 1 || !spread) {
       ck<<<(int)gc, kProjT, Sm::kCross, st>>>(a);
       if (cudaPeekAtLastError() != cudaSuccess) return QL_ERR_CUDA;
     } else if (launch_dependent(ck, (int)gc, kProjT, Sm::kCross, st, a) != cudaSuccess) {
       return QL_ERR_CUDA;
     }
     count_launch();
-    if (launch_dependent(cross_reduce_kernel<S>, (KC * NC + kReduceT - 1) / kReduceT, kReduceT, 0, st, a, KC, NC, (int)gc) !=
-        cudaSuccess)
+    constexpr int gr = (KC * NC + kReduceT - 1) / kReduceT;
+    if (!spread) {
+      cross_reduce_kernel<S><<<gr, kReduceT, 0, st>>>(a, KC, NC, (int)gc);
+      if (cudaPeekAtLastError() != cudaSuccess) return QL_ERR_CUDA;
+    } else if (launch_dependent(cross_reduce_kernel<S>, gr, kReduceT, 0, st, a, KC, NC, (int)gc) != cudaSuccess) {
       return QL_ERR_CUDA;
+    }
     a.tiles = utiles;
     count_launch();
-    if (launch_dependent(uk, (int)gu, UT, Sm::kUpdate, st, a) != cudaSuccess) return QL_ERR_CUDA;
+    if (!spread) {
+      uk<<<(int)gu, UT, Sm::kUpdate, st>>>(a);
+      if (cudaPeekAtLastError() != cudaSuccess) return QL_ERR_CUDA;
+    } else if (launch_dependent(uk, (int)gu, UT, Sm::kUpdate, st, a) != cudaSuccess) {
+      return QL_ERR_CUDA;
+    }
   }
   return QL_OK;
 }
@@ -412,11 +427,11 @@ ql_status ql_project_out(int64_t m, int64_t k, const void* Y, int64_t ldy, int64
   w.partials = w.cpass + (size_t)kMaxN * kMaxN;
   if (dtype == QL_F64) {
     ProjArgs<double> a{m, (int)k, (int)n, static_cast<const double*>(Y), ldy, static_cast<const double*>(X), ldx,
-                       static_cast<double*>(W), ldw, C, ldc, 1, w, 0, 0};
+                       static_cast<double*>(W), ldw, C, ldc, 1, w, 0, 0, 0};
     return proj_dispatch(a, st);
   }
   ProjArgs<float> a{m, (int)k, (int)n, static_cast<const float*>(Y), ldy, static_cast<const float*>(X), ldx,
-                    static_cast<float*>(W), ldw, C, ldc, 1, w, 0, 0};
+                    static_cast<float*>(W), ldw, C, ldc, 1, w, 0, 0, 0};
   return proj_dispatch(a, st);
 }
 

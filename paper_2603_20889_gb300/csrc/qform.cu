@@ -11,8 +11,9 @@
 //
 // Bound: 13 FP32 operations per product and row (m = 2^23, n = 16: 378 us at the measured FP32
 // rate, against 323 us of HBM).  Measured there 1638 us with one row per thread, a column fetched
-// at a time and block-wide tiles, 1195 us now; 4000000 x 32 2393 -> 1430 us, 2097152 x 64 5015 ->
-// 3994 us, 4000001 x 8 381 -> 263 us.  What is left is latency (fixed-latency stalls at 5 to 24
+// at a time and block-wide tiles, 1190 us now; 4000000 x 32 2393 -> 1430 us, 2097152 x 64 5015 ->
+// 3994 us, 4000001 x 8 381 -> 263 us; few rows, spread over the SMs, 1000 x 31 68 -> 61 us; FP32
+// 1048576 x 64 1760 -> 1305 us.  What is left is latency (fixed-latency stalls at 5 to 24
 // warps per SM) and the conversions of X and of the results (three FP64-pipe instructions each,
 // 640 us of that pipe at n = 16, overlapped; assembling the doubles with integer instructions
 // instead measured slower, 1605 us).
@@ -36,7 +37,7 @@ struct QformArgs {
   int64_t ldq;
   int32_t* info;
   int64_t tiles;  // blocks of 64 rows
-  int spread;     // fewer blocks than warps: adjacent blocks go to different CTAs
+  int cta_step, warp_step;  // first block of a warp = CTA x cta_step + warp x warp_step
   int pair;       // two adjacent rows of every column can be read and written in one access
 };
 
@@ -122,9 +123,7 @@ __global__ void __launch_bounds__(QformSmem<NC, S>::T, QformSmem<NC, S>::kCtas) 
   const int64_t nw = (int64_t)gridDim.x * (T / 32);
   X2* mine = xs + tid;  // column k of this thread's rows at mine[k T]
   using S2 = typename std::conditional<sizeof(S) == 8, double2, float2>::type;
-  const int warp = tid >> 5;
-  for (int64_t t = a.spread ? blockIdx.x + (int64_t)warp * gridDim.x : (int64_t)blockIdx.x * (T / 32) + warp; t < a.tiles;
-       t += nw) {
+  for (int64_t t = (int64_t)blockIdx.x * a.cta_step + (tid >> 5) * a.warp_step; t < a.tiles; t += nw) {
     const int64_t row = t * 64 + 2 * lane;
     const bool live0 = row < a.m, live1 = row + 1 < a.m;
     const bool whole = a.pair && t * 64 + 64 <= a.m;  // uniform in the warp
@@ -256,10 +255,12 @@ static ql_status qform_launch_one(QformArgs<S> a, cudaStream_t stream) {
   // (and, while one CTA per SM has the warps, one copy of R^{-1} is formed per SM)
   const int64_t sms = device_sm_count();
   int64_t g = sms * (occ < 1 ? 1 : occ);
-  a.spread = a.tiles < g * (Sm::T / 32) ? 1 : 0;
+  const bool spread = a.tiles < g * (Sm::T / 32);
   if (a.tiles <= sms * (Sm::T / 32)) g = sms;
   if (g > a.tiles) g = a.tiles;
   if (g < 1) g = 1;
+  a.cta_step = spread ? 1 : Sm::T / 32;
+  a.warp_step = spread ? (int)g : 1;
   count_launch();
   kern<<<(int)g, Sm::T, Sm::kBytes, stream>>>(a);
   return cudaPeekAtLastError() == cudaSuccess ? QL_OK : QL_ERR_CUDA;
@@ -313,9 +314,9 @@ extern "C" ql_status ql_q_from_r(int64_t m, int64_t n, const void* X, ql_dtype d
     return QL_ERR_ALIGN;
   cudaStream_t st = (cudaStream_t)stream;
   if (dtype == QL_F64) {
-    QformArgs<double> a{m, (int)n, static_cast<const double*>(X), ldx, R, ldr, static_cast<double*>(Q), ldq, info, 0, 0, 0};
+    QformArgs<double> a{m, (int)n, static_cast<const double*>(X), ldx, R, ldr, static_cast<double*>(Q), ldq, info, 0, 0, 0, 0};
     return qform_dispatch(a, st);
   }
-  QformArgs<float> a{m, (int)n, static_cast<const float*>(X), ldx, R, ldr, static_cast<float*>(Q), ldq, info, 0, 0, 0};
+  QformArgs<float> a{m, (int)n, static_cast<const float*>(X), ldx, R, ldr, static_cast<float*>(Q), ldq, info, 0, 0, 0, 0};
   return qform_dispatch(a, st);
 }
