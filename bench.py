@@ -412,7 +412,7 @@ def run_ours(args, rank, world, local_rank):
     out = {
         "metric": METRIC, "value": round(value, 2), "unit": "GB/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": round(ms_step, 3), "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": "f32x2", "data": "synthetic",
+        "vs_baseline": None, "dtype": "fp64 (exact sums of bf16 digits)", "data": "synthetic",
         "config": {"workload": WORKLOAD, "storage": "f64",
                    "arith": "exact integer Gram of 56-bit digits (bf16 tensor cores), 125-bit fixed-point Cholesky; "
                             "double-float for n <= 2",

@@ -25,10 +25,12 @@
  *   - The return value reports only synchronous errors (argument checks, launch errors).
  *     64-bit sizes are used throughout; m * ld may exceed 2^31.
  *
- * Arithmetic.  The m-proportional loops run in "double-float" arithmetic (an unevaluated
- * sum of two floats, about 48 significant bits) on the FP32 pipes by default, because the
- * FP64 pipe of this GPU is about 60x slower than its FP32 pipes; the n x n steps (R-tree,
- * Cholesky, eigensolve, back-substitution) always run in FP64.  Inputs whose magnitudes
+ * Arithmetic.  By default no m-proportional loop runs in FP64, whose pipe is about 60x slower
+ * than the FP32 pipes on this GPU.  From 3 columns R comes from an exact integer Gram matrix
+ * of X in fixed point (tensor cores) and a 125-bit fixed-point Cholesky; fewer columns, what that
+ * cannot answer, Q and the projections run in "double-float" arithmetic (an unevaluated sum of
+ * two floats, about 48 significant bits).  The other n x n steps (R-tree, FP64 Cholesky,
+ * eigensolve, back-substitution) run in FP64.  Inputs whose magnitudes
  * fall outside the double-float range (see ql_set_arith) are detected on the device and
  * recomputed by the FP64 kernels inside the same call, with no host round trip.
  */
@@ -110,11 +112,15 @@ size_t ql_workspace_bytes(ql_method method, int64_t m, int64_t n, ql_dtype dtype
 
 /*
  * Q-less TSQR (Sec. 3.2, Algorithms 2-4): the R of X for any condition number.
- * For n >= 3 the first launch forms X^T X exactly (X rounded to 2^-56 of each column's
- * largest entry, every product and sum an integer) and factors it in 125-bit fixed point:
- * the same R, with an error below the Householder tiles'.  Columns dependent to about 2^-40
- * of their norm (a pivot below 2^-80) are left to the Householder launch behind it, which
- * otherwise exits at once and which is the only one for n <= 2 (n <= 4 below 2^14 rows): every CTA streams its row blocks of X
+ * For n >= 3 the first launch forms X^T X in integers and factors it in 125-bit fixed point.
+ * An entry x is rounded once, to |dx| <= 2^-53 of the largest entry that its CTA has met in the
+ * column: a columnwise backward error of at most sqrt(m) max|x| 2^-53, below the Householder
+ * tiles' for columns of entries of similar size.  A few heavy rows above light ones lose the light
+ * rows' low bits; where R depends on them (a column with light entries whose R_kk is below four
+ * times its largest entry), the Householder launch behind it computes R, which otherwise
+ * exits at once.  A column dependent on earlier ones to 2^-48 of its norm (a pivot below 2^-96)
+ * gives a zero row of R.  The Householder launch is the only one for n <= 2, m < n and n = 3, 4
+ * below 2^12 rows: every CTA streams its row blocks of X
  * through shared memory, factors [R; W] in place with Householder reflectors (Algorithm 4),
  * and the per-CTA triangles are merged by a "last CTA done" R-tree (Algorithm 2, stage 2)
  * inside the same launch.  An FP64 fallback launch follows that exits at once unless the
@@ -127,7 +133,8 @@ ql_status ql_tsqr_qless(int64_t m, int64_t n, const void* X, ql_dtype dtype, int
 
 /*
  * TSQR for callers that cannot allocate device memory (the paper has no counterpart: it is
- * an interface addition of this library).  Same computation, arguments, argument and
+ * an interface addition of this library).  The R of ql_tsqr_qless, always by the Householder
+ * tiles (48-bit arithmetic also where that entry takes the exact pass); same arguments, argument and
  * alignment checks (QL_ERR_ARG, QL_ERR_ALIGN before any device work) and tuned grid as
  * ql_tsqr_qless, without the workspace: code running while its stream is captured into a
  * CUDA graph may not call cudaMalloc, host callbacks must not, and extensions of
@@ -150,9 +157,10 @@ ql_status ql_tsqr_qless_noalloc(int64_t m, int64_t n, const void* X, ql_dtype dt
  * Both Cholesky factorisations, R1^{-1} and R2 R1 run on the device in FP64.  A
  * non-positive pivot sets info = {QL_ERR_NOT_SPD, pivot} (+1000 for the second pass) and
  * fills R with NaN.  Reliable for kappa_2(X) up to about 1e6 (the Gram squares kappa).
- * For n >= 3 the first pass is exact (see ql_tsqr_qless): while every pivot of C stays above
- * 2^-46 of its column, R1 from the fixed-point Cholesky is already the R that both passes
- * give, with a smaller error, and the second pass ends at once.
+ * For n >= 3 the first pass is exact (see ql_tsqr_qless): where the FP64 Cholesky of C does not
+ * break down (certain while every pivot stays above 2^-46 of its column), R1 from the fixed-point
+ * Cholesky is already the R that both passes give, with a smaller error, and the second pass
+ * ends at once; with up to 8 columns not where light rows are lost.
  */
 ql_status ql_cholqr2_qless(int64_t m, int64_t n, const void* X, ql_dtype dtype, int64_t ldx, double* R,
                            int64_t ldr, int32_t* info, void* ws, size_t ws_bytes, void* stream);
@@ -215,7 +223,7 @@ ql_status ql_q_from_r(int64_t m, int64_t n, const void* X, ql_dtype dtype, int64
  *   C1 = Y^T X,  W1 = X - Y C1,  C2 = Y^T W1,  W = W1 - Y C2,
  * W (device, m x n of dtype, ld ldw; may be X itself) receives the projected block and C
  * (device double k x n, ld ldc >= k) the coefficients C1 + C2, so X = Y C + W.  The R of the
- * orthogonalised block is any Q-less call on W.  Four launches; the Y^T V products are
+ * orthogonalised block is any Q-less call on W.  Six launches; the Y^T V products are
  * reduced in a fixed order (reproducible).  ws: ql_project_workspace_bytes(k, n) bytes.
  */
 size_t ql_project_workspace_bytes(int64_t k, int64_t n);
@@ -261,11 +269,13 @@ typedef struct {
  * of a problem is its method_hint, or for QL_AUTO the autotune table entry of its
  * (m, n, dtype, kappa) class (ql_autotune), else Cholesky-QR2 from 24 columns when
  * 0 < kappa_hint <= 1e6 and TSQR otherwise; the Gram method needs n (+1 for least squares)
- * >= 9, narrower problems always run TSQR.  All problems run as work items (row-tile chunks)
- * of ONE persistent launch of the exact Gram pass (see ql_tsqr_qless); Cholesky-QR2 problems
+ * >= 9, narrower problems always run TSQR.  The problems run as work items (row-tile chunks)
+ * of ONE persistent launch: of the exact Gram pass (see ql_tsqr_qless), or of Householder tiles
+ * for a batch of problems of one or two columns or few rows only (and beside it in a mixed batch
+ * whose single columns have 2^21 rows together).  Cholesky-QR2 problems
  * asked for by method_hint keep a second pass per (column class, storage), which ends at once
- * unless a pivot fell below the method's limit.  A problem that leaves the double-float
- * range, or whose pivots fall below the limit of a TSQR call (QL_TSQR, QL_AUTO), is redone by
+ * unless the exact pass could not answer.  A problem that leaves the double-float
+ * range, or that the exact pass of a TSQR call (QL_TSQR, QL_AUTO) cannot answer, is redone by
  * a final gated Householder launch with per-problem R-trees.  The plan lives
  * in `ws` (ql_batch_workspace_bytes) and is rebuilt on every call.  Equivalent, problem by
  * problem, to the single-call entry points up to rounding order.

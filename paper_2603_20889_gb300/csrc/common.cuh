@@ -255,9 +255,6 @@ __host__ __device__ inline int df_emax_limit(int64_t m) {
 }
 
 // ---------------------------------------------------------------------------------------
-// cp.async staging (Ampere-style per-thread async copies; any element-aligned address).
-// ---------------------------------------------------------------------------------------
-// ---------------------------------------------------------------------------------------
 // Programmatic dependent launch.  A kernel launched with launch_dependent (internal.h) may
 // start while its predecessor in the stream still runs; pdl_wait returns once that one has
 // finished and its writes are visible (at once in an ordinary launch).  pdl_release lets the
@@ -267,6 +264,9 @@ __host__ __device__ inline int df_emax_limit(int64_t m) {
 QL_DEV void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 QL_DEV void pdl_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
+// ---------------------------------------------------------------------------------------
+// cp.async staging (Ampere-style per-thread async copies; any element-aligned address).
+// ---------------------------------------------------------------------------------------
 template <int I, int N, typename F>
 QL_DEV void static_for(F&& f) {
   if constexpr (I < N) {

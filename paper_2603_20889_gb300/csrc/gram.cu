@@ -1,6 +1,7 @@
-// Host launcher of the Q-less Gram methods (paper Sec. 3.1): Cholesky-QR2 (Algorithm 1)
-// and SVQB2.  Two launches per call (first pass, second pass); after the double-float
-// pair, two gated FP64 launches follow that run only if the range check fired.
+// Host launcher of the Q-less Gram methods (paper Sec. 3.1): Cholesky-QR2 (Algorithm 1), shifted
+// Cholesky-QR3 and SVQB2.  A clearing kernel, the first pass (exact from 3 columns, which then
+// usually writes R) and the later passes, which exit at once if it has; then as many gated FP64
+// launches that run only if the range check fired.
 #include "gram_launch.cuh"
 
 #include <cstdlib>
@@ -148,7 +149,7 @@ ql_status gram_launch(const GramCall& c, ql_arith arith) {
   return gram_dispatch<float, ArithF64>(c, w, 1);
 }
 
-// Workspace and launch of the exact pass for a TSQR call (n >= 2).  The caller clears the
+// Workspace and launch of the exact pass for a TSQR call (n >= 3).  The caller clears the
 // first *clear_bytes of `base` beforehand; flags[0] then asks for the FP64 launch and
 // flags[1] for the double-float Householder launch.
 size_t xgram_tsqr_bytes(int n) { return gram_layout(n, nullptr, nullptr); }

@@ -97,11 +97,13 @@ bool elem_aligned(const void* p, ql_dtype dt);
 ql_status check_matrix(int64_t m, int64_t n, const void* X, ql_dtype dt, int64_t ld, int nmax);
 // Output triangle R: non-null with ldr >= n (QL_ERR_ARG), 8-byte aligned (QL_ERR_ALIGN).
 ql_status check_r(const double* R, int64_t ldr, int64_t n);
-// Whether the Gram passes use the tensor-core kernels (double-float mode, n >= 9);
-// the environment variable QL_GRAM_SIMT=1 selects the SIMT kernels instead.
+// Whether the tensor-core kernels are used (double-float mode): the exact pass, of TSQR calls too,
+// and the later Gram passes from 9 columns; the environment variable QL_GRAM_SIMT=1 selects the
+// Householder tiles and the SIMT Gram kernels instead.
 bool tc_gram_enabled();
-// First Gram pass of the 16-, 32- and 64-column classes on the pipelined tcgen05 kernel
-// (default; QL_GRAM_PIPE=0 selects the per-tile kernels, for comparison).
+// First Gram pass of the Gram methods' 16-, 32- and 64-column classes, and the batched form, on the
+// exact kernel (default; QL_GRAM_PIPE=0 selects the per-tile kernels, for comparison; TSQR calls and
+// the Gram methods of up to 8 columns stay on the exact kernel).
 bool pipe_gram_enabled();
 // QL_GRAM_PIPE2=0: the later Gram passes of n <= 32 run on the per-tile mma.sync kernel instead
 // of the pipelined one (A/B comparisons).

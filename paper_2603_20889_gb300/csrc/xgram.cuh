@@ -2,9 +2,9 @@
 // over X, in the 4-, 8-, 16-, 32- and 64-column classes, for TSQR calls and, while their further
 // passes could not change R, for the Gram methods.
 //
-// Measured against the double-float Householder tiles (which stay for columns dependent to
-// about 2^-40 and the narrow calls of exact_route) and the Gram methods' own passes (which stay
-// beyond the limits in xg_finish): TSQR m = 2^25, n = 4 917 -> 383 us; m = 2^23, n = 8, 16, 32
+// Measured against the double-float Householder tiles (which stay for calls that lose light rows,
+// see light_floor, and those that exact_route leaves them) and the Gram methods' own passes (which
+// stay beyond the limits in xg_finish): TSQR m = 2^25, n = 4 917 -> 383 us; m = 2^23, n = 8, 16, 32
 // 213, 406, 783 us (2.5, 2.6, 2.7 TB/s of X); m = 2^22, n = 64 21.1 -> 2.11 ms, Cholesky-QR2
 // 8.30 -> 2.11 ms; SVQB2 10^6 x 32 3.89 -> 0.20 ms; shifted Cholesky-QR3 300007 x 24 871 ->
 // 114 us; least squares 2^24 x 31, FP32-stored, 19.3 -> 1.48 ms; 131072 x 8 145 -> 42 us.
@@ -20,10 +20,13 @@
 // core stays an integer of at most 2^24 (exact), the read-outs fold them into 128-bit
 // integers and the CTAs add those into one integer accumulator of 320 bits per entry of C.
 // The Gram matrix of the rounded X is therefore exact: no product is dropped, no sum rounds,
-// and the result does not depend on the order of tiles, CTAs or atomics.  That is what lets
+// and the sums do not depend on the order of tiles, CTAs or atomics (the rounding follows the
+// running maxima of each CTA, so it does on the partition into CTAs).  That is what lets
 // one pass serve TSQR: with C exact, a Cholesky factorisation in 125-bit fixed point
-// (xg_cholesky) loses kappa^2 2^-120 instead of kappa^2 2^-53, so the R it gives is limited
-// by the 2^-56 rounding of X (a backward error, like Householder's) up to kappa ~ 2^40.
+// (xg_cholesky) loses kappa^2 2^-99, 2^-111 when refined, instead of kappa^2 2^-53, so the R it
+// gives is limited by the rounding of X: a scale stands 2 to 3 bits above the maximum that set it,
+// so half a step is 2^-54 to 2^-53 of the largest entry that the CTA has met in the column, a
+// columnwise backward error of up to sqrt(m) max|x| 2^-53.  (It is not a rowwise one: light_floor.)
 //
 //  * Roles and tiles: 16 slicer warps cut tiles of 4096 elements (KT = 4096 / NC rows) into
 //    digit planes and read the accumulators out; one warp issues the tensor-map copies two
@@ -468,10 +471,11 @@ QL_DEV double wide_to_double(const Wide320& a, int e) {
 // operation and nothing to cancellation.  Integer multiplies run on the ALUs at full rate,
 // where FP64 (1/64 of the FP32 rate) or double-double would not: a double-double version of
 // the same factorisation needs about 0.9 M FP64 operations at n = 64, 0.2 ms on one SM.
+// (The divisions lose 2^-99, see fx_div_pivot, where they are not refined.)
 // 1 / sqrt(pivot) is formed in integers too, by one lane, while the other warps update the
-// trailing rows (a chain of dependent FP64 instructions took several times as long).  A pivot below 2^-80 of its
-// column (kappa above about 2^40), zero or negative stops the factorisation; a column that
-// is zero altogether gives a zero row of R.
+// trailing rows (a chain of dependent FP64 instructions took several times as long).  A pivot below
+// 2^-min_bits of its column, zero or negative stops the factorisation; a column that is zero
+// altogether gives a zero row of R.  (What then happens is in xg_finish.)
 // ---------------------------------------------------------------------------------------
 constexpr int kFx = 125;
 
@@ -1279,8 +1283,10 @@ template <int NC, typename S>
 __global__ void __launch_bounds__(XgShape<NC>::T, 1)
     xgram_kernel(const __grid_constant__ GramArgs<S> a, const __grid_constant__ CUtensorMap map) {
   extern __shared__ __align__(1024) unsigned char smem_umma[];
-  // The workspace is cleared by the kernel before this one, which this one may overlap (X itself
-  // was complete before that kernel started): nothing in it is read or added to before pdl_wait.
+  // The kernel before this one, which this one may overlap, is an ordinary launch (so X was
+  // complete before it started) that clears the head of the workspace alone: nothing in the head,
+  // flags and integer accumulators, is touched before pdl_wait.  The CTA's own 128-bit sums (fbuf)
+  // are used before it; they must never be cleared there.
   pdl_release();
   const uint32_t tbase = xg_cta_begin<NC, S>(smem_umma);
   PipeBars bars;
